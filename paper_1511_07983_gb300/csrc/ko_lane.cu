@@ -79,6 +79,21 @@ __device__ __forceinline__ int nth_unused(uint32_t used, uint32_t all, unsigned 
     return __ffs((int)u) - 1;
 }
 
+// Store a simulation (its column and registers) as a node state.
+template <class SH, class SIM>
+__device__ __forceinline__ void save_node(const SIM &sim, uint32_t *node)
+{
+    uint4 *dst = reinterpret_cast<uint4 *>(node);
+#pragma unroll 13
+    for (int f = 0; f < SH::kWords / 4; f++)
+        __stcg(dst + f, make_uint4(sim.W(4 * f), sim.W(4 * f + 1), sim.W(4 * f + 2), sim.W(4 * f + 3)));
+    uint32_t r[kRegWords];
+    sim.regs_out(r);
+#pragma unroll
+    for (int f = 0; f < kRegWords / 4; f++)
+        __stcg(dst + SH::kWords / 4 + f, make_uint4(r[4 * f], r[4 * f + 1], r[4 * f + 2], r[4 * f + 3]));
+}
+
 enum Phase : int { PH_FETCH = 0, PH_NEXT, PH_START, PH_EVENT, PH_FINAL, PH_PLACED, PH_DONE };
 
 template <int T, class SH>
@@ -195,17 +210,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                         phase = PH_START;
                     }
                 } else {
-                    if (depth >= d0 && n - depth >= 2) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(slab + (depth - d0) * kSaveWords);
-#pragma unroll 13
-                        for (int f = 0; f < kWords / 4; f++)
-                            __stcg(dst + f, make_uint4(sim.W(4 * f), sim.W(4 * f + 1), sim.W(4 * f + 2), sim.W(4 * f + 3)));
-                        uint32_t r[kRegWords];
-                        sim.regs_out(r);
-#pragma unroll
-                        for (int f = 0; f < kRegWords / 4; f++)
-                            __stcg(dst + kWords / 4 + f, make_uint4(r[4 * f], r[4 * f + 1], r[4 * f + 2], r[4 * f + 3]));
-                    }
+                    if (depth >= d0 && n - depth >= 2) save_node<SH>(sim, slab + (depth - d0) * kSaveWords);
                     phase = PH_NEXT;
                 }
             }
@@ -269,6 +274,8 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                     depth = 0;
                     perm = 0;
                     sim.init();
+                    // an empty prefix: the root, to which the walk backs up, is a saved node too
+                    if (d0 == 0 && n >= 2) save_node<SH>(sim, slab);
                     phase = PH_NEXT;
                     break;
                 }

@@ -174,3 +174,25 @@ def test_partly_overflowing_sets_full_space(ko, seed, state):
     assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
         (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"])
     assert np.array_equal(hist, st["hist"])
+
+
+@pytest.mark.parametrize("state", STATES)
+def test_whole_space_items_beside_deeper_walks(ko, state):
+    """Sets whose single work item is their whole space (N - 1 <= saved levels,
+    an empty prefix) in one launch with larger sets: the walk backs up to the
+    root, whose node state shares the threads' slab with the other sets'."""
+    sets = [synth.gen_set("sets10", 40 + i, n=n) for i, n in enumerate([8, 7, 5, 5, 4, 4, 3, 3, 2, 1] * 6)]
+    gpus = [ko.Gpu.from_set(s).configure(lanes=1, levels=4, lane_state=state) for s in sets]
+    b = ko.Batch(gpus)
+    res, _ = b.run()
+    moved = b.fallback_items()
+    b.close()
+    for s, r in zip(sets, res):
+        h = oracle.heuristic(s.gpu, s.kernels)
+        st = oracle.exhaustive_stats(s.gpu, s.kernels, oracle.makespan(s.gpu, s.kernels, h),
+                                     makespans=oracle.makespans_idx(s.gpu, s.kernels, first=0,
+                                                                    count=math.factorial(s.n)))
+        assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
+            (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"]), s.n
+    # the largest state finishes these small GPUs' items itself (the smaller ones may hand some over)
+    assert state > 0 or moved == 0

@@ -137,9 +137,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                     if (slot < a.ov_cap) a.ov_list[slot] = rec;
                     phase = PH_FETCH;
                 } else if (last) {
-                    phase = PH_FINAL;
-                } else if (left == 0) {
-                    phase = PH_PLACED;
+                    phase = PH_FINAL;  // the queue empties only in place_partial
                 }
             }
         } else {
@@ -154,7 +152,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                     if (slot < a.ov_cap) a.ov_list[slot] = rec;
                     phase = PH_FETCH;
                 } else {
-                    phase = PH_PLACED;
+                    phase = left > 0 ? PH_EVENT : PH_PLACED;
                 }
             }
             __syncwarp();

@@ -1,26 +1,40 @@
 // One simulation per thread: the block-dispatch model (Sec. 2 dispatch rule,
-// durations fixed at burst end from the SM's SumC / SumM) advanced one event at
-// a time by a single thread, touching only the SMs an event changes.
+// durations fixed at burst end from the SM's SumC / SumM) advanced by a single
+// thread, one run of SMs at a time.
 //
-// State.  SMs with identical state form runs of consecutive SM indices, kept
-// in SM order (run j+1 starts where run j ends).  A run holds usage (registers,
-// blocks and warps packed in one word, shared memory, SumC, SumM), the earliest
-// end of its started groups, and a 64-bit mask of the slots it holds in a pool
-// of groups.  A group is the blocks of one kernel started in one burst on every
-// SM of a run (kernel, blocks per SM, end).  When a run splits, both halves
-// keep the groups already started, which then sit in both masks; a group that
-// is still pending (its burst is open) is copied to a new slot for the new
-// half, so each pending group has exactly one owner run, whose SumC / SumM
-// fixes its duration when the burst closes.
+// State.  SMs with identical state form a run of consecutive SM indices; the
+// runs themselves are kept in no particular order (a split appends the new run).
+// A run holds usage (registers, blocks and warps packed in one word, shared
+// memory, SumC, SumM), the earliest end of its groups, and a list of up to ten
+// 6-bit slot numbers into a pool of groups, sorted by end.  A group is the
+// blocks of one kernel started in one burst on every SM of a run (kernel,
+// blocks per SM, end).  When a run splits, both halves list the groups already
+// started; a group that is still pending (its burst is open) is copied to a
+// new slot for the new half, so each pending group has exactly one owner run,
+// whose SumC / SumM fixes its duration when the burst closes.
 //
-// Per event only the runs whose earliest end is the event time are touched:
-// their ending groups are released, and the head kernel is offered to exactly
-// those runs (every other run was full for it when the last burst ended).
-// Measured on the N=12 / 148-SM set: about 11 runs and 34 groups live, 1.3 runs
-// released and 1.3 groups started per event, a split every 15 events; the last
-// burst of an order can split up to 13 runs.  56 slots hold every group of
-// about 99 % of the 120-order work items; the rest move on to the run-length
-// passes.
+// Events.  Between a kernel's first and last burst the queue holds more blocks
+// than any event frees room for, so a run whose groups end takes its full
+// capacity whatever the other runs do: event() takes ONE run per call --
+// release, capacity, placement and durations of that run alone -- also when
+// several runs end at the same time (the rest wait in `todo`).  Only the burst
+// that would empty the queue needs all its runs together: event() then reports
+// the last burst, and place_partial() releases the runs still in `todo`, takes
+// back what the burst had placed and fills all of them jointly.  A step without
+// loops over runs keeps the 32 simulations of a warp in step.
+//
+// What bounds it: instruction issue at the lanes that are active (a warp's
+// threads wait for each other at the control step) and the latency of nine
+// warps per SM; it moves no data to speak of.  The loops over released runs
+// and their slots that an event step had before made a warp run as long as its
+// worst thread.  All 39.9M orders of an 11-kernel / 148-SM set: 470 ms with the
+// looping event step over ordered runs, 260 ms with this one; 3.6M orders of a
+// ten-kernel / 15-SM set 31.9 -> 22.6 ms.
+//
+// Measured on the N=12 / 148-SM set: about 11 runs and 34 groups live, 1.24
+// runs released per event, 34 events per order, a split every 15 events.  56
+// slots hold every group of about 99 % of the 120-order work items; the rest
+// move on to the run-length passes.
 //
 // Layout.  The state of one simulation is a column of kWords 32-bit words in
 // shared memory, word f of the thread's column at col[f * STRIDE]; with STRIDE
@@ -54,25 +68,25 @@ namespace kolane {
 // shared memory; a work item that needs more is handed on (see LaneSim).
 template <int RUNS, int POOL>
 struct Shape {
-    static_assert(RUNS <= 16 && POOL <= 64 && POOL % 2 == 0, "run and slot masks are 32 and 64 bits");
+    static_assert(RUNS <= 16 && POOL <= 62 && POOL % 2 == 0, "run masks are 32 bits; slot 63 marks an empty list entry");
     static constexpr int kRuns = RUNS;   // runs one simulation may hold
     static constexpr int kPool = POOL;   // group slots of one simulation
-    static constexpr unsigned long long kPoolAll = POOL == 64 ? ~0ull : ((1ull << POOL) - 1ull);
+    static constexpr unsigned long long kPoolAll = (1ull << POOL) - 1ull;
     static constexpr int W_RB = 0;                 // run: first SM | SM count << 16
     static constexpr int W_RU = W_RB + RUNS;       // run: registers | blocks << 19 | warps << 25 in use per SM
     static constexpr int W_RS = W_RU + RUNS;       // run: shared memory in use per SM
     static constexpr int W_RC = W_RS + RUNS;       // run: SumC
     static constexpr int W_RM = W_RC + RUNS;       // run: SumM
-    static constexpr int W_RE = W_RM + RUNS;       // run: earliest end of its started groups (where valid)
-    static constexpr int W_RG0 = W_RE + RUNS;      // run: pool slots 0..31 it holds
-    static constexpr int W_RG1 = W_RG0 + RUNS;     // run: pool slots 32..63
-    static constexpr int W_GE = W_RG1 + RUNS;      // slot: end (mod 2^32)
+    static constexpr int W_RE = W_RM + RUNS;       // run: earliest end of its listed groups (where it lists any)
+    static constexpr int W_L0 = W_RE + RUNS;       // run: its listed groups' slots in order of end, low word
+    static constexpr int W_L1 = W_L0 + RUNS;       // run: high word
+    static constexpr int W_GE = W_L1 + RUNS;       // slot: end (mod 2^32)
     static constexpr int W_GD = W_GE + POOL;       // slots 2w, 2w+1: 16-bit descriptors
     static constexpr int kWords = W_GD + POOL / 2; // 8 words per run, 1.5 per slot
-    static constexpr int kSaveWords = kWords + 12; // with the registers of a node state
+    static constexpr int kSaveWords = kWords + 8;  // with the registers of a node state
     static_assert(kWords % 4 == 0, "node states are copied in 16-byte pieces");
 };
-// The shapes the one-thread simulator is built for: 14 runs / 56 slots (200
+// The shapes the one-thread simulator is built for: 14 runs / 56 slots (196
 // words), 12 / 40 (156 words), 10 / 32 (128 words).
 using ShapeL = Shape<14, 56>;
 using ShapeM = Shape<12, 40>;
@@ -82,9 +96,12 @@ using ShapeS = Shape<10, 32>;
 constexpr uint32_t kDescKernel = 31u, kDescOwnerShift = 11;
 // Packed usage word: registers in bits 0-18, blocks 19-24, warps 25-31.
 constexpr uint32_t kRegMask = (1u << 19) - 1u;
+// Slot lists: ten 6-bit entries from bit 0 of a 64-bit word, 63 = none; bits 60-63 stay set.
+constexpr int kListBits = 6, kListLen = 10;
+constexpr uint32_t kNoSlot = 63u;
 
 // Registers saved with a node state (beside the column words).
-constexpr int kRegWords = 12;
+constexpr int kRegWords = 8;
 
 // The set's limits, per thread.
 struct Limits {
@@ -92,18 +109,6 @@ struct Limits {
     uint32_t ccap, mcap;
     int cshift, mshift;
 };
-
-// floor(x / d) for 0 <= x <= 2^24, d >= 1, clamped to 63: the quotient of
-// min(x, 63 d) estimated with a float reciprocal (error far below one unit at
-// that size) and corrected once by an exact integer check.
-KO_HD int quot63(int x, int d, float rcp)
-{
-    const int xc = x < d * 63 ? x : d * 63;
-    int q = (int)((float)xc * rcp);
-    if ((q + 1) * d <= xc) q++;
-    if (q * d > xc) q--;
-    return q;
-}
 
 KO_HD int ffs64(unsigned long long v)
 {
@@ -121,13 +126,13 @@ KO_HD int ffs32(uint32_t v)
     return __builtin_ffs((int)v) - 1;
 #endif
 }
-
-// Insert a copy of bit j at position j + 1 (bits above move up one).
-KO_HD uint32_t dup_bit(uint32_t x, int j)
+KO_HD int msb32(uint32_t v)  // index of the highest set bit, v != 0
 {
-    const uint32_t lo = x & ((2u << j) - 1u);
-    const uint32_t hi = (x >> (j + 1)) << (j + 2);
-    return lo | hi | (((x >> j) & 1u) << (j + 1));
+#ifdef __CUDA_ARCH__
+    return 31 - __clz((int)v);
+#else
+    return 31 - __builtin_clz(v);
+#endif
 }
 
 // Per-run 8-bit values (up to 16 runs) in two 64-bit words.
@@ -139,12 +144,6 @@ struct Bytes16 {
         const int sh = (j & 7) * 8;
         const unsigned long long m = ~(0xffull << sh), b = (unsigned long long)(v & 0xff) << sh;
         if (j < 8) lo = (lo & m) | b; else hi = (hi & m) | b;
-    }
-    // insert a copy of byte j at j + 1 (bytes above move up one)
-    KO_HD void dup(int j)
-    {
-        for (int i = 15; i > j + 1; i--) set(i, get(i - 1));
-        set(j + 1, get(j));
     }
 };
 
@@ -163,29 +162,41 @@ struct LaneSim {
     static constexpr int kRuns = SH::kRuns, kPool = SH::kPool, kWords = SH::kWords;
     static constexpr unsigned long long kPoolAll = SH::kPoolAll;
     static constexpr int W_RB = SH::W_RB, W_RU = SH::W_RU, W_RS = SH::W_RS, W_RC = SH::W_RC, W_RM = SH::W_RM,
-                         W_RE = SH::W_RE, W_RG0 = SH::W_RG0, W_RG1 = SH::W_RG1, W_GE = SH::W_GE, W_GD = SH::W_GD;
+                         W_RE = SH::W_RE, W_L0 = SH::W_L0, W_L1 = SH::W_L1, W_GE = SH::W_GE, W_GD = SH::W_GD;
     uint32_t *col;            // word f at col[f * STRIDE]
     KLoad kl;                 // kernel constants by id
     Limits L;
     unsigned long long t;     // clock
-    unsigned long long tmx;   // latest end given to any group so far
     unsigned long long freeg; // free pool slots
-    unsigned long long pend;  // slots started in the open burst
-    int p;                    // round-robin pointer (an SM index)
+    unsigned long long rel;   // slots released at t, free once every run ending at t is released
+    unsigned long long pend;  // slots started at t: not listed yet (burst open), or placed by event()
+    int p;                    // round-robin pointer (an SM index) when the burst began
     int nr;                   // runs
     int run_limit;
-    uint32_t rv;              // runs whose W_RE holds the earliest end of a started group
     int fail;
+    uint32_t fresh, todo;     // runs whose earliest end is t; those event() has not taken yet
+    int pmax, pbest;          // event()'s placements at t: largest capacity, and how far past p its
+                              // cyclically last SM lies (what the pointer moves by when t passes)
     // head kernel
     int hk, hr, hs, hw, hc, hm;
     uint32_t hpk;             // registers | 1 << 19 | warps << 25
-    float frr, frs, frw;      // reciprocals of registers, shared memory, warps
-    // the last offer: per-run caps, SM-weighted total, maximum, offered runs
+    float frr, frs, frw, fsb; // reciprocals of registers, shared memory, warps (rounded down)
+    // the last offer: per-run caps, SM-weighted total, maximum, runs that take blocks
     Bytes16 caps;
     int ctotal, cmax;
     uint32_t celig;
 
     KO_HD uint32_t &W(int f) const { return col[f * STRIDE]; }
+#ifdef __CUDA_ARCH__
+    KO_HD uint32_t gd(int g) const
+    {
+        return reinterpret_cast<const uint16_t *>(col + (W_GD + (g >> 1)) * STRIDE)[g & 1];
+    }
+    KO_HD void set_gd(int g, uint32_t v) const
+    {
+        reinterpret_cast<uint16_t *>(col + (W_GD + (g >> 1)) * STRIDE)[g & 1] = (uint16_t)v;
+    }
+#else
     KO_HD uint32_t gd(int g) const { return (W(W_GD + (g >> 1)) >> ((g & 1) * 16)) & 0xffffu; }
     KO_HD void set_gd(int g, uint32_t v) const
     {
@@ -193,28 +204,32 @@ struct LaneSim {
         const int sh = (g & 1) * 16;
         x = (x & ~(0xffffu << sh)) | (v << sh);
     }
-    KO_HD unsigned long long gmask(int j) const
+#endif
+    KO_HD unsigned long long list(int j) const
     {
-        return (unsigned long long)W(W_RG0 + j) | ((unsigned long long)W(W_RG1 + j) << 32);
+        return (unsigned long long)W(W_L0 + j) | ((unsigned long long)W(W_L1 + j) << 32);
     }
-    KO_HD void set_gmask(int j, unsigned long long m) const
+    KO_HD void set_list(int j, unsigned long long l) const
     {
-        W(W_RG0 + j) = (uint32_t)m;
-        W(W_RG1 + j) = (uint32_t)(m >> 32);
+        W(W_L0 + j) = (uint32_t)l;
+        W(W_L1 + j) = (uint32_t)(l >> 32);
     }
+    // the list without its first entry
+    KO_HD static unsigned long long pop(unsigned long long l) { return (l >> kListBits) | (0x3full << 58); }
 
     KO_HD void init()
     {
         W(W_RB) = (uint32_t)L.S << 16;
         W(W_RU) = 0; W(W_RS) = 0; W(W_RC) = 0; W(W_RM) = 0;
-        set_gmask(0, 0);
+        set_list(0, ~0ull);
         nr = 1;
         t = 0;
-        tmx = 0;
         p = 0;
         freeg = kPoolAll;
+        rel = 0;
         pend = 0;
-        rv = 0;
+        fresh = todo = 0;
+        pmax = pbest = 0;
         fail = 0;
     }
 
@@ -223,94 +238,127 @@ struct LaneSim {
         const KParam q = kl.full(k);
         hk = k; hr = q.r; hs = q.s; hw = q.w; hc = q.c; hm = q.m;
         hpk = (uint32_t)q.r | (1u << 19) | ((uint32_t)q.w << 25);
-        // quot63 corrects its estimate exactly, so an approximate reciprocal will do
+        // A quotient of at most 40 estimated with one of these lies within 1 below the true one and
+        // never above it: the reciprocal, the conversion and the product each err by less than 2^-21
+        // relative, and the factor takes 2^-18 off (cap() corrects the estimate exactly).
+        const float down = 1.0f - 1.0f / 262144.0f;
 #ifdef __CUDA_ARCH__
-        frr = __fdividef(1.0f, (float)q.r);
-        frw = __fdividef(1.0f, (float)q.w);
-        frs = q.s > 0 ? __fdividef(1.0f, (float)q.s) : 0.0f;
+        frr = __fdividef(down, (float)q.r);
+        frw = __fdividef(down, (float)q.w);
+        frs = q.s > 0 ? __fdividef(down, (float)q.s) : 0.0f;
 #else
-        frr = 1.0f / (float)q.r;
-        frw = 1.0f / (float)q.w;
-        frs = q.s > 0 ? 1.0f / (float)q.s : 0.0f;
+        frr = down / (float)q.r;
+        frw = down / (float)q.w;
+        frs = q.s > 0 ? down / (float)q.s : 0.0f;
 #endif
+        fsb = q.s > 0 ? 0.0f : 40.0f;  // no shared memory: that limit never binds
     }
 
-    // Blocks of the head kernel one SM of run j still takes.
-    KO_HD int cap(int j) const
+    // Blocks of the head kernel an SM with usage u / us still takes: the least
+    // quotient of free resources, estimated in floating point and raised by one
+    // where one block more fits all of them.  At most 32 (the block limit).
+    KO_HD int cap(uint32_t u, uint32_t us) const
     {
-        const uint32_t u = W(W_RU + j);
-        int c = L.Bk - (int)((u >> 19) & 63u);
-        const int qr = quot63(L.R - (int)(u & kRegMask), hr, frr);
-        const int qw = quot63(L.W - (int)(u >> 25), hw, frw);
-        c = qr < c ? qr : c;
-        c = qw < c ? qw : c;
-        if (hs > 0) {
-            const int qs = quot63(L.Sh - (int)W(W_RS + j), hs, frs);
-            c = qs < c ? qs : c;
+        const int xr = L.R - (int)(u & kRegMask), xw = L.W - (int)(u >> 25), xs = L.Sh - (int)us;
+        const int xb = L.Bk - (int)((u >> 19) & 63u);
+        float f = (float)xr * frr;
+        const float fw = (float)xw * frw, fs = (float)xs * frs + fsb;
+        f = fw < f ? fw : f;
+        f = fs < f ? fs : f;
+        f = f < 40.0f ? f : 40.0f;
+        int q = (int)f;
+        if ((q + 1) * hr <= xr && (q + 1) * hw <= xw && (q + 1) * hs <= xs) q++;
+        return q < xb ? q : xb;
+    }
+
+    KO_HD uint32_t duration(uint32_t c, uint32_t m, uint32_t sc, uint32_t sm) const
+    {
+        // every factor fits 32 bits (c, m <= 2^24; SumC, SumM < 2^30; caps <= 2^30), so each
+        // product is one 32 x 32 -> 64-bit multiply; every duration is below 2^31
+        const uint32_t scc = sc > L.ccap ? sc : L.ccap, smm = sm > L.mcap ? sm : L.mcap;
+        const unsigned long long pc = (unsigned long long)c * scc + (L.ccap - 1u);
+        const unsigned long long pm = (unsigned long long)m * smm + (L.mcap - 1u);
+        const uint32_t dc = (uint32_t)(L.cshift >= 0 ? pc >> L.cshift : pc / L.ccap);
+        const uint32_t dm = (uint32_t)(L.mshift >= 0 ? pm >> L.mshift : pm / L.mcap);
+        return dc > dm ? dc : dm;
+    }
+
+    // Insert slot g, which ends at t + dur, into list l in order of end (after
+    // equal ends); `first` tells whether it became the earliest.  Ends are read
+    // four at a time, so the loads of a turn overlap.
+    KO_HD unsigned long long insert(unsigned long long l, int g, uint32_t dur, bool &first)
+    {
+        const uint32_t t32 = (uint32_t)t;
+        if (((l >> (kListBits * (kListLen - 1))) & 63u) != kNoSlot) { fail = 1; return l; }
+        int pos = 0;
+        unsigned long long rest = l;
+        for (;;) {
+            int in = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+            for (int i = 0; i < 4; i++) {
+                const uint32_t s = (uint32_t)(rest >> (kListBits * i)) & 63u;
+                const uint32_t e = W(W_GE + (int)(s < (uint32_t)kPool ? s : 0u)) - t32;
+                in += (s != kNoSlot && e <= dur) ? 1 : 0;
+            }
+            pos += in;
+            if (in < 4) break;
+            rest = (rest >> (4 * kListBits)) | (~0ull << (64 - 4 * kListBits));
         }
-        return c > 0 ? c : 0;
+        first = pos == 0;
+        const unsigned long long below = (1ull << (kListBits * pos)) - 1ull;
+        return (l & below) | ((unsigned long long)g << (kListBits * pos)) | ((l & ~below) << kListBits) | (0xfull << 60);
+    }
+
+    // Take the free slot for q blocks per SM of the head kernel on run j.
+    KO_HD int take_slot(int j, int q)
+    {
+        const int g = ffs64(freeg);
+        freeg &= freeg - 1;
+        pend |= 1ull << g;
+        set_gd(g, (uint32_t)hk | ((uint32_t)(q - 1) << 5) | ((uint32_t)j << kDescOwnerShift));
+        return g;
     }
 
     // Start q blocks per SM of the head kernel on run j as a new pending group.
     KO_HD void add_group(int j, int q)
     {
         if (freeg == 0) { fail = 1; return; }
-        const int g = ffs64(freeg);
-        freeg &= freeg - 1;
-        pend |= 1ull << g;
-        set_gd(g, (uint32_t)hk | ((uint32_t)(q - 1) << 5) | ((uint32_t)j << kDescOwnerShift));
-        set_gmask(j, gmask(j) | (1ull << g));
+        take_slot(j, q);
         W(W_RU + j) += (uint32_t)q * hpk;
         W(W_RS + j) += (uint32_t)(q * hs);
         W(W_RC + j) += (uint32_t)(q * hc);
         W(W_RM + j) += (uint32_t)(q * hm);
     }
 
-    // Split run j after x SMs (0 < x < its count): run j keeps the first x, a
-    // new run j+1 takes the rest; runs above move up one.  The caller's
-    // per-run registers (bit masks, caps) are shifted by the caller.
+    // Split run j after x SMs (0 < x < its count): run j keeps the first x, the
+    // new run `nr` takes the rest.
     KO_HD bool split(int j, int x)
     {
         if (nr >= run_limit) { fail = 1; return false; }
-        for (int i = nr - 1; i > j; i--) {
-            W(W_RB + i + 1) = W(W_RB + i);
-            W(W_RU + i + 1) = W(W_RU + i);
-            W(W_RS + i + 1) = W(W_RS + i);
-            W(W_RC + i + 1) = W(W_RC + i);
-            W(W_RM + i + 1) = W(W_RM + i);
-            W(W_RE + i + 1) = W(W_RE + i);
-            W(W_RG0 + i + 1) = W(W_RG0 + i);
-            W(W_RG1 + i + 1) = W(W_RG1 + i);
-        }
+        const int k = nr++;
         const uint32_t rb = W(W_RB + j);
         const uint32_t beg = rb & 0xffffu, cnt = rb >> 16;
         W(W_RB + j) = beg | ((uint32_t)x << 16);
-        W(W_RB + j + 1) = (beg + (uint32_t)x) | ((cnt - (uint32_t)x) << 16);
-        W(W_RU + j + 1) = W(W_RU + j);
-        W(W_RS + j + 1) = W(W_RS + j);
-        W(W_RC + j + 1) = W(W_RC + j);
-        W(W_RM + j + 1) = W(W_RM + j);
-        W(W_RE + j + 1) = W(W_RE + j);
-        rv = dup_bit(rv, j);
-        nr++;
-        // pending groups owned by runs above j move up with their runs
-        for (unsigned long long pm = pend; pm; pm &= pm - 1) {
-            const int g = ffs64(pm);
-            const uint32_t d = gd(g);
-            if ((int)(d >> kDescOwnerShift) > j) set_gd(g, d + (1u << kDescOwnerShift));
-        }
+        W(W_RB + k) = (beg + (uint32_t)x) | ((cnt - (uint32_t)x) << 16);
+        W(W_RU + k) = W(W_RU + j);
+        W(W_RS + k) = W(W_RS + j);
+        W(W_RC + k) = W(W_RC + j);
+        W(W_RM + k) = W(W_RM + j);
+        W(W_RE + k) = W(W_RE + j);
+        W(W_L0 + k) = W(W_L0 + j);
+        W(W_L1 + k) = W(W_L1 + j);
         // run j's pending groups: the new run gets its own copies
-        unsigned long long m1 = gmask(j);
-        for (unsigned long long pm = m1 & pend; pm; pm &= pm - 1) {
-            const int g = ffs64(pm);
+        for (unsigned long long pm = pend; pm; pm &= pm - 1) {
+            const uint32_t d = gd(ffs64(pm));
+            if ((int)(d >> kDescOwnerShift) != j) continue;
             if (freeg == 0) { fail = 1; return false; }
             const int g2 = ffs64(freeg);
             freeg &= freeg - 1;
             pend |= 1ull << g2;
-            set_gd(g2, (gd(g) & ((1u << kDescOwnerShift) - 1u)) | ((uint32_t)(j + 1) << kDescOwnerShift));
-            m1 = (m1 & ~(1ull << g)) | (1ull << g2);
+            set_gd(g2, (d & ((1u << kDescOwnerShift) - 1u)) | ((uint32_t)k << kDescOwnerShift));
         }
-        set_gmask(j + 1, m1);
         return true;
     }
 
@@ -321,26 +369,40 @@ struct LaneSim {
         caps.lo = caps.hi = 0ull;
         ctotal = 0;
         cmax = 0;
-        celig = elig;
         // runs with room for one block (four compares) take the exact capacity
         uint32_t room = 0;
-        for (uint32_t e = elig; e; e &= e - 1) {
-            const int j = ffs32(e);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int j = 0; j < kRuns; j++) {
+            if (!((elig >> j) & 1u)) continue;
             const uint32_t u = W(W_RU + j);
             const bool fits = (int)((u >> 19) & 63u) < L.Bk && (int)(u & kRegMask) + hr <= L.R &&
                               (int)(u >> 25) + hw <= L.W && (int)W(W_RS + j) + hs <= L.Sh;
             room |= (fits ? 1u : 0u) << j;
         }
-        uint32_t take = 0;
         for (uint32_t e = room; e; e &= e - 1) {
             const int j = ffs32(e);
-            const int c = cap(j);
+            const int c = cap(W(W_RU + j), W(W_RS + j));
             caps.set(j, c);
             ctotal += (int)(W(W_RB + j) >> 16) * c;
             cmax = c > cmax ? c : cmax;
-            take |= (c > 0 ? 1u : 0u) << j;
         }
-        celig = take;  // the placement steps visit only runs that take blocks
+        celig = room;  // the placement steps visit only runs that take blocks
+    }
+
+    // How far past p (in SMs, cyclically) the last SM of the run rb lies, 1..S.
+    KO_HD int last_past(uint32_t rb) const
+    {
+        const int b = (int)(rb & 0xffffu), d = b + (int)(rb >> 16) - p;
+        if (b < p && d > 0) return L.S;  // p lies inside: its last SM from p on is p - 1
+        return d <= 0 ? d + L.S : d;
+    }
+
+    KO_HD void move_pointer(int by)
+    {
+        p += by;
+        if (p >= L.S) p -= L.S;
     }
 
     // Every SM of the offered runs takes its full capacity (ctotal <= left);
@@ -348,33 +410,24 @@ struct LaneSim {
     // cyclically from p.
     KO_HD void place_full(int &left)
     {
-        const int S = L.S;
-        const int pm1 = p == 0 ? S - 1 : p - 1;
         int best = 0;
         for (uint32_t e = celig; e; e &= e - 1) {
             const int j = ffs32(e);
             const int c = caps.get(j);
-            if (c == 0) continue;
             add_group(j, c);
             if (c == cmax) {
-                const uint32_t rb = W(W_RB + j);
-                const int b = (int)(rb & 0xffffu), n = (int)(rb >> 16);
-                int pos;
-                if (pm1 >= b && pm1 < b + n) pos = S;
-                else { pos = b + n - p; if (pos <= 0) pos += S; }
+                const int pos = last_past(W(W_RB + j));
                 best = pos > best ? pos : best;
             }
         }
-        p += best;
-        if (p >= S) p -= S;
+        move_pointer(best);
         left -= ctotal;
     }
 
     // The offered runs hold more room than `left` blocks (ctotal > left): the
     // water-fill stops inside a sweep, cutting runs at p and where it stops.
-    KO_HD void place_partial(int &left)
+    KO_HD void water_fill(int &left)
     {
-        const int S = L.S;
         uint32_t elig = celig;
         // smallest sweep count L with F(L) = sum cnt * min(cap, L) >= left
         int lo = 1, hi = cmax;
@@ -390,110 +443,123 @@ struct LaneSim {
         }
         const int Lsw = lo;
         int filled = 0;
+        uint32_t last = 0;  // runs whose SMs can take a block in the last sweep
         for (uint32_t e = elig; e; e &= e - 1) {
             const int j = ffs32(e);
             const int c = caps.get(j);
             filled += (int)(W(W_RB + j) >> 16) * (c < Lsw - 1 ? c : Lsw - 1);
+            last |= (c >= Lsw ? 1u : 0u) << j;
         }
         const int rem = left - filled;  // 1 .. number of SMs with cap >= Lsw
-        // the run holding p; cut it at p when its SMs take a block in the last sweep
-        int jp = 0;
-        for (int j = 0; j < nr; j++) {
+        // cut the run that holds p at p when its SMs can take a block in the last sweep
+        for (uint32_t e = last; e; e &= e - 1) {
+            const int j = ffs32(e);
             const uint32_t rb = W(W_RB + j);
             const int b = (int)(rb & 0xffffu), n = (int)(rb >> 16);
-            if (b <= p && p < b + n) jp = j;
-        }
-        uint32_t plus = 0;
-        {
-            const uint32_t rb = W(W_RB + jp);
-            const int b = (int)(rb & 0xffffu);
-            if (((elig >> jp) & 1u) && caps.get(jp) >= Lsw && b < p) {
-                if (!split(jp, p - b)) return;
-                elig = dup_bit(elig, jp);
-                caps.dup(jp);
-                jp++;
+            if (b < p && p < b + n) {
+                if (!split(j, p - b)) return;
+                caps.set(nr - 1, caps.get(j));
+                elig |= 1u << (nr - 1);
+                last |= 1u << (nr - 1);
+                break;
             }
         }
-        // walk the runs cyclically from jp, one more block to each SM with cap >= Lsw
-        int acc = 0, newp = p, j = jp;
-        for (int it = 0; it < nr; it++, j = j + 1 == nr ? 0 : j + 1) {
-            if (!((elig >> j) & 1u) || caps.get(j) < Lsw) continue;
+        // visit those runs cyclically from p, one more block to each of their SMs
+        uint32_t plus = 0;
+        int acc = 0, newp = p;
+        while (last) {
+            int j = 0, best = 0x7fffffff;
+            for (uint32_t e = last; e; e &= e - 1) {
+                const int i = ffs32(e);
+                int d = (int)(W(W_RB + i) & 0xffffu) - p;
+                if (d < 0) d += L.S;
+                if (d < best) { best = d; j = i; }
+            }
+            last &= ~(1u << j);
+            plus |= 1u << j;
             const uint32_t rb = W(W_RB + j);
-            const int b = (int)(rb & 0xffffu), n = (int)(rb >> 16);
+            const int n = (int)(rb >> 16);
             if (acc + n >= rem) {
                 const int x = rem - acc;
                 if (x < n) {
                     if (!split(j, x)) return;
-                    elig = dup_bit(elig, j);
-                    plus = dup_bit(plus, j) & ~(1u << (j + 1));
-                    caps.dup(j);
+                    caps.set(nr - 1, caps.get(j));
+                    elig |= 1u << (nr - 1);
                 }
-                plus |= 1u << j;
-                newp = b + x;
+                newp = (int)(rb & 0xffffu) + x;
                 break;
             }
             acc += n;
-            plus |= 1u << j;
         }
-        p = newp >= S ? newp - S : newp;
+        p = newp >= L.S ? newp - L.S : newp;
         for (uint32_t e = elig; e; e &= e - 1) {
-            const int jj = ffs32(e);
-            const int c = caps.get(jj);
-            const int q = (c < Lsw - 1 ? c : Lsw - 1) + (int)((plus >> jj) & 1u);
-            if (q > 0) add_group(jj, q);
+            const int j = ffs32(e);
+            const int c = caps.get(j);
+            const int q = (c < Lsw - 1 ? c : Lsw - 1) + (int)((plus >> j) & 1u);
+            if (q > 0) add_group(j, q);
         }
         left = 0;
     }
 
-    // One dispatch burst of the head kernel with `left` blocks queued over the
-    // runs in `elig`.
-    KO_HD void burst(int &left, uint32_t elig)
+    // A run's state while event() or place_partial() works on it.
+    struct RunState {
+        uint32_t u, s, c, m, re;
+        unsigned long long l;
+    };
+
+    // Release the groups of run j that end at t.
+    KO_HD RunState release(int j)
     {
-        offer(elig);
-        if (ctotal == 0) return;
-        if (ctotal <= left) place_full(left);
-        else place_partial(left);
+        const uint32_t now = (uint32_t)t;
+        RunState r{W(W_RU + j), W(W_RS + j), W(W_RC + j), W(W_RM + j), 0u, list(j)};
+        for (;;) {
+            const uint32_t s0 = (uint32_t)r.l & 63u;
+            const int g = (int)(s0 < (uint32_t)kPool ? s0 : 0u);  // a run released here lists a group
+            const uint32_t d = gd(g);
+            const KRel q = kl.rel((int)(d & kDescKernel));
+            r.l = pop(r.l);
+            const uint32_t nx = (uint32_t)r.l & 63u;
+            const bool more = nx != kNoSlot;
+            r.re = W(W_GE + (int)(more ? nx : 0u));
+            const uint32_t nb = ((d >> 5) & 63u) + 1u;
+            r.u -= nb * q.pk;
+            r.s -= nb * q.s;
+            r.c -= nb * q.c;
+            r.m -= nb * q.m;
+            rel |= 1ull << g;
+            if (!more || r.re != now) break;
+        }
+        return r;
     }
 
-    KO_HD uint32_t duration(int k, uint32_t sc, uint32_t sm) const
+    KO_HD void store(int j, const RunState &r) const
     {
-        // every factor fits 32 bits (c, m <= 2^24; SumC, SumM < 2^30; caps <= 2^30), so each
-        // product is one 32 x 32 -> 64-bit multiply
-        const KRel q = kl.rel(k);
-        const uint32_t scc = sc > L.ccap ? sc : L.ccap, smm = sm > L.mcap ? sm : L.mcap;
-        const unsigned long long pc = (unsigned long long)(uint32_t)q.c * scc + (L.ccap - 1u);
-        const unsigned long long pmm = (unsigned long long)(uint32_t)q.m * smm + (L.mcap - 1u);
-        const unsigned long long dc = L.cshift >= 0 ? pc >> L.cshift : pc / L.ccap;
-        const unsigned long long dm = L.mshift >= 0 ? pmm >> L.mshift : pmm / L.mcap;
-        return (uint32_t)(dc > dm ? dc : dm);
+        W(W_RU + j) = r.u; W(W_RS + j) = r.s; W(W_RC + j) = r.c; W(W_RM + j) = r.m;
+        W(W_RE + j) = r.re;
+        set_list(j, r.l);
     }
 
-    // Fix the durations of the groups started in the open burst.
+    // Fix the durations of the pending groups and list them.
     KO_HD void close_burst()
     {
-        const uint32_t t32 = (uint32_t)t;
         for (unsigned long long pm = pend; pm; pm &= pm - 1) {
             const int g = ffs64(pm);
             const uint32_t d = gd(g);
             const int j = (int)(d >> kDescOwnerShift);
-            const uint32_t dur = duration((int)(d & kDescKernel), W(W_RC + j), W(W_RM + j));
-            const uint32_t e = t32 + dur;
-            W(W_GE + g) = e;
-            tmx = t + dur > tmx ? t + dur : tmx;
-            if ((rv >> j) & 1u) {
-                const uint32_t re = W(W_RE + j);
-                if (e - t32 < re - t32) W(W_RE + j) = e;
-            } else {
-                W(W_RE + j) = e;
-                rv |= 1u << j;
-            }
+            const KRel q = kl.rel((int)(d & kDescKernel));
+            const uint32_t dur = duration(q.c, q.m, W(W_RC + j), W(W_RM + j));
+            W(W_GE + g) = (uint32_t)t + dur;
+            bool first = false;
+            set_list(j, insert(list(j), g, dur, first));
+            if (first) W(W_RE + j) = (uint32_t)t + dur;
         }
         pend = 0;
     }
 
-    // Jump to the earliest end and release every group ending then; returns
-    // the runs that released blocks (the only ones with room for the head).
-    KO_HD uint32_t advance()
+    // Jump to the earliest end of a run.  While blocks are queued and the burst
+    // is closed every run lists a group (an empty SM takes a block of any
+    // kernel), so every run's earliest end is valid.
+    KO_HD void advance()
     {
         const uint32_t t32 = (uint32_t)t;
         uint32_t e[kRuns];
@@ -502,53 +568,23 @@ struct LaneSim {
 #pragma unroll
 #endif
         for (int j = 0; j < kRuns; j++) {
-            e[j] = 0;
-            if ((rv >> j) & 1u) {
-                e[j] = W(W_RE + j);
-                const uint32_t d = e[j] - t32;
-                dmin = d < dmin ? d : dmin;
-            }
+            e[j] = 0xffffffffu;
+            if (j < nr) e[j] = W(W_RE + j) - t32;
+            dmin = e[j] < dmin ? e[j] : dmin;
         }
-        if (dmin == 0xffffffffu) { fail = 1; return 0; }
-        t += dmin;
-        const uint32_t now = t32 + dmin;
-        uint32_t fresh = 0;
+        fresh = 0;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
         for (int j = 0; j < kRuns; j++)
-            if (((rv >> j) & 1u) && e[j] == now) fresh |= 1u << j;
-        unsigned long long rel = 0;
-        for (uint32_t f = fresh; f; f &= f - 1) {
-            const int j = ffs32(f);
-            const unsigned long long m = gmask(j);
-            // which of the run's groups end now, and the earliest end of the rest
-            unsigned long long gone = 0;
-            uint32_t nm = 0xffffffffu;
-            for (unsigned long long mm = m; mm; mm &= mm - 1) {
-                const int g = ffs64(mm);
-                const uint32_t dd = W(W_GE + g) - now;
-                if (dd == 0) gone |= 1ull << g;
-                else nm = dd < nm ? dd : nm;
-            }
-            uint32_t u = W(W_RU + j), us = W(W_RS + j), sc = W(W_RC + j), sm = W(W_RM + j);
-            for (unsigned long long mm = gone; mm; mm &= mm - 1) {
-                const uint32_t d = gd(ffs64(mm));
-                const KRel q = kl.rel((int)(d & kDescKernel));
-                const uint32_t nb = ((d >> 5) & 63u) + 1u;
-                u -= nb * q.pk;
-                us -= nb * q.s;
-                sc -= nb * q.c;
-                sm -= nb * q.m;
-            }
-            set_gmask(j, m & ~gone);
-            W(W_RU + j) = u; W(W_RS + j) = us; W(W_RC + j) = sc; W(W_RM + j) = sm;
-            if (nm != 0xffffffffu) W(W_RE + j) = now + nm;
-            else rv &= ~(1u << j);
-            rel |= gone;
-        }
+            if (e[j] == dmin) fresh |= 1u << j;
+        t += dmin;
+        todo = fresh;
         freeg |= rel;
-        return fresh;
+        rel = 0;
+        pend = 0;
+        move_pointer(pbest);
+        pmax = pbest = 0;
     }
 
     // Queue all blocks of kernel k behind the current queue: the first burst
@@ -557,55 +593,144 @@ struct LaneSim {
     {
         set_head(k);
         int left = kl.full(k).b;
-        burst(left, (nr >= 32 ? 0xffffffffu : ((1u << nr) - 1u)));
+        offer((1u << nr) - 1u);
+        if (ctotal > left) water_fill(left);
+        else if (ctotal > 0) place_full(left);
         return left;
     }
 
-    // One event while the head kernel still has queued blocks: close the open
-    // burst, advance to the next end, release, and place the head kernel where
-    // every offered SM takes its full capacity.  Returns true when the offered
-    // room exceeds the queue instead; the caller then finishes the burst with
-    // place_partial (the kernel's last burst).  `mask`: the threads of the warp
-    // that run this event step together; they reconverge after each stage.
+    // One run's event while the head kernel has queued blocks and the burst is
+    // closed: release what ends, place the head kernel's full capacity and list
+    // the new group.  Returns true, with nothing placed on this run, when that
+    // would empty the queue: the caller finishes the burst with place_partial.
+    // `mask`: the threads of the warp that run this step together; they
+    // reconverge after each stage.
     KO_HD bool event(int &left, unsigned mask)
     {
-        close_burst();
+        if (todo == 0) advance();
         KO_RECONVERGE(mask);
-        const uint32_t fresh = advance();
+        const int j = ffs32(todo);
+        todo &= todo - 1;
+        RunState r = release(j);
         KO_RECONVERGE(mask);
-        offer(fail ? 0u : fresh);  // a failed simulation still reaches every reconvergence point
-        KO_RECONVERGE(mask);
-        if (fail || ctotal == 0) return false;
-        if (ctotal <= left) {
-            place_full(left);
-            return false;
+        if (todo == 0) {  // every holder of the slots released at t has let go
+            freeg |= rel;
+            rel = 0;
         }
-        return true;
+        const int q = cap(r.u, r.s);
+        const uint32_t rb = W(W_RB + j);
+        const int take = q * (int)(rb >> 16);
+        const bool last = take >= left && take > 0;
+        if (take > 0 && !last) {
+            if (freeg == 0) fail = 1;
+            else {
+                const int g = take_slot(j, q);
+                r.u += (uint32_t)q * hpk;
+                r.s += (uint32_t)(q * hs);
+                r.c += (uint32_t)(q * hc);
+                r.m += (uint32_t)(q * hm);
+                const uint32_t dur = duration((uint32_t)hc, (uint32_t)hm, r.c, r.m);
+                W(W_GE + g) = (uint32_t)t + dur;
+                bool first = false;
+                r.l = insert(r.l, g, dur, first);
+                if (first) r.re = (uint32_t)t + dur;
+                left -= take;
+                const int pos = last_past(rb);
+                pbest = q > pmax ? pos : (q == pmax && pos > pbest ? pos : pbest);
+                pmax = q > pmax ? q : pmax;
+            }
+        }
+        KO_RECONVERGE(mask);
+        store(j, r);
+        return last && !fail;
     }
 
-    // Close the final burst; the makespan is the latest end of any group.
+    // The burst in which event() reported that the queue would empty: release
+    // the runs it has not taken, take back what it placed, and fill the runs
+    // that ended at t jointly.  The burst stays open unless blocks are left.
+    KO_HD void place_partial(int &left)
+    {
+        for (; todo; todo &= todo - 1) {
+            const int j = ffs32(todo);
+            store(j, release(j));
+        }
+        freeg |= rel;
+        rel = 0;
+        for (; pend; pend &= pend - 1) {
+            const int g = ffs64(pend);
+            const uint32_t d = gd(g), q = ((d >> 5) & 63u) + 1u;
+            const int j = (int)(d >> kDescOwnerShift);
+            W(W_RU + j) -= q * hpk;
+            W(W_RS + j) -= q * (uint32_t)hs;
+            W(W_RC + j) -= q * (uint32_t)hc;
+            W(W_RM + j) -= q * (uint32_t)hm;
+            left += (int)q * (int)(W(W_RB + j) >> 16);
+            freeg |= 1ull << g;
+            // out of the list
+            const unsigned long long all = list(j);
+            int at = 0;
+            while (at < kListLen && ((uint32_t)(all >> (kListBits * at)) & 63u) != (uint32_t)g) at++;
+            const unsigned long long keep = (1ull << (kListBits * at)) - 1ull;
+            const unsigned long long nl = (all & keep) | (pop(all) & ~keep);
+            set_list(j, nl);
+            const uint32_t head = (uint32_t)nl & 63u;
+            if (head != kNoSlot) W(W_RE + j) = W(W_GE + (int)head);
+        }
+        pmax = pbest = 0;
+        offer(fresh);
+        if (ctotal > left) water_fill(left);
+        else place_full(left);
+        if (left > 0) close_burst();
+    }
+
+    // The makespan: the latest end of any group, the pending ones' included
+    // (groups that have left ended by t).
     KO_HD long long finish()
     {
-        close_burst();
-        return (long long)tmx;
+        const uint32_t t32 = (uint32_t)t;
+        uint32_t d = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int j = 0; j < kRuns; j++) {
+            if (j < nr) {
+                const unsigned long long none = ~list(j) & ((1ull << 60) - 1ull);  // zero entries are empty
+                if (none) {
+                    const uint32_t hi = (uint32_t)(none >> 32), lo = (uint32_t)none;
+                    const int bit = hi ? 32 + msb32(hi) : msb32(lo);
+                    const int g = (int)((list(j) >> (bit / kListBits * kListBits)) & 63u);
+                    const uint32_t e = W(W_GE + g) - t32;
+                    d = e > d ? e : d;
+                }
+            }
+        }
+        for (unsigned long long pm = pend; pm; pm &= pm - 1) {
+            const uint32_t w = gd(ffs64(pm));
+            const int j = (int)(w >> kDescOwnerShift);
+            const KRel q = kl.rel((int)(w & kDescKernel));
+            const uint32_t e = duration(q.c, q.m, W(W_RC + j), W(W_RM + j));
+            d = e > d ? e : d;
+        }
+        return (long long)(t + d);
     }
 
-    // Registers of a node state.
+    // Registers of a node state (the queue is empty, the burst open).
     KO_HD void regs_out(uint32_t *r) const
     {
         r[0] = (uint32_t)t; r[1] = (uint32_t)(t >> 32);
         r[2] = (uint32_t)freeg; r[3] = (uint32_t)(freeg >> 32);
         r[4] = (uint32_t)pend; r[5] = (uint32_t)(pend >> 32);
-        r[6] = (uint32_t)p; r[7] = (uint32_t)nr; r[8] = rv;
-        r[9] = (uint32_t)tmx; r[10] = (uint32_t)(tmx >> 32); r[11] = 0;
+        r[6] = (uint32_t)p; r[7] = (uint32_t)nr;
     }
     KO_HD void regs_in(const uint32_t *r)
     {
         t = (unsigned long long)r[0] | ((unsigned long long)r[1] << 32);
         freeg = (unsigned long long)r[2] | ((unsigned long long)r[3] << 32);
         pend = (unsigned long long)r[4] | ((unsigned long long)r[5] << 32);
-        p = (int)r[6]; nr = (int)r[7]; rv = r[8];
-        tmx = (unsigned long long)r[9] | ((unsigned long long)r[10] << 32);
+        p = (int)r[6]; nr = (int)r[7];
+        rel = 0;
+        fresh = todo = 0;
+        pmax = pbest = 0;
         fail = 0;
     }
 };

@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
         if (!control) {
             if (phase == PH_EVENT) {
                 const bool last = sim.event(left, busy);
-                if (!sim.fail && ++events > total_blocks + 64) sim.fail = 1;  // each event frees >= 1 block
+                // a step frees a block, or takes one of the first burst's runs or pending groups
+                if (!sim.fail && ++events > total_blocks + 256) sim.fail = 1;
                 if (sim.fail) {
                     const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
                     if (slot < a.ov_cap) a.ov_list[slot] = rec;
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                     if (slot < a.ov_cap) a.ov_list[slot] = rec;
                     phase = PH_FETCH;
                 } else {
-                    phase = left > 0 ? PH_EVENT : PH_PLACED;
+                    phase = PH_PLACED;
                 }
             }
             __syncwarp();
@@ -298,18 +299,9 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
             }
             __syncwarp();
             if (phase == PH_START) {  // one call site for every kernel start
-                left = sim.start_kernel(cand);
-                // blocks still queued: the start burst has ended, so its durations are fixed
-                // here, together, rather than by the first event of each thread
-                if (left > 0) sim.close_burst();
+                left = sim.begin_kernel(cand);
                 events = 0;
-                if (sim.fail) {
-                    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                    if (slot < a.ov_cap) a.ov_list[slot] = rec;
-                    phase = PH_FETCH;
-                } else {
-                    phase = left > 0 ? PH_EVENT : PH_PLACED;
-                }
+                phase = PH_EVENT;
             }
         }
         if (!__any_sync(kAll, phase != PH_DONE)) break;

@@ -72,7 +72,7 @@ struct Shape {
     static constexpr int kRuns = RUNS;   // runs one simulation may hold
     static constexpr int kPool = POOL;   // group slots of one simulation
     static constexpr unsigned long long kPoolAll = (1ull << POOL) - 1ull;
-    static constexpr int W_RB = 0;                 // run: first SM | SM count << 16
+    static constexpr int W_RB = 0;                 // run: first SM | SM count << 11 | capacity at the last offer << 22
     static constexpr int W_RU = W_RB + RUNS;       // run: registers | blocks << 19 | warps << 25 in use per SM
     static constexpr int W_RS = W_RU + RUNS;       // run: shared memory in use per SM
     static constexpr int W_RC = W_RS + RUNS;       // run: SumC
@@ -100,8 +100,23 @@ constexpr uint32_t kRegMask = (1u << 19) - 1u;
 constexpr int kListBits = 6, kListLen = 10;
 constexpr uint32_t kNoSlot = 63u;
 
+// Run word: N_SM <= 1024, so a first SM and a count take 11 bits each.
+constexpr uint32_t kSmMask = 0x7ffu;
+constexpr int kCntShift = 11, kCapShift = 22;
+constexpr uint32_t kSpanMask = (1u << kCapShift) - 1u;
+
 // Registers saved with a node state (beside the column words).
 constexpr int kRegWords = 8;
+
+// a / b for capacities that are no power of two; one copy of the long division.
+#ifdef __CUDACC__
+static __host__ __device__ __noinline__ uint32_t quotient(unsigned long long a, uint32_t b)
+#else
+static inline uint32_t quotient(unsigned long long a, uint32_t b)
+#endif
+{
+    return (uint32_t)(a / b);
+}
 
 // The set's limits, per thread.
 struct Limits {
@@ -126,26 +141,6 @@ KO_HD int ffs32(uint32_t v)
     return __builtin_ffs((int)v) - 1;
 #endif
 }
-KO_HD int msb32(uint32_t v)  // index of the highest set bit, v != 0
-{
-#ifdef __CUDA_ARCH__
-    return 31 - __clz((int)v);
-#else
-    return 31 - __builtin_clz(v);
-#endif
-}
-
-// Per-run 8-bit values (up to 16 runs) in two 64-bit words.
-struct Bytes16 {
-    unsigned long long lo, hi;
-    KO_HD int get(int j) const { return (int)(((j < 8 ? lo : hi) >> ((j & 7) * 8)) & 0xffu); }
-    KO_HD void set(int j, int v)
-    {
-        const int sh = (j & 7) * 8;
-        const unsigned long long m = ~(0xffull << sh), b = (unsigned long long)(v & 0xff) << sh;
-        if (j < 8) lo = (lo & m) | b; else hi = (hi & m) | b;
-    }
-};
 
 // Kernel constants a simulation looks up by kernel id: all of them, and the
 // packed record the release and duration steps read (one 16-byte load).
@@ -166,25 +161,25 @@ struct LaneSim {
     uint32_t *col;            // word f at col[f * STRIDE]
     KLoad kl;                 // kernel constants by id
     Limits L;
-    unsigned long long t;     // clock
-    unsigned long long freeg; // free pool slots
-    unsigned long long rel;   // slots released at t, free once every run ending at t is released
-    unsigned long long pend;  // slots started at t: not listed yet (burst open), or placed by event()
-    int p;                    // round-robin pointer (an SM index) when the burst began
-    int nr;                   // runs
+    unsigned long long t;      // clock
+    unsigned long long freeg;  // free pool slots
+    unsigned long long rel;    // slots released at t, free once every run ending at t is released
+    unsigned long long pend;   // slots of groups started at t that are not listed yet (burst open)
+    unsigned long long placed; // slots event() started and listed in this burst, for the head kernel
+    int p;                     // round-robin pointer (an SM index) when the burst began
+    int nr;                    // runs
     int run_limit;
     int fail;
-    uint32_t fresh, todo;     // runs whose earliest end is t; those event() has not taken yet
-    int pmax, pbest;          // event()'s placements at t: largest capacity, and how far past p its
-                              // cyclically last SM lies (what the pointer moves by when t passes)
+    uint32_t fresh, todo;      // runs the burst offers the head kernel; those event() has not taken yet
+    int ends;                  // the runs in `fresh` have groups ending at t (0: the kernel's first burst)
+    int drain;                 // the burst empties the queue: runs in `todo` are released, not filled
+    int pmax, pbest;           // event()'s placements at t: largest capacity, and how far past p its
+                               // cyclically last SM lies (what the pointer moves by when t passes)
+    uint32_t tail, dburst;     // latest end of the groups listed before t, and of those listed at t, minus t
     // head kernel
     int hk, hr, hs, hw, hc, hm;
     uint32_t hpk;             // registers | 1 << 19 | warps << 25
     float frr, frs, frw, fsb; // reciprocals of registers, shared memory, warps (rounded down)
-    // the last offer: per-run caps, SM-weighted total, maximum, runs that take blocks
-    Bytes16 caps;
-    int ctotal, cmax;
-    uint32_t celig;
 
     KO_HD uint32_t &W(int f) const { return col[f * STRIDE]; }
 #ifdef __CUDA_ARCH__
@@ -219,17 +214,26 @@ struct LaneSim {
 
     KO_HD void init()
     {
-        W(W_RB) = (uint32_t)L.S << 16;
+        W(W_RB) = (uint32_t)L.S << kCntShift;
         W(W_RU) = 0; W(W_RS) = 0; W(W_RC) = 0; W(W_RM) = 0;
         set_list(0, ~0ull);
         nr = 1;
         t = 0;
         p = 0;
         freeg = kPoolAll;
-        rel = 0;
         pend = 0;
+        tail = 0;
+        settle();
+    }
+
+    // No burst in progress beyond the pending groups (a node state's registers).
+    KO_HD void settle()
+    {
+        rel = placed = 0;
         fresh = todo = 0;
+        ends = drain = 0;
         pmax = pbest = 0;
+        dburst = 0;
         fail = 0;
     }
 
@@ -278,8 +282,8 @@ struct LaneSim {
         const uint32_t scc = sc > L.ccap ? sc : L.ccap, smm = sm > L.mcap ? sm : L.mcap;
         const unsigned long long pc = (unsigned long long)c * scc + (L.ccap - 1u);
         const unsigned long long pm = (unsigned long long)m * smm + (L.mcap - 1u);
-        const uint32_t dc = (uint32_t)(L.cshift >= 0 ? pc >> L.cshift : pc / L.ccap);
-        const uint32_t dm = (uint32_t)(L.mshift >= 0 ? pm >> L.mshift : pm / L.mcap);
+        const uint32_t dc = L.cshift >= 0 ? (uint32_t)(pc >> L.cshift) : quotient(pc, L.ccap);
+        const uint32_t dm = L.mshift >= 0 ? (uint32_t)(pm >> L.mshift) : quotient(pm, L.mcap);
         return dc > dm ? dc : dm;
     }
 
@@ -289,7 +293,7 @@ struct LaneSim {
     KO_HD unsigned long long insert(unsigned long long l, int g, uint32_t dur, bool &first)
     {
         const uint32_t t32 = (uint32_t)t;
-        if (((l >> (kListBits * (kListLen - 1))) & 63u) != kNoSlot) { fail = 1; return l; }
+        if (((l >> (kListBits * (kListLen - 1))) & 63u) != kNoSlot) fail = 1;  // full: the item is handed on
         int pos = 0;
         unsigned long long rest = l;
         for (;;) {
@@ -303,7 +307,7 @@ struct LaneSim {
                 in += (s != kNoSlot && e <= dur) ? 1 : 0;
             }
             pos += in;
-            if (in < 4) break;
+            if (in < 4) break;  // at most three turns: entries past the tenth read as none
             rest = (rest >> (4 * kListBits)) | (~0ull << (64 - 4 * kListBits));
         }
         first = pos == 0;
@@ -311,12 +315,11 @@ struct LaneSim {
         return (l & below) | ((unsigned long long)g << (kListBits * pos)) | ((l & ~below) << kListBits) | (0xfull << 60);
     }
 
-    // Take the free slot for q blocks per SM of the head kernel on run j.
+    // A free slot for q blocks per SM of the head kernel on run j (freeg != 0).
     KO_HD int take_slot(int j, int q)
     {
         const int g = ffs64(freeg);
         freeg &= freeg - 1;
-        pend |= 1ull << g;
         set_gd(g, (uint32_t)hk | ((uint32_t)(q - 1) << 5) | ((uint32_t)j << kDescOwnerShift));
         return g;
     }
@@ -325,7 +328,7 @@ struct LaneSim {
     KO_HD void add_group(int j, int q)
     {
         if (freeg == 0) { fail = 1; return; }
-        take_slot(j, q);
+        pend |= 1ull << take_slot(j, q);
         W(W_RU + j) += (uint32_t)q * hpk;
         W(W_RS + j) += (uint32_t)(q * hs);
         W(W_RC + j) += (uint32_t)(q * hc);
@@ -334,14 +337,13 @@ struct LaneSim {
 
     // Split run j after x SMs (0 < x < its count): run j keeps the first x, the
     // new run `nr` takes the rest.
-    KO_HD bool split(int j, int x)
+    KO_HD void split(int j, int x)
     {
-        if (nr >= run_limit) { fail = 1; return false; }
+        if (nr >= run_limit) { fail = 1; return; }
         const int k = nr++;
         const uint32_t rb = W(W_RB + j);
-        const uint32_t beg = rb & 0xffffu, cnt = rb >> 16;
-        W(W_RB + j) = beg | ((uint32_t)x << 16);
-        W(W_RB + k) = (beg + (uint32_t)x) | ((cnt - (uint32_t)x) << 16);
+        W(W_RB + j) = (rb & ~(kSmMask << kCntShift)) | ((uint32_t)x << kCntShift);
+        W(W_RB + k) = rb + (uint32_t)x - ((uint32_t)x << kCntShift);
         W(W_RU + k) = W(W_RU + j);
         W(W_RS + k) = W(W_RS + j);
         W(W_RC + k) = W(W_RC + j);
@@ -352,49 +354,22 @@ struct LaneSim {
         // run j's pending groups: the new run gets its own copies
         for (unsigned long long pm = pend; pm; pm &= pm - 1) {
             const uint32_t d = gd(ffs64(pm));
-            if ((int)(d >> kDescOwnerShift) != j) continue;
-            if (freeg == 0) { fail = 1; return false; }
-            const int g2 = ffs64(freeg);
-            freeg &= freeg - 1;
-            pend |= 1ull << g2;
-            set_gd(g2, (d & ((1u << kDescOwnerShift) - 1u)) | ((uint32_t)k << kDescOwnerShift));
+            if ((int)(d >> kDescOwnerShift) == j) {
+                if (freeg == 0) fail = 1;
+                else {
+                    const int g2 = ffs64(freeg);
+                    freeg &= freeg - 1;
+                    pend |= 1ull << g2;
+                    set_gd(g2, (d & ((1u << kDescOwnerShift) - 1u)) | ((uint32_t)k << kDescOwnerShift));
+                }
+            }
         }
-        return true;
-    }
-
-    // Capacities of the head kernel on the runs in `elig` (every other run has
-    // no room for it): per-run caps, their SM-weighted total and maximum.
-    KO_HD void offer(uint32_t elig)
-    {
-        caps.lo = caps.hi = 0ull;
-        ctotal = 0;
-        cmax = 0;
-        // runs with room for one block (four compares) take the exact capacity
-        uint32_t room = 0;
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-        for (int j = 0; j < kRuns; j++) {
-            if (!((elig >> j) & 1u)) continue;
-            const uint32_t u = W(W_RU + j);
-            const bool fits = (int)((u >> 19) & 63u) < L.Bk && (int)(u & kRegMask) + hr <= L.R &&
-                              (int)(u >> 25) + hw <= L.W && (int)W(W_RS + j) + hs <= L.Sh;
-            room |= (fits ? 1u : 0u) << j;
-        }
-        for (uint32_t e = room; e; e &= e - 1) {
-            const int j = ffs32(e);
-            const int c = cap(W(W_RU + j), W(W_RS + j));
-            caps.set(j, c);
-            ctotal += (int)(W(W_RB + j) >> 16) * c;
-            cmax = c > cmax ? c : cmax;
-        }
-        celig = room;  // the placement steps visit only runs that take blocks
     }
 
     // How far past p (in SMs, cyclically) the last SM of the run rb lies, 1..S.
     KO_HD int last_past(uint32_t rb) const
     {
-        const int b = (int)(rb & 0xffffu), d = b + (int)(rb >> 16) - p;
+        const int b = (int)(rb & kSmMask), d = b + (int)((rb >> kCntShift) & kSmMask) - p;
         if (b < p && d > 0) return L.S;  // p lies inside: its last SM from p on is p - 1
         return d <= 0 ? d + L.S : d;
     }
@@ -405,113 +380,16 @@ struct LaneSim {
         if (p >= L.S) p -= L.S;
     }
 
-    // Every SM of the offered runs takes its full capacity (ctotal <= left);
-    // the last block lands on the SM with cap == cmax that comes last
-    // cyclically from p.
-    KO_HD void place_full(int &left)
-    {
-        int best = 0;
-        for (uint32_t e = celig; e; e &= e - 1) {
-            const int j = ffs32(e);
-            const int c = caps.get(j);
-            add_group(j, c);
-            if (c == cmax) {
-                const int pos = last_past(W(W_RB + j));
-                best = pos > best ? pos : best;
-            }
-        }
-        move_pointer(best);
-        left -= ctotal;
-    }
-
-    // The offered runs hold more room than `left` blocks (ctotal > left): the
-    // water-fill stops inside a sweep, cutting runs at p and where it stops.
-    KO_HD void water_fill(int &left)
-    {
-        uint32_t elig = celig;
-        // smallest sweep count L with F(L) = sum cnt * min(cap, L) >= left
-        int lo = 1, hi = cmax;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            int f = 0;
-            for (uint32_t e = elig; e; e &= e - 1) {
-                const int j = ffs32(e);
-                const int c = caps.get(j);
-                f += (int)(W(W_RB + j) >> 16) * (c < mid ? c : mid);
-            }
-            if (f >= left) hi = mid; else lo = mid + 1;
-        }
-        const int Lsw = lo;
-        int filled = 0;
-        uint32_t last = 0;  // runs whose SMs can take a block in the last sweep
-        for (uint32_t e = elig; e; e &= e - 1) {
-            const int j = ffs32(e);
-            const int c = caps.get(j);
-            filled += (int)(W(W_RB + j) >> 16) * (c < Lsw - 1 ? c : Lsw - 1);
-            last |= (c >= Lsw ? 1u : 0u) << j;
-        }
-        const int rem = left - filled;  // 1 .. number of SMs with cap >= Lsw
-        // cut the run that holds p at p when its SMs can take a block in the last sweep
-        for (uint32_t e = last; e; e &= e - 1) {
-            const int j = ffs32(e);
-            const uint32_t rb = W(W_RB + j);
-            const int b = (int)(rb & 0xffffu), n = (int)(rb >> 16);
-            if (b < p && p < b + n) {
-                if (!split(j, p - b)) return;
-                caps.set(nr - 1, caps.get(j));
-                elig |= 1u << (nr - 1);
-                last |= 1u << (nr - 1);
-                break;
-            }
-        }
-        // visit those runs cyclically from p, one more block to each of their SMs
-        uint32_t plus = 0;
-        int acc = 0, newp = p;
-        while (last) {
-            int j = 0, best = 0x7fffffff;
-            for (uint32_t e = last; e; e &= e - 1) {
-                const int i = ffs32(e);
-                int d = (int)(W(W_RB + i) & 0xffffu) - p;
-                if (d < 0) d += L.S;
-                if (d < best) { best = d; j = i; }
-            }
-            last &= ~(1u << j);
-            plus |= 1u << j;
-            const uint32_t rb = W(W_RB + j);
-            const int n = (int)(rb >> 16);
-            if (acc + n >= rem) {
-                const int x = rem - acc;
-                if (x < n) {
-                    if (!split(j, x)) return;
-                    caps.set(nr - 1, caps.get(j));
-                    elig |= 1u << (nr - 1);
-                }
-                newp = (int)(rb & 0xffffu) + x;
-                break;
-            }
-            acc += n;
-        }
-        p = newp >= L.S ? newp - L.S : newp;
-        for (uint32_t e = elig; e; e &= e - 1) {
-            const int j = ffs32(e);
-            const int c = caps.get(j);
-            const int q = (c < Lsw - 1 ? c : Lsw - 1) + (int)((plus >> j) & 1u);
-            if (q > 0) add_group(j, q);
-        }
-        left = 0;
-    }
-
-    // A run's state while event() or place_partial() works on it.
+    // A run's state while a step works on it.
     struct RunState {
         uint32_t u, s, c, m, re;
         unsigned long long l;
     };
 
-    // Release the groups of run j that end at t.
-    KO_HD RunState release(int j)
+    // Release the groups of the run that end at t.
+    KO_HD void release(RunState &r)
     {
         const uint32_t now = (uint32_t)t;
-        RunState r{W(W_RU + j), W(W_RS + j), W(W_RC + j), W(W_RM + j), 0u, list(j)};
         for (;;) {
             const uint32_t s0 = (uint32_t)r.l & 63u;
             const int g = (int)(s0 < (uint32_t)kPool ? s0 : 0u);  // a run released here lists a group
@@ -529,31 +407,6 @@ struct LaneSim {
             rel |= 1ull << g;
             if (!more || r.re != now) break;
         }
-        return r;
-    }
-
-    KO_HD void store(int j, const RunState &r) const
-    {
-        W(W_RU + j) = r.u; W(W_RS + j) = r.s; W(W_RC + j) = r.c; W(W_RM + j) = r.m;
-        W(W_RE + j) = r.re;
-        set_list(j, r.l);
-    }
-
-    // Fix the durations of the pending groups and list them.
-    KO_HD void close_burst()
-    {
-        for (unsigned long long pm = pend; pm; pm &= pm - 1) {
-            const int g = ffs64(pm);
-            const uint32_t d = gd(g);
-            const int j = (int)(d >> kDescOwnerShift);
-            const KRel q = kl.rel((int)(d & kDescKernel));
-            const uint32_t dur = duration(q.c, q.m, W(W_RC + j), W(W_RM + j));
-            W(W_GE + g) = (uint32_t)t + dur;
-            bool first = false;
-            set_list(j, insert(list(j), g, dur, first));
-            if (first) W(W_RE + j) = (uint32_t)t + dur;
-        }
-        pend = 0;
     }
 
     // Jump to the earliest end of a run.  While blocks are queued and the burst
@@ -579,92 +432,131 @@ struct LaneSim {
         for (int j = 0; j < kRuns; j++)
             if (e[j] == dmin) fresh |= 1u << j;
         t += dmin;
+        tail = (tail > dburst ? tail : dburst) - dmin;
+        dburst = 0;
         todo = fresh;
-        freeg |= rel;
-        rel = 0;
-        pend = 0;
+        ends = 1;
+        placed = 0;
         move_pointer(pbest);
         pmax = pbest = 0;
     }
 
-    // Queue all blocks of kernel k behind the current queue: the first burst
-    // offers it every run.  Returns the blocks still queued.
-    KO_HD int start_kernel(int k)
+    // Queue all blocks of kernel k behind the current queue: its first burst
+    // offers it the runs with room for one block (four compares; every other
+    // run is skipped), which event() then takes one by one.  Returns the blocks
+    // queued.
+    KO_HD int begin_kernel(int k)
     {
         set_head(k);
-        int left = kl.full(k).b;
-        offer((1u << nr) - 1u);
-        if (ctotal > left) water_fill(left);
-        else if (ctotal > 0) place_full(left);
-        return left;
+        uint32_t room = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int j = 0; j < kRuns; j++) {
+            if (j < nr) {
+                const uint32_t u = W(W_RU + j);
+                const bool fits = (int)((u >> 19) & 63u) < L.Bk && (int)(u & kRegMask) + hr <= L.R &&
+                                  (int)(u >> 25) + hw <= L.W && (int)W(W_RS + j) + hs <= L.Sh;
+                room |= (fits ? 1u : 0u) << j;
+            }
+        }
+        fresh = todo = room;
+        ends = 0;
+        placed = 0;
+        return kl.full(k).b;
     }
 
-    // One run's event while the head kernel has queued blocks and the burst is
-    // closed: release what ends, place the head kernel's full capacity and list
-    // the new group.  Returns true, with nothing placed on this run, when that
-    // would empty the queue: the caller finishes the burst with place_partial.
-    // `mask`: the threads of the warp that run this step together; they
-    // reconverge after each stage.
+    // One step while the head kernel has queued blocks, for one run:
+    //   a run of the burst in progress (`todo`): release what ends, place the
+    //     head kernel's full capacity and list the new group;
+    //   none left: list one group that was pending when the kernel's first
+    //     burst began (its run's SumC / SumM are final now);
+    //   neither: the next event begins.
+    // Returns true when this burst empties the queue; the caller finishes it
+    // with place_partial.  `mask`: the threads of the warp that run this step
+    // together; they reconverge after each stage.
     KO_HD bool event(int &left, unsigned mask)
     {
-        if (todo == 0) advance();
+        if (todo == 0 && pend == 0) advance();
         KO_RECONVERGE(mask);
-        const int j = ffs32(todo);
-        todo &= todo - 1;
-        RunState r = release(j);
+        const bool listing = todo == 0;
+        int g = 0, j;
+        uint32_t kc = (uint32_t)hc, km = (uint32_t)hm;
+        if (listing) {
+            g = ffs64(pend);
+            pend &= pend - 1;
+            const uint32_t d = gd(g);
+            j = (int)(d >> kDescOwnerShift);
+            const KRel q = kl.rel((int)(d & kDescKernel));
+            kc = q.c;
+            km = q.m;
+        } else {
+            j = ffs32(todo);
+            todo &= todo - 1;
+        }
+        RunState r{W(W_RU + j), W(W_RS + j), W(W_RC + j), W(W_RM + j), W(W_RE + j), list(j)};
+        const uint32_t rb = W(W_RB + j);
+        if (!listing && ends) release(r);
         KO_RECONVERGE(mask);
         if (todo == 0) {  // every holder of the slots released at t has let go
             freeg |= rel;
             rel = 0;
         }
-        const int q = cap(r.u, r.s);
-        const uint32_t rb = W(W_RB + j);
-        const int take = q * (int)(rb >> 16);
-        const bool last = take >= left && take > 0;
-        if (take > 0 && !last) {
-            if (freeg == 0) fail = 1;
-            else {
-                const int g = take_slot(j, q);
-                r.u += (uint32_t)q * hpk;
-                r.s += (uint32_t)(q * hs);
-                r.c += (uint32_t)(q * hc);
-                r.m += (uint32_t)(q * hm);
-                const uint32_t dur = duration((uint32_t)hc, (uint32_t)hm, r.c, r.m);
-                W(W_GE + g) = (uint32_t)t + dur;
-                bool first = false;
-                r.l = insert(r.l, g, dur, first);
-                if (first) r.re = (uint32_t)t + dur;
-                left -= take;
-                const int pos = last_past(rb);
-                pbest = q > pmax ? pos : (q == pmax && pos > pbest ? pos : pbest);
-                pmax = q > pmax ? q : pmax;
+        bool put = listing;
+        if (!listing) {
+            const int q = cap(r.u, r.s);
+            const int take = q * (int)((rb >> kCntShift) & kSmMask);
+            if (take >= left && take > 0) drain = 1;
+            if (q > 0 && !drain) {
+                if (freeg == 0) fail = 1;
+                else {
+                    g = take_slot(j, q);
+                    placed |= 1ull << g;
+                    r.u += (uint32_t)q * hpk;
+                    r.s += (uint32_t)(q * hs);
+                    r.c += (uint32_t)(q * hc);
+                    r.m += (uint32_t)(q * hm);
+                    left -= take;
+                    const int pos = last_past(rb);
+                    pbest = q > pmax ? pos : (q == pmax && pos > pbest ? pos : pbest);
+                    pmax = q > pmax ? q : pmax;
+                    put = true;
+                }
             }
         }
         KO_RECONVERGE(mask);
-        store(j, r);
-        return last && !fail;
+        if (put) {
+            const uint32_t dur = duration(kc, km, r.c, r.m);
+            W(W_GE + g) = (uint32_t)t + dur;
+            dburst = dur > dburst ? dur : dburst;
+            bool first = false;
+            r.l = insert(r.l, g, dur, first);
+            if (first) r.re = (uint32_t)t + dur;
+        }
+        KO_RECONVERGE(mask);
+        W(W_RU + j) = r.u; W(W_RS + j) = r.s; W(W_RC + j) = r.c; W(W_RM + j) = r.m;
+        W(W_RE + j) = r.re;
+        set_list(j, r.l);
+        if (!ends && drain) todo = 0;  // nothing ends in a first burst: no run left to release
+        return drain && todo == 0 && !fail;
     }
 
-    // The burst in which event() reported that the queue would empty: release
-    // the runs it has not taken, take back what it placed, and fill the runs
-    // that ended at t jointly.  The burst stays open unless blocks are left.
+    // The burst that empties the queue: take back what event() placed in it and
+    // fill its runs jointly.  Blocks go round-robin over the SMs with room, so
+    // every SM ends with min(capacity, L - 1) blocks of this burst and the first
+    // ones past p with more room have one more; runs are cut at p and where the
+    // last sweep stops.  The burst stays open for the next kernel.
     KO_HD void place_partial(int &left)
     {
-        for (; todo; todo &= todo - 1) {
-            const int j = ffs32(todo);
-            store(j, release(j));
-        }
-        freeg |= rel;
-        rel = 0;
-        for (; pend; pend &= pend - 1) {
-            const int g = ffs64(pend);
+        for (; placed; placed &= placed - 1) {
+            const int g = ffs64(placed);
             const uint32_t d = gd(g), q = ((d >> 5) & 63u) + 1u;
             const int j = (int)(d >> kDescOwnerShift);
             W(W_RU + j) -= q * hpk;
             W(W_RS + j) -= q * (uint32_t)hs;
             W(W_RC + j) -= q * (uint32_t)hc;
             W(W_RM + j) -= q * (uint32_t)hm;
-            left += (int)q * (int)(W(W_RB + j) >> 16);
+            left += (int)q * (int)((W(W_RB + j) >> kCntShift) & kSmMask);
             freeg |= 1ull << g;
             // out of the list
             const unsigned long long all = list(j);
@@ -676,34 +568,100 @@ struct LaneSim {
             const uint32_t head = (uint32_t)nl & 63u;
             if (head != kNoSlot) W(W_RE + j) = W(W_GE + (int)head);
         }
+        drain = 0;
+        dburst = 0;
         pmax = pbest = 0;
-        offer(fresh);
-        if (ctotal > left) water_fill(left);
-        else place_full(left);
-        if (left > 0) close_burst();
+        // capacities, kept in the runs' words
+        uint32_t elig = 0;
+        int cmax = 0;
+        for (uint32_t e = fresh; e; e &= e - 1) {
+            const int j = ffs32(e);
+            const int c = cap(W(W_RU + j), W(W_RS + j));
+            const uint32_t rb = W(W_RB + j) & kSpanMask;
+            W(W_RB + j) = rb | ((uint32_t)c << kCapShift);
+            cmax = c > cmax ? c : cmax;
+            elig |= (c > 0 ? 1u : 0u) << j;
+        }
+        // smallest sweep count L with F(L) = sum cnt * min(cap, L) >= left (total >= left)
+        int lo = 1, hi = cmax;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            int f = 0;
+            for (uint32_t e = elig; e; e &= e - 1) {
+                const uint32_t rb = W(W_RB + ffs32(e));
+                const int c = (int)(rb >> kCapShift);
+                f += (int)((rb >> kCntShift) & kSmMask) * (c < mid ? c : mid);
+            }
+            if (f >= left) hi = mid; else lo = mid + 1;
+        }
+        const int Lsw = lo;
+        // runs whose SMs can take a block in the last sweep; of those, the one that holds p past its start
+        uint32_t last = 0, cut = 0;
+        int rem = left;
+        for (uint32_t e = elig; e; e &= e - 1) {
+            const int j = ffs32(e);
+            const uint32_t rb = W(W_RB + j);
+            const int c = (int)(rb >> kCapShift), b = (int)(rb & kSmMask), n = (int)((rb >> kCntShift) & kSmMask);
+            rem -= n * (c < Lsw - 1 ? c : Lsw - 1);
+            if (c >= Lsw) {
+                last |= 1u << j;
+                if (b < p && p < b + n) cut = 1u << j;
+            }
+        }
+        // rem = 1 .. number of SMs with cap >= L.  Visit those runs cyclically from p, one more block
+        // to each of their SMs; a run is split where p or the sweep's end lies inside it.
+        uint32_t plus = 0;
+        int acc = 0, newp = p;
+        bool going = last != 0;
+        while (going) {
+            int j = 0, x;
+            if (cut) {
+                j = ffs32(cut);
+                x = p - (int)(W(W_RB + j) & kSmMask);
+            } else {
+                int best = 0x7fffffff;
+                for (uint32_t e = last; e; e &= e - 1) {
+                    const int i = ffs32(e);
+                    int d = (int)(W(W_RB + i) & kSmMask) - p;
+                    if (d < 0) d += L.S;
+                    if (d < best) { best = d; j = i; }
+                }
+                last &= ~(1u << j);
+                plus |= 1u << j;
+                const uint32_t rb = W(W_RB + j);
+                const int n = (int)((rb >> kCntShift) & kSmMask);
+                x = 0;
+                if (acc + n >= rem) {
+                    x = rem - acc;
+                    newp = (int)(rb & kSmMask) + x;
+                    if (x == n) x = 0;
+                    last = 0;
+                }
+                acc += n;
+            }
+            if (x > 0) {
+                split(j, x);
+                elig |= 1u << (nr - 1);
+                if (cut) last |= 1u << (nr - 1);
+            }
+            cut = 0;
+            going = last != 0 && !fail;
+        }
+        p = newp >= L.S ? newp - L.S : newp;
+        for (uint32_t e = elig; e; e &= e - 1) {
+            const int j = ffs32(e);
+            const int c = (int)(W(W_RB + j) >> kCapShift);
+            const int q = (c < Lsw - 1 ? c : Lsw - 1) + (int)((plus >> j) & 1u);
+            if (q > 0) add_group(j, q);
+        }
+        left = 0;
     }
 
     // The makespan: the latest end of any group, the pending ones' included
     // (groups that have left ended by t).
-    KO_HD long long finish()
+    KO_HD long long finish() const
     {
-        const uint32_t t32 = (uint32_t)t;
-        uint32_t d = 0;
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-        for (int j = 0; j < kRuns; j++) {
-            if (j < nr) {
-                const unsigned long long none = ~list(j) & ((1ull << 60) - 1ull);  // zero entries are empty
-                if (none) {
-                    const uint32_t hi = (uint32_t)(none >> 32), lo = (uint32_t)none;
-                    const int bit = hi ? 32 + msb32(hi) : msb32(lo);
-                    const int g = (int)((list(j) >> (bit / kListBits * kListBits)) & 63u);
-                    const uint32_t e = W(W_GE + g) - t32;
-                    d = e > d ? e : d;
-                }
-            }
-        }
+        uint32_t d = tail;
         for (unsigned long long pm = pend; pm; pm &= pm - 1) {
             const uint32_t w = gd(ffs64(pm));
             const int j = (int)(w >> kDescOwnerShift);
@@ -720,18 +678,31 @@ struct LaneSim {
         r[0] = (uint32_t)t; r[1] = (uint32_t)(t >> 32);
         r[2] = (uint32_t)freeg; r[3] = (uint32_t)(freeg >> 32);
         r[4] = (uint32_t)pend; r[5] = (uint32_t)(pend >> 32);
-        r[6] = (uint32_t)p; r[7] = (uint32_t)nr;
+        r[6] = (uint32_t)p | ((uint32_t)nr << 16); r[7] = tail;
     }
     KO_HD void regs_in(const uint32_t *r)
     {
         t = (unsigned long long)r[0] | ((unsigned long long)r[1] << 32);
         freeg = (unsigned long long)r[2] | ((unsigned long long)r[3] << 32);
         pend = (unsigned long long)r[4] | ((unsigned long long)r[5] << 32);
-        p = (int)r[6]; nr = (int)r[7];
-        rel = 0;
-        fresh = todo = 0;
-        pmax = pbest = 0;
-        fail = 0;
+        p = (int)(r[6] & 0xffffu); nr = (int)(r[6] >> 16);
+        tail = r[7];
+        settle();
+    }
+
+    // The first burst of kernel k and the close of a burst as whole calls, for
+    // callers that do not step event() themselves.
+    KO_HD int start_kernel(int k)
+    {
+        int left = begin_kernel(k);
+        while (todo && !fail)
+            if (event(left, 0u)) place_partial(left);
+        return left;
+    }
+    KO_HD void close_burst()
+    {
+        int left = 1;  // listing takes no blocks
+        while (pend && !fail) event(left, 0u);
     }
 };
 

@@ -288,6 +288,40 @@ __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__
     }
 }
 
+// Raw features: FP32 rows [B x 192] to the BF16 operands of the layers -- xb
+// row-major, and (training) xt transposed for the weight gradients.  Bound by
+// the host link that fills x, not by this pass (B = 65536: 50 MB read, 25 MB
+// written).  A block takes 64 rows: coalesced 16-byte reads, 8-byte row stores,
+// and the transposed rows leave through shared memory (a 66-element pitch
+// spreads a column over the banks) as 128-byte segments.  The host used to
+// round and transpose element by element: 24.4 ms of a 65,536-row prediction.
+constexpr int kFeatRows = 64, kFeatPitch = kFeatRows + 2;
+__global__ void __launch_bounds__(256) features_bf16_kernel(const float *__restrict__ x, int B, uint16_t *xb,
+                                                            uint16_t *xt)
+{
+    __shared__ uint16_t tile[kMlpIn * kFeatPitch];
+    const long long row0 = (long long)blockIdx.x * kFeatRows;
+    constexpr int kQuads = kMlpIn / 4;
+    for (int i = threadIdx.x; i < kFeatRows * kQuads; i += blockDim.x) {
+        const int r = i / kQuads, f = (i - r * kQuads) * 4;
+        const long long at = (row0 + r) * kMlpIn + f;
+        const float4 v = __ldcs(reinterpret_cast<const float4 *>(x + at));
+        const uint16_t h[4] = {bf16_bits(v.x), bf16_bits(v.y), bf16_bits(v.z), bf16_bits(v.w)};
+        *reinterpret_cast<uint2 *>(xb + at) =
+            make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16));
+        if (xt)
+#pragma unroll
+            for (int q = 0; q < 4; q++) tile[(f + q) * kFeatPitch + r] = h[q];
+    }
+    if (!xt) return;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kMlpIn * (kFeatRows / 2); i += blockDim.x) {
+        const int f = i / (kFeatRows / 2), r = (i - f * (kFeatRows / 2)) * 2;
+        *reinterpret_cast<uint32_t *>(xt + (long long)f * B + row0 + r) =
+            *reinterpret_cast<const uint32_t *>(&tile[f * kFeatPitch + r]);
+    }
+}
+
 // y[b] = A3[b] . w4 + b4: eight threads per row, thread c sums columns
 // 32c .. 32c + 31 as a chain of fused multiply-adds in column order, and the
 // eight partials combine as ((p0 + p1) + (p2 + p3)) + ((p4 + p5) + (p6 + p7))
@@ -619,6 +653,13 @@ cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *sid, co
     const long long blocks = ((long long)B + 32 * kEncWarps - 1) / (32 * kEncWarps);
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
     encode_kernel<<<grid, kEncWarps * 32, 0, st>>>(rows, row_stride, sid, pick, set_n, kfeat, gfeat, B, x, xt);
+    ko_count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t ko_mlp_features(const float *x, int B, uint16_t *xb, uint16_t *xt, cudaStream_t st)
+{
+    features_bf16_kernel<<<(unsigned)(B / kFeatRows), 256, 0, st>>>(x, B, xb, xt);
     ko_count_launch();
     return cudaGetLastError();
 }

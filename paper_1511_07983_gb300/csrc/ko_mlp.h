@@ -62,6 +62,9 @@ cudaError_t ko_mlp_gemm_f32(const uint16_t *A, int lda, const uint16_t *Bt, int 
 cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *sid, const int *pick,
                           const int *set_n, const float *kfeat, const float *gfeat, int B, uint16_t *x,
                           uint16_t *xt, cudaStream_t st);
+// FP32 features x [B x 192] (device, B % 64 == 0) rounded to BF16 (nearest, ties to even) into xb and,
+// if xt is non-null, transposed into xt [192 x B].
+cudaError_t ko_mlp_features(const float *x, int B, uint16_t *xb, uint16_t *xt, cudaStream_t st);
 cudaError_t ko_mlp_out_fwd(const uint16_t *a3, const uint16_t *w4, const float *b4, int B, float *y,
                            cudaStream_t st);
 // The backward kernels sum per-block partials (workspace `part`, at least

@@ -269,29 +269,15 @@ ko_status adam(ko_model *md, float lr, cudaStream_t st)
     return refresh_bf16(md, st);
 }
 
-uint16_t host_bf16(float x)
+// Features of raw rows x [B x 192] (host floats) into a0 and, for training, a0t:
+// copied to the device as they are (into `da`, which the backward pass only
+// writes later) and rounded there.
+ko_status upload_features(ko_model *md, const float *x, int B, bool train, cudaStream_t st)
 {
-    uint32_t u;
-    std::memcpy(&u, &x, 4);
-    u += 0x7FFFu + ((u >> 16) & 1u);
-    return (uint16_t)(u >> 16);
-}
-
-// Features of raw rows x [B x 192] (host floats) into a0 / a0t.
-ko_status upload_features(ko_model *md, const float *x, int B, cudaStream_t st)
-{
-    std::vector<uint16_t> h((size_t)B * kMlpIn), ht((size_t)B * kMlpIn);
-    for (int b = 0; b < B; b++)
-        for (int f = 0; f < kMlpIn; f++) {
-            const uint16_t v = host_bf16(x[(size_t)b * kMlpIn + f]);
-            h[(size_t)b * kMlpIn + f] = v;
-            ht[(size_t)f * B + b] = v;
-        }
-    if (cudaMemcpyAsync(md->a0, h.data(), h.size() * 2, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(md->a0t, ht.data(), ht.size() * 2, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+    static_assert(kMlpIn <= kHidden, "the FP32 rows fit the input-gradient buffer");
+    if (cudaMemcpyAsync(md->da, x, sizeof(float) * (size_t)B * kMlpIn, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return KO_ERR_CUDA;
-    return KO_OK;
+    return cuda_ok(ko_mlp_features(md->da, B, md->a0, train ? md->a0t : nullptr, st));
 }
 
 }  // namespace
@@ -385,7 +371,7 @@ ko_status ko_model_raw(ko_model *md, const float *x, const float *t, int B, floa
     if (B < 64 || B % 64) return KO_ERR_ARG;
     ko_status s = ensure_acts(md, B);
     if (s) return s;
-    if ((s = upload_features(md, x, B, st))) return s;
+    if ((s = upload_features(md, x, B, t != nullptr, st))) return s;
     if ((s = forward(md, B, t != nullptr, st))) return s;
     if (t) {
         if (cudaMemcpyAsync(md->t, t, sizeof(float) * B, cudaMemcpyHostToDevice, st) != cudaSuccess ||

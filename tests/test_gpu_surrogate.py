@@ -317,3 +317,23 @@ def test_trained_network_gain(ko):
     for m in models.values():
         m.close()
     assert guided_wins["mixed"] > 16 and guided_wins["mixed"] >= guided_wins["untrained"], guided_wins
+
+
+@pytest.mark.parametrize("B", [64, 192, 4160])
+def test_raw_features_are_rounded_as_the_oracle_rounds(ko, B):
+    """Features that are no BF16 values -- random, and exact ties between two of
+    them -- give the same bits as the oracle's rounding of them, in the forward
+    pass (rows) and in the weight gradients (the transposed copy too)."""
+    rng = np.random.default_rng(B)
+    x = rng.standard_normal((B, 192)).astype(np.float32)
+    ties = mlp.bf16(x[:, ::3]).view(np.uint32) + np.uint32(0x8000)
+    x[:, ::3] = ties.view(np.float32)
+    t = rng.standard_normal(B).astype(np.float32)
+    m = ko.Model()
+    m.set_params(_flat(_params(11)))
+    rounded = mlp.bf16(x)
+    assert not np.array_equal(rounded, x)
+    assert np.array_equal(m.predict(x), m.predict(rounded))
+    (g0, l0), (g1, l1) = m.grad(x, t), m.grad(rounded, t)
+    assert np.array_equal(g0, g1)
+    assert l0 == l1

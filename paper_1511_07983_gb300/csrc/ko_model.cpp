@@ -293,6 +293,8 @@ ko_model *ko_model_new(uint64_t seed, ko_status *err)
               dalloc(&md->w3, (size_t)kHidden * kHidden) && dalloc(&md->w3t, (size_t)kHidden * kHidden) &&
               dalloc(&md->w4b, (size_t)kHidden) && dalloc(&md->loss, 1 << 16) && dalloc(&md->tc_err, 1);
     if (!ok) { delete md; *err = KO_ERR_NOMEM; return nullptr; }
+    // new device memory holds whatever was there before: the flag must start clear
+    if (cudaMemset(md->tc_err, 0, sizeof(int)) != cudaSuccess) { delete md; *err = KO_ERR_CUDA; return nullptr; }
     // He-normal initialisation from a counter-based generator (zero biases,
     // zero weights on the padded input features)
     std::vector<float> h(kParams, 0.0f);

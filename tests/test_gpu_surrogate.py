@@ -337,3 +337,19 @@ def test_raw_features_are_rounded_as_the_oracle_rounds(ko, B):
     (g0, l0), (g1, l1) = m.grad(x, t), m.grad(rounded, t)
     assert np.array_equal(g0, g1)
     assert l0 == l1
+
+
+def test_new_model_in_used_device_memory(ko):
+    """A model's error flag must not be read from memory that an earlier
+    allocation left non-zero: predictions of a model created right after many
+    small buffers full of ones were freed."""
+    import ctypes
+    rt = ctypes.CDLL("/usr/local/cuda/lib64/libcudart.so")
+    ptrs = [ctypes.c_void_p() for _ in range(4096)]
+    for p in ptrs:
+        assert rt.cudaMalloc(ctypes.byref(p), 512) == 0
+        assert rt.cudaMemset(p, 0xFF, 512) == 0
+    for p in ptrs:
+        assert rt.cudaFree(p) == 0
+    x = np.zeros((128, 192), dtype=np.float32)
+    assert np.isfinite(ko.Model(seed=3).predict(x)).all()

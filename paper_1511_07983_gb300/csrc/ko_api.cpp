@@ -396,6 +396,7 @@ ko_status ko_eval_orders(ko_gpu *g, const uint64_t *idx, const int8_t *orders, i
         c.count = n;
         c.d0 = N;
         c.mode = idx ? 1 : 2;
+        KoRoute route(&g->fast, ko_list_choice(g->h, n), st);
         if ((s = upload_meta(g, st))) return fail(s);
         KoWork w = work_for(g, 1);
         w.idx = idx ? (const uint64_t *)d_in : nullptr;
@@ -439,6 +440,7 @@ ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, long long *refs,
     ko_status s = check_cuda(ko_launch_accum_reset(d_acc, 1, st));
     if (s) return s;
     if (fast_ok(g)) {
+        KoRoute route(&g->fast, ko_space_choice(g->h), st);
         KoWork lv;
         exhaustive_chunk(g, &lv);
         if ((s = upload_meta(g, st))) return s;
@@ -528,6 +530,7 @@ ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t 
         c0.d0 = N;
         c0.mode = 2;
         for (int i = 0; i < N; i++) g->h_meta.perm[i] = (int8_t)ord[i];
+        KoRoute route(&g->fast, ko_space_choice(g->h), st);
         KoWork lv;
         exhaustive_chunk(g, &lv);
         if ((s = upload_meta(g, st))) return fail(s);
@@ -606,10 +609,12 @@ ko_status ko_set_option(ko_gpu *g, int32_t key, int64_t value)
     case KO_OPT_LANES:
         if (value != 1 && value != 16 && value != 32) return fail(KO_ERR_ARG);
         g->fast.lanes = (int)value;
+        g->fast.chosen = true;
         break;
     case KO_OPT_LEVELS:
         if (value < 0 || value > 6) return fail(KO_ERR_ARG);
         g->fast.levels = (int)value;
+        g->fast.chosen = true;
         break;
     case KO_OPT_SIMPLE_ONLY:
         if (value != 0 && value != 1) return fail(KO_ERR_ARG);
@@ -622,10 +627,12 @@ ko_status ko_set_option(ko_gpu *g, int32_t key, int64_t value)
     case KO_OPT_STACK_GLOBAL:
         if (value != 0 && value != 1) return fail(KO_ERR_ARG);
         g->fast.stack_global = (int)value;
+        g->fast.chosen = true;
         break;
     case KO_OPT_LANE_STATE:
         if (value < 0 || value > 2) return fail(KO_ERR_ARG);
         g->fast.lane_shape = (int)value;
+        g->fast.chosen = true;
         break;
     default:
         return fail(KO_ERR_ARG);
@@ -665,6 +672,7 @@ ko_status ko_autotune(ko_gpu *g, const char *cache_path, void *stream)
     g->fast.levels = levels;
     g->fast.stack_global = stack;
     g->fast.lane_shape = shape;
+    g->fast.chosen = true;
     return ok();
 }
 
@@ -687,6 +695,7 @@ ko_status ko_batch_autotune(ko_gpu *const *sets, int32_t nsets, const char *cach
         sets[i]->fast.levels = levels[i];
         sets[i]->fast.stack_global = stack[i];
         sets[i]->fast.lane_shape = shape[i];
+        sets[i]->fast.chosen = true;
     }
     return ok();
 }

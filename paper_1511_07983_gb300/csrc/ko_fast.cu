@@ -875,6 +875,100 @@ int ko_fast_d0(const KoFastState &fs, int n)
 
 size_t ko_fast_smem_levels_cap() { return kMaxLevels; }
 
+// The one-thread simulator's packed usage word holds this set's limits (its
+// kernel hands every other set's items on).
+static bool packs(const KoSet &h) { return h.R < (1 << 19) && h.W <= 127; }
+
+// Lists of explicit orders: an order costs a whole simulation whatever the
+// list's length, so a short list is bound by one simulation's latency (a warp
+// per simulation is the quickest) and a long one by throughput (a thread per
+// simulation).  Measured, us for 32 lanes / one thread per order:
+//   1,024 orders  N=8, 13 SMs 127 / 210   N=12, 148 SMs 411 / 870   N=20, 13 SMs 634 / 1519
+//   4,096                     192 / 216                 559 / 914               1093 / 1635
+//   16,384                    495 / 227                1545 / 1016              3165 / 1752
+//   100,003 (16 lanes / one) 2039 / 570                6912 / 2073             13710 / 3959
+// The one-thread state holds 14 runs: on more than 32 SMs that is enough for
+// up to 13 kernels (under 3 % of random orders overflow in 31 of 32 sampled
+// sets; 14 kernels: 34 to 76 %); beyond, 32 lanes (16,384 orders of N=20 on
+// 148 SMs: 4.0 ms, 16 lanes 7.2 ms, one thread 8.0 ms).
+KoChoice ko_list_choice(const KoSet &h, long long count)
+{
+    const bool holds = packs(h) && (h.S <= 32 || h.n <= 13);
+    return count > 6144 && holds ? KoChoice{1, 1, 0} : KoChoice{32, 1, 0};
+}
+
+// Whole spaces: the work items of a space are its prefixes, each walked by one
+// simulation.  Up to 6! orders fill no chip however they are split, so a
+// warp takes one order (N=5, 148 SMs: 96 us; one 16-lane segment for the
+// whole space 3.9 ms).  Larger spaces go to one thread per item with the most
+// levels that still leave four items for every thread, and none where even
+// single orders do not (N=8, 13 SMs: 0.23 ms without levels, 0.31 with one, 6.4
+// with the state's default; N=9, 148 SMs: 2.1 ms with one level, 4.9 with three,
+// 22 with the default).  The 12-run state holds spaces on up to 16 SMs (N=9,
+// 13 SMs: 1.21 ms against 1.44 with 14 runs); on 148 SMs it hands on too many
+// items (N=10: 20.6 against 16.2 ms).
+KoChoice ko_space_choice(const KoSet &h)
+{
+    const int n = h.n;
+    if (n <= 6) return KoChoice{32, 0, 0};
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long want = 4ll * sms * 288;
+    const int deepest = h.S <= 16 ? 3 : 4;  // a deeper item that overflows hands on more orders
+    int levels = 0;
+    long long items = 1;
+    for (int i = 2; i <= n; i++) items *= i;
+    while (levels < deepest && levels + 1 < n && items / (levels + 2) >= want) items /= ++levels + 1;
+    if (!packs(h)) return KoChoice{16, levels, 0};
+    return KoChoice{1, levels, h.S <= 16 ? 1 : 0};
+}
+
+namespace {
+
+size_t gstack_need(int levels)
+{
+    // pass 1: at most 8 blocks of 8 segments per SM, 16 saved lanes per level
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int lv = levels < 1 ? 1 : (levels > kMaxLevels ? kMaxLevels : levels);
+    return sizeof(int) * (size_t)sms * 8 * 8 * lv * (state_words(kG) * 16 + 4);
+}
+
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) return false;
+    cudaGetLastError();
+    return true;
+}
+
+}  // namespace
+
+KoRoute::KoRoute(KoFastState *state, KoChoice c, cudaStream_t st, bool always)
+    : fs(state), lanes(state->lanes), levels(state->levels), shape(state->lane_shape), stack(state->stack_global)
+{
+    if (fs->chosen && !always) return;
+    fs->stack_global = 1;
+    if (capturing(st) && (fs->gstack_bytes < gstack_need(c.levels) ||
+                          (c.lanes == 1 && fs->lslab_bytes < ko_lane_slab_bytes(c.levels, c.shape)))) {
+        while (fs->levels > 1 && fs->gstack_bytes < gstack_need(fs->levels)) fs->levels--;
+        return;
+    }
+    fs->lanes = c.lanes;
+    fs->levels = c.levels;
+    fs->lane_shape = c.shape;
+}
+
+KoRoute::~KoRoute()
+{
+    fs->lanes = lanes;
+    fs->levels = levels;
+    fs->lane_shape = shape;
+    fs->stack_global = stack;
+}
+
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st)
 {
     // a pass abandons an item at most once, so lists as long as the launch's work lose none
@@ -883,11 +977,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     if (fs->ov_cap < want) {
         // a stream being captured cannot take a free or a malloc: the caller
         // must size the lists with an uncaptured launch first
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return KO_ERR_STATE;
-        }
+        if (capturing(st)) return KO_ERR_STATE;
         const size_t need = sizeof(FastBuf) + sizeof(unsigned long long) * 3 * (size_t)want;
         cudaFree(fs->buf);
         fs->buf = nullptr;
@@ -912,11 +1002,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         // one-thread-per-order pass: a node-state slab for every thread it runs
         const size_t need = ko_lane_slab_bytes(w.levels < 1 ? 1 : w.levels, fs->lane_shape);
         if (fs->lslab_bytes < need) {
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-                cudaGetLastError();
-                return KO_ERR_STATE;
-            }
+            if (capturing(st)) return KO_ERR_STATE;
             cudaFree(fs->lslab);
             fs->lslab = nullptr;
             fs->lslab_bytes = 0;
@@ -928,20 +1014,11 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         }
     }
     if (fs->stack_global) {
-        // pass 1: at most 8 blocks of 8 segments per SM, 16 saved lanes per level
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int lv = w.levels < 1 ? 1 : (w.levels > kMaxLevels ? kMaxLevels : w.levels);
-        const size_t need = sizeof(int) * (size_t)sms * 8 * 8 * lv * (state_words(kG) * 16 + 4);
+        const size_t need = gstack_need(w.levels);
         if (fs->gstack_bytes < need) {
             // a stream being captured cannot take a free or a malloc: the
             // caller must size the slab with an uncaptured launch first
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-                cudaGetLastError();
-                return KO_ERR_STATE;
-            }
+            if (capturing(st)) return KO_ERR_STATE;
             cudaFree(fs->gstack);
             fs->gstack = nullptr;
             fs->gstack_bytes = 0;

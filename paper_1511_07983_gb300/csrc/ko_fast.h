@@ -59,6 +59,7 @@ struct KoFastState {
     int run_limit = 32;         // cap on runs per simulation (tests force the hand-over)
     int stack_global = 1;       // DFS node states in global memory (1) or shared memory (0)
     int lane_shape = 0;         // one-thread pass state: 0 = 14 runs / 56 group slots, 1 = 12 / 40, 2 = 10 / 32
+    bool chosen = false;        // lanes, levels or state were set or tuned: no choice by size (KoRoute)
     void *gstack = nullptr;     // global slab for node states
     size_t gstack_bytes = 0;
     void *lslab = nullptr;      // node-state slab of the one-thread-per-order pass
@@ -74,6 +75,28 @@ bool ko_fast_applicable(const KoSet &h);
 
 // Prefix depth for exhaustive work items of an n-kernel set.
 int ko_fast_d0(const KoFastState &fs, int n);
+
+// How a launch runs: threads per simulation, saved DFS levels, one-thread state.
+struct KoChoice {
+    int lanes, levels, shape;
+};
+// For `count` explicit orders of a set, and for a set's whole space.
+KoChoice ko_list_choice(const KoSet &h, long long count);
+KoChoice ko_space_choice(const KoSet &h);
+
+// Puts a choice into a state whose options were left alone (`always`: into any)
+// for the launches of one call and restores the state's own options at the end
+// of the scope.  A stream being captured takes no allocation: where the state's
+// slabs are too small for the choice, the options it had are used, with as few
+// levels as its slab holds.
+struct KoRoute {
+    KoFastState *fs;
+    int lanes, levels, shape, stack;
+    KoRoute(KoFastState *state, KoChoice c, cudaStream_t st, bool always = false);
+    ~KoRoute();
+    KoRoute(const KoRoute &) = delete;
+    KoRoute &operator=(const KoRoute &) = delete;
+};
 
 // Enqueue one run-length launch over `w` (counters reset here) followed by the
 // device-side fallback for abandoned items.  Fills the counter fields of w.

@@ -238,3 +238,57 @@ def test_edge_gpus_match_oracle(ko, case):
     assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
         (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"])
     assert np.array_equal(hist, st["hist"])
+
+
+# ------------------------------------------------ choice by size (options left alone)
+
+@pytest.mark.parametrize("gpu", [(13, 65536, 49152, 64, 16), (148, 65536, 233472, 64, 32),
+                                 (16, 65536, 49152, 128, 16), (33, 1 << 19, 98304, 64, 32)])
+@pytest.mark.parametrize("n", [1, 2, 6, 7, 8])
+def test_default_space_equals_every_pinned_choice(ko, n, gpu):
+    # N around the lines of the rule, 16 and more SMs, limits outside the packed usage word
+    s = synth.random_set(700 + n, n, gpu=gpu, blk=(1, 5 * gpu[0]), c=(100, 30000))
+    want = oracle.makespans_idx(s.gpu, s.kernels, first=0, count=math.factorial(n))
+    with ko.Gpu.from_set(s) as g:
+        assert np.array_equal(_all(g, n), want)
+        assert ko.ko_get_option(g.h, ko.KO_OPT_LANES) == 16      # the handle's options stay
+        assert ko.ko_get_option(g.h, ko.KO_OPT_LEVELS) == 4
+
+
+@pytest.mark.parametrize("workload,n", [("single8", 8), ("single12", 13), ("single12", 14), ("large", 24)])
+@pytest.mark.parametrize("count", [6144, 6145])
+def test_default_list_equals_a_pinned_choice(ko, workload, n, count):
+    s = synth.gen_set(workload, 5, n=n)
+    rows = synth.random_orders(count, n, count).astype(np.int8)
+    rows[3, 0] = rows[3, 1]                                      # not a permutation
+    with ko.Gpu.from_set(s) as g:
+        got = g.eval_orders(orders=rows)
+    with ko.Gpu.from_set(s) as g:
+        g.configure(lanes=32)
+        want = g.eval_orders(orders=rows)
+    assert np.array_equal(got, want) and got[3] == -1
+    pick = np.arange(0, count, 61)
+    pick = pick[pick != 3]
+    assert np.array_equal(got[pick], oracle.makespans_orders(s.gpu, s.kernels, rows[pick].astype(np.int32)))
+
+
+def test_captured_list_after_a_space_only(ko):
+    """A captured call takes no allocation: with the slabs of an earlier space
+    (whose one-thread state is smaller) and a short list, a long list keeps the
+    handle's options."""
+    import torch
+    s = synth.gen_set("single8", 3, n=9)
+    rows = torch.from_numpy(synth.random_orders(8, 9, 9000).astype(np.int8)).cuda()
+    with ko.Gpu.from_set(s) as g:
+        _all(g, 9)
+        g.eval_orders(orders=rows[:100], out=torch.zeros(100, dtype=torch.int64, device="cuda"))
+        torch.cuda.synchronize()
+        out = torch.zeros(9000, dtype=torch.int64, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            g.eval_orders(orders=rows, out=out)
+        graph.replay()
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+        want = g.eval_orders(orders=rows.cpu().numpy())
+    assert np.array_equal(got, want)

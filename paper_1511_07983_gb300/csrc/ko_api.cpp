@@ -446,6 +446,7 @@ ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, long long *refs,
         if ((s = upload_meta(g, st))) return s;
         KoWork w = work_for(g, 1);
         w.levels = lv.levels;
+        w.space = true;
         w.refs = refs;
         w.accs = d_acc;
         w.out = d_out;
@@ -541,6 +542,7 @@ ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t 
         if ((s = check_cuda(ko_launch_accum_reset(g->d_acc, 1, st)))) return fail(s);
         KoWork w1 = work_for(g, 1);
         w1.levels = lv.levels;
+        w1.space = true;
         w1.refs = &g->d_meta->ref;
         w1.accs = g->d_acc;
         w1.out = g->d_ms;
@@ -731,6 +733,13 @@ ko_batch *ko_batch_create(ko_gpu *const *sets, int32_t nsets, int32_t nbins)
         lanes[i] = sets[i]->fast.lanes;
         stack[i] = sets[i]->fast.stack_global;
         shape[i] = sets[i]->fast.lane_shape;
+        if (!sets[i]->fast.chosen && ko_fast_applicable(sets[i]->h)) {
+            const KoChoice c = ko_space_choice(sets[i]->h, false);
+            lanes[i] = c.lanes;
+            levels[i] = c.levels;
+            shape[i] = c.shape;
+            stack[i] = 1;
+        }
     }
     ko_status err = KO_OK;
     ko_batch *b = ko_batch_build(hs.data(), levels.data(), lanes.data(), stack.data(), shape.data(), nsets, nbins,

@@ -111,6 +111,7 @@ ko_status enqueue(ko_batch *b, cudaStream_t st)
         x.accs = b->d_accs;
         x.out = b->d_ms;
         x.levels = gr.levels;
+        x.space = true;
         b->fast.lanes = gr.lanes;
         b->fast.stack_global = gr.stack;
         b->fast.lane_shape = gr.shape;
@@ -251,6 +252,7 @@ ko_batch *ko_batch_build(const KoSet *const *sets, const int *levels, const int 
         none.nchunks = 1;
         none.n_items = 0;
         none.levels = gr.levels;
+        none.space = true;
         none.reserve_items = longest;
         b->fast.lanes = gr.lanes;
         b->fast.stack_global = gr.stack;
@@ -296,10 +298,10 @@ ko_status ko_batch_exec(ko_batch *b, ko_rank *out, uint64_t *hist, bool hist_dev
         cudaGetLastError();
         return KO_ERR_CUDA;
     }
-    // reset, the reference-order passes (three), each group's passes (three, four with the one-thread pass)
-    ko_count_launch(b->nsets * (b->nbins > 0 ? 1 : 0) + 4 + 3 * (int)b->groups.size() +
-                    (int)std::count_if(b->groups.begin(), b->groups.end(),
-                                       [](const ko_batch::Group &g) { return g.lanes == 1; }));
+    // reset, the reference-order passes (three), each group's passes (three, and one or two one-thread ones)
+    int launches = b->nsets * (b->nbins > 0 ? 1 : 0) + 4;
+    for (const ko_batch::Group &g : b->groups) launches += 3 + (g.lanes != 1 ? 0 : g.shape == 0 ? 1 : 2);
+    ko_count_launch(launches);
     if (hist && b->nbins > 0) {
         const size_t bytes = sizeof(unsigned long long) * b->nbins * b->nsets;
         if (cudaMemcpyAsync(hist, b->d_hist, bytes, hist_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -307,11 +309,11 @@ ko_status ko_batch_exec(ko_batch *b, ko_rank *out, uint64_t *hist, bool hist_dev
             return KO_ERR_CUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return KO_ERR_CUDA;
-    unsigned long long cnt[2] = {0, 0};
+    unsigned long long cnt = 0;
     const unsigned long long *dc = ko_fast_overflow_counter(&b->fast);
-    if (dc && cudaMemcpy(cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost) == cudaSuccess)
-        b->fast.last_overflow = cnt[0];
-    if (cnt[0] > b->fast.ov_cap || cnt[1] > b->fast.ov_cap) return KO_ERR_STATE;  // cannot happen
+    if (dc && cudaMemcpy(&cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost) == cudaSuccess)
+        b->fast.last_overflow = cnt;
+    if (cnt > b->fast.ov_cap) return KO_ERR_STATE;  // cannot happen
     for (int i = 0; i < b->nsets; i++) {
         const KoAccum &a = b->h_accs[i];
         const long long mh = b->h_refs[i];

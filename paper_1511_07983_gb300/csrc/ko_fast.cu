@@ -36,7 +36,10 @@
 //   kG groups in one run, abandons its work item and records it; a second
 //   pass with 32 lanes and 16 group slots re-runs the recorded items, and the
 //   simple simulator takes whatever that pass abandons, all on the stream.
+#include <algorithm>
+
 #include "ko_fast.h"
+#include "ko_units.cuh"
 
 namespace {
 
@@ -645,27 +648,43 @@ fast_kernel(KoWork a)
     if (sim.sg.lane == 0) st.clear();
     sim.init_sms(0);  // a segment without an item still takes part in the warp's event steps
 
+    // a pass over abandoned items takes them in parts where whole ones would leave segments idle
+    __shared__ kounits::Numbering units;
+    if (threadIdx.x == 0) {
+        if (a.item_list) {
+            units = kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, a.space ? a.levels : 0,
+                                         (unsigned long long)gridDim.x * kSegs);
+        } else {
+            units.units = (unsigned long long)a.n_items;
+        }
+    }
+    __syncthreads();
+
     // The warp's segments take consecutive items together and walk them in step: every
     // whole-warp operation below (the fetch's shuffles, the walk's vote, the event vote in
     // place_kernel) is reached by all segments of the warp equally often, and the only exit
     // from this loop is the same for the whole warp.
     constexpr int kPerWarp = 32 / LANES;
     for (;;) {
-        unsigned long long base = 0, lim = 0;
-        if ((threadIdx.x & 31) == 0) {
-            base = atomicAdd(a.counter, (unsigned long long)kPerWarp);
-            lim = (unsigned long long)a.n_items;
-            if (a.item_list)  // pass over items a previous pass abandoned
-                lim = *a.item_count < a.ov_cap ? *a.item_count : a.ov_cap;
-        }
+        unsigned long long base = 0;
+        if ((threadIdx.x & 31) == 0) base = atomicAdd(a.counter, (unsigned long long)kPerWarp);
         base = __shfl_sync(kAll, base, 0);
-        lim = __shfl_sync(kAll, lim, 0);
-        if (base >= lim) break;
+        if (base >= units.units) break;
         unsigned long long item = base + half;
-        bool have = item < lim;  // an odd tail leaves the last segment without an item
-        if (have && a.item_list) item = a.item_list[item];
+        bool have = item < units.units;  // an odd tail leaves the last segment without a unit
+        unsigned part = 0, list_part = 0;
+        int cut = 0, list_cut = 0;
+        if (have && a.item_list) {
+            const kounits::Unit un = kounits::unit_at(units, item);
+            const unsigned long long entry = a.item_list[un.item];
+            item = entry & kounits::kItemMask;
+            list_part = (unsigned)((entry >> kounits::kItemBits) & kounits::kPartMask);
+            list_cut = (int)(entry >> (kounits::kItemBits + kounits::kPartBits));
+            part = un.part;
+            cut = un.x;
+        }
         have = have && item < (unsigned long long)a.n_items;
-        // the index an abandoned item is recorded under: the later passes take items in plain
+        // the entry an abandoned item is recorded under: the later passes take items in plain
         // order, so a reordered prefix is recorded as the item that plain order maps to it
         unsigned long long rec = item;
 
@@ -675,8 +694,19 @@ fast_kernel(KoWork a)
         int n = 0, d0 = 0, depth = 0;
         uint32_t all = 0, used = 0;
         bool first_child = true;
+        KoChunk ch{};
         if (have) {
-            const KoChunk ch = a.chunks[find_chunk(a.chunks, a.nchunks, (long long)item)];
+            ch = a.chunks[find_chunk(a.chunks, a.nchunks, (long long)item)];
+            if (a.item_list) {
+                const kounits::Unit un =
+                    kounits::cut_unit(item, list_part, list_cut, ch.mode == 0 ? a.sets[ch.set].n - ch.d0 : 0, cut, part);
+                have = un.valid;
+                part = un.part;
+                cut = un.x;
+                rec = kounits::entry_of(item, part, cut);
+            }
+        }
+        if (have) {
             if (ch.set != loaded) {
                 load_set<LANES>(K, a.sets + ch.set, sim.sg);
                 loaded = ch.set;
@@ -708,7 +738,7 @@ fast_kernel(KoWork a)
                     used |= 1u << v;
                 }
             } else {
-                d0 = ch.d0;
+                d0 = ch.d0 + cut;
                 unsigned long long j = (unsigned long long)(ch.list_off + local);
                 // swap partners pair up only in a pass over whole chunks; an item taken from a
                 // list of abandoned items is run as the item it names
@@ -717,7 +747,7 @@ fast_kernel(KoWork a)
                                         (unsigned long long)(ch.list_off + ch.count));
                     rec = (unsigned long long)ch.first + (j - (unsigned long long)ch.list_off);
                 }
-                const unsigned long long first = j * c_fact[n - d0];
+                const unsigned long long first = j * c_fact[n - ch.d0] + part * c_fact[n - d0];
                 outpos = ch.out_off + (long long)first;
                 lehmer_prefix(n, first, d0, perm, used);
             }
@@ -806,6 +836,7 @@ fast_kernel(KoWork a)
             if (sim.fail) {
                 const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
                 if (slot < a.ov_cap) a.ov_list[slot] = rec;
+                if (!a.item_list) atomicAdd(a.abandoned, 1ull);
             } else {
                 st.add(is);
             }
@@ -814,10 +845,15 @@ fast_kernel(KoWork a)
     if (sim.sg.lane == 0) st.flush(a.accs, st_set);
 }
 
+// Lists of abandoned units: one per pass that can abandon any (two one-thread
+// passes, the 16-lane and the wide one).
+constexpr int kLists = 4;
+
 // Device buffer layout inside KoFastState::buf.
 struct FastBuf {
-    unsigned long long counter[3], ov_count[3], fb_counter, pad[1];
-    unsigned long long ov_list[1];   // KoFastState::ov_cap entries per pass
+    unsigned long long counter[kLists], ov_count[kLists], fb_counter, abandoned;
+    unsigned int part_seen[kPartSeen / 32];
+    unsigned long long ov_list[1];   // KoFastState::ov_cap entries per list
 };
 
 constexpr size_t kFallbackScratch = size_t(256) << 20;
@@ -843,7 +879,7 @@ cudaError_t launch(const KoWork &a, cudaStream_t st)
     }
     const long long work = a.item_list ? (long long)a.ov_cap : a.n_items;
     const long long blocks_needed = (work + kThreads / LANES - 1) / (kThreads / LANES);
-    if (blocks > blocks_needed) blocks = blocks_needed;
+    if (blocks > blocks_needed && !(a.item_list && a.space)) blocks = blocks_needed;
     if (blocks < 1) blocks = 1;
     fast_kernel<LANES, G, SAVE><<<(unsigned)blocks, kThreads, smem, st>>>(a);
     ko_count_launch();
@@ -906,19 +942,20 @@ KoChoice ko_list_choice(const KoSet &h, long long count)
 // with the state's default; N=9, 148 SMs: 2.1 ms with one level, 4.9 with three,
 // 22 with the default).  The 12-run state holds spaces on up to 16 SMs (N=9,
 // 13 SMs: 1.21 ms against 1.44 with 14 runs); on 148 SMs it hands on too many
-// items (N=10: 20.6 against 16.2 ms).
-KoChoice ko_space_choice(const KoSet &h)
+// items (N=10: 20.6 against 16.2 ms).  In a batch every set takes one thread per
+// item: its other sets fill the chip, and each choice is a launch of its own.
+KoChoice ko_space_choice(const KoSet &h, bool alone)
 {
     const int n = h.n;
-    if (n <= 6) return KoChoice{32, 0, 0};
+    if (n <= 6 && alone) return KoChoice{32, 0, 0};
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long want = 4ll * sms * 288;
+    const unsigned long long want = 4ull * sms * 288;
     const int deepest = h.S <= 16 ? 3 : 4;  // a deeper item that overflows hands on more orders
     int levels = 0;
-    long long items = 1;
-    for (int i = 2; i <= n; i++) items *= i;
+    unsigned long long items = 1;
+    for (int i = 2; i <= n; i++) items *= (unsigned long long)i;
     while (levels < deepest && levels + 1 < n && items / (levels + 2) >= want) items /= ++levels + 1;
     if (!packs(h)) return KoChoice{16, levels, 0};
     return KoChoice{1, levels, h.S <= 16 ? 1 : 0};
@@ -952,7 +989,7 @@ KoRoute::KoRoute(KoFastState *state, KoChoice c, cudaStream_t st, bool always)
     if (fs->chosen && !always) return;
     fs->stack_global = 1;
     if (capturing(st) && (fs->gstack_bytes < gstack_need(c.levels) ||
-                          (c.lanes == 1 && fs->lslab_bytes < ko_lane_slab_bytes(c.levels, c.shape)))) {
+                          (c.lanes == 1 && fs->lslab_bytes < std::max(ko_lane_slab_bytes(c.levels, c.shape), ko_lane_slab_bytes(c.levels, 0))))) {
         while (fs->levels > 1 && fs->gstack_bytes < gstack_need(fs->levels)) fs->levels--;
         return;
     }
@@ -971,14 +1008,18 @@ KoRoute::~KoRoute()
 
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st)
 {
-    // a pass abandons an item at most once, so lists as long as the launch's work lose none
+    // a pass abandons a unit at most once, so lists as long as the units a pass may number lose none
     unsigned long long want = (unsigned long long)(w.n_items > w.reserve_items ? w.n_items : w.reserve_items);
+    if (fs->lanes == 1 && w.space) {
+        const unsigned long long threads = (unsigned long long)std::max(ko_lane_threads(fs->lane_shape), ko_lane_threads(0));
+        want += threads * kounits::parts(w.levels + 1, 1) + (threads + 1) * kounits::parts(w.levels + 1, 2);
+    }
     want = ((want < 1024 ? 1024 : want) + 1023) & ~1023ull;
     if (fs->ov_cap < want) {
         // a stream being captured cannot take a free or a malloc: the caller
         // must size the lists with an uncaptured launch first
         if (capturing(st)) return KO_ERR_STATE;
-        const size_t need = sizeof(FastBuf) + sizeof(unsigned long long) * 3 * (size_t)want;
+        const size_t need = sizeof(FastBuf) + sizeof(unsigned long long) * kLists * (size_t)want;
         cudaFree(fs->buf);
         fs->buf = nullptr;
         fs->cap = 0;
@@ -1000,7 +1041,8 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     const bool lane = fs->lanes == 1;
     if (lane) {
         // one-thread-per-order pass: a node-state slab for every thread it runs
-        const size_t need = ko_lane_slab_bytes(w.levels < 1 ? 1 : w.levels, fs->lane_shape);
+        const int lv = w.levels < 1 ? 1 : w.levels;
+        const size_t need = std::max(ko_lane_slab_bytes(lv, fs->lane_shape), ko_lane_slab_bytes(lv, 0));
         if (fs->lslab_bytes < need) {
             if (capturing(st)) return KO_ERR_STATE;
             cudaFree(fs->lslab);
@@ -1035,30 +1077,36 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     if (w.levels < 1) w.levels = 1;
     if (w.levels > kMaxLevels) w.levels = kMaxLevels;
     w.ov_cap = fs->ov_cap;
-    w.item_list = nullptr;
-    w.item_count = nullptr;
-    int list = 0;  // abandoned-item list the next pass writes
+    w.abandoned = &fb->abandoned;
+    w.part_seen = fb->part_seen;
+    int list = 0;  // list the next pass writes; it reads the one before
+    auto next_pass = [&](KoWork &x) {
+        x.counter = &fb->counter[list];
+        x.item_list = list ? fb->ov_list + (list - 1) * fs->ov_cap : nullptr;
+        x.item_count = list ? &fb->ov_count[list - 1] : nullptr;
+        x.ov_count = &fb->ov_count[list];
+        x.ov_list = fb->ov_list + list * fs->ov_cap;
+        list++;
+    };
     cudaError_t e = cudaSuccess;
     if (lane) {
-        // pass 0: all items, one simulation per thread
+        // all items, one simulation per thread; what a smaller state cannot hold goes to the largest
+        // one before any run-length pass (48 mixed sets in one graph: the 16-lane pass over what the
+        // 12-run state handed on took 51 of 180 ms)
         KoWork w0 = w;
-        w0.counter = &fb->counter[2];
-        w0.ov_count = &fb->ov_count[0];
-        w0.ov_list = fb->ov_list;
         w0.gstack = (int *)fs->lslab;
         w0.gstack_words = (long long)(fs->lslab_bytes / sizeof(int));
-        if ((e = ko_launch_lane(w0, fs->lane_shape, st)) != cudaSuccess) {
-            cudaGetLastError();
-            return KO_ERR_CUDA;
+        for (int shape = fs->lane_shape;; shape = 0) {
+            next_pass(w0);
+            if ((e = ko_launch_lane(w0, shape, st)) != cudaSuccess) {
+                cudaGetLastError();
+                return KO_ERR_CUDA;
+            }
+            if (shape == 0) break;
         }
-        w.item_list = fb->ov_list;
-        w.item_count = &fb->ov_count[0];
-        list = 1;
     }
-    // pass 1: all items (or those pass 0 abandoned), 16 lanes per run-length simulation, 8 group slots
-    w.counter = &fb->counter[0];
-    w.ov_count = &fb->ov_count[list];
-    w.ov_list = fb->ov_list + list * fs->ov_cap;
+    // all items (or those the one-thread passes abandoned), 16 or 32 lanes per simulation, 8 group slots
+    next_pass(w);
     w.gstack = fs->stack_global ? (int *)fs->gstack : nullptr;
     w.gstack_words = fs->stack_global ? (long long)(fs->gstack_bytes / sizeof(int)) : 0;
     e = fs->lanes == 32 ? launch<32, kG, 16>(w, st) : launch<16, kG, 16>(w, st);
@@ -1066,22 +1114,17 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         cudaGetLastError();
         return KO_ERR_CUDA;
     }
-    // pass 2: the items pass 1 abandoned, 32 lanes and 16 group slots per run
+    // the items that pass abandoned, 32 lanes and 16 group slots per run
     KoWork w2 = w;
     w2.gstack = nullptr;  // the wide pass keeps its (32-lane) node states in shared memory
     w2.gstack_words = 0;
-    w2.counter = &fb->counter[1];
-    w2.item_list = fb->ov_list + list * fs->ov_cap;
-    w2.item_count = &fb->ov_count[list];
-    w2.ov_count = &fb->ov_count[list + 1];
-    w2.ov_list = fb->ov_list + (list + 1) * fs->ov_cap;
-    w2.run_limit = fs->run_limit;
+    next_pass(w2);
     e = launch<32, kGWide, 32>(w2, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return KO_ERR_CUDA;
     }
-    // pass 3: whatever is left, simple simulator
+    // whatever is left, simple simulator
     KoWork w3 = w2;
     w3.fb_counter = &fb->fb_counter;
     e = ko_launch_fallback(w3, fs->fb_scratch, fs->fb_bytes, max_slab_bytes, st);
@@ -1094,7 +1137,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
 
 const unsigned long long *ko_fast_overflow_counter(const KoFastState *fs)
 {
-    return fs->buf ? &((const FastBuf *)fs->buf)->ov_count[0] : nullptr;
+    return fs->buf ? &((const FastBuf *)fs->buf)->abandoned : nullptr;
 }
 
 void ko_fast_release(KoFastState *fs)

@@ -18,6 +18,8 @@ struct KoChunk {
     long long out_off;   // added to the output position (mode 0: Lehmer index; 1/2: item)
 };
 
+constexpr int kPartSeen = 1 << 17;  // items with parts a first pass may number (bits of KoWork::part_seen)
+
 // Parameters of one simulator launch (passed by value to the kernels).
 struct KoWork {
     const KoSet *sets;
@@ -32,12 +34,15 @@ struct KoWork {
     int64_t *out;                     // makespans, or null
     unsigned long long *counter;      // next work item
     unsigned long long *ov_count;     // items abandoned by the run-length simulator
-    unsigned long long *ov_list;      // their global item indices
+    unsigned long long *ov_list;      // their list entries (ko_units.cuh)
+    unsigned long long *abandoned;    // work items the first pass abandoned (whole or in part)
+    unsigned int *part_seen;          // first pass: items with an abandoned part, one bit each
     unsigned long long ov_cap;
     unsigned long long *fb_counter;   // next abandoned item for the fallback
     const unsigned long long *item_list;   // non-null: work items are item_list[0 .. *item_count)
     const unsigned long long *item_count;
     int levels;                       // saved DFS levels per segment
+    bool space;                       // the chunks are prefixes (mode 0): their items may be cut into parts
     int run_limit;                    // runs one simulation may hold
     int *gstack;                      // non-null: DFS node states in this global slab, not shared memory
     long long gstack_words;           // words of gstack (bounds the segments that may use it)
@@ -80,9 +85,10 @@ int ko_fast_d0(const KoFastState &fs, int n);
 struct KoChoice {
     int lanes, levels, shape;
 };
-// For `count` explicit orders of a set, and for a set's whole space.
+// For `count` explicit orders of a set, and for a set's whole space (`alone`: the
+// only one of its launch).
 KoChoice ko_list_choice(const KoSet &h, long long count);
-KoChoice ko_space_choice(const KoSet &h);
+KoChoice ko_space_choice(const KoSet &h, bool alone = true);
 
 // Puts a choice into a state whose options were left alone (`always`: into any)
 // for the launches of one call and restores the state's own options at the end
@@ -102,8 +108,8 @@ struct KoRoute {
 // device-side fallback for abandoned items.  Fills the counter fields of w.
 // Asynchronous, graph-capturable (no host synchronisation) once an earlier
 // launch outside capture has sized the buffers: each abandoned-item list holds
-// max(w.n_items, w.reserve_items) entries, so no abandoned item is ever lost
-// (a pass abandons an item at most once).
+// the units a pass may number (ko_units.cuh), so no abandoned item is ever lost
+// (a pass abandons a unit at most once).
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st);
 
 // One-thread-per-order pass (ko_lane.cu) over the items of `w` (counters and
@@ -111,9 +117,9 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
 // ko_lane_slab_bytes(w.levels, shape) bytes); shape as KoFastState::lane_shape.
 cudaError_t ko_launch_lane(const KoWork &w, int shape, cudaStream_t st);
 size_t ko_lane_slab_bytes(int levels, int shape);
+long long ko_lane_threads(int shape);  // simulations a full launch runs at a time
 
-// Device address of the count of items the first pass of the last launch
-// abandoned (followed by the count the wide second pass abandoned).
+// Device address of the count of items the first pass of the last launch abandoned.
 const unsigned long long *ko_fast_overflow_counter(const KoFastState *fs);
 
 void ko_fast_release(KoFastState *fs);

@@ -17,6 +17,7 @@
 // simulation holds is recorded for the run-length simulator, which re-runs it.
 #include "ko_fast.h"
 #include "ko_lane_sim.cuh"
+#include "ko_units.cuh"
 
 namespace {
 
@@ -94,6 +95,23 @@ __device__ __forceinline__ void save_node(const SIM &sim, uint32_t *node)
         __stcg(dst + SH::kWords / 4 + f, make_uint4(r[4 * f], r[4 * f + 1], r[4 * f + 2], r[4 * f + 3]));
 }
 
+// Record a unit for the next pass, and its item among those the first pass
+// abandoned: items from `cut_from` on may have several such parts.
+__device__ __forceinline__ void abandon(const KoWork &a, unsigned long long rec, unsigned long long cut_from)
+{
+    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
+    if (slot < a.ov_cap) a.ov_list[slot] = rec;
+    if (a.item_list) return;
+    const unsigned long long item = rec & kounits::kItemMask;
+    bool seen = false;
+    if (item >= cut_from) {
+        const unsigned long long i = item - cut_from;  // < the grid's threads
+        const unsigned bit = 1u << (i & 31u);
+        if (i < (unsigned long long)kPartSeen) seen = (atomicOr(&a.part_seen[i >> 5], bit) & bit) != 0u;
+    }
+    if (!seen) atomicAdd(a.abandoned, 1ull);
+}
+
 enum Phase : int { PH_FETCH = 0, PH_NEXT, PH_START, PH_EVENT, PH_FINAL, PH_PLACED, PH_DONE };
 
 template <int T, class SH>
@@ -110,6 +128,16 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
     uint32_t *slab = reinterpret_cast<uint32_t *>(a.gstack) + gtid * levels * kSaveWords;
     // a thread without slab room takes no work (the host sizes the grid so this never happens)
     int phase = (gtid + 1) * levels * kSaveWords <= a.gstack_words ? PH_FETCH : PH_DONE;
+
+    // the pass's units: parts of items where whole items would leave threads idle
+    __shared__ kounits::Numbering units;
+    if (threadIdx.x == 0) {
+        const int lv = a.space ? levels : 0;
+        const unsigned long long threads = (unsigned long long)gridDim.x * T;
+        units = a.item_list ? kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, lv, threads)
+                            : kounits::number_space((unsigned long long)a.n_items, lv, threads);
+    }
+    __syncthreads();
 
     // current work item
     const KoSet *set = nullptr;
@@ -134,8 +162,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                 // a step frees a block, or takes one of the first burst's runs or pending groups
                 if (!sim.fail && ++events > total_blocks + 256) sim.fail = 1;
                 if (sim.fail) {
-                    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                    if (slot < a.ov_cap) a.ov_list[slot] = rec;
+                    abandon(a, rec, units.a);
                     phase = PH_FETCH;
                 } else if (last) {
                     phase = PH_FINAL;  // the queue empties only in place_partial
@@ -149,8 +176,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
             if (phase == PH_FINAL) {  // the head kernel's last burst, deferred from its event
                 sim.place_partial(left);
                 if (sim.fail) {
-                    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                    if (slot < a.ov_cap) a.ov_list[slot] = rec;
+                    abandon(a, rec, units.a);
                     phase = PH_FETCH;
                 } else {
                     phase = PH_PLACED;
@@ -217,13 +243,22 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
             if (phase == PH_FETCH) {
                 for (;;) {  // until an item starts or the list is exhausted
                     const unsigned long long base = atomicAdd(a.counter, 1ull);
-                    unsigned long long lim = (unsigned long long)a.n_items;
-                    if (a.item_list) lim = *a.item_count < a.ov_cap ? *a.item_count : a.ov_cap;
-                    if (base >= lim) { phase = PH_DONE; break; }
-                    unsigned long long item = a.item_list ? a.item_list[base] : base;
+                    if (base >= units.units) { phase = PH_DONE; break; }
+                    kounits::Unit un = kounits::unit_at(units, base);
+                    unsigned part = 0;
+                    int fixed = 0;
+                    if (a.item_list) {
+                        const unsigned long long entry = a.item_list[un.item];
+                        un.item = entry & kounits::kItemMask;
+                        part = (unsigned)((entry >> kounits::kItemBits) & kounits::kPartMask);
+                        fixed = (int)(entry >> (kounits::kItemBits + kounits::kPartBits));
+                    }
+                    const unsigned long long item = un.item;
                     if (item >= (unsigned long long)a.n_items) continue;
-                    rec = item;
                     const KoChunk ch = a.chunks[lane_find_chunk(a.chunks, a.nchunks, (long long)item)];
+                    un = kounits::cut_unit(item, part, fixed, ch.mode == 0 ? a.sets[ch.set].n - ch.d0 : 0, un.x, un.part);
+                    if (!un.valid) continue;
+                    rec = kounits::entry_of(item, un.part, un.x);
                     set_id = ch.set;
                     set = a.sets + ch.set;
                     n = set->n;
@@ -253,9 +288,10 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                             seen |= 1u << v;
                         }
                     } else {
-                        d0 = ch.d0;
+                        d0 = ch.d0 + un.x;
                         const unsigned long long first =
-                            (unsigned long long)(ch.list_off + local) * c_lane_fact[n - d0];
+                            (unsigned long long)(ch.list_off + local) * c_lane_fact[n - ch.d0] +
+                            (unsigned long long)un.part * c_lane_fact[n - d0];
                         outpos = ch.out_off + (long long)first;
                         lk = first;
                     }
@@ -264,8 +300,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
                         continue;
                     }
                     if (set->R >= (1 << 19) || set->W > 127) {  // outside the packed usage word
-                        const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                        if (slot < a.ov_cap) a.ov_list[slot] = rec;
+                        abandon(a, rec, units.a);
                         continue;
                     }
                     mn = ~0ull; mx = 0; nb = ne = nw = 0;
@@ -347,7 +382,10 @@ cudaError_t launch_lane(const KoWork &a, cudaStream_t st)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int levels = a.levels < 1 ? 1 : a.levels;
-    const long long work = a.item_list ? (long long)a.ov_cap : a.n_items;
+    // units the pass may number: of a list, as many as the grid has threads
+    long long work = a.item_list ? (long long)a.ov_cap : a.n_items;
+    if (a.space && a.item_list) work = (long long)sms * T;
+    else if (a.space && work < (long long)sms * T) work *= kounits::parts(levels + 1, 2);
     const long long needed = (work + T - 1) / T;
     if (needed < sms && work > 0) {
         // fewer items than SMs x T: blocks of kSmallT threads, one item per thread at most
@@ -367,6 +405,16 @@ cudaError_t launch_lane(const KoWork &a, cudaStream_t st)
 }
 
 }  // namespace
+
+long long ko_lane_threads(int shape)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return (long long)sms * (shape == 2   ? lane_threads<ShapeS>()
+                             : shape == 1 ? lane_threads<ShapeM>()
+                                          : lane_threads<ShapeL>());
+}
 
 size_t ko_lane_slab_bytes(int levels, int shape)
 {

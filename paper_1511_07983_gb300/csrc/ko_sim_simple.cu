@@ -21,6 +21,7 @@
 
 #include "ko_internal.h"
 #include "ko_fast.h"
+#include "ko_units.cuh"
 
 namespace {
 
@@ -300,8 +301,8 @@ __device__ __forceinline__ int find_chunk_simple(const KoChunk *chunks, int nchu
     return lo;
 }
 
-// Re-runs the work items the run-length simulator abandoned: one warp per
-// item, lanes split the item's orders; same outputs and accumulators.
+// Re-runs the units the run-length simulator abandoned: one warp per
+// unit, lanes split the unit's orders; same outputs and accumulators.
 __global__ void __launch_bounds__(kThreads)
 fallback_kernel(KoWork w, void *scratch, size_t per_thread)
 {
@@ -313,21 +314,25 @@ fallback_kernel(KoWork w, void *scratch, size_t per_thread)
         if (lane == 0) e = atomicAdd(w.fb_counter, 1ull);
         e = __shfl_sync(0xffffffffu, e, 0);
         if (e >= total) break;
-        const long long item = (long long)w.ov_list[e];
+        const unsigned long long entry = w.ov_list[e];
+        const long long item = (long long)(entry & kounits::kItemMask);
+        const unsigned long long part = (entry >> kounits::kItemBits) & kounits::kPartMask;
+        const int cut = (int)(entry >> (kounits::kItemBits + kounits::kPartBits));
         const KoChunk ch = w.chunks[find_chunk_simple(w.chunks, w.nchunks, item)];
         const KoSet &d = w.sets[ch.set];
         const Slab st = slab_at(scratch, per_thread, d.S, d.Bk, slot);
         const int n = d.n;
         const long long local = item - ch.first;
         const long long ref = w.refs ? w.refs[ch.set] : d.ref_makespan;
-        const unsigned long long span = ch.mode == 0 ? c_fact[n - ch.d0] : 1ull;
+        const unsigned long long span = ch.mode == 0 ? c_fact[n - ch.d0 - cut] : 1ull;
         unsigned long long lmin = ~0ull, lmax = 0, nb = 0, ne = 0, nw = 0;
         for (unsigned long long o = lane; o < span; o += 32) {
             int8_t perm[KO_MAX_KERNELS];
             bool ok = true;
             long long outpos;
             if (ch.mode == 0) {
-                const unsigned long long k = (unsigned long long)(ch.list_off + local) * span + o;
+                const unsigned long long k =
+                    (unsigned long long)(ch.list_off + local) * c_fact[n - ch.d0] + part * span + o;
                 outpos = ch.out_off + (long long)k;
                 unrank(n, k, perm);
             } else if (ch.mode == 1) {

@@ -223,6 +223,7 @@ double ko_tune_measure(KoFastState *fs, const KoSet &h, const KoSet *d_set, KoCh
     w.n_items = items;
     w.accs = d_acc;
     w.levels = n - 1 - d0 > 0 ? n - 1 - d0 : 1;
+    w.space = true;
     return time_candidate(fs, w, d_acc, 1, items * span, cand.lanes, cand.stack, cand.shape, ko_slab_bytes(h.S, h.Bk),
                           reps, st);
 }
@@ -348,6 +349,7 @@ ko_status ko_tune_batch(const KoSet *const *hs, int nsets, const char *cache_pat
                 w.n_items = first;
                 w.accs = d_accs;
                 w.levels = std::max(1, h0.n - 1 - d0);
+                w.space = true;
                 const double r = time_candidate(&fs, w, d_accs, (int)sample.size(), orders, c.lanes, c.stack,
                                                 c.shape, slab, warmed ? 1 : 2, st);
                 warmed = true;

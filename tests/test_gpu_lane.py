@@ -196,3 +196,30 @@ def test_whole_space_items_beside_deeper_walks(ko, state):
             (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"]), s.n
     # the largest state finishes these small GPUs' items itself (the smaller ones may hand some over)
     assert state > 0 or moved == 0
+
+
+@pytest.mark.parametrize("workload,n,levels,state,run_limit", [
+    ("sets10", 8, 2, 0, 6), ("sets10", 8, 5, 1, 6), ("sets10", 7, 6, 2, 4),
+    ("single12", 9, 2, 0, 32), ("single12", 9, 3, 2, 32), ("single12", 9, 5, 1, 32), ("single12", 10, 2, 1, 32)])
+def test_cut_items_cover_the_space_once(ko, workload, n, levels, state, run_limit):
+    """A pass cuts its last items (all of them below one item per thread) into
+    parts, and so do the passes over what it abandons (a run limit makes many):
+    every order's makespan and one count per order, as without parts."""
+    import torch
+    s = synth.gen_set(workload, 6, n=n)
+    n_all = math.factorial(n)
+    h = list(range(n))
+    with ko.Gpu.from_set(s) as g:
+        g.configure(lanes=16, levels=3)
+        want = torch.empty(n_all, dtype=torch.int64, device="cuda")
+        g.eval_all(want)
+        rw, hw = g.rank_order(h, nbins=512)
+    with ko.Gpu.from_set(s) as g:
+        g.configure(lanes=1, levels=levels, lane_state=state, run_limit=run_limit)
+        got = torch.full((n_all,), -7, dtype=torch.int64, device="cuda")
+        g.eval_all(got)
+        moved = g.last_fallback_items()
+        rg, hg = g.rank_order(h, nbins=512)
+    assert torch.equal(got, want)
+    assert rg == rw and np.array_equal(hg, hw)
+    assert moved <= n_all // math.factorial(min(levels, n - 1) + 1) and (run_limit == 32 or moved > 0)

@@ -54,10 +54,7 @@ bool is_device_ptr(const void *p)
 
 // Small per-call device records of a handle.
 struct Meta {
-    KoChunk chunk[2];                 // [0] heuristic order (mode 2), [1] the main work
-    long long ref;                    // reference makespan written by the heuristic pass
-    long long pad;
-    int8_t perm[KO_MAX_KERNELS + 8];  // heuristic / ranked order
+    KoChunk chunk;  // the call's work
 };
 
 }  // namespace
@@ -157,23 +154,23 @@ ko_status upload_meta(ko_gpu *g, cudaStream_t st)
     return KO_OK;
 }
 
-KoWork work_for(ko_gpu *g, int chunk)
+KoWork work_for(ko_gpu *g)
 {
     KoWork w{};
     w.sets = g->d_set;
-    w.chunks = &g->d_meta->chunk[chunk];
+    w.chunks = &g->d_meta->chunk;
     w.nchunks = 1;
-    w.n_items = g->h_meta.chunk[chunk].count;
+    w.n_items = g->h_meta.chunk.count;
     w.levels = 1;
     return w;
 }
 
-// Exhaustive chunk (all N! orders as prefix items) into h_meta.chunk[1].
+// Exhaustive chunk (all N! orders as prefix items) into h_meta.chunk.
 void exhaustive_chunk(ko_gpu *g, KoWork *w_levels)
 {
     const int N = g->h.n;
     const int d0 = ko_fast_d0(g->fast, N);
-    KoChunk &c = g->h_meta.chunk[1];
+    KoChunk &c = g->h_meta.chunk;
     c = KoChunk{};
     c.first = 0;
     c.count = kFactorial[N] / kFactorial[N - d0];
@@ -391,14 +388,14 @@ ko_status ko_eval_orders(ko_gpu *g, const uint64_t *idx, const int8_t *orders, i
     int64_t *d_out = out_dev ? makespan_out : (int64_t *)stage;
     bool used_fast = false;
     if (fast_ok(g)) {
-        KoChunk &c = g->h_meta.chunk[1];
+        KoChunk &c = g->h_meta.chunk;
         c = KoChunk{};
         c.count = n;
         c.d0 = N;
         c.mode = idx ? 1 : 2;
         KoRoute route(&g->fast, ko_list_choice(g->h, n), st);
         if ((s = upload_meta(g, st))) return fail(s);
-        KoWork w = work_for(g, 1);
+        KoWork w = work_for(g);
         w.idx = idx ? (const uint64_t *)d_in : nullptr;
         w.perms = idx ? nullptr : (const int8_t *)d_in;
         w.out = d_out;
@@ -432,9 +429,8 @@ ko_status ko_eval_orders(ko_gpu *g, const uint64_t *idx, const int8_t *orders, i
 
 namespace {
 
-// All N! makespans into d_out (device, nullable) and the accumulator, on
-// `st`; with `refs` the counts compare against *refs (device).
-ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, long long *refs, cudaStream_t st)
+// All N! makespans into d_out (device, nullable) and the accumulator, on `st`.
+ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, cudaStream_t st)
 {
     const int64_t total = kFactorial[g->h.n];
     ko_status s = check_cuda(ko_launch_accum_reset(d_acc, 1, st));
@@ -444,10 +440,9 @@ ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, long long *refs,
         KoWork lv;
         exhaustive_chunk(g, &lv);
         if ((s = upload_meta(g, st))) return s;
-        KoWork w = work_for(g, 1);
+        KoWork w = work_for(g);
         w.levels = lv.levels;
         w.space = true;
-        w.refs = refs;
         w.accs = d_acc;
         w.out = d_out;
         return fast_launch_timed(g, w, st);
@@ -455,28 +450,6 @@ ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, long long *refs,
     if ((s = simple_scratch(g, total))) return s;
     return check_cuda(ko_launch_simple(g->d_set, g->h, nullptr, nullptr, 0, total, d_out, d_acc,
                                        g->scratch, g->scratch_bytes, st));
-}
-
-ko_status makespan_of(ko_gpu *g, const int32_t *order, int64_t *m, cudaStream_t st)
-{
-    const int N = g->h.n;
-    int8_t perm[KO_MAX_KERNELS];
-    for (int i = 0; i < N; i++) perm[i] = (int8_t)order[i];
-    ko_status s = grow(&g->d_stage, &g->stage_cap, 256 + sizeof(int64_t));
-    if (s) return s;
-    int8_t *d_perm = (int8_t *)g->d_stage;
-    int64_t *d_m = (int64_t *)((char *)g->d_stage + 256);
-    if (cudaMemcpyAsync(d_perm, perm, N, cudaMemcpyHostToDevice, st) != cudaSuccess) return KO_ERR_CUDA;
-    g->h2d += N;
-    if ((s = simple_scratch(g, 1))) return s;
-    if ((s = check_cuda(ko_launch_simple(g->d_set, g->h, d_perm, nullptr, 0, 1, d_m, nullptr,
-                                         g->scratch, g->scratch_bytes, st))))
-        return s;
-    if (cudaMemcpyAsync(m, d_m, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return KO_ERR_CUDA;
-    g->d2h += sizeof(int64_t);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return KO_ERR_CUDA;
-    return KO_OK;
 }
 
 }  // namespace
@@ -492,7 +465,7 @@ ko_status ko_eval_all(ko_gpu *g, int64_t *makespans_out, void *stream)
     g->h.ref_makespan = 0;
     ko_status s = prepare(g, st);
     if (s) return fail(s);
-    if ((s = exhaustive(g, makespans_out, g->d_acc, nullptr, st))) return fail(s);
+    if ((s = exhaustive(g, makespans_out, g->d_acc, st))) return fail(s);
     g->fast_pending = fast_ok(g);
     return ok();
 }
@@ -516,44 +489,22 @@ ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t 
         ko_heuristic_host(g->h, ord.data());
     }
     const int64_t total = kFactorial[N];
+    // the ranked order's position in the space: lexicographic (Lehmer) index
+    int64_t at = 0;
+    for (int i = 0; i < N; i++) {
+        int smaller = 0;
+        for (int j = i + 1; j < N; j++) smaller += ord[j] < ord[i];
+        at += smaller * kFactorial[N - 1 - i];
+    }
     g->h.ref_makespan = 0;
     ko_status s = prepare(g, st);
     if (s) return fail(s);
     if ((s = grow((void **)&g->d_ms, &g->ms_cap, sizeof(int64_t) * total))) return fail(s);
-    int64_t mh = 0;
     const bool fast = fast_ok(g);
-    if (fast) {
-        // pass 1: makespan of the ranked order into d_meta->ref (device);
-        // pass 2: all N! orders, counted against that reference
-        KoChunk &c0 = g->h_meta.chunk[0];
-        c0 = KoChunk{};
-        c0.count = 1;
-        c0.d0 = N;
-        c0.mode = 2;
-        for (int i = 0; i < N; i++) g->h_meta.perm[i] = (int8_t)ord[i];
-        KoRoute route(&g->fast, ko_space_choice(g->h), st);
-        KoWork lv;
-        exhaustive_chunk(g, &lv);
-        if ((s = upload_meta(g, st))) return fail(s);
-        KoWork w0 = work_for(g, 0);
-        w0.perms = g->d_meta->perm;
-        w0.out = (int64_t *)&g->d_meta->ref;
-        if ((s = ko_fast_launch(&g->fast, w0, ko_slab_bytes(g->h.S, g->h.Bk), st))) return fail(s);
-        if ((s = check_cuda(ko_launch_accum_reset(g->d_acc, 1, st)))) return fail(s);
-        KoWork w1 = work_for(g, 1);
-        w1.levels = lv.levels;
-        w1.space = true;
-        w1.refs = &g->d_meta->ref;
-        w1.accs = g->d_acc;
-        w1.out = g->d_ms;
-        if ((s = fast_launch_timed(g, w1, st))) return fail(s);
-    } else {
-        if ((s = makespan_of(g, ord.data(), &mh, st))) return fail(s);
-        if (mh < 0) return fail(KO_ERR_STATE);
-        g->h.ref_makespan = mh;
-        if ((s = prepare(g, st))) return fail(s);
-        if ((s = exhaustive(g, g->d_ms, g->d_acc, nullptr, st))) return fail(s);
-    }
+    if ((s = check_cuda(ko_launch_accum_reset(g->d_acc + 1, 1, st)))) return fail(s);
+    if ((s = exhaustive(g, g->d_ms, g->d_acc, st))) return fail(s);
+    unsigned long long *dh = nullptr;
+    const bool hist_dev = hist && is_device_ptr(hist);
     if (hist) {
         if (g->hist_cap < nbins) {
             cudaFree(g->d_hist);
@@ -565,40 +516,35 @@ ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t 
             }
             g->hist_cap = nbins;
         }
-        const bool hist_dev = is_device_ptr(hist);
-        unsigned long long *dh = hist_dev ? (unsigned long long *)hist : g->d_hist;
+        dh = hist_dev ? (unsigned long long *)hist : g->d_hist;
         if (cudaMemsetAsync(dh, 0, sizeof(unsigned long long) * nbins, st) != cudaSuccess)
             return fail(KO_ERR_CUDA);
-        if ((s = check_cuda(ko_launch_histogram(g->d_ms, total, g->d_acc, dh, nbins, st))))
-            return fail(s);
-        if (!hist_dev) {
-            if (cudaMemcpyAsync(hist, dh, sizeof(unsigned long long) * nbins, cudaMemcpyDeviceToHost,
-                                st) != cudaSuccess)
-                return fail(KO_ERR_CUDA);
-            g->d2h += (long long)sizeof(unsigned long long) * nbins;
-        }
     }
-    KoAccum acc;
-    if (cudaMemcpyAsync(&acc, g->d_acc, sizeof(KoAccum), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return fail(KO_ERR_CUDA);
-    g->d2h += sizeof(KoAccum);
-    if (fast) {
-        if (cudaMemcpyAsync(&mh, &g->d_meta->ref, sizeof(mh), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if ((s = check_cuda(ko_launch_histogram(g->d_ms, total, g->d_acc, dh, hist ? nbins : 0, st, at, g->d_acc + 1))))
+        return fail(s);
+    if (hist && !hist_dev) {
+        if (cudaMemcpyAsync(hist, dh, sizeof(unsigned long long) * nbins, cudaMemcpyDeviceToHost, st) != cudaSuccess)
             return fail(KO_ERR_CUDA);
-        g->d2h += sizeof(mh);
+        g->d2h += (long long)sizeof(unsigned long long) * nbins;
     }
+    KoAccum res[2];  // the space's statistics; the counts against the ranked order and its makespan
+    if (cudaMemcpyAsync(res, g->d_acc, sizeof(res), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        return fail(KO_ERR_CUDA);
+    g->d2h += sizeof(res);
     if (cudaStreamSynchronize(st) != cudaSuccess) return fail(KO_ERR_CUDA);
     if (fast && (s = fast_after_sync(g))) return fail(s);
+    const KoAccum &acc = res[0], &cnt = res[1];
+    const int64_t mh = (int64_t)cnt.min;
     if (acc.failed || mh < 0) return fail(KO_ERR_STATE);
     out->min = (int64_t)acc.min;
     out->max = (int64_t)acc.max;
     out->makespan = mh;
     out->n_total = (uint64_t)total;
-    out->n_better = acc.n_better;
-    out->n_equal = acc.n_equal;
-    out->n_worse = acc.n_worse;
-    out->percentile = 100.0 * (double)(acc.n_worse + acc.n_equal) / (double)total;
-    out->percentile_strict = 100.0 * (double)acc.n_worse / (double)total;
+    out->n_better = cnt.n_better;
+    out->n_equal = cnt.n_equal;
+    out->n_worse = cnt.n_worse;
+    out->percentile = 100.0 * (double)(cnt.n_worse + cnt.n_equal) / (double)total;
+    out->percentile_strict = 100.0 * (double)cnt.n_worse / (double)total;
     out->speedup_over_worst = (double)out->max / (double)mh;
     out->deviation_from_optimal = (double)(mh - out->min) / (double)out->min;
     return ok();

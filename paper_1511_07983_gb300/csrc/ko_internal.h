@@ -67,9 +67,12 @@ cudaError_t ko_launch_simple(const KoSet *d_set, const KoSet &h_set, const int8_
                              cudaStream_t stream);
 
 // Histogram of `count` makespans with bin = (M - min) * nbins / (max - min + 1),
-// min / max read from acc on the device; hist (device, nbins u64) is added to.
+// min / max read from acc on the device; hist (device, nbins u64; unused when
+// nbins is 0) is added to.  With `counts` (reset before), the makespans better
+// than, equal to and worse than ms[ref_at] are counted there, and min = ms[ref_at].
 cudaError_t ko_launch_histogram(const int64_t *ms, int64_t count, const KoAccum *acc,
-                                unsigned long long *hist, int32_t nbins, cudaStream_t stream);
+                                unsigned long long *hist, int32_t nbins, cudaStream_t stream,
+                                int64_t ref_at = 0, KoAccum *counts = nullptr);
 
 // Resets an accumulator to (min = max u64, max = 0, counts = 0).
 cudaError_t ko_launch_accum_reset(KoAccum *acc, int count, cudaStream_t stream);

@@ -171,6 +171,13 @@ gemm_nt_kernel(const uint16_t *__restrict__ A, int lda, const uint16_t *__restri
     }
 }
 
+__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
+{
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
 // ---------------------------------------------------------------- encoding
 
 // x[b] = features of order rows[b] of set sid[b]: kernel at position p goes to
@@ -189,38 +196,33 @@ __device__ __forceinline__ int slot_position(int n, int slot)
     return pos;
 }
 
-// One thread per row, a warp per 32 consecutive rows.  Per block: the slot ->
-// position map of every N and -- for a single set (no sid) -- the set's
-// kernel and global features.  Per warp step: the 32 rows' order bytes are
-// copied to shared memory with coalesced loads (contiguous rows, no pick);
+// Rows of one set.  One thread per row, a warp per 32 consecutive rows.  Per
+// block: the slot -> position map of the set's N and its kernel and global
+// features.  Per warp step: the 32 rows' order bytes are copied to shared memory
+// with coalesced loads;
 // each thread produces its row's 192 features in order (slot by slot: one
 // kernel index, its 7 features; then the globals and the zero padding),
 // packs them two BF16 to a word (round to nearest even) and writes them to a
 // per-warp staging area (row pitch 400 bytes: conflict-free 16-byte stores);
 // the warp then stores its 32 rows (12,288 contiguous bytes) 16 bytes per
-// lane.  xt (training) gets the transposed copy value by value.
+// lane.
 constexpr int kEncWarps = 2, kEncPitch = 100;  // staging row pitch in words
 __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__restrict__ rows, int row_stride,
-                                                                const int *__restrict__ sid,
-                                                                const int *__restrict__ pick,
                                                                 const int *__restrict__ set_n,
                                                                 const float *__restrict__ kfeat,
                                                                 const float *__restrict__ gfeat, int B,
-                                                                uint16_t *x, uint16_t *xt)
+                                                                uint16_t *x)
 {
-    __shared__ int8_t s_pos[kMaxK + 1][kSlots];
+    __shared__ int8_t s_pos[kSlots];
     __shared__ float s_kf[kMaxK * kSlotFeat + kGlobals];
     __shared__ __align__(16) int8_t s_rows[kEncWarps][32 * kMaxK];
     __shared__ __align__(16) uint32_t s_out[kEncWarps][32 * kEncPitch];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < (kMaxK + 1) * kSlots; i += blockDim.x)
-        s_pos[i / kSlots][i % kSlots] = (int8_t)slot_position(i / kSlots, i % kSlots);
-    if (!sid) {
-        for (int i = threadIdx.x; i < kMaxK * kSlotFeat; i += blockDim.x) s_kf[i] = kfeat[i];
-        for (int i = threadIdx.x; i < kGlobals; i += blockDim.x) s_kf[kMaxK * kSlotFeat + i] = gfeat[i];
-    }
+    for (int i = threadIdx.x; i < kSlots; i += blockDim.x) s_pos[i] = (int8_t)slot_position(set_n[0], i);
+    for (int i = threadIdx.x; i < kMaxK * kSlotFeat; i += blockDim.x) s_kf[i] = kfeat[i];
+    for (int i = threadIdx.x; i < kGlobals; i += blockDim.x) s_kf[kMaxK * kSlotFeat + i] = gfeat[i];
     __syncthreads();
-    const bool stage = !pick && row_stride <= kMaxK;
+    const bool stage = row_stride <= kMaxK;
     const long long wsteps = ((long long)B + 31) / 32;
     for (long long ws = (long long)blockIdx.x * kEncWarps + warp; ws < wsteps;
          ws += (long long)gridDim.x * kEncWarps) {
@@ -240,13 +242,8 @@ __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__
             __syncwarp();
         }
         if (lane < nrows) {
-            const int b = base + lane;
-            const int src = pick ? pick[b] : b;
-            const int set = sid ? sid[src] : 0;
-            const int n = set_n[set];
-            const int8_t *row = stage ? &s_rows[warp][lane * row_stride] : rows + (size_t)src * row_stride;
-            const float *kf = sid ? kfeat + (size_t)set * kMaxK * kSlotFeat : s_kf;
-            const float *gf = sid ? gfeat + (size_t)set * kGlobals : s_kf + kMaxK * kSlotFeat;
+            const int8_t *row = stage ? &s_rows[warp][lane * row_stride] : rows + (size_t)(base + lane) * row_stride;
+            const float *kf = s_kf, *gf = s_kf + kMaxK * kSlotFeat;
             uint32_t *out = &s_out[warp][lane * kEncPitch];
             float v[8];
             auto put = [&](int f, float val) {  // f is a constant after unrolling
@@ -259,16 +256,11 @@ __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__
                         memcpy(&w[h], &p2, sizeof(uint32_t));
                     }
                     *reinterpret_cast<uint4 *>(out + (f >> 3) * 4) = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (xt) {
-#pragma unroll
-                        for (int h = 0; h < 8; h++)
-                            xt[(size_t)((f & ~7) + h) * B + b] = (uint16_t)(w[h >> 1] >> ((h & 1) * 16));
-                    }
                 }
             };
 #pragma unroll
             for (int slot = 0; slot < kSlots; slot++) {
-                const int pos = s_pos[n][slot];
+                const int pos = s_pos[slot];
                 const int k = pos >= 0 ? (int)row[pos] : -1;
 #pragma unroll
                 for (int q = 0; q < kSlotFeat; q++) put(slot * kSlotFeat + q, k >= 0 ? kf[k * kSlotFeat + q] : 0.0f);
@@ -285,6 +277,68 @@ __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__
             const int r = i / (kMlpIn / 8), c = i % (kMlpIn / 8);
             dst[i] = *reinterpret_cast<const uint4 *>(&s_out[warp][r * kEncPitch + c * 4]);
         }
+    }
+}
+
+// A training batch.  A block takes 32 rows: 32 threads draw their picks; 768
+// (row, slot) pairs look up their kernel; 6,144 features are gathered (the sets'
+// tables stay in L1) into a tile whose odd pitch spreads both readings over the
+// banks, and leave as 16-byte pieces of rows and as 64-byte runs of the
+// transposed copy.  The inference encoder's one thread per row wrote that copy
+// two bytes at a time: 18.5 us for 4,096 rows (caches cold) and 5.8 for picks and
+// targets in two more kernels; 12.5 us for all of it here.
+constexpr int kBatchRows = 32, kBatchPitch = kMlpIn + 2;  // 97 words
+__global__ void __launch_bounds__(256) batch_kernel(const int8_t *__restrict__ rows, int row_stride,
+                                                    const int *__restrict__ sid, const float *__restrict__ targets,
+                                                    long long pool, unsigned long long seed,
+                                                    const int *__restrict__ set_n, const float *__restrict__ kfeat,
+                                                    const float *__restrict__ gfeat, int B, uint16_t *x, uint16_t *xt,
+                                                    float *t)
+{
+    __shared__ int s_src[kBatchRows], s_set[kBatchRows], s_n[kBatchRows];
+    __shared__ int8_t s_kern[kBatchRows][kSlots];
+    __shared__ uint16_t tile[kBatchRows * kBatchPitch];
+    const int r0 = blockIdx.x * kBatchRows;
+    if (threadIdx.x < kBatchRows) {
+        const int b = r0 + threadIdx.x;
+        const int src = (int)(mix64(seed + (unsigned long long)b * 0x9E3779B97F4A7C15ull) % (unsigned long long)pool);
+        s_src[threadIdx.x] = src;
+        s_set[threadIdx.x] = sid[src];
+        s_n[threadIdx.x] = set_n[sid[src]];
+        t[b] = targets[src];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBatchRows * kSlots; i += blockDim.x) {
+        const int r = i / kSlots, slot = i - r * kSlots;
+        const int pos = slot_position(s_n[r], slot);
+        s_kern[r][slot] = pos >= 0 ? rows[(size_t)s_src[r] * row_stride + pos] : (int8_t)-1;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kBatchRows * kMlpIn; i += blockDim.x) {
+        const int r = i / kMlpIn, f = i - r * kMlpIn;
+        float v = 0.0f;
+        if (f < kSlots * kSlotFeat) {
+            const int slot = f / kSlotFeat, k = s_kern[r][slot];
+            if (k >= 0) v = kfeat[((size_t)s_set[r] * kMaxK + k) * kSlotFeat + (f - slot * kSlotFeat)];
+        } else if (f < kSlots * kSlotFeat + kGlobals) {
+            v = gfeat[(size_t)s_set[r] * kGlobals + (f - kSlots * kSlotFeat)];
+        }
+        tile[r * kBatchPitch + f] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+    }
+    __syncthreads();
+    const uint32_t *words = reinterpret_cast<const uint32_t *>(tile);
+    for (int i = threadIdx.x; i < kBatchRows * (kMlpIn / 8); i += blockDim.x) {
+        const int r = i / (kMlpIn / 8), c = i - r * (kMlpIn / 8);
+        const uint32_t *w = words + r * (kBatchPitch / 2) + c * 4;
+        *reinterpret_cast<uint4 *>(x + (size_t)(r0 + r) * kMlpIn + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    for (int i = threadIdx.x; i < kMlpIn * (kBatchRows / 8); i += blockDim.x) {
+        const int f = i >> 2, c = (i & 3) * 8;
+        uint32_t w[4];
+#pragma unroll
+        for (int h = 0; h < 4; h++)
+            w[h] = (uint32_t)tile[(c + 2 * h) * kBatchPitch + f] | ((uint32_t)tile[(c + 2 * h + 1) * kBatchPitch + f] << 16);
+        *reinterpret_cast<uint4 *>(xt + (size_t)f * B + r0 + c) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -353,105 +407,213 @@ __global__ void out_fwd_kernel(const uint16_t *__restrict__ a3, const uint16_t *
     if (b < B && c == 0) y[b] = s + b4[0];
 }
 
-// Output layer backward: dy = 2 (y - t) / B; loss sum; dw4 = sum dy * A3; db4 = sum dy;
-// dZ3 = dy * w4 * [A3 > 0] (fp32 for the bias gradient, bf16 + transposed for GEMMs).
-// Each block writes its partial sums (rows r0 .. r0+31) to part[blockIdx.x]:
-// dw4 partials, db3 partials, loss, db4; part_sum_kernel adds them up in
-// block order, so the gradients do not depend on the order blocks finish in.
-constexpr int kPartOut = 2 * kHidden + 2;
-
-__global__ void out_bwd_kernel(const float *__restrict__ y, const float *__restrict__ t,
-                               const uint16_t *__restrict__ a3, const uint16_t *__restrict__ w4, int B,
-                               float *part, uint16_t *dz, uint16_t *dzt)
+// Output layer of a training step, forward and backward.  y as out_fwd_kernel
+// (eight threads per row, its order of sums); dy = 2 (y - t) / B; loss sum;
+// dw4 = sum dy * A3; db4 = sum dy; dZ3 = dy * w4 * [A3 > 0] (fp32 for the bias
+// gradient, bf16 row-major and transposed for the GEMMs).  A block takes 32
+// rows; thread k then walks column k down them, holding the column's sums and
+// its 32 BF16 values, which leave as 64 contiguous bytes of the transposed copy
+// (two-byte stores before: 30 us for 4,096 rows and 4 for the separate forward
+// pass; 6.1 us for both here).  Sums of a block go to part[blockIdx.x]: dw4, db3,
+// loss, db4; finish_kernel adds the blocks up in order, so the gradients do not
+// depend on the order blocks finish in.
+constexpr int kOutRows = 32;
+__global__ void __launch_bounds__(kHidden) out_train_kernel(const uint16_t *__restrict__ a3,
+                                                            const uint16_t *__restrict__ w4,
+                                                            const float *__restrict__ b4, const float *__restrict__ t,
+                                                            int B, float *y, uint16_t *dz, uint16_t *dzt, float *part)
 {
-    __shared__ float s_dw[kHidden], s_db[kHidden];
-    for (int k = threadIdx.x; k < kHidden; k += blockDim.x) { s_dw[k] = 0.0f; s_db[k] = 0.0f; }
-    __syncthreads();
-    const int rows_per_block = 32;
-    const int r0 = blockIdx.x * rows_per_block;
-    float lsum = 0.0f, dbsum = 0.0f;
-    for (int r = r0; r < r0 + rows_per_block && r < B; r++) {
-        const float d = y[r] - t[r];
-        const float dy = 2.0f * d / (float)B;
-        if (threadIdx.x == 0) { lsum += d * d; dbsum += dy; }
-        for (int k = threadIdx.x; k < kHidden; k += blockDim.x) {
-            const float a = bf16_val(a3[(size_t)r * kHidden + k]);
-            s_dw[k] += dy * a;
-            const float g = a > 0.0f ? dy * bf16_val(w4[k]) : 0.0f;
-            s_db[k] += g;
-            const uint16_t bits = bf16_bits(g);
-            dz[(size_t)r * kHidden + k] = bits;
-            dzt[(size_t)k * B + r] = bits;
+    __shared__ float s_d[kOutRows], s_dy[kOutRows];
+    const int r0 = blockIdx.x * kOutRows, k = threadIdx.x;
+    {
+        const int r = k >> 3, c = k & 7;
+        const uint4 *src = reinterpret_cast<const uint4 *>(a3 + (size_t)(r0 + r) * kHidden + c * 32);
+        const uint16_t *w = w4 + c * 32;
+        float s = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint4 v = src[q];
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int h = 0; h < 4; h++) {
+                s = __fmaf_rn(__uint_as_float(u[h] << 16), bf16_val(w[8 * q + 2 * h]), s);
+                s = __fmaf_rn(__uint_as_float(u[h] & 0xFFFF0000u), bf16_val(w[8 * q + 2 * h + 1]), s);
+            }
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        if (c == 0) {
+            const float out = s + b4[0];
+            y[r0 + r] = out;
+            const float d = out - t[r0 + r];
+            s_d[r] = d;
+            s_dy[r] = 2.0f * d / (float)B;
         }
     }
     __syncthreads();
-    float *mine = part + (size_t)blockIdx.x * kPartOut;
-    for (int k = threadIdx.x; k < kHidden; k += blockDim.x) {
-        mine[k] = s_dw[k];
-        mine[kHidden + k] = s_db[k];
+    const float w = bf16_val(w4[k]);
+    float dw = 0.0f, db = 0.0f;
+    uint32_t col[kOutRows / 2];
+#pragma unroll
+    for (int r = 0; r < kOutRows; r++) {
+        const float dy = s_dy[r];
+        const float a = bf16_val(a3[(size_t)(r0 + r) * kHidden + k]);
+        dw += dy * a;
+        const float g = a > 0.0f ? dy * w : 0.0f;
+        db += g;
+        const uint32_t bits = bf16_bits(g);
+        dz[(size_t)(r0 + r) * kHidden + k] = (uint16_t)bits;
+        col[r >> 1] = r & 1 ? col[r >> 1] | (bits << 16) : bits;
     }
-    if (threadIdx.x == 0) {
+    uint4 *dt = reinterpret_cast<uint4 *>(dzt + (size_t)k * B + r0);
+#pragma unroll
+    for (int q = 0; q < 4; q++) dt[q] = make_uint4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
+    float *mine = part + (size_t)blockIdx.x * kPartOut;
+    mine[k] = dw;
+    mine[kHidden + k] = db;
+    if (k == 0) {
+        float lsum = 0.0f, dbsum = 0.0f;
+        for (int r = 0; r < kOutRows; r++) {
+            lsum += s_d[r] * s_d[r];
+            dbsum += s_dy[r];
+        }
         mine[2 * kHidden] = lsum;
         mine[2 * kHidden + 1] = dbsum;
     }
 }
 
-// Hidden-layer ReLU backward: dZ = dA * [A > 0]; bias-gradient partials per
-// block (fp32) into part[blockIdx.x]; dZ as bf16 row-major and transposed.
-__global__ void relu_bwd_kernel(const float *__restrict__ da, const uint16_t *__restrict__ a, int B,
-                                float *part, uint16_t *dz, uint16_t *dzt)
+// Hidden-layer ReLU backward behind the mma.sync input gradient: dZ = dA * [A > 0];
+// bias-gradient partials per block (fp32) into part[blockIdx.x]; dZ as bf16
+// row-major and transposed.  Thread k walks column k down 32 rows, as above.
+__global__ void __launch_bounds__(kHidden) relu_bwd_kernel(const float *__restrict__ da,
+                                                           const uint16_t *__restrict__ a, int B, float *part,
+                                                           uint16_t *dz, uint16_t *dzt)
 {
-    __shared__ float s_db[kHidden];
-    for (int k = threadIdx.x; k < kHidden; k += blockDim.x) s_db[k] = 0.0f;
-    __syncthreads();
-    const int rows_per_block = 32;
-    const int r0 = blockIdx.x * rows_per_block;
-    for (int r = r0; r < r0 + rows_per_block && r < B; r++) {
-        for (int k = threadIdx.x; k < kHidden; k += blockDim.x) {
-            const size_t i = (size_t)r * kHidden + k;
-            const float g = bf16_val(a[i]) > 0.0f ? da[i] : 0.0f;
-            s_db[k] += g;
-            const uint16_t bits = bf16_bits(g);
-            dz[i] = bits;
-            dzt[(size_t)k * B + r] = bits;
-        }
+    const int r0 = blockIdx.x * kOutRows, k = threadIdx.x;
+    float db = 0.0f;
+    uint32_t col[kOutRows / 2];
+#pragma unroll
+    for (int r = 0; r < kOutRows; r++) {
+        const size_t i = (size_t)(r0 + r) * kHidden + k;
+        const float g = bf16_val(a[i]) > 0.0f ? da[i] : 0.0f;
+        db += g;
+        const uint32_t bits = bf16_bits(g);
+        dz[i] = (uint16_t)bits;
+        col[r >> 1] = r & 1 ? col[r >> 1] | (bits << 16) : bits;
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < kHidden; k += blockDim.x) part[(size_t)blockIdx.x * kHidden + k] = s_db[k];
+    uint4 *dt = reinterpret_cast<uint4 *>(dzt + (size_t)k * B + r0);
+#pragma unroll
+    for (int q = 0; q < 4; q++) dt[q] = make_uint4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
+    part[(size_t)blockIdx.x * kHidden + k] = db;
 }
 
-// Column sums of nblk rows of `width` partials, rows added in order.  Columns
-// [0, span) go to lo[c], [span, 2 span) to hi[c - span], column 2 span to *s0
-// and 2 span + 1 to *s1.
-struct PartDst {
-    float *lo, *hi, *s0, *s1;
-    int span;
-};
-__global__ void part_sum_kernel(const float *__restrict__ part, int nblk, int width, PartDst dst)
+// Adam on the FP32 master weights.
+__device__ __forceinline__ float adam_step(const KoMlpAdam &o, long long i, float gi)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= width) return;
+    const float mi = o.b1 * o.m[i] + (1.0f - o.b1) * gi;
+    const float vi = o.b2 * o.v[i] + (1.0f - o.b2) * gi * gi;
+    o.m[i] = mi;
+    o.v[i] = vi;
+    const float mh = mi / o.c1, vh = vi / o.c2;
+    const float pi = o.p[i] - o.lr * mh / (sqrtf(vh) + o.eps);
+    o.p[i] = pi;
+    return pi;
+}
+
+// End of a backward pass (see ko_mlp_finish) in one launch; it took eleven
+// (slice sums, partial sums, Adam, BF16 copies; 62 us with cold caches, 14.6 now).  Blocks [0, 176): 32 x 32 tiles
+// of the three weight matrices -- a thread adds its elements' slices in order
+// (all loads of one element in flight together), updates them and leaves the BF16
+// value in a tile from which both layouts are written in 64-byte runs.  The last
+// 33 blocks: 32 columns of the per-32-row partials each, loaded by eight warps,
+// added in row order by the first.
+constexpr int kFinTile = 32, kFinW1 = kMlpIn / kFinTile * (kHidden / kFinTile), kFinW = kHidden / kFinTile * (kHidden / kFinTile);
+constexpr int kFinTiles = kFinW1 + 2 * kFinW, kFinSums = (kPartOut + 2 * kHidden + 31) / 32;
+constexpr int kFinRows = 128;  // partial rows held at a time
+__global__ void __launch_bounds__(256) finish_kernel(float *__restrict__ g, const float *__restrict__ wg1,
+                                                     const float *__restrict__ wg2, const float *__restrict__ wg3,
+                                                     int slices, const float *__restrict__ part_out,
+                                                     const float *__restrict__ part2, const float *__restrict__ part1,
+                                                     int nblk, float *loss_sum, const KoMlpAdam o)
+{
+    __shared__ uint16_t tile[kFinTile][kFinTile + 2];
+    __shared__ float rows[kFinRows][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool adam = o.on;
+    int blk = blockIdx.x;
+    if (blk < kFinTiles) {
+        const float *src = wg1;
+        long long off = kOffW1;
+        uint16_t *wk = nullptr, *wt = o.w1t;
+        int K = kMlpIn;
+        if (blk >= kFinW1) {
+            const bool third = blk >= kFinW1 + kFinW;
+            blk -= third ? kFinW1 + kFinW : kFinW1;
+            src = third ? wg3 : wg2;
+            off = third ? kOffW3 : kOffW2;
+            wk = third ? o.w3 : o.w2;
+            wt = third ? o.w3t : o.w2t;
+            K = kHidden;
+        }
+        const int k0 = blk / (kHidden / kFinTile) * kFinTile, n0 = blk % (kHidden / kFinTile) * kFinTile;
+#pragma unroll
+        for (int q = 0; q < kFinTile / 8; q++) {
+            const int kr = warp + q * 8;
+            const long long i = (long long)(k0 + kr) * kHidden + n0 + lane;
+            float gi;
+            if (src) {
+                gi = 0.0f;
+#pragma unroll 8
+                for (int s = 0; s < slices; s++) gi += src[(size_t)s * kHidden * kHidden + i];
+                g[off + i] = gi;
+            } else {
+                gi = g[off + i];
+            }
+            if (adam) {
+                const uint16_t b = bf16_bits(adam_step(o, off + i, gi));
+                tile[kr][lane] = b;
+                if (wk) wk[i] = b;
+            }
+        }
+        if (!adam) return;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kFinTile / 8; q++) {
+            const int n = warp + q * 8;
+            wt[(size_t)(n0 + n) * K + k0 + lane] = tile[lane][n];
+        }
+        return;
+    }
+    // columns: dw4 [0, 256), db3 [256, 512), loss 512, db4 513, db2 [514, 770), db1 [770, 1026)
+    const int c = (blk - kFinTiles) * 32 + lane;
+    const float *col = nullptr;
+    int width = kHidden;
+    if (c < kPartOut) { col = part_out + c; width = kPartOut; }
+    else if (c < kPartOut + kHidden) col = part2 + (c - kPartOut);
+    else if (c < kPartOut + 2 * kHidden) col = part1 + (c - kPartOut - kHidden);
     float acc = 0.0f;
-    for (int b = 0; b < nblk; b++) acc += part[(size_t)b * width + c];
-    if (c < dst.span) dst.lo[c] = acc;
-    else if (c < 2 * dst.span) dst.hi[c - dst.span] = acc;
-    else if (c == 2 * dst.span) *dst.s0 = acc;
-    else *dst.s1 = acc;
-}
-
-// Adam on the FP32 master weights, then refresh the BF16 copies the GEMMs read.
-__global__ void adam_kernel(float *p, float *m, float *v, const float *g, long long count, float lr,
-                            float b1, float b2, float eps, float c1, float c2)
-{
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / c1, vh = vi / c2;
-        p[i] -= lr * mh / (sqrtf(vh) + eps);
+    for (int b0 = 0; b0 < nblk; b0 += kFinRows) {
+        const int have = nblk - b0 < kFinRows ? nblk - b0 : kFinRows;
+        __syncthreads();
+        if (col)
+            for (int r = warp; r < have; r += 8) rows[r][lane] = col[(size_t)(b0 + r) * width];
+        __syncthreads();
+        if (warp == 0 && col)
+#pragma unroll 8
+            for (int r = 0; r < have; r++) acc += rows[r][lane];
+    }
+    if (warp != 0 || !col) return;
+    if (c == 2 * kHidden) { *loss_sum = acc; return; }
+    const long long at = c < kHidden       ? kOffW4 + c
+                         : c < 2 * kHidden ? kOffB3 + (c - kHidden)
+                         : c < kPartOut    ? kOffB4
+                         : c < kPartOut + kHidden ? kOffB2 + (c - kPartOut)
+                                                  : kOffB1 + (c - kPartOut - kHidden);
+    g[at] = acc;
+    if (adam) {
+        const float pn = adam_step(o, at, acc);
+        if (c < kHidden) o.w4b[c] = bf16_bits(pn);
     }
 }
 
@@ -534,13 +696,6 @@ __global__ void select_emit_kernel(const float *__restrict__ y, long long n, con
     }
 }
 
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z)
-{
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
 // Uniform random permutations (Fisher-Yates) from a counter-based SplitMix64
 // stream per row: row r uses mix64(seed + (r * 2^6 + step) * golden).
 __global__ void random_orders_kernel(int8_t *rows, int stride, long long count, int n,
@@ -601,18 +756,6 @@ __global__ void neighbours_kernel(const int8_t *__restrict__ base, int beam, int
     for (int i = 0; i < kMaxK; i++) o[i] = i < n ? p[i] : (int8_t)0;
 }
 
-__global__ void random_pick_kernel(int *pick, int B, long long pool, unsigned long long seed)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) pick[b] = (int)(mix64(seed + (unsigned long long)b * 0x9E3779B97F4A7C15ull) % (unsigned long long)pool);
-}
-
-__global__ void gather_f32_kernel(const float *src, const int *pick, int B, float *dst)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) dst[b] = src[pick[b]];
-}
-
 __global__ void gather_rows_kernel(const int8_t *src, int stride, const int *pick, int B, int8_t *dst)
 {
     const int b = blockIdx.x;
@@ -642,9 +785,8 @@ cudaError_t ko_mlp_gemm_f32(const uint16_t *A, int lda, const uint16_t *Bt, int 
     return cudaGetLastError();
 }
 
-cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *sid, const int *pick,
-                          const int *set_n, const float *kfeat, const float *gfeat, int B, uint16_t *x,
-                          uint16_t *xt, cudaStream_t st)
+cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *set_n, const float *kfeat,
+                          const float *gfeat, int B, uint16_t *x, cudaStream_t st)
 {
     if (B <= 0) return cudaSuccess;
     int dev = 0, sms = 0;
@@ -652,7 +794,18 @@ cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *sid, co
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long blocks = ((long long)B + 32 * kEncWarps - 1) / (32 * kEncWarps);
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
-    encode_kernel<<<grid, kEncWarps * 32, 0, st>>>(rows, row_stride, sid, pick, set_n, kfeat, gfeat, B, x, xt);
+    encode_kernel<<<grid, kEncWarps * 32, 0, st>>>(rows, row_stride, set_n, kfeat, gfeat, B, x);
+    ko_count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t ko_mlp_batch(const int8_t *rows, int row_stride, const int *sid, const float *targets, long long pool,
+                         unsigned long long seed, const int *set_n, const float *kfeat, const float *gfeat, int B,
+                         uint16_t *x, uint16_t *xt, float *t, cudaStream_t st)
+{
+    if (B % kBatchRows) return cudaErrorInvalidValue;
+    batch_kernel<<<(unsigned)(B / kBatchRows), 256, 0, st>>>(rows, row_stride, sid, targets, pool, seed, set_n, kfeat,
+                                                            gfeat, B, x, xt, t);
     ko_count_launch();
     return cudaGetLastError();
 }
@@ -672,36 +825,30 @@ cudaError_t ko_mlp_out_fwd(const uint16_t *a3, const uint16_t *w4, const float *
     return cudaGetLastError();
 }
 
-size_t ko_mlp_part_floats(int B) { return (size_t)((B + 31) / 32) * kPartOut; }
-
-cudaError_t ko_mlp_out_bwd(const float *y, const float *t, const uint16_t *a3, const uint16_t *w4, int B,
-                           float *loss_sum, float *dw4, float *db4, float *db3, uint16_t *dz,
-                           uint16_t *dzt, float *part, cudaStream_t st)
+cudaError_t ko_mlp_out_train(const uint16_t *a3, const uint16_t *w4, const float *b4, const float *t, int B, float *y,
+                             uint16_t *dz, uint16_t *dzt, float *part, cudaStream_t st)
 {
-    const int nblk = (B + 31) / 32;
-    out_bwd_kernel<<<nblk, 256, 0, st>>>(y, t, a3, w4, B, part, dz, dzt);
-    // columns: dw4 [0, 256), db3 [256, 512), loss 512, db4 513
-    PartDst d{dw4, db3, loss_sum, db4, kHidden};
-    part_sum_kernel<<<(2 * kHidden + 2 + 255) / 256, 256, 0, st>>>(part, nblk, kPartOut, d);
-    ko_count_launch(2);
+    if (B % kOutRows) return cudaErrorInvalidValue;
+    out_train_kernel<<<(unsigned)(B / kOutRows), kHidden, 0, st>>>(a3, w4, b4, t, B, y, dz, dzt, part);
+    ko_count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t ko_mlp_relu_bwd(const float *da, const uint16_t *a, int B, float *db, uint16_t *dz,
-                            uint16_t *dzt, float *part, cudaStream_t st)
+cudaError_t ko_mlp_relu_bwd(const float *da, const uint16_t *a, int B, uint16_t *dz, uint16_t *dzt, float *part,
+                            cudaStream_t st)
 {
-    const int nblk = (B + 31) / 32;
-    relu_bwd_kernel<<<nblk, 256, 0, st>>>(da, a, B, part, dz, dzt);
-    PartDst d{db, nullptr, nullptr, nullptr, kHidden};
-    part_sum_kernel<<<(kHidden + 255) / 256, 256, 0, st>>>(part, nblk, kHidden, d);
-    ko_count_launch(2);
+    if (B % kOutRows) return cudaErrorInvalidValue;
+    relu_bwd_kernel<<<(unsigned)(B / kOutRows), kHidden, 0, st>>>(da, a, B, part, dz, dzt);
+    ko_count_launch();
     return cudaGetLastError();
 }
 
-cudaError_t ko_mlp_adam(float *p, float *m, float *v, const float *g, long long count, float lr, float b1,
-                        float b2, float eps, float c1, float c2, cudaStream_t st)
+cudaError_t ko_mlp_finish(float *g, const float *wg1, const float *wg2, const float *wg3, int slices,
+                          const float *part_out, const float *part2, const float *part1, int B, float *loss_sum,
+                          const KoMlpAdam &adam, cudaStream_t st)
 {
-    adam_kernel<<<256, 256, 0, st>>>(p, m, v, g, count, lr, b1, b2, eps, c1, c2);
+    finish_kernel<<<kFinTiles + kFinSums, 256, 0, st>>>(g, wg1, wg2, wg3, slices, part_out, part2, part1,
+                                                       (int)ko_mlp_part_rows(B), loss_sum, adam);
     ko_count_launch();
     return cudaGetLastError();
 }
@@ -752,15 +899,6 @@ cudaError_t ko_mlp_targets(const int64_t *ms, const int *sid, const double *log2
     if (blocks < 1) blocks = 1;
     targets_kernel<<<(unsigned)blocks, 256, 0, st>>>(ms, sid, log2_lb, n, t);
     ko_count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t ko_mlp_pick(int *pick, int B, long long pool, unsigned long long seed, const float *t_src,
-                        float *t_dst, cudaStream_t st)
-{
-    random_pick_kernel<<<(B + 255) / 256, 256, 0, st>>>(pick, B, pool, seed);
-    gather_f32_kernel<<<(B + 255) / 256, 256, 0, st>>>(t_src, pick, B, t_dst);
-    ko_count_launch(2);
     return cudaGetLastError();
 }
 

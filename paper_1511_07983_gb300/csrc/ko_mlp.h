@@ -47,36 +47,60 @@ cudaError_t ko_mlp_layer_tc_out(const uint16_t *A, const uint16_t *Wt, int M, in
 // ([256][ldt] BF16, ldt % 8 == 0).  Same shapes as ko_mlp_layer_tc.
 cudaError_t ko_mlp_layer_tc_t(const uint16_t *A, const uint16_t *Wt, int M, int K, const float *bias, uint16_t *out,
                               uint16_t *out_t, long long ldt, int *err, cudaStream_t st);
-// tcgen05 input gradient: outf[M][256] = A Wt^T in FP32 (M % 128 == 0, K in {192, 256}).
-cudaError_t ko_mlp_layer_tc_f32(const uint16_t *A, const uint16_t *Wt, int M, int K, float *outf, int *err,
-                                cudaStream_t st);
-// tcgen05 weight gradient: out[M][256] (row stride ldo) = A Bt^T with
-// A [M][Kdim] (row stride lda), Bt [256][Kdim] (row stride ldb), M <= 256,
-// Kdim % 256 == 0; split-K over 256-wide slices into `work`
-// (ko_mlp_wgrad_tc_workspace bytes), summed in a fixed order.
-size_t ko_mlp_wgrad_tc_workspace(int M, long long Kdim);
+// tcgen05 input gradient with the ReLU's backward pass: g = dz W^T (FP32) where
+// act > 0, else 0; out[M][256] = bf16(g) (nullable), out_t[256][ldt] its
+// transpose, part[M / 32][256] the column sums of each 32 rows in row order
+// (M % 128 == 0, ldt % 8 == 0, K = 256).
+cudaError_t ko_mlp_dgrad_tc(const uint16_t *dz, const uint16_t *W, int M, const uint16_t *act, uint16_t *out,
+                            uint16_t *out_t, long long ldt, float *part, int *err, cudaStream_t st);
+// tcgen05 weight gradient A Bt^T with A [M][Kdim] (row stride lda), Bt [256][Kdim]
+// (row stride ldb), M <= 256, Kdim % 256 == 0: split-K, one partial matrix
+// [256][256] per 256-wide slice in `work` (ko_mlp_wgrad_tc_floats floats), for
+// ko_mlp_finish to add up in slice order.
+int ko_mlp_wgrad_tc_slices(long long Kdim);
+size_t ko_mlp_wgrad_tc_floats(long long Kdim);
 cudaError_t ko_mlp_wgrad_tc(const uint16_t *A, long long lda, const uint16_t *Bt, long long ldb, int M,
-                            long long Kdim, float *out, int ldo, float *work, int *err, cudaStream_t st);
+                            long long Kdim, float *work, int *err, cudaStream_t st);
 cudaError_t ko_mlp_gemm_f32(const uint16_t *A, int lda, const uint16_t *Bt, int ldb, int M, int N, int K,
                             float *out, int ldo, cudaStream_t st);
-cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *sid, const int *pick,
-                          const int *set_n, const float *kfeat, const float *gfeat, int B, uint16_t *x,
-                          uint16_t *xt, cudaStream_t st);
+// Encoded orders (rows of one set) x [B x 192].
+cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *set_n, const float *kfeat,
+                          const float *gfeat, int B, uint16_t *x, cudaStream_t st);
 // FP32 features x [B x 192] (device, B % 64 == 0) rounded to BF16 (nearest, ties to even) into xb and,
 // if xt is non-null, transposed into xt [192 x B].
 cudaError_t ko_mlp_features(const float *x, int B, uint16_t *xb, uint16_t *xt, cudaStream_t st);
+// A training batch: B uniform picks of the labelled pool (row b takes pool entry
+// mix64(seed + b golden) % pool), their encoded orders x [B x 192] and xt
+// [192 x B], and their targets (B % 32 == 0).
+cudaError_t ko_mlp_batch(const int8_t *rows, int row_stride, const int *sid, const float *targets, long long pool,
+                         unsigned long long seed, const int *set_n, const float *kfeat, const float *gfeat, int B,
+                         uint16_t *x, uint16_t *xt, float *t, cudaStream_t st);
 cudaError_t ko_mlp_out_fwd(const uint16_t *a3, const uint16_t *w4, const float *b4, int B, float *y,
                            cudaStream_t st);
-// The backward kernels sum per-block partials (workspace `part`, at least
-// ko_mlp_part_floats(B) floats) in a fixed order: gradients are reproducible.
-size_t ko_mlp_part_floats(int B);
-cudaError_t ko_mlp_out_bwd(const float *y, const float *t, const uint16_t *a3, const uint16_t *w4, int B,
-                           float *loss_sum, float *dw4, float *db4, float *db3, uint16_t *dz,
-                           uint16_t *dzt, float *part, cudaStream_t st);
-cudaError_t ko_mlp_relu_bwd(const float *da, const uint16_t *a, int B, float *db, uint16_t *dz,
-                            uint16_t *dzt, float *part, cudaStream_t st);
-cudaError_t ko_mlp_adam(float *p, float *m, float *v, const float *g, long long count, float lr, float b1,
-                        float b2, float eps, float c1, float c2, cudaStream_t st);
+// Partial sums of the backward pass, one row per 32 batch rows: [514] of the
+// output layer (dw4, db3, loss, db4), then [256] each of db2 and db1.
+constexpr int kPartOut = 2 * kHidden + 2;
+inline size_t ko_mlp_part_rows(int B) { return (size_t)(B + 31) / 32; }
+// Output layer of a training step: y, and dZ3 (row-major and transposed) with
+// its partial sums into part [rows x 514].
+cudaError_t ko_mlp_out_train(const uint16_t *a3, const uint16_t *w4, const float *b4, const float *t, int B, float *y,
+                             uint16_t *dz, uint16_t *dzt, float *part, cudaStream_t st);
+// dZ = dA where a > 0, row-major and transposed, column sums per 32 rows into part.
+cudaError_t ko_mlp_relu_bwd(const float *da, const uint16_t *a, int B, uint16_t *dz, uint16_t *dzt, float *part,
+                            cudaStream_t st);
+// End of a backward pass: gradients into g -- a weight matrix from its `slices`
+// split-K partials (null: already in g), biases, w4 and the loss sum from the
+// partial rows, everything added in a fixed order -- and, with adam.on, one
+// Adam step on p, m, v and the BF16 copies the GEMMs read.
+struct KoMlpAdam {
+    bool on;
+    float *p, *m, *v;
+    uint16_t *w1t, *w2, *w2t, *w3, *w3t, *w4b;
+    float lr, b1, b2, eps, c1, c2;
+};
+cudaError_t ko_mlp_finish(float *g, const float *wg1, const float *wg2, const float *wg3, int slices,
+                          const float *part_out, const float *part2, const float *part1, int B, float *loss_sum,
+                          const KoMlpAdam &adam, cudaStream_t st);
 cudaError_t ko_mlp_weights_bf16(const float *w, int K, int N, uint16_t *wk, uint16_t *wt, cudaStream_t st);
 cudaError_t ko_mlp_topk(const float *y, long long n, int k, uint32_t *state, unsigned int *hist,
                         unsigned int *counters, int *out, cudaStream_t st);
@@ -84,8 +108,6 @@ cudaError_t ko_mlp_random_orders(int8_t *rows, int stride, long long count, int 
                                  cudaStream_t st);
 cudaError_t ko_mlp_targets(const int64_t *ms, const int *sid, const double *log2_lb, long long n, float *t,
                            cudaStream_t st);
-cudaError_t ko_mlp_pick(int *pick, int B, long long pool, unsigned long long seed, const float *t_src,
-                        float *t_dst, cudaStream_t st);
 cudaError_t ko_mlp_neighbours(const int8_t *base, int beam, int n, int8_t *out, cudaStream_t st);
 cudaError_t ko_mlp_gather_rows(const int8_t *src, int stride, const int *pick, int B, int8_t *dst,
                                cudaStream_t st);

@@ -2,17 +2,28 @@
 // form C[m][n] = sum_k A[m][k] * Bt[n][k] with BF16 operands, both K-major,
 // and an FP32 accumulator in TMEM:
 //
-//   tc_layer_kernel<MODE>  M rows (a multiple of 128), N = 256, K in {192, 256}:
-//                          Bt (256 x K) is loaded once per CTA and 128-row
-//                          tiles of A stream through (persistent grid).
+//   tc_layer_kernel<MODE, NT>  M rows (a multiple of 128), N = 256, K in {192, 256}:
+//                          NT rows of Bt (NT x K) are loaded once per CTA and
+//                          128-row tiles of A stream through (persistent grid).
 //       MODE 0  out   = bf16(relu(C + bias))               (inference, forward)
 //       MODE 1  out   = bf16(relu(C + bias)), out_t = its transpose (training
 //                       forward: out_t feeds the weight gradients)
-//       MODE 2  outf  = C in FP32                           (input gradients)
-//   tc_wgrad_kernel        M <= 256, N = 256, K a multiple of 256 (the batch):
+//       MODE 3  out   = bf16(C where the layer's activation is positive, else
+//                       0), out_t = its transpose, and the bias gradient's
+//                       partial sums per 32 rows (input gradients with the
+//                       ReLU's backward pass)
+//   tc_wgrad_kernel<NT>    M <= 256, N = 256, K a multiple of 256 (the batch):
 //                          split-K, one 256-wide K slice per CTA, FP32 partial
-//                          tiles to a workspace; wgrad_reduce_kernel sums the
-//                          slices in a fixed order (deterministic).
+//                          128 x NT tiles to a workspace; the optimiser's
+//                          kernel sums the slices in a fixed order.
+//                          NT (columns per CTA): a training batch has few
+//                          128-row tiles (4,096 rows: 32), so at NT = 256 they
+//                          occupied 32 of 152 SMs, each loading 192 KB before
+//                          its first MMA; column blocks of 128 or 64 spread the
+//                          loads and the epilogue while they still fit one wave
+//                          (4,096 rows, cold caches: forward layer 16.2 -> 9.5 us,
+//                          weight gradient 15.0 -> 8.1; input gradient 17.1 and a
+//                          39.6 us ReLU pass behind it -> 10.8 for both).
 //   tc_ws_kernel<OUT>      the MODE 0 layer, warp-specialised: TMA producer,
 //                          MMA issuer and epilogue warps over a ring of
 //                          128-byte-swizzled A stages and two TMEM
@@ -34,12 +45,13 @@
 //    and columns 128 (w / 4) .. +127, 32 columns at a time with
 //    tcgen05.ld.32x32b.x32.  MODE 0 passes each 32 x 64-byte BF16 piece through
 //    a per-warp staging area (16-byte slots XOR-rotated by row, conflict-free
-//    both ways) so a store writes 8 whole 64-byte row segments.  MODE 1 stages
-//    the 32 x 32 piece as one word per value with a row stride of 33 words,
-//    which makes both the row-wise and the column-wise reads conflict-free,
-//    and writes out and out_t (64 contiguous bytes per lane) from it.
-// Shared memory (at most 226 KB) keeps one CTA per SM, so a TMEM allocation
-// (256 columns; 512 in tc_ws_kernel) never waits for another CTA.
+//    both ways) so a store writes 8 whole 64-byte row segments.  MODEs 1 and 3
+//    stage the 32 x 32 piece as one word per value with a row stride of 33
+//    words, which makes both the row-wise and the column-wise reads
+//    conflict-free, and write out and out_t (64 contiguous bytes per lane) from it.
+// Shared memory (96 to 226 KB) keeps at most two CTAs per SM where they allocate
+// 64 TMEM columns and one where they allocate more (512 in tc_ws_kernel), so an
+// allocation never waits for another CTA.
 #include <cstdint>
 #include <cstring>
 
@@ -107,12 +119,13 @@ __device__ __forceinline__ void tc_fill(uint8_t *dst, const uint16_t *src, int r
     }
 }
 
-// K/16 MMAs of the 128 x K tile in `sa` against the 256 x K operand in `sb`,
+// K/16 MMAs of the 128 x K tile in `sa` against the NT x K operand in `sb`,
 // then a commit to `mbar` (called by one thread).
+template <int NT>
 __device__ __forceinline__ void tc_mma(uint32_t tmem, const uint8_t *sa, const uint8_t *sb, int K, uint64_t *mbar)
 {
     const uint32_t sbo = (uint32_t)(K / 8) * 128u;
-    const uint32_t idesc = instr_desc(kTileM, kTileN);
+    const uint32_t idesc = instr_desc(kTileM, NT);
     for (int k = 0; k < K / 16; k++) {
         // a 16-wide K step covers two core matrices along K
         const uint64_t ad = smem_desc(saddr(sa) + (uint32_t)k * 256u, 128u, sbo);
@@ -177,34 +190,36 @@ __device__ __forceinline__ void tc_fence_sync()
 // tensor core's async proxy before each MMA batch; the mbarrier phase
 // alternates per tile.  The next tile's A operand is requested as soon as the
 // current MMAs complete, so its load overlaps the epilogue.
-template <int MODE>
+template <int MODE, int NT>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt, int K, int tiles,
-                const float *__restrict__ bias, uint16_t *__restrict__ out, uint16_t *__restrict__ out_t,
-                long long ldt, float *__restrict__ outf, int *err)
+                const float *__restrict__ bias, const uint16_t *__restrict__ act, uint16_t *__restrict__ out,
+                uint16_t *__restrict__ out_t, long long ldt, float *__restrict__ part, int *err)
 {
+    static_assert(NT % 64 == 0 && NT <= kTileN, "two column halves of whole 32-column pieces");
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int quarter = warp & 3, col0 = (warp >> 2) * (kTileN / 2);
+    const int quarter = warp & 3, col0 = (warp >> 2) * (NT / 2);
+    const int n0 = blockIdx.y * NT;                  // first of this CTA's columns
     uint8_t *sa = smem;                              // 128 x K
-    uint8_t *sb = smem + (size_t)kTileM * K * 2;     // 256 x K
-    float *sbias = (float *)(sb + (size_t)kTileN * K * 2);  // 256
-    uint32_t *stage = (uint32_t *)(sbias + kTileN) + warp * 32 * (MODE == 1 ? kStageTWords : kStageRowWords);
+    uint8_t *sb = smem + (size_t)kTileM * K * 2;     // NT x K
+    float *sbias = (float *)(sb + (size_t)NT * K * 2);  // NT
+    uint32_t *stage = (uint32_t *)(sbias + NT) + warp * 32 * (MODE == 0 ? kStageRowWords : kStageTWords);
 
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(saddr(&tmem_base)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(&tmem_base)), "n"(NT));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(saddr(&mbar)));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
     }
-    tc_fill(sb, Wt, kTileN, kTileN, K, K);
+    tc_fill(sb, Wt + (size_t)n0 * K, NT, NT, K, K);
     asm volatile("cp.async.commit_group;\n" ::);
-    if (MODE != 2)
-        for (int i = tid; i < kTileN; i += blockDim.x) sbias[i] = bias[i];
+    if (MODE != 3)
+        for (int i = tid; i < NT; i += blockDim.x) sbias[i] = bias[n0 + i];
     tc_fence_sync();
     const uint32_t tmem = tmem_base;
     auto load_a = [&](int tile) {
@@ -220,7 +235,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
         asm volatile("cp.async.wait_all;\n" ::);
         asm volatile("fence.proxy.async.shared::cta;\n" ::);
         tc_fence_sync();
-        if (tid == 0) tc_mma(tmem, sa, sb, K, &mbar);
+        if (tid == 0) tc_mma<NT>(tmem, sa, sb, K, &mbar);
         if (!tc_wait(&mbar, phase, err)) {
             ok = false;
         } else {
@@ -228,17 +243,54 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
             // the MMAs have read the A tile: start loading the next one under the epilogue
             if (tile + (int)gridDim.x < tiles) load_a(tile + gridDim.x);
             const int row0 = m0 + quarter * 32;
-            for (int c0 = col0; c0 < col0 + kTileN / 2; c0 += 32) {
+            for (int c0 = col0; c0 < col0 + NT / 2; c0 += 32) {
                 uint32_t v[32];
-                tc_ld32(tmem, quarter, c0, v);
-                if constexpr (MODE == 2) {
-                    float4 *dst = (float4 *)(outf + (size_t)(row0 + lane) * kTileN + c0);
+                if constexpr (MODE == 3) {
+                    // this row's activations, loaded under the accumulator's read
+                    uint4 gate[4];
+                    const uint4 *src = (const uint4 *)(act + (size_t)(row0 + lane) * kTileN + n0 + c0);
 #pragma unroll
-                    for (int q = 0; q < 8; q++)
-                        dst[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                             __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+                    for (int q = 0; q < 4; q++) gate[q] = __ldg(src + q);
+                    tc_ld32(tmem, quarter, c0, v);
+#pragma unroll
+                    for (int j = 0; j < 16; j++) {
+                        const uint32_t w = j % 4 == 0 ? gate[j / 4].x : j % 4 == 1 ? gate[j / 4].y
+                                                      : j % 4 == 2 ? gate[j / 4].z : gate[j / 4].w;
+                        stage[lane * kStageTWords + 2 * j] = __uint_as_float(w << 16) > 0.0f ? v[2 * j] : 0u;
+                        stage[lane * kStageTWords + 2 * j + 1] =
+                            __uint_as_float(w & 0xFFFF0000u) > 0.0f ? v[2 * j + 1] : 0u;
+                    }
+                    __syncwarp();
+                    if (out) {
+#pragma unroll
+                        for (int it = 0; it < 4; it++) {
+                            const int r = it * 8 + (lane >> 2), q = lane & 3;
+                            const float *f = (const float *)stage + r * kStageTWords + q * 8;
+                            *(uint4 *)(out + (size_t)(row0 + r) * kTileN + n0 + c0 + q * 8) =
+                                make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]),
+                                           pack_bf16(f[6], f[7]));
+                        }
+                    }
+                    // column c0 + lane: its 32 rows, and their sum in row order
+                    uint32_t col[16];
+                    float sum = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < 16; j++) {
+                        const float g0 = __uint_as_float(stage[(2 * j) * kStageTWords + lane]);
+                        const float g1 = __uint_as_float(stage[(2 * j + 1) * kStageTWords + lane]);
+                        sum += g0;
+                        sum += g1;
+                        col[j] = pack_bf16(g0, g1);
+                    }
+                    uint4 *dt = (uint4 *)(out_t + (size_t)(n0 + c0 + lane) * ldt + row0);
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        dt[q] = make_uint4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
+                    part[(size_t)(row0 >> 5) * kTileN + n0 + c0 + lane] = sum;
+                    __syncwarp();
                     continue;
                 } else {
+                tc_ld32(tmem, quarter, c0, v);
                 uint32_t packed[16];
 #pragma unroll
                 for (int j = 0; j < 16; j++) {
@@ -258,7 +310,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
                     for (int it = 0; it < 4; it++) {
                         const int r = it * 8 + (lane >> 2), q = lane & 3;
                         const uint4 w = *(const uint4 *)(stage + r * 16 + ((q + (r >> 1)) & 3) * 4);
-                        *(uint4 *)(out + (size_t)(row0 + r) * kTileN + c0 + q * 8) = w;
+                        *(uint4 *)(out + (size_t)(row0 + r) * kTileN + n0 + c0 + q * 8) = w;
                     }
                     __syncwarp();
                 } else {
@@ -276,7 +328,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
                         const uint32_t *src = stage + r * kStageTWords + q * 8;
                         const uint4 w = make_uint4(src[0] | (src[1] << 16), src[2] | (src[3] << 16),
                                                    src[4] | (src[5] << 16), src[6] | (src[7] << 16));
-                        *(uint4 *)(out + (size_t)(row0 + r) * kTileN + c0 + q * 8) = w;
+                        *(uint4 *)(out + (size_t)(row0 + r) * kTileN + n0 + c0 + q * 8) = w;
                     }
                     // transpose: lane c writes column c0 + c's 32 rows (64 contiguous bytes of out_t)
                     uint32_t col[16];
@@ -284,7 +336,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
                     for (int j = 0; j < 16; j++)
                         col[j] = stage[(2 * j) * kStageTWords + lane] |
                                  (stage[(2 * j + 1) * kStageTWords + lane] << 16);
-                    uint4 *dt = (uint4 *)(out_t + (size_t)(c0 + lane) * ldt + row0);
+                    uint4 *dt = (uint4 *)(out_t + (size_t)(n0 + c0 + lane) * ldt + row0);
 #pragma unroll
                     for (int q = 0; q < 4; q++)
                         dt[q] = make_uint4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
@@ -297,7 +349,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
         tc_fence_sync();
     }
     asm volatile("cp.async.wait_all;\n" ::);
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "n"(NT));
 }
 
 // One 2-D TMA box copy into shared memory, completion counted in bytes on mbar.
@@ -627,10 +679,11 @@ bool encode_operand_sw128(CUtensorMap *map, const uint16_t *base, long long rows
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Weight gradient slice: CTA (mt, s) multiplies rows 128 mt.. of A (M x Kdim,
-// row stride lda) by all 256 rows of Bt (256 x Kdim, row stride ldb) over the
-// K slice 256 s .. 256 s + 255 and writes the FP32 128 x 256 partial tile to
-// part[s][128 mt ..][0 .. 256).
+// Weight gradient slice: CTA (mt, s, nt) multiplies rows 128 mt.. of A (M x Kdim,
+// row stride lda) by rows NT nt.. of Bt (256 x Kdim, row stride ldb) over the
+// K slice 256 s .. 256 s + 255 and writes the FP32 128 x NT partial tile to
+// part[s][128 mt ..][NT nt ..].
+template <int NT>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 tc_wgrad_kernel(const uint16_t *__restrict__ A, long long lda, const uint16_t *__restrict__ Bt, long long ldb,
                 int M, float *__restrict__ part, int mpad, int *err)
@@ -639,14 +692,14 @@ tc_wgrad_kernel(const uint16_t *__restrict__ A, long long lda, const uint16_t *_
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int quarter = warp & 3, col0 = (warp >> 2) * (kTileN / 2);
+    const int quarter = warp & 3, col0 = (warp >> 2) * (NT / 2);
     const int mt = blockIdx.x, s = blockIdx.y;
-    const int m0 = mt * kTileM;
+    const int m0 = mt * kTileM, n0 = blockIdx.z * NT;
     const long long k0 = (long long)s * kSliceK;
     uint8_t *sa = smem;                                 // 128 x 256
-    uint8_t *sb = smem + (size_t)kTileM * kSliceK * 2;  // 256 x 256
+    uint8_t *sb = smem + (size_t)kTileM * kSliceK * 2;  // NT x 256
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(saddr(&tmem_base)));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(saddr(&tmem_base)), "n"(NT));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
     if (tid == 0) {
@@ -654,17 +707,17 @@ tc_wgrad_kernel(const uint16_t *__restrict__ A, long long lda, const uint16_t *_
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
     }
     tc_fill(sa, A + (size_t)m0 * lda + k0, kTileM, M - m0, lda, kSliceK);
-    tc_fill(sb, Bt + k0, kTileN, kTileN, ldb, kSliceK);
+    tc_fill(sb, Bt + (size_t)n0 * ldb + k0, NT, NT, ldb, kSliceK);
     asm volatile("cp.async.commit_group;\n" ::);
     asm volatile("cp.async.wait_all;\n" ::);
     asm volatile("fence.proxy.async.shared::cta;\n" ::);
     tc_fence_sync();
     const uint32_t tmem = tmem_base;
-    if (tid == 0) tc_mma(tmem, sa, sb, kSliceK, &mbar);
+    if (tid == 0) tc_mma<NT>(tmem, sa, sb, kSliceK, &mbar);
     if (tc_wait(&mbar, 0, err)) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
-        float *dst_row = part + ((size_t)s * mpad + m0 + quarter * 32 + lane) * kTileN;
-        for (int c0 = col0; c0 < col0 + kTileN / 2; c0 += 32) {
+        float *dst_row = part + ((size_t)s * mpad + m0 + quarter * 32 + lane) * kTileN + n0;
+        for (int c0 = col0; c0 < col0 + NT / 2; c0 += 32) {
             uint32_t v[32];
             tc_ld32(tmem, quarter, c0, v);
             float4 *dst = (float4 *)(dst_row + c0);
@@ -675,19 +728,7 @@ tc_wgrad_kernel(const uint16_t *__restrict__ A, long long lda, const uint16_t *_
         }
     }
     tc_fence_sync();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
-}
-
-// out[m][n] = sum over slices s = 0, 1, ... of part[s][m][n], m < M (fixed order).
-__global__ void wgrad_reduce_kernel(const float *__restrict__ part, int slices, int mpad, int M,
-                                    float *__restrict__ out, int ldo)
-{
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)M * kTileN) return;
-    const int m = (int)(i / kTileN), n = (int)(i % kTileN);
-    float acc = 0.0f;
-    for (int s = 0; s < slices; s++) acc += part[((size_t)s * mpad + m) * kTileN + n];
-    out[(size_t)m * ldo + n] = acc;
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "n"(NT));
 }
 
 int max_dyn_smem()
@@ -698,26 +739,49 @@ int max_dyn_smem()
     return v;
 }
 
-template <int MODE>
-cudaError_t launch_layer(const uint16_t *A, const uint16_t *Wt, int M, int K, const float *bias, uint16_t *out,
-                         uint16_t *out_t, long long ldt, float *outf, int *err, cudaStream_t st)
+int sm_count()
 {
-    if (M % kTileM || (K != 192 && K != 256)) return cudaErrorInvalidValue;
-    const int stage_words = MODE == 1 ? kStageTWords : kStageRowWords;
-    const size_t smem = (size_t)(kTileM + kTileN) * K * 2 + sizeof(float) * kTileN +
-                        (kThreadsTc / 32) * 32 * stage_words * sizeof(uint32_t);
-    if ((long long)smem > (long long)max_dyn_smem()) return cudaErrorInvalidValue;
-    cudaError_t e =
-        cudaFuncSetAttribute(tc_layer_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tiles = M / kTileM;
-    const int grid = tiles < sms ? tiles : sms;
-    tc_layer_kernel<MODE><<<grid, kThreadsTc, smem, st>>>(A, Wt, K, tiles, bias, out, out_t, ldt, outf, err);
+    return sms;
+}
+
+template <int MODE, int NT>
+cudaError_t launch_layer_nt(const uint16_t *A, const uint16_t *Wt, int M, int K, const float *bias,
+                            const uint16_t *act, uint16_t *out, uint16_t *out_t, long long ldt, float *part,
+                            int *err, cudaStream_t st)
+{
+    const int stage_words = MODE == 0 ? kStageRowWords : kStageTWords;
+    const size_t smem = (size_t)(kTileM + NT) * K * 2 + sizeof(float) * NT +
+                        (kThreadsTc / 32) * 32 * stage_words * sizeof(uint32_t);
+    if ((long long)smem > (long long)max_dyn_smem()) return cudaErrorInvalidValue;
+    cudaError_t e =
+        cudaFuncSetAttribute(tc_layer_kernel<MODE, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int tiles = M / kTileM, room = sm_count() / (kTileN / NT);
+    const dim3 grid(tiles < room ? tiles : (room > 0 ? room : 1), kTileN / NT);
+    tc_layer_kernel<MODE, NT><<<grid, kThreadsTc, smem, st>>>(A, Wt, K, tiles, bias, act, out, out_t, ldt, part, err);
     ko_count_launch();
     return cudaGetLastError();
+}
+
+// Columns per CTA: the fewest whose CTAs still run in one wave (see above).
+int columns_per_cta(int tiles)
+{
+    const int sms = sm_count();
+    return 4 * tiles <= sms ? 64 : 2 * tiles <= sms ? 128 : 256;
+}
+
+template <int MODE>
+cudaError_t launch_layer(const uint16_t *A, const uint16_t *Wt, int M, int K, const float *bias, const uint16_t *act,
+                         uint16_t *out, uint16_t *out_t, long long ldt, float *part, int *err, cudaStream_t st)
+{
+    if (M % kTileM || (K != 192 && K != 256)) return cudaErrorInvalidValue;
+    const int nt = columns_per_cta(M / kTileM);
+    if (nt == 64) return launch_layer_nt<MODE, 64>(A, Wt, M, K, bias, act, out, out_t, ldt, part, err, st);
+    if (nt == 128) return launch_layer_nt<MODE, 128>(A, Wt, M, K, bias, act, out, out_t, ldt, part, err, st);
+    return launch_layer_nt<MODE, 256>(A, Wt, M, K, bias, act, out, out_t, ldt, part, err, st);
 }
 
 // Launch tc_ws_kernel<OUT> with as many 16 KB A stages as fit beside the
@@ -759,7 +823,7 @@ cudaError_t ko_mlp_layer_tc(const uint16_t *A, const uint16_t *Wt, int M, int K,
     if (M % kTileM || (K != 192 && K != 256)) return cudaErrorInvalidValue;
     const cudaError_t e = launch_ws<false>(A, Wt, M, K, bias, out, nullptr, nullptr, nullptr, err, st);
     if (e != cudaErrorNotSupported) return e;
-    return launch_layer<0>(A, Wt, M, K, bias, out, nullptr, 0, nullptr, err, st);
+    return launch_layer<0>(A, Wt, M, K, bias, nullptr, out, nullptr, 0, nullptr, err, st);
 }
 
 cudaError_t ko_mlp_layer_tc_out(const uint16_t *A, const uint16_t *Wt, int M, int K, const float *bias,
@@ -769,7 +833,7 @@ cudaError_t ko_mlp_layer_tc_out(const uint16_t *A, const uint16_t *Wt, int M, in
     if (M % kTileM || (K != 192 && K != 256)) return cudaErrorInvalidValue;
     const cudaError_t e = launch_ws<true>(A, Wt, M, K, bias, nullptr, w4, b4, y, err, st);
     if (e != cudaErrorNotSupported) return e;
-    const cudaError_t e2 = launch_layer<0>(A, Wt, M, K, bias, out, nullptr, 0, nullptr, err, st);
+    const cudaError_t e2 = launch_layer<0>(A, Wt, M, K, bias, nullptr, out, nullptr, 0, nullptr, err, st);
     if (e2 != cudaSuccess) return e2;
     return ko_mlp_out_fwd(out, w4, b4, M, y, st);
 }
@@ -778,37 +842,49 @@ cudaError_t ko_mlp_layer_tc_t(const uint16_t *A, const uint16_t *Wt, int M, int 
                               uint16_t *out_t, long long ldt, int *err, cudaStream_t st)
 {
     if (ldt % 8) return cudaErrorInvalidValue;  // 16-byte stores into out_t rows
-    return launch_layer<1>(A, Wt, M, K, bias, out, out_t, ldt, nullptr, err, st);
+    return launch_layer<1>(A, Wt, M, K, bias, nullptr, out, out_t, ldt, nullptr, err, st);
 }
 
-cudaError_t ko_mlp_layer_tc_f32(const uint16_t *A, const uint16_t *Wt, int M, int K, float *outf, int *err,
-                                cudaStream_t st)
+cudaError_t ko_mlp_dgrad_tc(const uint16_t *dz, const uint16_t *W, int M, const uint16_t *act, uint16_t *out,
+                            uint16_t *out_t, long long ldt, float *part, int *err, cudaStream_t st)
 {
-    return launch_layer<2>(A, Wt, M, K, nullptr, nullptr, nullptr, 0, outf, err, st);
+    if (ldt % 8) return cudaErrorInvalidValue;  // 16-byte stores into out_t rows
+    return launch_layer<3>(dz, W, M, kHidden, nullptr, act, out, out_t, ldt, part, err, st);
 }
 
-size_t ko_mlp_wgrad_tc_workspace(int M, long long Kdim)
+int ko_mlp_wgrad_tc_slices(long long Kdim) { return (int)(Kdim / kSliceK); }
+
+size_t ko_mlp_wgrad_tc_floats(long long Kdim)
 {
-    const int mpad = (M + kTileM - 1) / kTileM * kTileM;
-    return sizeof(float) * (size_t)(Kdim / kSliceK) * mpad * kTileN;
+    return (size_t)ko_mlp_wgrad_tc_slices(Kdim) * 2 * kTileM * kTileN;
 }
+
+namespace {
+
+template <int NT>
+cudaError_t launch_wgrad(const uint16_t *A, long long lda, const uint16_t *Bt, long long ldb, int M, int mt,
+                         int slices, float *work, int *err, cudaStream_t st)
+{
+    const size_t smem = (size_t)(kTileM + NT) * kSliceK * 2;
+    if ((long long)smem > (long long)max_dyn_smem()) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(tc_wgrad_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    tc_wgrad_kernel<NT><<<dim3(mt, slices, kTileN / NT), kThreadsTc, smem, st>>>(A, lda, Bt, ldb, M, work,
+                                                                                2 * kTileM, err);
+    ko_count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
 
 cudaError_t ko_mlp_wgrad_tc(const uint16_t *A, long long lda, const uint16_t *Bt, long long ldb, int M,
-                            long long Kdim, float *out, int ldo, float *work, int *err, cudaStream_t st)
+                            long long Kdim, float *work, int *err, cudaStream_t st)
 {
     if (M < 1 || M > 2 * kTileM || Kdim < kSliceK || Kdim % kSliceK || lda % 8 || ldb % 8)
         return cudaErrorInvalidValue;
-    const size_t smem = (size_t)(kTileM + kTileN) * kSliceK * 2;
-    if ((long long)smem > (long long)max_dyn_smem()) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tc_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int mt = (M + kTileM - 1) / kTileM, slices = (int)(Kdim / kSliceK);
-    const int mpad = mt * kTileM;
-    tc_wgrad_kernel<<<dim3(mt, slices), kThreadsTc, smem, st>>>(A, lda, Bt, ldb, M, work, mpad, err);
-    ko_count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const long long n = (long long)M * kTileN;
-    wgrad_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(work, slices, mpad, M, out, ldo);
-    ko_count_launch();
-    return cudaGetLastError();
+    const int mt = (M + kTileM - 1) / kTileM, slices = ko_mlp_wgrad_tc_slices(Kdim);
+    const int nt = columns_per_cta(mt * slices);
+    if (nt == 64) return launch_wgrad<64>(A, lda, Bt, ldb, M, mt, slices, work, err, st);
+    if (nt == 128) return launch_wgrad<128>(A, lda, Bt, ldb, M, mt, slices, work, err, st);
+    return launch_wgrad<256>(A, lda, Bt, ldb, M, mt, slices, work, err, st);
 }

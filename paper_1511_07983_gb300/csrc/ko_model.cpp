@@ -72,33 +72,47 @@ struct ko_model {
     float *p = nullptr, *m = nullptr, *v = nullptr, *g = nullptr;
     uint16_t *w1t = nullptr, *w2 = nullptr, *w2t = nullptr, *w3 = nullptr, *w3t = nullptr, *w4b = nullptr;
     long long step = 0;
-    int cap = 0;  // batch capacity of the activation buffers
+    int cap = 0, cap_wide = 0, cap_train = 0;  // batch capacity of the buffers of a forward pass, of `da`,
+                                               // and of the training buffers
     uint16_t *a0 = nullptr, *a0t = nullptr, *a1 = nullptr, *a1t = nullptr, *a2 = nullptr, *a2t = nullptr,
-             *a3 = nullptr, *dz = nullptr, *dzt = nullptr;
+             *a3 = nullptr, *dz = nullptr, *dz2 = nullptr, *dzt = nullptr;
     float *y = nullptr, *t = nullptr, *da = nullptr, *loss = nullptr;
-    float *part = nullptr;     // per-block bias-gradient partials (summed in a fixed order)
-    int *pick = nullptr;
+    float *part = nullptr;     // per-32-row partial sums of the backward pass (summed in a fixed order)
     KoFastState fast{};
     int tc_forward = 1;        // inference layers on tcgen05 (1) or mma.sync (0)
     int tc_train = 1;          // training GEMMs on tcgen05 (1) or mma.sync (0)
     float *wg_work = nullptr;  // split-K partials of the tcgen05 weight gradients
-    size_t wg_bytes = 0;
+    size_t wg_floats = 0;
     int chunk = 262144;        // candidate rows per forward pass of the proposal paths
     int *tc_err = nullptr;     // device flag: a tcgen05 completion wait gave up
     int polish = 64;           // exact descent steps after a guided search (0: none)
 
-    void free_acts()
+    void free_forward()
     {
-        cudaFree(a0); cudaFree(a0t); cudaFree(a1); cudaFree(a1t); cudaFree(a2); cudaFree(a2t); cudaFree(a3);
-        cudaFree(dz); cudaFree(dzt); cudaFree(y); cudaFree(t); cudaFree(da); cudaFree(pick); cudaFree(part);
-        a0 = a0t = a1 = a1t = a2 = a2t = a3 = dz = dzt = nullptr;
-        y = t = da = part = nullptr;
-        pick = nullptr;
+        cudaFree(a0); cudaFree(a1); cudaFree(a2); cudaFree(a3); cudaFree(y);
+        a0 = a1 = a2 = a3 = nullptr;
+        y = nullptr;
         cap = 0;
+    }
+    void free_wide()
+    {
+        cudaFree(da);
+        da = nullptr;
+        cap_wide = 0;
+    }
+    void free_train()
+    {
+        cudaFree(a0t); cudaFree(a1t); cudaFree(a2t); cudaFree(dz); cudaFree(dz2); cudaFree(dzt); cudaFree(t);
+        cudaFree(part);
+        a0t = a1t = a2t = dz = dz2 = dzt = nullptr;
+        t = part = nullptr;
+        cap_train = 0;
     }
     ~ko_model()
     {
-        free_acts();
+        free_forward();
+        free_wide();
+        free_train();
         cudaFree(p); cudaFree(m); cudaFree(v); cudaFree(g); cudaFree(loss); cudaFree(tc_err); cudaFree(wg_work);
         cudaFree(w1t); cudaFree(w2); cudaFree(w2t); cudaFree(w3); cudaFree(w3t); cudaFree(w4b);
         ko_fast_release(&fast);
@@ -107,20 +121,46 @@ struct ko_model {
 
 namespace {
 
-ko_status ensure_acts(ko_model *md, int B)
+// Activations for a forward pass of B rows.
+ko_status ensure_forward(ko_model *md, int B)
 {
     if (md->cap >= B) return KO_OK;
-    md->free_acts();
+    md->free_forward();
     const size_t in = (size_t)B * kMlpIn, hid = (size_t)B * kHidden;
-    bool ok = dalloc(&md->a0, in) && dalloc(&md->a0t, in) && dalloc(&md->a1, hid) && dalloc(&md->a1t, hid) &&
-              dalloc(&md->a2, hid) && dalloc(&md->a2t, hid) && dalloc(&md->a3, hid) && dalloc(&md->dz, hid) &&
-              dalloc(&md->dzt, hid) && dalloc(&md->y, (size_t)B) && dalloc(&md->t, (size_t)B) &&
-              dalloc(&md->da, hid) && dalloc(&md->pick, (size_t)B) && dalloc(&md->part, ko_mlp_part_floats(B));
-    if (!ok) {
-        md->free_acts();
+    if (!dalloc(&md->a0, in) || !dalloc(&md->a1, hid) || !dalloc(&md->a2, hid) || !dalloc(&md->a3, hid) ||
+        !dalloc(&md->y, (size_t)B)) {
+        md->free_forward();
         return KO_ERR_NOMEM;
     }
     md->cap = B;
+    return KO_OK;
+}
+
+// The FP32 [B x 256] buffer of raw features and mma.sync input gradients.
+ko_status ensure_wide(ko_model *md, int B)
+{
+    if (md->cap_wide >= B) return KO_OK;
+    md->free_wide();
+    if (!dalloc(&md->da, (size_t)B * kHidden)) return KO_ERR_NOMEM;
+    md->cap_wide = B;
+    return KO_OK;
+}
+
+// Everything a training step of B rows needs.
+ko_status ensure_train(ko_model *md, int B)
+{
+    ko_status s;
+    if ((s = ensure_forward(md, B)) || (s = ensure_wide(md, B))) return s;
+    if (md->cap_train >= B) return KO_OK;
+    md->free_train();
+    const size_t in = (size_t)B * kMlpIn, hid = (size_t)B * kHidden;
+    if (!dalloc(&md->a0t, in) || !dalloc(&md->a1t, hid) || !dalloc(&md->a2t, hid) || !dalloc(&md->dz, hid) ||
+        !dalloc(&md->dz2, hid) || !dalloc(&md->dzt, hid) || !dalloc(&md->t, (size_t)B) ||
+        !dalloc(&md->part, ko_mlp_part_rows(B) * (kPartOut + 2 * kHidden))) {
+        md->free_train();
+        return KO_ERR_NOMEM;
+    }
+    md->cap_train = B;
     return KO_OK;
 }
 
@@ -153,7 +193,8 @@ ko_status refresh_bf16(ko_model *md, cudaStream_t st)
 }
 
 // Forward over a0 (B rows, B % 64 == 0); with `train` the transposed
-// activations for the weight gradients are written too.
+// activations for the weight gradients are written too, and the output layer is
+// left to backward().
 ko_status forward(ko_model *md, int B, bool train, cudaStream_t st)
 {
     ko_status s;
@@ -165,9 +206,7 @@ ko_status forward(ko_model *md, int B, bool train, cudaStream_t st)
             if ((s = cuda_ok(ko_mlp_layer_tc_t(md->a1, md->w2t, B, kHidden, md->p + kOffB2, md->a2, md->a2t, B,
                                                md->tc_err, st))))
                 return s;
-            if ((s = cuda_ok(ko_mlp_layer_tc(md->a2, md->w3t, B, kHidden, md->p + kOffB3, md->a3, md->tc_err, st))))
-                return s;
-            return cuda_ok(ko_mlp_out_fwd(md->a3, md->w4b, md->p + kOffB4, B, md->y, st));
+            return cuda_ok(ko_mlp_layer_tc(md->a2, md->w3t, B, kHidden, md->p + kOffB3, md->a3, md->tc_err, st));
         }
         if (e != cudaErrorInvalidValue) return cuda_ok(e);
         cudaGetLastError();
@@ -189,84 +228,76 @@ ko_status forward(ko_model *md, int B, bool train, cudaStream_t st)
     if ((s = cuda_ok(ko_mlp_gemm_relu(md->a2, kHidden, md->w3t, kHidden, B, kHidden, kHidden, md->p + kOffB3,
                                       md->a3, kHidden, nullptr, 0, st))))
         return s;
-    return cuda_ok(ko_mlp_out_fwd(md->a3, md->w4b, md->p + kOffB4, B, md->y, st));
+    return train ? KO_OK : cuda_ok(ko_mlp_out_fwd(md->a3, md->w4b, md->p + kOffB4, B, md->y, st));
 }
 
-// Gradients of the mean squared error into md->g (zeroed here); loss sum
-// added to *loss_dev.
-// tcgen05 weight and input gradients (B % 256 == 0), the mma.sync ones otherwise.
-ko_status wgrad(ko_model *md, const uint16_t *at, int M, int B, float *out, cudaStream_t st)
+// Weight gradient of a layer with activations `at` (transposed, M rows): split-K
+// partials on tcgen05 (B % 256 == 0) into *parts, or straight into `out` on mma.sync.
+ko_status wgrad(ko_model *md, const uint16_t *at, int M, int B, float *out, float *work, const float **parts,
+                cudaStream_t st)
 {
-    if (md->tc_train && B % 256 == 0) {
-        const size_t need = ko_mlp_wgrad_tc_workspace(M, B);
-        if (md->wg_bytes < need) {
-            cudaFree(md->wg_work);
-            md->wg_work = nullptr;
-            md->wg_bytes = 0;
-            if (cudaMalloc(&md->wg_work, need) != cudaSuccess) {
-                cudaGetLastError();
-                return KO_ERR_NOMEM;
-            }
-            md->wg_bytes = need;
-        }
-        const cudaError_t e = ko_mlp_wgrad_tc(at, B, md->dzt, B, M, B, out, kHidden, md->wg_work, md->tc_err, st);
+    *parts = nullptr;
+    if (work) {
+        const cudaError_t e = ko_mlp_wgrad_tc(at, B, md->dzt, B, M, B, work, md->tc_err, st);
+        if (e == cudaSuccess) *parts = work;
         if (e != cudaErrorInvalidValue) return cuda_ok(e);
         cudaGetLastError();
     }
     return cuda_ok(ko_mlp_gemm_f32(at, B, md->dzt, B, M, kHidden, B, out, kHidden, st));
 }
 
-ko_status dgrad(ko_model *md, const uint16_t *w, int B, cudaStream_t st)
+// Gradient of a layer's input times its ReLU's derivative: reads dz, writes dz_out
+// (nullable), md->dzt and the bias partials.
+ko_status dgrad(ko_model *md, const uint16_t *w, const uint16_t *act, int B, const uint16_t *dz, uint16_t *dz_out,
+                float *part, cudaStream_t st)
 {
     if (md->tc_train && B % 128 == 0) {
-        const cudaError_t e = ko_mlp_layer_tc_f32(md->dz, w, B, kHidden, md->da, md->tc_err, st);
+        const cudaError_t e = ko_mlp_dgrad_tc(dz, w, B, act, dz_out, md->dzt, B, part, md->tc_err, st);
         if (e != cudaErrorInvalidValue) return cuda_ok(e);
         cudaGetLastError();
     }
-    return cuda_ok(ko_mlp_gemm_f32(md->dz, kHidden, w, kHidden, B, kHidden, kHidden, md->da, kHidden, st));
+    const ko_status s = cuda_ok(ko_mlp_gemm_f32(dz, kHidden, w, kHidden, B, kHidden, kHidden, md->da, kHidden, st));
+    if (s) return s;
+    return cuda_ok(ko_mlp_relu_bwd(md->da, act, B, dz_out ? dz_out : md->dz2, md->dzt, part, st));
 }
 
-ko_status backward(ko_model *md, int B, float *loss_dev, cudaStream_t st)
+// Output layer, gradients of the mean squared error into md->g and the loss sum
+// into *loss_dev; with `adam` an Adam step as well.
+ko_status backward(ko_model *md, int B, float *loss_dev, bool adam, float lr, cudaStream_t st)
 {
     ko_status s;
-    if (cudaMemsetAsync(md->g, 0, sizeof(float) * kParams, st) != cudaSuccess) return KO_ERR_CUDA;
-    if ((s = cuda_ok(ko_mlp_out_bwd(md->y, md->t, md->a3, md->w4b, B, loss_dev, md->g + kOffW4, md->g + kOffB4,
-                                    md->g + kOffB3, md->dz, md->dzt, md->part, st))))
-        return s;
-    if (md->tc_train) {
-        if ((s = wgrad(md, md->a2t, kHidden, B, md->g + kOffW3, st))) return s;
-        if ((s = dgrad(md, md->w3, B, st))) return s;
-        if ((s = cuda_ok(ko_mlp_relu_bwd(md->da, md->a2, B, md->g + kOffB2, md->dz, md->dzt, md->part, st)))) return s;
-        if ((s = wgrad(md, md->a1t, kHidden, B, md->g + kOffW2, st))) return s;
-        if ((s = dgrad(md, md->w2, B, st))) return s;
-        if ((s = cuda_ok(ko_mlp_relu_bwd(md->da, md->a1, B, md->g + kOffB1, md->dz, md->dzt, md->part, st)))) return s;
-        return wgrad(md, md->a0t, kMlpIn, B, md->g + kOffW1, st);
+    const size_t rows = ko_mlp_part_rows(B);
+    float *part_out = md->part, *part2 = part_out + rows * kPartOut, *part1 = part2 + rows * kHidden;
+    float *work = nullptr;
+    size_t per = 0;
+    if (md->tc_train && B % 256 == 0) {
+        per = ko_mlp_wgrad_tc_floats(B);
+        if (md->wg_floats < 3 * per) {
+            cudaFree(md->wg_work);
+            md->wg_work = nullptr;
+            md->wg_floats = 0;
+            if (!dalloc(&md->wg_work, 3 * per)) return KO_ERR_NOMEM;
+            md->wg_floats = 3 * per;
+        }
+        work = md->wg_work;
     }
-    // layer 3
-    if ((s = cuda_ok(ko_mlp_gemm_f32(md->a2t, B, md->dzt, B, kHidden, kHidden, B, md->g + kOffW3, kHidden, st))))
+    const float *wg1, *wg2, *wg3;
+    if ((s = cuda_ok(ko_mlp_out_train(md->a3, md->w4b, md->p + kOffB4, md->t, B, md->y, md->dz, md->dzt, part_out, st))))
         return s;
-    if ((s = cuda_ok(ko_mlp_gemm_f32(md->dz, kHidden, md->w3, kHidden, B, kHidden, kHidden, md->da, kHidden, st))))
-        return s;
-    if ((s = cuda_ok(ko_mlp_relu_bwd(md->da, md->a2, B, md->g + kOffB2, md->dz, md->dzt, md->part, st)))) return s;
-    // layer 2
-    if ((s = cuda_ok(ko_mlp_gemm_f32(md->a1t, B, md->dzt, B, kHidden, kHidden, B, md->g + kOffW2, kHidden, st))))
-        return s;
-    if ((s = cuda_ok(ko_mlp_gemm_f32(md->dz, kHidden, md->w2, kHidden, B, kHidden, kHidden, md->da, kHidden, st))))
-        return s;
-    if ((s = cuda_ok(ko_mlp_relu_bwd(md->da, md->a1, B, md->g + kOffB1, md->dz, md->dzt, md->part, st)))) return s;
-    // layer 1 (no input gradient needed)
-    return cuda_ok(ko_mlp_gemm_f32(md->a0t, B, md->dzt, B, kMlpIn, kHidden, B, md->g + kOffW1, kHidden, st));
-}
-
-ko_status adam(ko_model *md, float lr, cudaStream_t st)
-{
-    md->step++;
-    const float c1 = (float)(1.0 - std::pow(kBeta1, (double)md->step));
-    const float c2 = (float)(1.0 - std::pow(kBeta2, (double)md->step));
-    ko_status s = cuda_ok(ko_mlp_adam(md->p, md->m, md->v, md->g, kParams, lr, (float)kBeta1, (float)kBeta2,
-                                      (float)kEps, c1, c2, st));
-    if (s) return s;
-    return refresh_bf16(md, st);
+    if ((s = wgrad(md, md->a2t, kHidden, B, md->g + kOffW3, work, &wg3, st))) return s;
+    if ((s = dgrad(md, md->w3, md->a2, B, md->dz, md->dz2, part2, st))) return s;
+    if ((s = wgrad(md, md->a1t, kHidden, B, md->g + kOffW2, work ? work + per : nullptr, &wg2, st))) return s;
+    if ((s = dgrad(md, md->w2, md->a1, B, md->dz2, nullptr, part1, st))) return s;  // no input gradient of layer 1
+    if ((s = wgrad(md, md->a0t, kMlpIn, B, md->g + kOffW1, work ? work + 2 * per : nullptr, &wg1, st))) return s;
+    KoMlpAdam o{adam,  md->p, md->m, md->v, md->w1t, md->w2, md->w2t, md->w3, md->w3t, md->w4b,
+                lr,    (float)kBeta1, (float)kBeta2, (float)kEps, 1.0f, 1.0f};
+    if (adam) {
+        md->step++;
+        o.c1 = (float)(1.0 - std::pow(kBeta1, (double)md->step));
+        o.c2 = (float)(1.0 - std::pow(kBeta2, (double)md->step));
+    }
+    return cuda_ok(ko_mlp_finish(md->g, wg1, wg2, wg3, ko_mlp_wgrad_tc_slices(B), part_out, part2, part1, B, loss_dev,
+                                 o, st));
 }
 
 // Features of raw rows x [B x 192] (host floats) into a0 and, for training, a0t:
@@ -371,19 +402,18 @@ ko_status ko_model_raw(ko_model *md, const float *x, const float *t, int B, floa
                        float *loss_out, float lr, cudaStream_t st)
 {
     if (B < 64 || B % 64) return KO_ERR_ARG;
-    ko_status s = ensure_acts(md, B);
+    ko_status s = t ? ensure_train(md, B) : ensure_forward(md, B);
+    if (!s) s = ensure_wide(md, B);
     if (s) return s;
     if ((s = upload_features(md, x, B, t != nullptr, st))) return s;
     if ((s = forward(md, B, t != nullptr, st))) return s;
     if (t) {
-        if (cudaMemcpyAsync(md->t, t, sizeof(float) * B, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-            cudaMemsetAsync(md->loss, 0, sizeof(float), st) != cudaSuccess)
+        if (cudaMemcpyAsync(md->t, t, sizeof(float) * B, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return KO_ERR_CUDA;
-        if ((s = backward(md, B, md->loss, st))) return s;
+        if ((s = backward(md, B, md->loss, lr > 0.0f, lr, st))) return s;
         if (grad_out && cudaMemcpyAsync(grad_out, md->g, sizeof(float) * kParams, cudaMemcpyDeviceToHost, st) !=
                             cudaSuccess)
             return KO_ERR_CUDA;
-        if (lr > 0.0f && (s = adam(md, lr, st))) return s;
         float ls = 0.0f;
         if (cudaMemcpyAsync(&ls, md->loss, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
@@ -548,17 +578,13 @@ ko_status ko_model_train_sets(ko_model *md, const KoSet *const *hs, int nsets, l
         if (s) break;
         if ((s = label_pool(&md->fast, tb.sets, hs, nsets, pairs_per_set, rows, ms, d_chunks, st))) break;
         if ((s = cuda_ok(ko_mlp_targets(ms, sid, tb.log2_lb, pool, targets, st)))) break;
-        if ((s = ensure_acts(md, batch))) break;
-        if (cudaMemsetAsync(md->loss, 0, sizeof(float) * steps, st) != cudaSuccess) { s = KO_ERR_CUDA; break; }
+        if ((s = ensure_train(md, batch))) break;
         for (int it = 0; it < steps && !s; it++) {
-            if ((s = cuda_ok(ko_mlp_pick(md->pick, batch, pool, mix64(seed + 0x1000ull + it), targets, md->t, st))))
-                break;
-            if ((s = cuda_ok(ko_mlp_encode(rows, kMaxK, sid, md->pick, tb.set_n, tb.kfeat, tb.gfeat, batch, md->a0,
-                                           md->a0t, st))))
+            if ((s = cuda_ok(ko_mlp_batch(rows, kMaxK, sid, targets, pool, mix64(seed + 0x1000ull + it), tb.set_n,
+                                          tb.kfeat, tb.gfeat, batch, md->a0, md->a0t, md->t, st))))
                 break;
             if ((s = forward(md, batch, true, st))) break;
-            if ((s = backward(md, batch, md->loss + it, st))) break;
-            s = adam(md, lr, st);
+            s = backward(md, batch, md->loss + it, true, lr, st);
         }
         if (s) break;
         if (loss_curve) {
@@ -614,15 +640,15 @@ ko_status ko_model_propose_set(ko_model *md, const KoSet &h, long long n_cand, i
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!s) s = make_events(&e0, &e1);
-    if (!s) s = ensure_acts(md, C);
+    if (!s) s = ensure_forward(md, C);
     if (!s) {
         cudaEventRecord(e0, st);
         if (cudaMemsetAsync(rows, 0, (size_t)padded * kMaxK, st) != cudaSuccess) s = KO_ERR_CUDA;
         if (!s) s = cuda_ok(ko_mlp_random_orders(rows, kMaxK, n_cand, h.n, mix64(seed ^ 0xC0FFEEull), st));
         for (long long off = 0; off < n_cand && !s; off += C) {
             const long long c = n_cand - off < C ? n_cand - off : C;
-            if ((s = cuda_ok(ko_mlp_encode(rows + (size_t)off * kMaxK, kMaxK, nullptr, nullptr, tb.set_n, tb.kfeat,
-                                           tb.gfeat, C, md->a0, nullptr, st))))
+            if ((s = cuda_ok(ko_mlp_encode(rows + (size_t)off * kMaxK, kMaxK, tb.set_n, tb.kfeat, tb.gfeat, C,
+                                           md->a0, st))))
                 break;
             if ((s = forward(md, C, false, st))) break;
             if (cudaMemcpyAsync(y_all + off, md->y, sizeof(float) * c, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
@@ -719,7 +745,7 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
         return KO_OK;
     };
     if (!s) s = make_events(&e0, &e1);
-    if (!s) s = ensure_acts(md, C);
+    if (!s) s = ensure_forward(md, C);
     if (!s) {
         cudaEventRecord(e0, st);
         // screening
@@ -729,8 +755,8 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
         if (!s) s = cuda_ok(ko_mlp_random_orders(rows, kMaxK, n_cand, n, mix64(seed ^ 0xC0FFEEull), st));
         for (long long off = 0; off < n_cand && !s; off += C) {
             const long long c = n_cand - off < C ? n_cand - off : C;
-            if ((s = cuda_ok(ko_mlp_encode(rows + (size_t)off * kMaxK, kMaxK, nullptr, nullptr, tb.set_n, tb.kfeat,
-                                           tb.gfeat, C, md->a0, nullptr, st))))
+            if ((s = cuda_ok(ko_mlp_encode(rows + (size_t)off * kMaxK, kMaxK, tb.set_n, tb.kfeat, tb.gfeat, C,
+                                           md->a0, st))))
                 break;
             if ((s = forward(md, C, false, st))) break;
             if (cudaMemcpyAsync(y_all + off, md->y, sizeof(float) * c, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
@@ -750,8 +776,8 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
             const int q = nbase * per, qpad = (q + 127) / 128 * 128;
             for (int off = 0; off < qpad && !s; off += C) {
                 const int c = qpad - off < C ? qpad - off : C;
-                if ((s = cuda_ok(ko_mlp_encode(nb + (size_t)off * kMaxK, kMaxK, nullptr, nullptr, tb.set_n, tb.kfeat,
-                                               tb.gfeat, c, md->a0, nullptr, st))))
+                if ((s = cuda_ok(ko_mlp_encode(nb + (size_t)off * kMaxK, kMaxK, tb.set_n, tb.kfeat, tb.gfeat, c,
+                                               md->a0, st))))
                     break;
                 if ((s = forward(md, c, false, st))) break;
                 if (cudaMemcpyAsync(y_all + off, md->y, sizeof(float) * c, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
@@ -938,7 +964,7 @@ ko_status ko_model_features(const KoSet &h, const int8_t *orders, long long n, f
     for (long long i = 0; i < n; i++) std::memcpy(&hr[(size_t)i * kMaxK], orders + (size_t)i * h.n, h.n);
     std::vector<uint16_t> hx((size_t)n * kMlpIn);
     if (cudaMemcpyAsync(rows, hr.data(), hr.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) s = KO_ERR_CUDA;
-    if (!s) s = cuda_ok(ko_mlp_encode(rows, kMaxK, nullptr, nullptr, tb.set_n, tb.kfeat, tb.gfeat, (int)n, x, nullptr, st));
+    if (!s) s = cuda_ok(ko_mlp_encode(rows, kMaxK, tb.set_n, tb.kfeat, tb.gfeat, (int)n, x, st));
     if (!s && (cudaMemcpyAsync(hx.data(), x, hx.size() * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                cudaStreamSynchronize(st) != cudaSuccess))
         s = KO_ERR_CUDA;

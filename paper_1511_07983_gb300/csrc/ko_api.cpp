@@ -178,7 +178,7 @@ void exhaustive_chunk(ko_gpu *g, KoWork *w_levels)
     c.d0 = d0;
     c.mode = 0;
     *w_levels = KoWork{};
-    w_levels->levels = N - 1 - d0 > 0 ? N - 1 - d0 : 1;
+    w_levels->levels = N - 1 - d0;
 }
 
 ko_status fast_launch_timed(ko_gpu *g, const KoWork &w, cudaStream_t st)

@@ -918,19 +918,19 @@ static bool packs(const KoSet &h) { return h.R < (1 << 19) && h.W <= 127; }
 // Lists of explicit orders: an order costs a whole simulation whatever the
 // list's length, so a short list is bound by one simulation's latency (a warp
 // per simulation is the quickest) and a long one by throughput (a thread per
-// simulation).  Measured, us for 32 lanes / one thread per order:
-//   1,024 orders  N=8, 13 SMs 127 / 210   N=12, 148 SMs 411 / 870   N=20, 13 SMs 634 / 1519
-//   4,096                     192 / 216                 559 / 914               1093 / 1635
-//   16,384                    495 / 227                1545 / 1016              3165 / 1752
-//   100,003 (16 lanes / one) 2039 / 570                6912 / 2073             13710 / 3959
+// simulation).  Measured, us for a warp / a thread per order:
+//   1,024 orders  N=8, 13 SMs 76 / 218   N=12, 148 SMs 202 / 554   N=20, 13 SMs 364 / 1126
+//   8,192                    144 / 229                 418 / 959               794 / 1753
+//   16,384                   234 / 229                 723 / 985              1416 / 1758
+//   50,000                   599 / 376                1883 / 1476             3862 / 2848
 // The one-thread state holds 14 runs: on more than 32 SMs that is enough for
 // up to 13 kernels (under 3 % of random orders overflow in 31 of 32 sampled
-// sets; 14 kernels: 34 to 76 %); beyond, 32 lanes (16,384 orders of N=20 on
-// 148 SMs: 4.0 ms, 16 lanes 7.2 ms, one thread 8.0 ms).
+// sets; 14 kernels: 34 to 76 %); beyond, a warp per order (50,000 orders of N=20
+// on 148 SMs: 3.9 ms, 16 lanes 19.6, one thread 21.0).
 KoChoice ko_list_choice(const KoSet &h, long long count)
 {
     const bool holds = packs(h) && (h.S <= 32 || h.n <= 13);
-    return count > 6144 && holds ? KoChoice{1, 1, 0} : KoChoice{32, 1, 0};
+    return count > 16384 && holds ? KoChoice{1, 1, 0} : KoChoice{32, 1, 0};
 }
 
 // Whole spaces: the work items of a space are its prefixes, each walked by one
@@ -988,8 +988,11 @@ KoRoute::KoRoute(KoFastState *state, KoChoice c, cudaStream_t st, bool always)
 {
     if (fs->chosen && !always) return;
     fs->stack_global = 1;
-    if (capturing(st) && (fs->gstack_bytes < gstack_need(c.levels) ||
-                          (c.lanes == 1 && fs->lslab_bytes < std::max(ko_lane_slab_bytes(c.levels, c.shape), ko_lane_slab_bytes(c.levels, 0))))) {
+    // (a warp per order, the only choice of 32 lanes, needs no slab)
+    if (c.lanes != 32 && capturing(st) &&
+        (fs->gstack_bytes < gstack_need(c.levels) ||
+         (c.lanes == 1 && fs->lslab_bytes < std::max(ko_lane_slab_bytes(c.levels, c.shape),
+                                                     ko_lane_slab_bytes(c.levels, 0))))) {
         while (fs->levels > 1 && fs->gstack_bytes < gstack_need(fs->levels)) fs->levels--;
         return;
     }
@@ -1055,7 +1058,9 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
             fs->lslab_bytes = need;
         }
     }
-    if (fs->stack_global) {
+    const bool orders = !w.space || w.levels < 1;   // items are single orders
+    const bool warps = fs->lanes == 32 && orders;   // a warp each: no node states
+    if (fs->stack_global && !warps) {
         const size_t need = gstack_need(w.levels);
         if (fs->gstack_bytes < need) {
             // a stream being captured cannot take a free or a malloc: the
@@ -1104,6 +1109,19 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
             }
             if (shape == 0) break;
         }
+    }
+    if (warps) {
+        // its runs and groups are as many as the wide pass has
+        next_pass(w);
+        if ((e = ko_launch_warp(w, st)) == cudaSuccess) {
+            w.fb_counter = &fb->fb_counter;
+            e = ko_launch_fallback(w, fs->fb_scratch, fs->fb_bytes, max_slab_bytes, st);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return KO_ERR_CUDA;
+        }
+        return KO_OK;
     }
     // all items (or those the one-thread passes abandoned), 16 or 32 lanes per simulation, 8 group slots
     next_pass(w);

@@ -119,6 +119,10 @@ cudaError_t ko_launch_lane(const KoWork &w, int shape, cudaStream_t st);
 size_t ko_lane_slab_bytes(int levels, int shape);
 long long ko_lane_threads(int shape);  // simulations a full launch runs at a time
 
+// One warp per simulation (ko_warp.cu) over the items of `w` (counters and list
+// set): lists, or spaces of single orders (no saved levels).
+cudaError_t ko_launch_warp(const KoWork &w, cudaStream_t st);
+
 // Device address of the count of items the first pass of the last launch abandoned.
 const unsigned long long *ko_fast_overflow_counter(const KoFastState *fs);
 

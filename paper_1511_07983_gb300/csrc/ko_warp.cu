@@ -1,0 +1,423 @@
+// One simulation per warp, one run of SMs per lane: the pass over short lists of
+// explicit orders (and over spaces walked order by order), where the time of a
+// single simulation decides.
+//
+// Same model and runs as the run-length simulator (ko_fast.cu), laid out for a
+// short chain of dependent instructions per event:
+//   * runs are unordered (a split appends a lane), so a split moves no lanes;
+//   * a lane keeps what its SMs have free and the earliest end of its groups in
+//     registers and its groups (end, descriptor) in its own column of shared
+//     memory, free of bank conflicts; an event reads the column once, in one
+//     burst of independent loads, for what ends and for the next end;
+//   * between a kernel's first and last burst an event changes only the lanes
+//     whose groups end, and those take their full capacity, so the event is
+//     three warp reductions (next end, blocks taken, pointer) and one lane's
+//     work; the joint water-fill runs once per kernel, for the burst that
+//     empties the queue.
+// It is bound by instruction latency: a list of a few hundred orders is one or
+// two warps per SM sub-partition.  The run-length kernel took 3,200 cycles per
+// event here (its groups in registers behind select chains, two reductions more
+// per event, lanes shifted by every split).  570 orders, us before -> after:
+// N=8 on 13 SMs 124 -> 75, N=20 on 13 SMs 608 -> 342, N=20 on 148 SMs 573 -> 376.
+#include "ko_fast.h"
+#include "ko_units.cuh"
+
+namespace {
+
+constexpr unsigned kAll = 0xffffffffu;
+constexpr int kWarps = 4;        // at most, per block
+constexpr int kSlots16 = 16;     // group slots of a run
+constexpr int kPosBits = 12;     // a pointer move is 1 .. N_SM <= 1024
+
+__constant__ unsigned long long c_warp_fact[21] = {
+    1ull, 1ull, 2ull, 6ull, 24ull, 120ull, 720ull, 5040ull, 40320ull, 362880ull, 3628800ull,
+    39916800ull, 479001600ull, 6227020800ull, 87178291200ull, 1307674368000ull,
+    20922789888000ull, 355687428096000ull, 6402373705728000ull, 121645100408832000ull,
+    2432902008176640000ull};
+
+// One kernel's constants: a block's needs and cycles, blocks, and the reciprocals
+// of the needs rounded down (ko_lane_sim.cuh's cap() says why that is exact).
+struct __align__(16) WarpKern {
+    int r, s, w, c;
+    int m, b;
+    float frr, frs;
+    float frw, fsb;
+    int pad0, pad1;
+};
+
+struct WarpMem {
+    uint32_t end[kSlots16][32];
+    uint32_t desc[kSlots16][32];  // kernel | blocks per SM << 5
+    WarpKern k[KO_MAX_KERNELS];
+};
+
+// A lane's run and the simulation's warp-uniform state.
+struct WarpSim {
+    WarpMem &mem;
+    int lane;
+    int S;
+    uint32_t ccap, mcap;
+    int cshift, mshift;
+    // run
+    int beg, cnt, fr, fs, fw, fb;   // SMs; free registers, shared memory, warps, blocks of each
+    uint32_t sc, sm, re;            // SumC, SumM, earliest end of its groups (where it has any)
+    uint32_t used, pend;            // group slots in use; of groups whose burst is open
+    // simulation
+    unsigned long long t;
+    int p, nr;
+
+    __device__ void init(const KoSet *set)
+    {
+        beg = 0;
+        cnt = lane == 0 ? S : 0;
+        fr = set->R; fs = set->Sh; fw = set->W; fb = set->Bk;
+        sc = sm = re = 0;
+        used = pend = 0;
+        t = 0;
+        p = 0;
+        nr = 1;
+    }
+
+    __device__ __forceinline__ int cap(const WarpKern &h) const
+    {
+        float f = (float)fr * h.frr;
+        f = fminf(f, fminf((float)fw * h.frw, (float)fs * h.frs + h.fsb));
+        int q = (int)fminf(f, 40.0f);
+        if ((q + 1) * h.r <= fr && (q + 1) * h.w <= fw && (q + 1) * h.s <= fs) q++;
+        return min(q, fb);
+    }
+
+    __device__ __forceinline__ uint32_t duration(uint32_t c, uint32_t m) const
+    {
+        const unsigned long long pc = (unsigned long long)c * max(sc, ccap) + (ccap - 1u);
+        const unsigned long long pm = (unsigned long long)m * max(sm, mcap) + (mcap - 1u);
+        const uint32_t dc = cshift >= 0 ? (uint32_t)(pc >> cshift) : (uint32_t)(pc / ccap);
+        const uint32_t dm = mshift >= 0 ? (uint32_t)(pm >> mshift) : (uint32_t)(pm / mcap);
+        return max(dc, dm);
+    }
+
+    // q blocks per SM of kernel k as a new group; its slot, or -1 without one.
+    __device__ __forceinline__ int place(const WarpKern &h, int k, int q)
+    {
+        const int g = __ffs((int)(~used & 0xffffu)) - 1;
+        if (g < 0) return -1;
+        used |= 1u << g;
+        mem.desc[g][lane] = (uint32_t)k | ((uint32_t)q << 5);
+        fr -= q * h.r; fs -= q * h.s; fw -= q * h.w; fb -= q;
+        sc += (uint32_t)(q * h.c); sm += (uint32_t)(q * h.m);
+        return g;
+    }
+
+    __device__ __forceinline__ void start(int g, uint32_t dur)
+    {
+        const uint32_t t32 = (uint32_t)t;
+        mem.end[g][lane] = t32 + dur;
+        // the slots besides g decide whether `re` holds an end
+        if ((used & ~pend & ~(1u << g)) == 0u || dur < re - t32) re = t32 + dur;
+    }
+
+    // Durations of the groups whose burst closes now.
+    __device__ void close_burst()
+    {
+        while (__any_sync(kAll, pend != 0u)) {
+            if (pend) {
+                const int g = __ffs((int)pend) - 1;
+                const WarpKern &q = mem.k[mem.desc[g][lane] & 31u];
+                start(g, duration((uint32_t)q.c, (uint32_t)q.m));
+                pend &= pend - 1u;
+            }
+        }
+    }
+
+    // Release the groups that end at t; `re` becomes the earliest end of the rest.
+    __device__ __forceinline__ void release()
+    {
+        const uint32_t now = (uint32_t)t;
+        uint32_t gone = 0, next = 0xffffffffu;
+#pragma unroll
+        for (int g = 0; g < 8; g++) {
+            const uint32_t d = mem.end[g][lane] - now;
+            if ((used >> g) & 1u) {
+                if (d == 0u) gone |= 1u << g; else next = min(next, d);
+            }
+        }
+        if (used >> 8) {
+#pragma unroll
+            for (int g = 8; g < kSlots16; g++) {
+                const uint32_t d = mem.end[g][lane] - now;
+                if ((used >> g) & 1u) {
+                    if (d == 0u) gone |= 1u << g; else next = min(next, d);
+                }
+            }
+        }
+        used &= ~gone;
+        re = now + next;
+        do {  // a run is released because a group of it ends
+            const int g = __ffs((int)gone) - 1;
+            gone &= gone - 1u;
+            const uint32_t d = mem.desc[g][lane];
+            const WarpKern &k = mem.k[d & 31u];
+            const int q = (int)(d >> 5);
+            fr += q * k.r; fs += q * k.s; fw += q * k.w; fb += q;
+            sc -= (uint32_t)(q * k.c); sm -= (uint32_t)(q * k.m);
+        } while (gone);
+    }
+
+    // How far past p (in SMs, cyclically) the run's last SM lies, 1 .. S.
+    __device__ __forceinline__ int last_past() const
+    {
+        const int d = beg + cnt - p;
+        if (beg < p && d > 0) return S;  // p lies inside: its last SM from p on is p - 1
+        return d <= 0 ? d + S : d;
+    }
+
+    // Lane j keeps the run's first x SMs (0 < x < its count); lane nr takes the rest.
+    __device__ void split(int j, int x)
+    {
+        const int k = nr++;
+        __syncwarp();
+        if (lane < kSlots16) {
+            mem.end[lane][k] = mem.end[lane][j];
+            mem.desc[lane][k] = mem.desc[lane][j];
+        }
+        const int b = __shfl_sync(kAll, beg, j), n = __shfl_sync(kAll, cnt, j);
+        const int r = __shfl_sync(kAll, fr, j), s = __shfl_sync(kAll, fs, j), w = __shfl_sync(kAll, fw, j),
+                  bl = __shfl_sync(kAll, fb, j);
+        const uint32_t c = __shfl_sync(kAll, sc, j), m = __shfl_sync(kAll, sm, j), e = __shfl_sync(kAll, re, j);
+        const uint32_t masks = __shfl_sync(kAll, used | (pend << 16), j);
+        if (lane == j) cnt = x;
+        if (lane == k) {
+            beg = b + x; cnt = n - x;
+            fr = r; fs = s; fw = w; fb = bl;
+            sc = c; sm = m; re = e;
+            used = masks & 0xffffu; pend = masks >> 16;
+        }
+        __syncwarp();
+    }
+
+    // The burst that empties the queue: `left` blocks over lanes with room q, of
+    // which there is more in all.  Every SM ends with min(room, L - 1) blocks of
+    // it and the first ones past p with more room have one more; runs are cut at p
+    // and where the last sweep stops.  False if a run or a slot is missing.
+    __device__ bool place_last(const WarpKern &h, int kern, int left, int q, int run_limit)
+    {
+        int lo = 1, hi = (int)__reduce_max_sync(kAll, (unsigned)q);
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if ((int)__reduce_add_sync(kAll, (unsigned)(cnt * min(q, mid))) >= left) hi = mid; else lo = mid + 1;
+        }
+        const int rem = left - (int)__reduce_add_sync(kAll, (unsigned)(cnt * min(q, lo - 1)));  // >= 1
+        const unsigned inside = __ballot_sync(kAll, q >= lo && beg < p && p < beg + cnt);
+        if (inside) {
+            if (nr >= run_limit) return false;
+            const int j = __ffs((int)inside) - 1, k = nr;
+            const int room = __shfl_sync(kAll, q, j);
+            split(j, p - __shfl_sync(kAll, beg, j));
+            if (lane == k) q = room;
+        }
+        // the runs with room in the last sweep, in cyclic order from p: SMs before this one
+        const bool in = q >= lo && cnt > 0;
+        const int e = in ? cnt : 0;
+        int d = beg - p;
+        if (d < 0) d += S;
+        int before = 0;
+        for (unsigned m = __ballot_sync(kAll, in); m; m &= m - 1u) {
+            const int j = __ffs((int)m) - 1;
+            const int dj = __shfl_sync(kAll, d, j), ej = __shfl_sync(kAll, e, j);
+            if (dj < d) before += ej;
+        }
+        int give = min(q, lo - 1) + (in && before < rem ? 1 : 0);
+        const unsigned here = __ballot_sync(kAll, in && before < rem && rem <= before + e);
+        const int star = __ffs((int)here) - 1;  // exactly one: 1 <= rem <= SMs with room
+        const int x = rem - __shfl_sync(kAll, before, star);
+        p = __shfl_sync(kAll, beg, star) + x;
+        if (p >= S) p -= S;
+        if (x < __shfl_sync(kAll, cnt, star)) {
+            if (nr >= run_limit) return false;
+            const int k = nr;
+            const int room = __shfl_sync(kAll, give, star);
+            split(star, x);
+            if (lane == k) give = room - 1;
+        }
+        bool ok = true;
+        if (give > 0) {
+            const int g = place(h, kern, give);
+            ok = g >= 0;
+            if (ok) pend |= 1u << g;
+        }
+        return __all_sync(kAll, ok);
+    }
+
+    // Queue all blocks of kernel `kern` behind the current queue and simulate until
+    // the last of them is placed (its burst stays open).  False if the state
+    // cannot hold it.
+    __device__ bool place_kernel(int kern, int limit, int run_limit)
+    {
+        const WarpKern h = mem.k[kern];
+        int left = h.b;
+        bool fresh = cnt > 0, first = true;
+        for (int it = 0; it < limit; it++) {
+            const int q = fresh ? cap(h) : 0;
+            const int total = (int)__reduce_add_sync(kAll, (unsigned)(q * cnt));
+            if (total > left) return place_last(h, kern, left, q, run_limit);
+            // every lane in it takes its room; p moves past the last SM with the most
+            unsigned key = q > 0 ? ((unsigned)q << kPosBits) | (unsigned)last_past() : 0u;
+            if (q > 0 && used == 0xffffu) key = 0xffffffffu;
+            const unsigned top = __reduce_max_sync(kAll, key);
+            if (top == 0xffffffffu) return false;
+            p += (int)(top & ((1u << kPosBits) - 1u));
+            if (p >= S) p -= S;
+            left -= total;
+            if (q > 0) {
+                const int g = place(h, kern, q);
+                if (left == 0 || first) pend |= 1u << g;
+                else start(g, duration((uint32_t)h.c, (uint32_t)h.m));
+            }
+            if (left == 0) return true;
+            if (first) close_burst();
+            first = false;
+            // the earliest end of all
+            const uint32_t rel = used ? re - (uint32_t)t : 0xffffffffu;
+            const uint32_t dmin = __reduce_min_sync(kAll, rel);
+            if (dmin == 0xffffffffu) return false;
+            t += dmin;
+            fresh = rel == dmin;
+            if (fresh) release();
+            __syncwarp();
+        }
+        return false;  // each event frees a block: not reached
+    }
+
+    // Close the last burst; the makespan is the latest end.
+    __device__ unsigned long long finish()
+    {
+        close_burst();
+        const uint32_t now = (uint32_t)t;
+        uint32_t last = 0;
+#pragma unroll
+        for (int g = 0; g < kSlots16; g++)
+            if ((used >> g) & 1u) last = max(last, mem.end[g][lane] - now);
+        return t + __reduce_max_sync(kAll, last);
+    }
+};
+
+__global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
+{
+    __shared__ WarpMem mems[kWarps];
+    const int lane = threadIdx.x & 31;
+    WarpSim sim{mems[threadIdx.x >> 5], lane};
+    const int run_limit = a.run_limit < 32 ? a.run_limit : 32;
+    int loaded = -1, n = 0, limit = 0;
+    const KoSet *set = nullptr;
+    for (;;) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(a.counter, 1ull);
+        item = __shfl_sync(kAll, item, 0);
+        if (item >= (unsigned long long)a.n_items) break;
+        int lo = 0, hi = a.nchunks - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.chunks[mid].first <= (long long)item) lo = mid; else hi = mid - 1;
+        }
+        const KoChunk ch = a.chunks[lo];
+        if (ch.set != loaded) {
+            loaded = ch.set;
+            set = a.sets + ch.set;
+            n = set->n;
+            int blocks = 0;
+            __syncwarp();
+            if (lane < n) {
+                const KoKern k = set->k[lane];
+                const float down = 1.0f - 1.0f / 262144.0f;
+                blocks = k.b;
+                sim.mem.k[lane] = WarpKern{k.r, k.s, k.w, k.c, k.m, k.b, __fdividef(down, (float)k.r),
+                                           k.s > 0 ? __fdividef(down, (float)k.s) : 0.0f,
+                                           __fdividef(down, (float)k.w), k.s > 0 ? 0.0f : 40.0f, 0, 0};
+            }
+            limit = (int)__reduce_add_sync(kAll, (unsigned)blocks) + 64;
+            sim.S = set->S;
+            sim.ccap = (uint32_t)set->ccap; sim.mcap = (uint32_t)set->mcap;
+            sim.cshift = set->cshift; sim.mshift = set->mshift;
+            __syncwarp();
+        }
+        // lane d holds the kernel at position d
+        const long long local = (long long)item - ch.first;
+        long long outpos = ch.out_off + local;
+        int mine = -1;
+        bool valid = true;
+        if (ch.mode == 2) {
+            const int8_t *row = a.perms + ch.list_off + local * (a.perm_stride ? a.perm_stride : n);
+            const int v = lane < n ? row[lane] : 0;
+            const bool range = lane >= n || (v >= 0 && v < n);
+            const unsigned seen = __reduce_or_sync(kAll, lane < n && range ? 1u << v : 0u);
+            valid = __all_sync(kAll, range) && seen == (n < 32 ? (1u << n) - 1u : kAll);
+            mine = v;
+        } else {
+            // a Lehmer index; a prefix of all kernels but one leaves no choice either
+            unsigned long long k;
+            if (ch.mode == 1) {
+                k = a.idx[ch.list_off + local];
+                valid = k < c_warp_fact[n];
+            } else {
+                k = (unsigned long long)(ch.list_off + local) * c_warp_fact[n - ch.d0];
+                outpos = ch.out_off + (long long)k;
+            }
+            unsigned rest = (1u << n) - 1u;
+            for (int d = 0; valid && d < n; d++) {
+                const unsigned long long f = c_warp_fact[n - 1 - d];
+                const unsigned digit = (unsigned)(k / f);
+                k -= (unsigned long long)digit * f;
+                unsigned u = rest;
+                for (unsigned q = 0; q < digit; q++) u &= u - 1u;
+                const int v = __ffs((int)u) - 1;
+                rest &= ~(1u << v);
+                if (lane == d) mine = v;
+            }
+        }
+        if (!valid) {
+            if (lane == 0 && a.out) a.out[outpos] = -1;
+            continue;
+        }
+        sim.init(set);
+        bool ok = true;
+        for (int d = 0; ok && d < n; d++) ok = sim.place_kernel(__shfl_sync(kAll, mine, d), limit, run_limit);
+        if (!ok) {
+            if (lane == 0) {
+                const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
+                if (slot < a.ov_cap) a.ov_list[slot] = kounits::entry_of(item, 0u, 0);
+                atomicAdd(a.abandoned, 1ull);
+            }
+            continue;
+        }
+        const unsigned long long ms = sim.finish();
+        if (lane == 0) {
+            if (a.out) a.out[outpos] = (int64_t)ms;
+            if (a.accs) {
+                KoAccum *acc = a.accs + ch.set;
+                const unsigned long long ref = (unsigned long long)(a.refs ? a.refs[ch.set] : set->ref_makespan);
+                atomicMin(&acc->min, ms);
+                atomicMax(&acc->max, ms);
+                atomicAdd(ms < ref ? &acc->n_better : ms == ref ? &acc->n_equal : &acc->n_worse, 1ull);
+            }
+        }
+    }
+}
+
+}  // namespace
+
+cudaError_t ko_launch_warp(const KoWork &a, cudaStream_t st)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // as few warps per block as give every warp one order, up to one per sub-partition
+    const long long per_sm = (a.n_items + sms - 1) / sms;
+    const int warps = per_sm < 1 ? 1 : per_sm < kWarps ? (int)per_sm : kWarps;
+    long long blocks = (a.n_items + warps - 1) / warps;
+    const long long resident = (long long)sms * 8;
+    if (blocks > resident) blocks = resident;
+    if (blocks < 1) blocks = 1;
+    warp_kernel<<<(unsigned)blocks, warps * 32, 0, st>>>(a);
+    ko_count_launch();
+    return cudaGetLastError();
+}

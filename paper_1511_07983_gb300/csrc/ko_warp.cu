@@ -14,11 +14,17 @@
 //     three warp reductions (next end, blocks taken, pointer) and one lane's
 //     work; the joint water-fill runs once per kernel, for the burst that
 //     empties the queue.
-// It is bound by instruction latency: a list of a few hundred orders is one or
-// two warps per SM sub-partition.  The run-length kernel took 3,200 cycles per
-// event here (its groups in registers behind select chains, two reductions more
-// per event, lanes shifted by every split).  570 orders, us before -> after:
-// N=8 on 13 SMs 124 -> 75, N=20 on 13 SMs 608 -> 342, N=20 on 148 SMs 573 -> 376.
+//   * the slot and descriptor of a lane's next group to end are at hand, so its
+//     release does not wait for a look through the column; its room and the
+//     duration of what it takes come before the reductions that decide whether
+//     the queue runs empty.
+// It is bound by instruction latency (570 orders of N=20 on 13 SMs, one warp per
+// SM sub-partition: 229 warp instructions per event at 4.2 cycles each, half of
+// that waits for the previous instruction).  The run-length kernel took 3,200
+// cycles per event here (its groups in registers behind select chains, two
+// reductions more per event, lanes shifted by every split).  570 orders, us
+// before -> after: N=8 on 13 SMs 124 -> 60, N=20 on 13 SMs 608 -> 268, N=20 on
+// 148 SMs 573 -> 283.
 #include "ko_fast.h"
 #include "ko_units.cuh"
 
@@ -51,6 +57,9 @@ struct WarpMem {
     WarpKern k[KO_MAX_KERNELS];
 };
 
+// a / b for capacities that are no power of two; one copy of the long division.
+__device__ __noinline__ uint32_t quotient(unsigned long long a, uint32_t b) { return (uint32_t)(a / b); }
+
 // A lane's run and the simulation's warp-uniform state.
 struct WarpSim {
     WarpMem &mem;
@@ -58,10 +67,13 @@ struct WarpSim {
     int S;
     uint32_t ccap, mcap;
     int cshift, mshift;
+    bool shifts;                    // both capacities are powers of two
     // run
     int beg, cnt, fr, fs, fw, fb;   // SMs; free registers, shared memory, warps, blocks of each
     uint32_t sc, sm, re;            // SumC, SumM, earliest end of its groups (where it has any)
     uint32_t used, pend;            // group slots in use; of groups whose burst is open
+    int rslot;                      // the group that ends at re: its slot and descriptor
+    uint32_t rdesc;
     // simulation
     unsigned long long t;
     int p, nr;
@@ -73,6 +85,8 @@ struct WarpSim {
         fr = set->R; fs = set->Sh; fw = set->W; fb = set->Bk;
         sc = sm = re = 0;
         used = pend = 0;
+        rslot = 0;
+        rdesc = 0;
         t = 0;
         p = 0;
         nr = 1;
@@ -87,13 +101,13 @@ struct WarpSim {
         return min(q, fb);
     }
 
-    __device__ __forceinline__ uint32_t duration(uint32_t c, uint32_t m) const
+    // Cycles of a block started when its SM's sums are c_sum / m_sum.
+    __device__ __forceinline__ uint32_t duration(uint32_t c, uint32_t m, uint32_t c_sum, uint32_t m_sum) const
     {
-        const unsigned long long pc = (unsigned long long)c * max(sc, ccap) + (ccap - 1u);
-        const unsigned long long pm = (unsigned long long)m * max(sm, mcap) + (mcap - 1u);
-        const uint32_t dc = cshift >= 0 ? (uint32_t)(pc >> cshift) : (uint32_t)(pc / ccap);
-        const uint32_t dm = mshift >= 0 ? (uint32_t)(pm >> mshift) : (uint32_t)(pm / mcap);
-        return max(dc, dm);
+        const unsigned long long pc = (unsigned long long)c * max(c_sum, ccap) + (ccap - 1u);
+        const unsigned long long pm = (unsigned long long)m * max(m_sum, mcap) + (mcap - 1u);
+        if (shifts) return max((uint32_t)(pc >> cshift), (uint32_t)(pm >> mshift));
+        return max(quotient(pc, ccap), quotient(pm, mcap));
     }
 
     // q blocks per SM of kernel k as a new group; its slot, or -1 without one.
@@ -108,12 +122,17 @@ struct WarpSim {
         return g;
     }
 
-    __device__ __forceinline__ void start(int g, uint32_t dur)
+    // Group g (descriptor d) ends at t + dur.
+    __device__ __forceinline__ void start(int g, uint32_t d, uint32_t dur)
     {
         const uint32_t t32 = (uint32_t)t;
         mem.end[g][lane] = t32 + dur;
         // the slots besides g decide whether `re` holds an end
-        if ((used & ~pend & ~(1u << g)) == 0u || dur < re - t32) re = t32 + dur;
+        if ((used & ~pend & ~(1u << g)) == 0u || dur < re - t32) {
+            re = t32 + dur;
+            rslot = g;
+            rdesc = d;
+        }
     }
 
     // Durations of the groups whose burst closes now.
@@ -122,45 +141,55 @@ struct WarpSim {
         while (__any_sync(kAll, pend != 0u)) {
             if (pend) {
                 const int g = __ffs((int)pend) - 1;
-                const WarpKern &q = mem.k[mem.desc[g][lane] & 31u];
-                start(g, duration((uint32_t)q.c, (uint32_t)q.m));
+                const uint32_t d = mem.desc[g][lane];
+                const WarpKern &q = mem.k[d & 31u];
+                start(g, d, duration((uint32_t)q.c, (uint32_t)q.m, sc, sm));
                 pend &= pend - 1u;
             }
         }
     }
 
-    // Release the groups that end at t; `re` becomes the earliest end of the rest.
+    // Release the groups that end at t -- the one at rslot and any others -- and
+    // find the earliest end of the rest.  The first group's descriptor is at hand
+    // since the last time the lane looked, so its constants load while the ends
+    // are read.
     __device__ __forceinline__ void release()
     {
         const uint32_t now = (uint32_t)t;
-        uint32_t gone = 0, next = 0xffffffffu;
-#pragma unroll
-        for (int g = 0; g < 8; g++) {
-            const uint32_t d = mem.end[g][lane] - now;
-            if ((used >> g) & 1u) {
-                if (d == 0u) gone |= 1u << g; else next = min(next, d);
-            }
-        }
-        if (used >> 8) {
-#pragma unroll
-            for (int g = 8; g < kSlots16; g++) {
-                const uint32_t d = mem.end[g][lane] - now;
-                if ((used >> g) & 1u) {
-                    if (d == 0u) gone |= 1u << g; else next = min(next, d);
-                }
-            }
-        }
-        used &= ~gone;
-        re = now + next;
-        do {  // a run is released because a group of it ends
-            const int g = __ffs((int)gone) - 1;
-            gone &= gone - 1u;
-            const uint32_t d = mem.desc[g][lane];
+        uint32_t gone = 1u << rslot, d = rdesc, next;
+        do {
             const WarpKern &k = mem.k[d & 31u];
             const int q = (int)(d >> 5);
-            fr += q * k.r; fs += q * k.s; fw += q * k.w; fb += q;
-            sc -= (uint32_t)(q * k.c); sm -= (uint32_t)(q * k.m);
-        } while (gone);
+            const int4 a = *reinterpret_cast<const int4 *>(&k);
+            const int km = k.m;
+            used &= ~gone;
+            uint32_t e[8];
+#pragma unroll
+            for (int g = 0; g < 8; g++) {
+                e[g] = mem.end[g][lane] - now;
+                if (!((used >> g) & 1u)) e[g] = 0xffffffffu;
+            }
+            next = min(min(min(e[0], e[1]), min(e[2], e[3])), min(min(e[4], e[5]), min(e[6], e[7])));
+            gone = 0;
+#pragma unroll
+            for (int g = 0; g < 8; g++) gone |= e[g] == next ? 1u << g : 0u;
+            if (used >> 8) {
+                for (uint32_t m = used >> 8; m; m &= m - 1u) {
+                    const int g = __ffs((int)m) + 7;
+                    const uint32_t x = mem.end[g][lane] - now;
+                    if (x < next) { next = x; gone = 0; }
+                    if (x == next) gone |= 1u << g;
+                }
+            }
+            gone &= used;
+            gone &= 0u - gone;  // the first of equal ones
+            rslot = gone ? __ffs((int)gone) - 1 : 0;
+            d = mem.desc[rslot][lane];
+            fr += q * a.x; fs += q * a.y; fw += q * a.z; fb += q;
+            sc -= (uint32_t)(q * a.w); sm -= (uint32_t)(q * km);
+        } while (next == 0u);
+        rdesc = d;
+        re = now + next;
     }
 
     // How far past p (in SMs, cyclically) the run's last SM lies, 1 .. S.
@@ -185,12 +214,15 @@ struct WarpSim {
                   bl = __shfl_sync(kAll, fb, j);
         const uint32_t c = __shfl_sync(kAll, sc, j), m = __shfl_sync(kAll, sm, j), e = __shfl_sync(kAll, re, j);
         const uint32_t masks = __shfl_sync(kAll, used | (pend << 16), j);
+        const uint32_t rd = __shfl_sync(kAll, rdesc, j);
+        const int rs = __shfl_sync(kAll, rslot, j);
         if (lane == j) cnt = x;
         if (lane == k) {
             beg = b + x; cnt = n - x;
             fr = r; fs = s; fw = w; fb = bl;
             sc = c; sm = m; re = e;
             used = masks & 0xffffu; pend = masks >> 16;
+            rdesc = rd; rslot = rs;
         }
         __syncwarp();
     }
@@ -248,6 +280,18 @@ struct WarpSim {
         return __all_sync(kAll, ok);
     }
 
+    // Every lane takes its room q: p moves past the last SM with the most.  False
+    // if a lane has no slot.
+    __device__ __forceinline__ bool move_pointer(int q)
+    {
+        unsigned key = q > 0 ? ((unsigned)q << kPosBits) | (unsigned)last_past() : 0u;
+        if (q > 0 && used == 0xffffu) key = 0xffffffffu;
+        const unsigned top = __reduce_max_sync(kAll, key);
+        p += (int)(top & ((1u << kPosBits) - 1u));
+        if (p >= S) p -= S;
+        return top != 0xffffffffu;
+    }
+
     // Queue all blocks of kernel `kern` behind the current queue and simulate until
     // the last of them is placed (its burst stays open).  False if the state
     // cannot hold it.
@@ -255,35 +299,41 @@ struct WarpSim {
     {
         const WarpKern h = mem.k[kern];
         int left = h.b;
-        bool fresh = cnt > 0, first = true;
-        for (int it = 0; it < limit; it++) {
-            const int q = fresh ? cap(h) : 0;
+        {   // the first burst continues the open one: every run is offered the kernel
+            const int q = cnt > 0 ? cap(h) : 0;
             const int total = (int)__reduce_add_sync(kAll, (unsigned)(q * cnt));
             if (total > left) return place_last(h, kern, left, q, run_limit);
-            // every lane in it takes its room; p moves past the last SM with the most
-            unsigned key = q > 0 ? ((unsigned)q << kPosBits) | (unsigned)last_past() : 0u;
-            if (q > 0 && used == 0xffffu) key = 0xffffffffu;
-            const unsigned top = __reduce_max_sync(kAll, key);
-            if (top == 0xffffffffu) return false;
-            p += (int)(top & ((1u << kPosBits) - 1u));
-            if (p >= S) p -= S;
+            if (!move_pointer(q)) return false;
             left -= total;
-            if (q > 0) {
-                const int g = place(h, kern, q);
-                if (left == 0 || first) pend |= 1u << g;
-                else start(g, duration((uint32_t)h.c, (uint32_t)h.m));
-            }
+            if (q > 0) pend |= 1u << place(h, kern, q);
             if (left == 0) return true;
-            if (first) close_burst();
-            first = false;
-            // the earliest end of all
+            close_burst();
+        }
+        for (int it = 0; it < limit; it++) {
             const uint32_t rel = used ? re - (uint32_t)t : 0xffffffffu;
             const uint32_t dmin = __reduce_min_sync(kAll, rel);
             if (dmin == 0xffffffffu) return false;
             t += dmin;
-            fresh = rel == dmin;
-            if (fresh) release();
+            int q = 0;
+            uint32_t dur = 0;
+            if (rel == dmin) {
+                release();
+                q = cap(h);
+                // the duration of what it takes, should the queue not run empty
+                dur = duration((uint32_t)h.c, (uint32_t)h.m, sc + (uint32_t)(q * h.c), sm + (uint32_t)(q * h.m));
+            }
             __syncwarp();
+            const int total = (int)__reduce_add_sync(kAll, (unsigned)(q * cnt));
+            if (total > left) return place_last(h, kern, left, q, run_limit);
+            if (!move_pointer(q)) return false;
+            left -= total;
+            if (q > 0) {
+                const int g = place(h, kern, q);
+                if (left == 0) pend |= 1u << g;
+                else start(g, (uint32_t)kern | ((uint32_t)q << 5), dur);
+            }
+            __syncwarp();
+            if (left == 0) return true;
         }
         return false;  // each event frees a block: not reached
     }
@@ -338,6 +388,7 @@ __global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
             sim.S = set->S;
             sim.ccap = (uint32_t)set->ccap; sim.mcap = (uint32_t)set->mcap;
             sim.cshift = set->cshift; sim.mshift = set->mshift;
+            sim.shifts = set->cshift >= 0 && set->mshift >= 0;
             __syncwarp();
         }
         // lane d holds the kernel at position d

@@ -110,10 +110,11 @@ struct WarpSim {
         return max(quotient(pc, ccap), quotient(pm, mcap));
     }
 
-    // q blocks per SM of kernel k as a new group; its slot, or -1 without one.
-    __device__ __forceinline__ int place(const WarpKern &h, int k, int q)
+    // q blocks per SM of kernel k as a new group in a slot outside `taken`; the
+    // slot, or -1 without one.
+    __device__ __forceinline__ int place(const WarpKern &h, int k, int q, uint32_t taken)
     {
-        const int g = __ffs((int)(~used & 0xffffu)) - 1;
+        const int g = __ffs((int)(~taken & 0xffffu)) - 1;
         if (g < 0) return -1;
         used |= 1u << g;
         mem.desc[g][lane] = (uint32_t)k | ((uint32_t)q << 5);
@@ -122,14 +123,13 @@ struct WarpSim {
         return g;
     }
 
-    // Group g (descriptor d) ends at t + dur.
-    __device__ __forceinline__ void start(int g, uint32_t d, uint32_t dur)
+    // Group g (descriptor d), started now, ends after dur.
+    __device__ __forceinline__ void start(uint32_t now, int g, uint32_t d, uint32_t dur)
     {
-        const uint32_t t32 = (uint32_t)t;
-        mem.end[g][lane] = t32 + dur;
+        mem.end[g][lane] = now + dur;
         // the slots besides g decide whether `re` holds an end
-        if ((used & ~pend & ~(1u << g)) == 0u || dur < re - t32) {
-            re = t32 + dur;
+        if ((used & ~pend & ~(1u << g)) == 0u || dur < re - now) {
+            re = now + dur;
             rslot = g;
             rdesc = d;
         }
@@ -143,19 +143,18 @@ struct WarpSim {
                 const int g = __ffs((int)pend) - 1;
                 const uint32_t d = mem.desc[g][lane];
                 const WarpKern &q = mem.k[d & 31u];
-                start(g, d, duration((uint32_t)q.c, (uint32_t)q.m, sc, sm));
+                start((uint32_t)t, g, d, duration((uint32_t)q.c, (uint32_t)q.m, sc, sm));
                 pend &= pend - 1u;
             }
         }
     }
 
-    // Release the groups that end at t -- the one at rslot and any others -- and
+    // Release the groups that end now -- the one at rslot and any others -- and
     // find the earliest end of the rest.  The first group's descriptor is at hand
     // since the last time the lane looked, so its constants load while the ends
     // are read.
-    __device__ __forceinline__ void release()
+    __device__ __forceinline__ void release(uint32_t now)
     {
-        const uint32_t now = (uint32_t)t;
         uint32_t gone = 1u << rslot, d = rdesc, next;
         do {
             const WarpKern &k = mem.k[d & 31u];
@@ -192,8 +191,8 @@ struct WarpSim {
         re = now + next;
     }
 
-    // How far past p (in SMs, cyclically) the run's last SM lies, 1 .. S.
-    __device__ __forceinline__ int last_past() const
+    // How far past `p` (in SMs, cyclically) the run's last SM lies, 1 .. S.
+    __device__ __forceinline__ int last_past(int p) const
     {
         const int d = beg + cnt - p;
         if (beg < p && d > 0) return S;  // p lies inside: its last SM from p on is p - 1
@@ -273,7 +272,7 @@ struct WarpSim {
         }
         bool ok = true;
         if (give > 0) {
-            const int g = place(h, kern, give);
+            const int g = place(h, kern, give, used);
             ok = g >= 0;
             if (ok) pend |= 1u << g;
         }
@@ -284,7 +283,7 @@ struct WarpSim {
     // if a lane has no slot.
     __device__ __forceinline__ bool move_pointer(int q)
     {
-        unsigned key = q > 0 ? ((unsigned)q << kPosBits) | (unsigned)last_past() : 0u;
+        unsigned key = q > 0 ? ((unsigned)q << kPosBits) | (unsigned)last_past(p) : 0u;
         if (q > 0 && used == 0xffffu) key = 0xffffffffu;
         const unsigned top = __reduce_max_sync(kAll, key);
         p += (int)(top & ((1u << kPosBits) - 1u));
@@ -292,9 +291,67 @@ struct WarpSim {
         return top != 0xffffffffu;
     }
 
+    // p after a burst in which lanes with key > 0 placed: past the last SM of those
+    // with the largest key.  p always lies where a run begins (it is set to the end
+    // of a run, and runs only ever split), so one such lane alone decides it;
+    // -1 where several do and `from`, the pointer before, is not known (< 0).
+    __device__ __forceinline__ int pointer_after(unsigned key, int from) const
+    {
+        const unsigned top = __reduce_max_sync(kAll, key);
+        const unsigned who = __ballot_sync(kAll, key == top);
+        if ((who & (who - 1u)) == 0u) {
+            const int end = __shfl_sync(kAll, beg + cnt, __ffs((int)who) - 1);
+            return end >= S ? end - S : end;
+        }
+        if (from < 0) return -1;
+        const int to = from + (int)__reduce_max_sync(kAll, key == top ? (unsigned)last_past(from) : 0u);
+        return to >= S ? to - S : to;
+    }
+
+    // The state a run has after its next event, worked out ahead of time.
+    struct Ahead {
+        int fr, fs, fw, fb;
+        uint32_t sc, sm, re, used, rdesc;
+        int rslot;
+        int q;   // blocks per SM it takes
+    };
+
+    // The run's next event: releases at `re`, room for the head kernel, the new
+    // group.  The run itself stays as it is; the new group may go to the released
+    // group's slot (put_back() restores that one) or a free one.
+    __device__ __forceinline__ void look_ahead(const WarpKern &h, int kern, Ahead &a)
+    {
+        const Ahead was{fr, fs, fw, fb, sc, sm, re, used, rdesc, rslot, 0};
+        release(was.re);
+        const int q = cap(h);
+        if (q > 0) {
+            const int g = place(h, kern, q, used | (was.used & ~(1u << was.rslot)));
+            start(was.re, g, (uint32_t)kern | ((uint32_t)q << 5), duration((uint32_t)h.c, (uint32_t)h.m, sc, sm));
+        }
+        a = Ahead{fr, fs, fw, fb, sc, sm, re, used, rdesc, rslot, q};
+        set(was);
+    }
+    __device__ __forceinline__ void set(const Ahead &a)
+    {
+        fr = a.fr; fs = a.fs; fw = a.fw; fb = a.fb;
+        sc = a.sc; sm = a.sm; re = a.re; used = a.used; rdesc = a.rdesc;
+        rslot = a.rslot;
+    }
+    __device__ __forceinline__ void put_back()
+    {
+        mem.end[rslot][lane] = re;
+        mem.desc[rslot][lane] = rdesc;
+    }
+
     // Queue all blocks of kernel `kern` behind the current queue and simulate until
     // the last of them is placed (its burst stays open).  False if the state
     // cannot hold it.
+    //
+    // Between the kernel's first burst and the one that empties the queue a run's
+    // events depend on no other run, so every lane has its next event worked out,
+    // and a turn takes, of all runs side by side, the next events before the
+    // earliest event that is not worked out yet -- if the queue is longer than what
+    // they take.
     __device__ bool place_kernel(int kern, int limit, int run_limit)
     {
         const WarpKern h = mem.k[kern];
@@ -305,35 +362,62 @@ struct WarpSim {
             if (total > left) return place_last(h, kern, left, q, run_limit);
             if (!move_pointer(q)) return false;
             left -= total;
-            if (q > 0) pend |= 1u << place(h, kern, q);
+            if (q > 0) pend |= 1u << place(h, kern, q, used);
             if (left == 0) return true;
             close_burst();
         }
+        Ahead a{};
+        if (used) look_ahead(h, kern, a);
+        __syncwarp();
         for (int it = 0; it < limit; it++) {
-            const uint32_t rel = used ? re - (uint32_t)t : 0xffffffffu;
-            const uint32_t dmin = __reduce_min_sync(kAll, rel);
-            if (dmin == 0xffffffffu) return false;
-            t += dmin;
-            int q = 0;
-            uint32_t dur = 0;
-            if (rel == dmin) {
-                release();
-                q = cap(h);
-                // the duration of what it takes, should the queue not run empty
-                dur = duration((uint32_t)h.c, (uint32_t)h.m, sc + (uint32_t)(q * h.c), sm + (uint32_t)(q * h.m));
+            const uint32_t now = (uint32_t)t, none = 0xffffffffu;
+            const uint32_t e1 = used ? re - now : none, e2 = used && a.used ? a.re - now : none;
+            const uint32_t bound = __reduce_min_sync(kAll, e2);
+            bool in = e1 < bound;
+            const int take = a.q * cnt;
+            int total = (int)__reduce_add_sync(kAll, in ? (unsigned)take : 0u);
+            uint32_t adv = __reduce_max_sync(kAll, in ? e1 : 0u);
+            int to = p;
+            if (total > 0 && total < left) {
+                // the pointer: the last of these bursts decides, with the one before it
+                // where several runs end together
+                const uint32_t at = in && a.q > 0 ? e1 : 0u;
+                const uint32_t last = __reduce_max_sync(kAll, at);
+                const unsigned key = at == last ? (unsigned)a.q : 0u;
+                to = pointer_after(key, -1);
+                if (to < 0) {
+                    const uint32_t prev = at == last ? 0u : at;
+                    const uint32_t before = __reduce_max_sync(kAll, prev);
+                    const int from = before ? pointer_after(prev == before ? (unsigned)a.q : 0u, -1) : p;
+                    if (from >= 0) to = pointer_after(key, from);
+                }
             }
-            __syncwarp();
-            const int total = (int)__reduce_add_sync(kAll, (unsigned)(q * cnt));
-            if (total > left) return place_last(h, kern, left, q, run_limit);
-            if (!move_pointer(q)) return false;
+            if (total >= left || to < 0) {  // the earliest end alone
+                adv = __reduce_min_sync(kAll, e1);
+                in = e1 == adv && used != 0u;
+                total = (int)__reduce_add_sync(kAll, in ? (unsigned)take : 0u);
+                if (total >= left) {        // the queue runs empty
+                    if (used) put_back();
+                    t += adv;
+                    if (in) release((uint32_t)t);
+                    __syncwarp();
+                    const int q = in ? cap(h) : 0;
+                    if (total > left) return place_last(h, kern, left, q, run_limit);
+                    if (!move_pointer(q)) return false;
+                    if (q > 0) pend |= 1u << place(h, kern, q, used);
+                    return true;
+                }
+                to = total > 0 ? pointer_after(in ? (unsigned)a.q : 0u, p) : p;
+            }
+            if (!__any_sync(kAll, in)) return false;  // nothing runs: not reached
+            p = to;
+            t += adv;
             left -= total;
-            if (q > 0) {
-                const int g = place(h, kern, q);
-                if (left == 0) pend |= 1u << g;
-                else start(g, (uint32_t)kern | ((uint32_t)q << 5), dur);
+            if (in) {
+                set(a);
+                if (used) look_ahead(h, kern, a);
             }
             __syncwarp();
-            if (left == 0) return true;
         }
         return false;  // each event frees a block: not reached
     }

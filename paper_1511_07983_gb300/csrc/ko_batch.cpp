@@ -97,7 +97,7 @@ ko_status enqueue(ko_batch *b, cudaStream_t st)
     w.perms = b->d_rows;
     w.out = (int64_t *)b->d_refs;
     w.levels = 1;
-    b->fast.lanes = 16;
+    b->fast.lanes = 32;  // a warp per ranked order
     b->fast.stack_global = 1;
     ko_status s = ko_fast_launch(&b->fast, w, b->slab, st);
     if (s) return s;
@@ -237,15 +237,12 @@ ko_batch *ko_batch_build(const KoSet *const *sets, const int *levels, const int 
         *err = KO_ERR_CUDA;
         return nullptr;
     }
-    // allocate the simulators' buffers outside capture: one empty launch with
-    // the reference-order pass's choice (16 lanes, global slab, 1 level), then
-    // one per group, each with its choice, its deepest levels and the longest list
+    // allocate the simulators' buffers outside capture: one empty launch per
+    // group, with its choice, its deepest levels and the longest list (the
+    // reference-order pass needs no more)
     long long longest = b->n_ref_items;
     for (const ko_batch::Group &gr : b->groups) longest = std::max(longest, gr.n_items);
-    std::vector<ko_batch::Group> sizing;
-    sizing.push_back(ko_batch::Group{16, 1, 0, 0, 0, 0, 1});
-    sizing.insert(sizing.end(), b->groups.begin(), b->groups.end());
-    for (const ko_batch::Group &gr : sizing) {
+    for (const ko_batch::Group &gr : b->groups) {
         KoWork none{};
         none.sets = b->d_sets;
         none.chunks = b->d_chunks;
@@ -298,9 +295,9 @@ ko_status ko_batch_exec(ko_batch *b, ko_rank *out, uint64_t *hist, bool hist_dev
         cudaGetLastError();
         return KO_ERR_CUDA;
     }
-    // reset, the reference-order passes (three), each group's passes (three, and one or two one-thread ones)
-    int launches = b->nsets * (b->nbins > 0 ? 1 : 0) + 4;
-    for (const ko_batch::Group &g : b->groups) launches += 3 + (g.lanes != 1 ? 0 : g.shape == 0 ? 1 : 2);
+    // reset, the reference-order passes (two), each group's passes (three; with one-thread ones two or three more)
+    int launches = b->nsets * (b->nbins > 0 ? 1 : 0) + 3;
+    for (const ko_batch::Group &g : b->groups) launches += 3 + (g.lanes != 1 ? 0 : g.shape == 0 ? 2 : 3);
     ko_count_launch(launches);
     if (hist && b->nbins > 0) {
         const size_t bytes = sizeof(unsigned long long) * b->nbins * b->nsets;

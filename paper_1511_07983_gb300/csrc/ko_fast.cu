@@ -652,8 +652,11 @@ fast_kernel(KoWork a)
     __shared__ kounits::Numbering units;
     if (threadIdx.x == 0) {
         if (a.item_list) {
-            units = kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, a.space ? a.levels : 0,
-                                         (unsigned long long)gridDim.x * kSegs);
+            const unsigned long long have = *a.item_count < a.ov_cap ? *a.item_count : a.ov_cap;
+            const int lv = a.space ? a.levels : 0;
+            kounits::Numbering singles;
+            units = kounits::number_list(have, lv, (unsigned long long)gridDim.x * kSegs);
+            if (a.singles_taken && kounits::number_singles(have, lv, a.ov_cap, singles)) units.units = 0;
         } else {
             units.units = (unsigned long long)a.n_items;
         }
@@ -851,7 +854,7 @@ constexpr int kLists = 4;
 
 // Device buffer layout inside KoFastState::buf.
 struct FastBuf {
-    unsigned long long counter[kLists], ov_count[kLists], fb_counter, abandoned;
+    unsigned long long counter[kLists + 1], ov_count[kLists], fb_counter, abandoned;
     unsigned int part_seen[kPartSeen / 32];
     unsigned long long ov_list[1];   // KoFastState::ov_cap entries per list
 };
@@ -918,19 +921,22 @@ static bool packs(const KoSet &h) { return h.R < (1 << 19) && h.W <= 127; }
 // Lists of explicit orders: an order costs a whole simulation whatever the
 // list's length, so a short list is bound by one simulation's latency (a warp
 // per simulation is the quickest) and a long one by throughput (a thread per
-// simulation).  Measured, us for a warp / a thread per order:
-//   1,024 orders  N=8, 13 SMs 76 / 218   N=12, 148 SMs 202 / 554   N=20, 13 SMs 364 / 1126
-//   8,192                    144 / 229                 418 / 959               794 / 1753
-//   16,384                   234 / 229                 723 / 985              1416 / 1758
-//   50,000                   599 / 376                1883 / 1476             3862 / 2848
+// simulation, whose time is flat up to the 43,776 that run at once).  Measured,
+// us for a warp / a thread per order:
+//              N=8, 13 SMs   N=10, 15     N=9, 148     N=12, 148      N=20, 13
+//   16,384      241 / 241    460 / 434    310 / 433    455 / 1020    982 / 1760
+//   32,768      407 / 252    843 / 470    567 / 463    864 / 1083   1846 / 1968
+//   50,000      598 / 378   1253 / 763    844 / 668   1269 / 1501   2744 / 2871
+//   100,003    1149 / 579   2380 / 1134  1636 / 1020  2479 / 2073   5389 / 3976
 // The one-thread state holds 14 runs: on more than 32 SMs that is enough for
 // up to 13 kernels (under 3 % of random orders overflow in 31 of 32 sampled
 // sets; 14 kernels: 34 to 76 %); beyond, a warp per order (50,000 orders of N=20
-// on 148 SMs: 3.9 ms, 16 lanes 19.6, one thread 21.0).
+// on 148 SMs: 2.3 ms, 16 lanes 19.6, one thread 21.1).
 KoChoice ko_list_choice(const KoSet &h, long long count)
 {
     const bool holds = packs(h) && (h.S <= 32 || h.n <= 13);
-    return count > 16384 && holds ? KoChoice{1, 1, 0} : KoChoice{32, 1, 0};
+    const long long line = h.n > 10 ? 53248 : h.S > 32 ? 28672 : 16384;
+    return count > line && holds ? KoChoice{1, 1, 0} : KoChoice{32, 1, 0};
 }
 
 // Whole spaces: the work items of a space are its prefixes, each walked by one
@@ -1123,8 +1129,23 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         }
         return KO_OK;
     }
-    // all items (or those the one-thread passes abandoned), 16 or 32 lanes per simulation, 8 group slots
+    // all items, or those the one-thread passes abandoned: these first order by order, a warp each (a
+    // few are done in one simulation's time: 100,003 orders of N=12, some 250 of them handed on, 2.2 ->
+    // 1.9 ms), or where there are too many, walked as items; 16 or 32 lanes per simulation, 8 group slots
+    if (lane) {
+        KoWork w1 = w;
+        next_pass(w1);
+        if ((e = ko_launch_warp(w1, st)) != cudaSuccess) {
+            cudaGetLastError();
+            return KO_ERR_CUDA;
+        }
+        list--;  // the walking pass reads and writes the same lists; only one of the two takes the items
+    }
     next_pass(w);
+    if (lane) {
+        w.counter = &fb->counter[kLists];
+        w.singles_taken = true;
+    }
     w.gstack = fs->stack_global ? (int *)fs->gstack : nullptr;
     w.gstack_words = fs->stack_global ? (long long)(fs->gstack_bytes / sizeof(int)) : 0;
     e = fs->lanes == 32 ? launch<32, kG, 16>(w, st) : launch<16, kG, 16>(w, st);
@@ -1134,6 +1155,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     }
     // the items that pass abandoned, 32 lanes and 16 group slots per run
     KoWork w2 = w;
+    w2.singles_taken = false;
     w2.gstack = nullptr;  // the wide pass keeps its (32-lane) node states in shared memory
     w2.gstack_words = 0;
     next_pass(w2);

@@ -43,6 +43,7 @@ struct KoWork {
     const unsigned long long *item_count;
     int levels;                       // saved DFS levels per segment
     bool space;                       // the chunks are prefixes (mode 0): their items may be cut into parts
+    bool singles_taken;               // list passes: the warp pass has taken a list it could cut to single orders
     int run_limit;                    // runs one simulation may hold
     int *gstack;                      // non-null: DFS node states in this global slab, not shared memory
     long long gstack_words;           // words of gstack (bounds the segments that may use it)
@@ -120,7 +121,8 @@ size_t ko_lane_slab_bytes(int levels, int shape);
 long long ko_lane_threads(int shape);  // simulations a full launch runs at a time
 
 // One warp per simulation (ko_warp.cu) over the items of `w` (counters and list
-// set): lists, or spaces of single orders (no saved levels).
+// set): lists, spaces of single orders (no saved levels), and lists of abandoned
+// units, which it leaves alone where their single orders outnumber a list.
 cudaError_t ko_launch_warp(const KoWork &w, cudaStream_t st);
 
 // Device address of the count of items the first pass of the last launch abandoned.

@@ -88,6 +88,16 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
     return u;
 }
 
+// The numbering of a list as single orders, if there are few enough of them (and
+// no more than a list holds) that running each from the start, a warp per order,
+// beats walking the items: 65,536 orders take about 2 ms, as walking one item does.
+__host__ __device__ inline bool number_singles(unsigned long long items, int levels, unsigned long long cap,
+                                               Numbering &u)
+{
+    u = number_list(items, levels, cap < 65536ull ? cap : 65536ull);
+    return levels + 1 - u.x2 <= 1;
+}
+
 // The item (or list entry) of unit `unit`, the part's number and its cut.
 __host__ __device__ inline Unit unit_at(const Numbering &u, unsigned long long unit)
 {

@@ -443,17 +443,43 @@ __global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
     const int run_limit = a.run_limit < 32 ? a.run_limit : 32;
     int loaded = -1, n = 0, limit = 0;
     const KoSet *set = nullptr;
+    kounits::Numbering units{};
+    if (a.item_list) {
+        const unsigned long long have = *a.item_count < a.ov_cap ? *a.item_count : a.ov_cap;
+        if (!kounits::number_singles(have, a.space ? a.levels : 0, a.ov_cap, units)) return;  // the next pass walks them
+    } else {
+        units.units = (unsigned long long)a.n_items;
+    }
     for (;;) {
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(a.counter, 1ull);
         item = __shfl_sync(kAll, item, 0);
-        if (item >= (unsigned long long)a.n_items) break;
+        if (item >= units.units) break;
+        unsigned part = 0, list_part = 0;
+        int cut = 0, list_cut = 0;
+        if (a.item_list) {
+            const kounits::Unit un = kounits::unit_at(units, item);
+            const unsigned long long entry = a.item_list[un.item];
+            item = entry & kounits::kItemMask;
+            list_part = (unsigned)((entry >> kounits::kItemBits) & kounits::kPartMask);
+            list_cut = (int)(entry >> (kounits::kItemBits + kounits::kPartBits));
+            part = un.part;
+            cut = un.x;
+            if (item >= (unsigned long long)a.n_items) continue;
+        }
         int lo = 0, hi = a.nchunks - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
             if (a.chunks[mid].first <= (long long)item) lo = mid; else hi = mid - 1;
         }
         const KoChunk ch = a.chunks[lo];
+        if (a.item_list) {
+            const kounits::Unit un =
+                kounits::cut_unit(item, list_part, list_cut, ch.mode == 0 ? a.sets[ch.set].n - ch.d0 : 0, cut, part);
+            if (!un.valid) continue;
+            part = un.part;
+            cut = un.x;
+        }
         if (ch.set != loaded) {
             loaded = ch.set;
             set = a.sets + ch.set;
@@ -494,7 +520,8 @@ __global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
                 k = a.idx[ch.list_off + local];
                 valid = k < c_warp_fact[n];
             } else {
-                k = (unsigned long long)(ch.list_off + local) * c_warp_fact[n - ch.d0];
+                k = (unsigned long long)(ch.list_off + local) * c_warp_fact[n - ch.d0] +
+                    part * c_warp_fact[n - ch.d0 - cut];
                 outpos = ch.out_off + (long long)k;
             }
             unsigned rest = (1u << n) - 1u;
@@ -519,8 +546,8 @@ __global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
         if (!ok) {
             if (lane == 0) {
                 const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                if (slot < a.ov_cap) a.ov_list[slot] = kounits::entry_of(item, 0u, 0);
-                atomicAdd(a.abandoned, 1ull);
+                if (slot < a.ov_cap) a.ov_list[slot] = kounits::entry_of(item, part, cut);
+                if (!a.item_list) atomicAdd(a.abandoned, 1ull);
             }
             continue;
         }
@@ -546,9 +573,10 @@ cudaError_t ko_launch_warp(const KoWork &a, cudaStream_t st)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // as few warps per block as give every warp one order, up to one per sub-partition
-    const long long per_sm = (a.n_items + sms - 1) / sms;
+    const long long work = a.item_list ? (long long)sms * kWarps : a.n_items;
+    const long long per_sm = (work + sms - 1) / sms;
     const int warps = per_sm < 1 ? 1 : per_sm < kWarps ? (int)per_sm : kWarps;
-    long long blocks = (a.n_items + warps - 1) / warps;
+    long long blocks = (work + warps - 1) / warps;
     const long long resident = (long long)sms * 8;
     if (blocks > resident) blocks = resident;
     if (blocks < 1) blocks = 1;

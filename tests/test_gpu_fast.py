@@ -255,8 +255,8 @@ def test_default_space_equals_every_pinned_choice(ko, n, gpu):
         assert ko.ko_get_option(g.h, ko.KO_OPT_LEVELS) == 4
 
 
-@pytest.mark.parametrize("workload,n", [("single8", 8), ("single12", 13), ("single12", 14), ("large", 24)])
-@pytest.mark.parametrize("count", [16384, 16385])
+@pytest.mark.parametrize("workload,n", [("single8", 8), ("single12", 9), ("single12", 13), ("single12", 14)])
+@pytest.mark.parametrize("count", [16384, 16385, 28673, 53249])
 def test_default_list_equals_a_pinned_choice(ko, workload, n, count):
     s = synth.gen_set(workload, 5, n=n)
     rows = synth.random_orders(count, n, count).astype(np.int8)

@@ -1193,6 +1193,9 @@ void ko_fast_release(KoFastState *fs)
     cudaFree(fs->lslab);
     fs->lslab = nullptr;
     fs->lslab_bytes = 0;
+    cudaFree(fs->arena);
+    fs->arena = nullptr;
+    fs->arena_bytes = 0;
     fs->buf = nullptr;
     fs->fb_scratch = nullptr;
     fs->cap = 0;

@@ -70,6 +70,8 @@ struct KoFastState {
     size_t gstack_bytes = 0;
     void *lslab = nullptr;      // node-state slab of the one-thread-per-order pass
     size_t lslab_bytes = 0;
+    void *arena = nullptr;      // search workspace, kept between calls (as large as the largest call's)
+    size_t arena_bytes = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around the last run-length launch
     double last_ms = -1.0;
     long long h2d = 0, d2h = 0;

@@ -656,22 +656,96 @@ __global__ void select_hist_kernel(const float *__restrict__ y, long long n, con
         if (h[i]) atomicAdd(&hist[i], h[i]);
 }
 
-// Fix the digit: state = {prefix, remaining k}; clears the histogram.
+// The digit whose bin holds the `need`-th smallest of a 256-bin histogram and how
+// many lie below it; one warp, eight bins a lane.
+__device__ __forceinline__ void select_digit(const unsigned int *hist, uint32_t need, int &digit, uint32_t &below)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) mine += hist[lane * 8 + i];
+    uint32_t upto = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += v;
+    }
+    const unsigned has = __ballot_sync(0xffffffffu, upto >= need);
+    const int owner = has ? __ffs((int)has) - 1 : 31;
+    int d = lane * 8 + 7;
+    uint32_t cum = upto - mine;
+    for (int i = 0; i < 8; i++) {
+        if (cum + hist[lane * 8 + i] >= need) { d = lane * 8 + i; break; }
+        if (i < 7) cum += hist[lane * 8 + i];
+    }
+    digit = __shfl_sync(0xffffffffu, d, owner);
+    below = __shfl_sync(0xffffffffu, cum, owner);
+}
+
+__global__ void select_init_kernel(uint32_t *state, uint32_t k, unsigned int *hist, unsigned int *counters)
+{
+    if (threadIdx.x == 0) { state[0] = 0u; state[1] = k; }
+    if (threadIdx.x < 2) counters[threadIdx.x] = 0u;
+    hist[threadIdx.x] = 0u;
+}
+
+// Fix the digit: state = {prefix, remaining k}; clears the histogram.  (One
+// thread over 256 bins in memory took 8.7 us of a 13 us digit.)
 __global__ void select_scan_kernel(uint32_t *state, int shift, unsigned int *hist)
 {
-    if (threadIdx.x == 0) {
-        uint32_t need = state[1];
-        uint32_t cum = 0;
-        int digit = 255;
-        for (int d = 0; d < 256; d++) {
-            if (cum + hist[d] >= need) { digit = d; break; }
-            cum += hist[d];
+    if (threadIdx.x < 32) {
+        int digit;
+        uint32_t below;
+        const uint32_t need = state[1];
+        select_digit(hist, need, digit, below);
+        if (threadIdx.x == 0) {
+            state[0] |= (uint32_t)digit << shift;
+            state[1] = need - below;
         }
-        state[0] |= (uint32_t)digit << shift;
-        state[1] = need - cum;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+    hist[threadIdx.x] = 0;
+}
+
+// Up to kSmallTopk keys: the four digits and the output in one block, the keys in
+// shared memory (the neighbourhoods of a search round; nine launches, two clears
+// and a copy before: 70 of a round's 340 us).
+constexpr int kSmallTopk = 8192;
+__global__ void __launch_bounds__(1024) select_small_kernel(const float *__restrict__ y, int n, int k, int *out)
+{
+    __shared__ uint32_t keys[kSmallTopk];
+    __shared__ unsigned int hist[256];
+    __shared__ uint32_t s_prefix, s_need;
+    __shared__ unsigned int s_out, s_eq;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = float_key(y[i]);
+    if (threadIdx.x == 0) { s_prefix = 0u; s_need = (uint32_t)k; s_out = s_eq = 0u; }
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        if (threadIdx.x < 256) hist[threadIdx.x] = 0u;
+        __syncthreads();
+        const uint32_t prefix = s_prefix, mask = shift == 24 ? 0u : (0xFFFFFFFFu << (shift + 8));
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            if ((keys[i] & mask) == prefix) atomicAdd(&hist[(keys[i] >> shift) & 255u], 1u);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            int digit;
+            uint32_t below;
+            select_digit(hist, s_need, digit, below);
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                s_prefix = prefix | ((uint32_t)digit << shift);
+                s_need -= below;
+            }
+        }
+        __syncthreads();
+    }
+    const uint32_t thr = s_prefix, quota = s_need;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t key = keys[i];
+        if (key < thr || (key == thr && atomicAdd(&s_eq, 1u) < quota)) {
+            const unsigned int at = atomicAdd(&s_out, 1u);
+            if (at < (unsigned)k) out[at] = i;
+        }
+    }
 }
 
 // Write the indices of the k smallest keys: all keys below the threshold and
@@ -728,17 +802,13 @@ __global__ void targets_kernel(const int64_t *ms, const int *sid, const double *
     }
 }
 
-// All single-step neighbours of `beam` base orders (rows of stride 24): first
-// the n(n-1)/2 swaps of two positions, then the n(n-1) moves of one kernel to
-// another position (the rest shift by one).  Row r = b * per + q.
-__global__ void neighbours_kernel(const int8_t *__restrict__ base, int beam, int n, int8_t *out)
+// Neighbour q of an n-kernel order: first the n(n-1)/2 swaps of two positions,
+// then the n(n-1) moves of one kernel to another position (the rest shift by one).
+__device__ __forceinline__ void write_neighbour(const int8_t *base, int n, int q, int8_t *o)
 {
-    const int swaps = n * (n - 1) / 2, per = swaps + n * (n - 1);
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= beam * per) return;
-    const int b = r / per, q = r % per;
+    const int swaps = n * (n - 1) / 2;
     int8_t p[kMaxK];
-    for (int i = 0; i < n; i++) p[i] = base[b * kMaxK + i];
+    for (int i = 0; i < n; i++) p[i] = base[i];
     if (q < swaps) {
         int i = 0, rem = q;
         while (rem >= n - 1 - i) { rem -= n - 1 - i; i++; }
@@ -752,8 +822,71 @@ __global__ void neighbours_kernel(const int8_t *__restrict__ base, int beam, int
         else { for (int i = from; i > to; i--) p[i] = p[i - 1]; }
         p[to] = v;
     }
-    int8_t *o = out + (size_t)r * kMaxK;
     for (int i = 0; i < kMaxK; i++) o[i] = i < n ? p[i] : (int8_t)0;
+}
+
+// All single-step neighbours of `beam` base orders (rows of stride 24).  Row r = b * per + q.
+__global__ void neighbours_kernel(const int8_t *__restrict__ base, int beam, int n, int8_t *out)
+{
+    const int per = n * (n - 1) / 2 + n * (n - 1);
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= beam * per) return;
+    write_neighbour(base + r / per * kMaxK, n, r % per, out + (size_t)r * kMaxK);
+}
+
+// A descent's step between two evaluations.  One block: the step is a few
+// microseconds between simulations of hundreds, but the host's part of it (two
+// copies back, the choice, two copies and three launches) was 70 of 340.
+constexpr int kDescendThreads = 512;
+__global__ void __launch_bounds__(kDescendThreads) descend_kernel(KoDescent *s, const int64_t *__restrict__ ms, int nq,
+                                                                  int n, int8_t *rows)
+{
+    __shared__ unsigned long long s_best[kDescendThreads / 32];
+    __shared__ int s_idx[kDescendThreads / 32];
+    __shared__ int8_t s_order[kMaxK];
+    __shared__ int s_done;
+    if (s->done) return;
+    // the lowest makespan, the lowest index among equal ones; a failed one (< 0) orders below all
+    unsigned long long best = ~0ull;
+    int at = 0x7fffffff;
+    for (int q = threadIdx.x; q < nq; q += kDescendThreads) {
+        const unsigned long long v = (unsigned long long)ms[q] ^ (1ull << 63);  // signed order
+        if (v < best) { best = v; at = q; }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long b2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int a2 = __shfl_xor_sync(0xffffffffu, at, o);
+        if (b2 < best || (b2 == best && a2 < at)) { best = b2; at = a2; }
+    }
+    if ((threadIdx.x & 31) == 0) { s_best[threadIdx.x >> 5] = best; s_idx[threadIdx.x >> 5] = at; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kDescendThreads / 32; w++)
+            if (s_best[w] < best || (s_best[w] == best && s_idx[w] < at)) { best = s_best[w]; at = s_idx[w]; }
+        const int64_t found = (int64_t)(best ^ (1ull << 63));
+        if (s->makespan < 0) {
+            s->makespan = ms[nq];
+            s->evals = 1;
+        }
+        s->evals += nq;
+        const bool bad = found < 0 || s->makespan < 0;
+        const bool better = !bad && found < s->makespan;
+        if (better) {
+            s->makespan = found;
+            s->steps++;
+            for (int i = 0; i < kMaxK; i++) s->order[i] = rows[(size_t)at * kMaxK + i];
+        }
+        if (bad) s->failed = 1;
+        s_done = !better || s->steps >= s->max_steps;
+        s->done = s_done;
+        for (int i = 0; i < kMaxK; i++) s_order[i] = s->order[i];
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q <= nq; q += kDescendThreads) {
+        if (s_done || q == nq) rows[(size_t)q * kMaxK] = -1;  // row nq: the first order, known now
+        else write_neighbour(s_order, n, q, rows + (size_t)q * kMaxK);
+    }
 }
 
 __global__ void gather_rows_kernel(const int8_t *src, int stride, const int *pick, int B, int8_t *dst)
@@ -863,12 +996,13 @@ cudaError_t ko_mlp_weights_bf16(const float *w, int K, int N, uint16_t *wk, uint
 cudaError_t ko_mlp_topk(const float *y, long long n, int k, uint32_t *state, unsigned int *hist,
                         unsigned int *counters, int *out, cudaStream_t st)
 {
-    // state = {prefix 0, remaining k}; hist and counters zeroed here
-    uint32_t init[2] = {0u, (uint32_t)k};
-    if (cudaMemcpyAsync(state, init, sizeof(init), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned int), st) != cudaSuccess ||
-        cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned int), st) != cudaSuccess)
+    if (n <= kSmallTopk) {
+        select_small_kernel<<<1, 1024, 0, st>>>(y, (int)n, k, out);
+        ko_count_launch();
         return cudaGetLastError();
+    }
+    select_init_kernel<<<1, 256, 0, st>>>(state, (uint32_t)k, hist, counters);
+    ko_count_launch();
     const int blocks = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
     for (int shift = 24; shift >= 0; shift -= 8) {
         select_hist_kernel<<<blocks, 256, 0, st>>>(y, n, state, shift, hist);
@@ -908,6 +1042,13 @@ cudaError_t ko_mlp_neighbours(const int8_t *base, int beam, int n, int8_t *out, 
     const int rows = beam * per;
     if (rows <= 0) return cudaSuccess;
     neighbours_kernel<<<(rows + 127) / 128, 128, 0, st>>>(base, beam, n, out);
+    ko_count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t ko_mlp_descend(KoDescent *s, const int64_t *ms, int nq, int n, int8_t *rows, cudaStream_t st)
+{
+    descend_kernel<<<1, kDescendThreads, 0, st>>>(s, ms, nq, n, rows);
     ko_count_launch();
     return cudaGetLastError();
 }

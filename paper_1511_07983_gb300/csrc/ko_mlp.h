@@ -109,5 +109,19 @@ cudaError_t ko_mlp_random_orders(int8_t *rows, int stride, long long count, int 
 cudaError_t ko_mlp_targets(const int64_t *ms, const int *sid, const double *log2_lb, long long n, float *t,
                            cudaStream_t st);
 cudaError_t ko_mlp_neighbours(const int8_t *base, int beam, int n, int8_t *out, cudaStream_t st);
+// One step of a steepest descent on the device: `ms` holds the makespans of the
+// `nq` neighbours of s->order in `rows` (those ko_mlp_neighbours would write,
+// stride 24) and, in its first step, of the order itself behind them.  Moves to
+// the best strictly better neighbour (the lowest index among equal ones) and
+// writes its neighbours, or ends the descent; rows of an ended one are no orders
+// (-1), which an evaluation passes over.
+struct KoDescent {
+    int64_t makespan;     // of `order`; < 0 before the first step
+    int64_t evals;
+    int32_t steps, max_steps;
+    int32_t done, failed;
+    int8_t order[kMaxK];
+};
+cudaError_t ko_mlp_descend(KoDescent *s, const int64_t *ms, int nq, int n, int8_t *rows, cudaStream_t st);
 cudaError_t ko_mlp_gather_rows(const int8_t *src, int stride, const int *pick, int B, int8_t *dst,
                                cudaStream_t st);

@@ -428,49 +428,102 @@ ko_status ko_model_raw(ko_model *md, const float *x, const float *t, int B, floa
 
 // ------------------------------------------------------------ set plumbing
 
+// Parts of one block of memory, 256-byte aligned; without a base it only counts.
+struct Carve {
+    char *base;
+    size_t size = 0;
+    explicit Carve(void *b) : base((char *)b) {}
+    template <typename T>
+    T *take(size_t n)
+    {
+        const size_t at = size;
+        size += (sizeof(T) * (n ? n : 1) + 255) / 256 * 256;
+        return base ? (T *)(base + at) : nullptr;
+    }
+};
+
+// The state's search workspace, at least `bytes` long (nothing of an earlier call
+// is in it or in flight on it, see ArenaUse).
+static ko_status ensure_arena(KoFastState *fs, size_t bytes)
+{
+    if (fs->arena_bytes >= bytes) return KO_OK;
+    cudaFree(fs->arena);
+    fs->arena = nullptr;
+    fs->arena_bytes = 0;
+    char *p = nullptr;
+    if (!dalloc(&p, bytes)) return KO_ERR_NOMEM;
+    fs->arena = p;
+    fs->arena_bytes = bytes;
+    return KO_OK;
+}
+
+// End of a call that used the arena: nothing is in flight on it, and no more than
+// kArenaKept stays allocated (4M candidates take 120 MB).
+constexpr size_t kArenaKept = size_t(256) << 20;
+struct ArenaUse {
+    KoFastState *fs;
+    cudaStream_t st;
+    ~ArenaUse()
+    {
+        cudaStreamSynchronize(st);
+        if (fs->arena_bytes <= kArenaKept) return;
+        cudaFree(fs->arena);
+        fs->arena = nullptr;
+        fs->arena_bytes = 0;
+    }
+};
+
+// Device copies of the sets and what the encoder reads of them, in one block.
 struct SetTables {
+    void *mem = nullptr;
     int *set_n = nullptr;
     float *kfeat = nullptr, *gfeat = nullptr;
     double *log2_lb = nullptr;
     KoSet *sets = nullptr;
-    ~SetTables()
+    void carve(Carve &c, int nsets)
     {
-        cudaFree(set_n); cudaFree(kfeat); cudaFree(gfeat); cudaFree(log2_lb); cudaFree(sets);
+        set_n = c.take<int>(nsets);
+        kfeat = c.take<float>((size_t)nsets * kMaxK * kSlotFeat);
+        gfeat = c.take<float>((size_t)nsets * kGlobals);
+        log2_lb = c.take<double>(nsets);
+        sets = c.take<KoSet>(nsets);
     }
+    ~SetTables() { cudaFree(mem); }
 };
 
 static ko_status build_tables(const KoSet *const *hs, int nsets, SetTables *tb, cudaStream_t st)
 {
-    std::vector<int> n(nsets);
-    std::vector<float> kf((size_t)nsets * kMaxK * kSlotFeat), gf((size_t)nsets * kGlobals);
-    std::vector<double> l2(nsets);
-    std::vector<KoSet> sets(nsets);
+    Carve count(nullptr);
+    tb->carve(count, nsets);
+    std::vector<char> host(count.size, 0);
+    SetTables ht;
+    Carve on_host(host.data());
+    ht.carve(on_host, nsets);
     for (int i = 0; i < nsets; i++) {
         int64_t lb = 0, ub = 0;
         ko_bounds_host(*hs[i], &lb, &ub);
-        n[i] = hs[i]->n;
-        ko_set_features(*hs[i], lb, kf.data() + (size_t)i * kMaxK * kSlotFeat, gf.data() + (size_t)i * kGlobals);
-        l2[i] = std::log2((double)(lb > 1 ? lb : 1));
-        sets[i] = *hs[i];
-        sets[i].ref_makespan = 0;
+        ht.set_n[i] = hs[i]->n;
+        ko_set_features(*hs[i], lb, ht.kfeat + (size_t)i * kMaxK * kSlotFeat, ht.gfeat + (size_t)i * kGlobals);
+        ht.log2_lb[i] = std::log2((double)(lb > 1 ? lb : 1));
+        ht.sets[i] = *hs[i];
+        ht.sets[i].ref_makespan = 0;
     }
-    if (!dalloc(&tb->set_n, nsets) || !dalloc(&tb->kfeat, kf.size()) || !dalloc(&tb->gfeat, gf.size()) ||
-        !dalloc(&tb->log2_lb, nsets) || !dalloc(&tb->sets, nsets))
-        return KO_ERR_NOMEM;
-    if (cudaMemcpyAsync(tb->set_n, n.data(), sizeof(int) * nsets, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(tb->kfeat, kf.data(), sizeof(float) * kf.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(tb->gfeat, gf.data(), sizeof(float) * gf.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(tb->log2_lb, l2.data(), sizeof(double) * nsets, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(tb->sets, sets.data(), sizeof(KoSet) * nsets, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+    char *mem = nullptr;
+    if (!dalloc(&mem, count.size)) return KO_ERR_NOMEM;
+    tb->mem = mem;
+    Carve on_device(mem);
+    tb->carve(on_device, nsets);
+    if (cudaMemcpyAsync(mem, host.data(), host.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return KO_ERR_CUDA;
     return KO_OK;
 }
 
 // Exact makespans of `count` rows (stride 24) of set `set` into out, with the
-// choice for that many orders (the state's own options are kept).
+// choice for that many orders (the state's own options are kept).  `upload`:
+// d_chunk does not describe these rows yet.
 static ko_status exact_rows(KoFastState *fs, const KoSet *d_sets, const KoSet &h, int set, const int8_t *rows,
-                            long long count, int64_t *out, KoChunk *d_chunk, cudaStream_t st)
+                            long long count, int64_t *out, KoChunk *d_chunk, cudaStream_t st, bool upload = true)
 {
     KoRoute route(fs, ko_list_choice(h, count), st, true);
     KoChunk c{};
@@ -478,7 +531,8 @@ static ko_status exact_rows(KoFastState *fs, const KoSet *d_sets, const KoSet &h
     c.set = set;
     c.d0 = h.n;
     c.mode = 2;
-    if (cudaMemcpyAsync(d_chunk, &c, sizeof(c), cudaMemcpyHostToDevice, st) != cudaSuccess) return KO_ERR_CUDA;
+    if (upload && cudaMemcpyAsync(d_chunk, &c, sizeof(c), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        return KO_ERR_CUDA;
     KoWork w{};
     w.sets = d_sets;
     w.chunks = d_chunk;
@@ -615,6 +669,14 @@ static ko_status best_of(const int64_t *d_ms, long long count, int64_t *best, lo
     return KO_OK;
 }
 
+// Rows of one forward pass over `rows` candidates: the model's chunk, or all of
+// them in whole 128-row tiles where they are fewer.
+static int chunk_rows(const ko_model *md, long long rows)
+{
+    const long long all = (rows + 127) / 128 * 128;
+    return all < md->chunk ? (int)all : md->chunk;
+}
+
 ko_status ko_model_propose_set(ko_model *md, const KoSet &h, long long n_cand, int top_k, uint64_t seed,
                                int32_t *best_order, int64_t *best_makespan, double *gpu_ms, cudaStream_t st)
 {
@@ -624,20 +686,32 @@ ko_status ko_model_propose_set(ko_model *md, const KoSet &h, long long n_cand, i
     SetTables tb;
     ko_status s = build_tables(hs, 1, &tb, st);
     if (s) return s;
-    const int C = md->chunk;
+    const int C = chunk_rows(md, n_cand);
     const long long padded = (n_cand + C - 1) / C * C;
-    int8_t *rows = nullptr, *top_rows = nullptr;
-    float *y_all = nullptr;
-    int *top_idx = nullptr;
-    int64_t *top_ms = nullptr;
-    uint32_t *sel_state = nullptr;
-    unsigned int *sel_hist = nullptr, *sel_cnt = nullptr;
-    KoChunk *d_chunk = nullptr;
-    if (!dalloc(&rows, (size_t)padded * kMaxK) || !dalloc(&y_all, (size_t)n_cand) || !dalloc(&top_idx, top_k) ||
-        !dalloc(&top_rows, (size_t)top_k * kMaxK) || !dalloc(&top_ms, top_k) || !dalloc(&sel_state, 2) ||
-        !dalloc(&sel_hist, 256) || !dalloc(&sel_cnt, 2) || !dalloc(&d_chunk, 1)) {
-        s = KO_ERR_NOMEM;
-    }
+    int8_t *rows, *top_rows;
+    float *y_all;
+    int *top_idx;
+    int64_t *top_ms;
+    uint32_t *sel_state;
+    unsigned int *sel_hist, *sel_cnt;
+    KoChunk *d_chunk;
+    auto carve = [&](Carve &c) {
+        rows = c.take<int8_t>((size_t)padded * kMaxK);
+        y_all = c.take<float>((size_t)n_cand);
+        top_idx = c.take<int>(top_k);
+        top_rows = c.take<int8_t>((size_t)top_k * kMaxK);
+        top_ms = c.take<int64_t>(top_k);
+        sel_state = c.take<uint32_t>(2);
+        sel_hist = c.take<unsigned int>(256);
+        sel_cnt = c.take<unsigned int>(2);
+        d_chunk = c.take<KoChunk>(1);
+    };
+    Carve need(nullptr);
+    carve(need);
+    ArenaUse use{&md->fast, st};
+    s = ensure_arena(&md->fast, need.size);
+    Carve mem(md->fast.arena);
+    if (!s) carve(mem);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!s) s = make_events(&e0, &e1);
     if (!s) s = ensure_forward(md, C);
@@ -675,8 +749,6 @@ ko_status ko_model_propose_set(ko_model *md, const KoSet &h, long long n_cand, i
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    cudaFree(rows); cudaFree(top_rows); cudaFree(y_all); cudaFree(top_idx); cudaFree(top_ms);
-    cudaFree(sel_state); cudaFree(sel_hist); cudaFree(sel_cnt); cudaFree(d_chunk);
     return s;
 }
 
@@ -699,24 +771,39 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
     SetTables tb;
     ko_status s = build_tables(hs, 1, &tb, st);
     if (s) return s;
-    const int C = md->chunk;
     const int k2 = 256;
-    const long long padded = (n_cand + C - 1) / C * C;
     const int per = n * (n - 1) / 2 + n * (n - 1);
     const int nb_rows = beam * per, nb_pad = (nb_rows + 127) / 128 * 128;
+    // rows per forward pass: no more than there are (the screening's or a round's)
+    const int C = chunk_rows(md, std::max<long long>(n_cand, nb_pad));
+    const long long padded = (n_cand + C - 1) / C * C;
     const int kmax = top_k > k2 ? top_k : k2;
-    int8_t *rows = nullptr, *top_rows = nullptr, *nb = nullptr, *base = nullptr;
-    float *y_all = nullptr;
-    int *top_idx = nullptr;
-    int64_t *top_ms = nullptr;
-    uint32_t *sel_state = nullptr;
-    unsigned int *sel_hist = nullptr, *sel_cnt = nullptr;
-    KoChunk *d_chunk = nullptr;
-    if (!dalloc(&rows, (size_t)padded * kMaxK) || !dalloc(&y_all, (size_t)std::max<long long>(n_cand, nb_pad)) ||
-        !dalloc(&top_idx, kmax) || !dalloc(&top_rows, (size_t)kmax * kMaxK) || !dalloc(&top_ms, kmax) ||
-        !dalloc(&nb, (size_t)nb_pad * kMaxK) || !dalloc(&base, (size_t)beam * kMaxK) || !dalloc(&sel_state, 2) ||
-        !dalloc(&sel_hist, 256) || !dalloc(&sel_cnt, 2) || !dalloc(&d_chunk, 1))
-        s = KO_ERR_NOMEM;
+    int8_t *rows, *top_rows, *nb, *base;
+    float *y_all;
+    int *top_idx;
+    int64_t *top_ms;
+    uint32_t *sel_state;
+    unsigned int *sel_hist, *sel_cnt;
+    KoChunk *d_chunk;
+    auto carve = [&](Carve &c) {
+        rows = c.take<int8_t>((size_t)padded * kMaxK);
+        y_all = c.take<float>((size_t)std::max<long long>(n_cand, nb_pad));
+        top_idx = c.take<int>(kmax);
+        top_rows = c.take<int8_t>((size_t)kmax * kMaxK);
+        top_ms = c.take<int64_t>(kmax);
+        nb = c.take<int8_t>((size_t)nb_pad * kMaxK);
+        base = c.take<int8_t>((size_t)beam * kMaxK);
+        sel_state = c.take<uint32_t>(2);
+        sel_hist = c.take<unsigned int>(256);
+        sel_cnt = c.take<unsigned int>(2);
+        d_chunk = c.take<KoChunk>(1);
+    };
+    Carve need(nullptr);
+    carve(need);
+    ArenaUse use{&md->fast, st};
+    s = ensure_arena(&md->fast, need.size);
+    Carve mem(md->fast.arena);
+    if (!s) carve(mem);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     struct Cand {
         int64_t ms;
@@ -818,8 +905,6 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
-    cudaFree(rows); cudaFree(top_rows); cudaFree(nb); cudaFree(base); cudaFree(y_all); cudaFree(top_idx);
-    cudaFree(top_ms); cudaFree(sel_state); cudaFree(sel_hist); cudaFree(sel_cnt); cudaFree(d_chunk);
     return s;
 }
 
@@ -865,25 +950,30 @@ ko_status ko_random_search_set(KoFastState *fs, const KoSet &h, long long n_orde
 }
 
 // Steepest-descent hill climbing with exact scoring.  Neighbours of the
-// current order come from the neighbours kernel (swaps of two positions, then
-// moves of one kernel to another position); every one is simulated exactly,
-// the lowest makespan wins (lowest neighbour index among equals) and the walk
-// moves only on a strict improvement.  One step = one H2D of the current order,
-// two launches and one D2H of the neighbours' makespans.
+// current order are swaps of two positions, then moves of one kernel to another
+// position; every one is simulated exactly, the lowest makespan wins (lowest
+// neighbour index among equals) and the walk moves only on a strict improvement.
+// The walk is on the device (ko_mlp_descend): an evaluation and the choice of the
+// next order follow each other without the host, which looks every kAhead steps
+// whether the descent has ended (the rows of an ended one are passed over).
+// The start is evaluated with its neighbours.
 ko_status ko_local_search_set(KoFastState *fs, const KoSet &h, const int32_t *start, bool moves, int max_iters,
                               int32_t *order_out, int64_t *makespan_out, int32_t *steps_out, int64_t *evals_out,
                               double *gpu_ms, cudaStream_t st)
 {
+    constexpr int kAhead = 3;
     const int n = h.n;
     if (n < 1 || max_iters < 0 || max_iters > (1 << 20)) return KO_ERR_ARG;
     if (!ko_fast_applicable(h)) return KO_ERR_OVERFLOW;
-    std::vector<int8_t> cur(kMaxK, 0);
+    KoDescent d{};
+    d.makespan = -1;
+    d.max_steps = max_iters;
     {
         std::vector<char> seen(n, 0);
         for (int i = 0; i < n; i++) {
             if (start[i] < 0 || start[i] >= n || seen[start[i]]) return KO_ERR_ARG;
             seen[start[i]] = 1;
-            cur[i] = (int8_t)start[i];
+            d.order[i] = (int8_t)start[i];
         }
     }
     const KoSet *hs[1] = {&h};
@@ -891,59 +981,55 @@ ko_status ko_local_search_set(KoFastState *fs, const KoSet &h, const int32_t *st
     ko_status s = build_tables(hs, 1, &tb, st);
     if (s) return s;
     const int swaps = n * (n - 1) / 2, per = swaps + n * (n - 1);
-    const int nq = moves ? per : swaps;
-    int8_t *base = nullptr, *nb = nullptr;
-    int64_t *ms = nullptr;
-    KoChunk *d_chunk = nullptr;
-    if (!dalloc(&base, kMaxK) || !dalloc(&nb, (size_t)(per > 0 ? per : 1) * kMaxK) ||
-        !dalloc(&ms, (size_t)(per > 0 ? per : 1) + 1) || !dalloc(&d_chunk, 1))
-        s = KO_ERR_NOMEM;
+    const int nq = max_iters > 0 ? (moves ? per : swaps) : 0;
+    Carve need(nullptr);
+    auto carve = [&](Carve &c, KoDescent **state, int8_t **rows, int64_t **ms, KoChunk **chunk) {
+        *state = c.take<KoDescent>(1);
+        *rows = c.take<int8_t>((size_t)(per + 1) * kMaxK);  // the neighbours kernel writes all of them
+        *ms = c.take<int64_t>((size_t)nq + 1);
+        *chunk = c.take<KoChunk>(1);
+    };
+    KoDescent *state;
+    int8_t *rows;
+    int64_t *ms;
+    KoChunk *d_chunk;
+    carve(need, &state, &rows, &ms, &d_chunk);
+    ArenaUse use{fs, st};
+    if ((s = ensure_arena(fs, need.size))) return s;
+    Carve mem(fs->arena);
+    carve(mem, &state, &rows, &ms, &d_chunk);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    int64_t cur_ms = -1, evals = 0;
-    int steps = 0;
-    std::vector<int64_t> hm((size_t)(nq > 0 ? nq : 1));
-    if (!s) s = make_events(&e0, &e1);
-    if (!s) {
-        cudaEventRecord(e0, st);
-        if (cudaMemcpyAsync(base, cur.data(), kMaxK, cudaMemcpyHostToDevice, st) != cudaSuccess) s = KO_ERR_CUDA;
-        if (!s) s = exact_rows(fs, tb.sets, h, 0, base, 1, ms + per, d_chunk, st);
-        if (!s && (cudaMemcpyAsync(&cur_ms, ms + per, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if ((s = make_events(&e0, &e1))) return s;
+    cudaEventRecord(e0, st);
+    if (cudaMemcpyAsync(state, &d, sizeof(d), cudaMemcpyHostToDevice, st) != cudaSuccess) s = KO_ERR_CUDA;
+    if (!s && nq > 0) s = cuda_ok(ko_mlp_neighbours(state->order, 1, n, rows, st));
+    if (!s && cudaMemcpyAsync(rows + (size_t)nq * kMaxK, state->order, kMaxK, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        s = KO_ERR_CUDA;
+    bool first = true;
+    while (!s && !d.done) {
+        for (int i = 0; i < kAhead && !s; i++) {
+            s = exact_rows(fs, tb.sets, h, 0, rows, nq + 1, ms, d_chunk, st, first);
+            first = false;
+            if (!s) s = cuda_ok(ko_mlp_descend(state, ms, nq, n, rows, st));
+        }
+        if (!s && (cudaMemcpyAsync(&d, state, sizeof(d), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                    cudaStreamSynchronize(st) != cudaSuccess))
             s = KO_ERR_CUDA;
-        if (!s && cur_ms < 0) s = KO_ERR_STATE;
-        evals = 1;
-        while (!s && steps < max_iters && nq > 0) {
-            if (cudaMemcpyAsync(base, cur.data(), kMaxK, cudaMemcpyHostToDevice, st) != cudaSuccess) { s = KO_ERR_CUDA; break; }
-            if ((s = cuda_ok(ko_mlp_neighbours(base, 1, n, nb, st)))) break;
-            if ((s = exact_rows(fs, tb.sets, h, 0, nb, nq, ms, d_chunk, st))) break;
-            if (cudaMemcpyAsync(hm.data(), ms, sizeof(int64_t) * nq, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaStreamSynchronize(st) != cudaSuccess) { s = KO_ERR_CUDA; break; }
-            evals += nq;
-            int bq = -1;
-            for (int q = 0; q < nq; q++) {
-                if (hm[q] < 0) { s = KO_ERR_STATE; break; }
-                if (bq < 0 || hm[q] < hm[bq]) bq = q;
-            }
-            if (s || hm[bq] >= cur_ms) break;
-            if (cudaMemcpy(cur.data(), nb + (size_t)bq * kMaxK, kMaxK, cudaMemcpyDeviceToHost) != cudaSuccess) { s = KO_ERR_CUDA; break; }
-            cur_ms = hm[bq];
-            steps++;
-        }
-        cudaEventRecord(e1, st);
-        if (!s && cudaStreamSynchronize(st) != cudaSuccess) s = KO_ERR_CUDA;
     }
+    if (!s && d.failed) s = KO_ERR_STATE;
+    cudaEventRecord(e1, st);
+    if (!s && cudaStreamSynchronize(st) != cudaSuccess) s = KO_ERR_CUDA;
     if (!s) {
         float t = 0.0f;
         cudaEventElapsedTime(&t, e0, e1);
         if (gpu_ms) *gpu_ms = t;
-        for (int i = 0; i < n; i++) order_out[i] = cur[i];
-        *makespan_out = cur_ms;
-        if (steps_out) *steps_out = steps;
-        if (evals_out) *evals_out = evals;
+        for (int i = 0; i < n; i++) order_out[i] = d.order[i];
+        *makespan_out = d.makespan;
+        if (steps_out) *steps_out = d.steps;
+        if (evals_out) *evals_out = d.evals;
     }
-    if (e0) cudaEventDestroy(e0);
-    if (e1) cudaEventDestroy(e1);
-    cudaFree(base); cudaFree(nb); cudaFree(ms); cudaFree(d_chunk);
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
     return s;
 }
 

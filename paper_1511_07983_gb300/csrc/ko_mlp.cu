@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(kEncWarps * 32) encode_kernel(const int8_t *__
     __shared__ __align__(16) int8_t s_rows[kEncWarps][32 * kMaxK];
     __shared__ __align__(16) uint32_t s_out[kEncWarps][32 * kEncPitch];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_wait();
     for (int i = threadIdx.x; i < kSlots; i += blockDim.x) s_pos[i] = (int8_t)slot_position(set_n[0], i);
     for (int i = threadIdx.x; i < kMaxK * kSlotFeat; i += blockDim.x) s_kf[i] = kfeat[i];
     for (int i = threadIdx.x; i < kGlobals; i += blockDim.x) s_kf[kMaxK * kSlotFeat + i] = gfeat[i];
@@ -299,6 +300,7 @@ __global__ void __launch_bounds__(256) batch_kernel(const int8_t *__restrict__ r
     __shared__ int8_t s_kern[kBatchRows][kSlots];
     __shared__ uint16_t tile[kBatchRows * kBatchPitch];
     const int r0 = blockIdx.x * kBatchRows;
+    pdl_wait();
     if (threadIdx.x < kBatchRows) {
         const int b = r0 + threadIdx.x;
         const int src = (int)(mix64(seed + (unsigned long long)b * 0x9E3779B97F4A7C15ull) % (unsigned long long)pool);
@@ -425,6 +427,7 @@ __global__ void __launch_bounds__(kHidden) out_train_kernel(const uint16_t *__re
 {
     __shared__ float s_d[kOutRows], s_dy[kOutRows];
     const int r0 = blockIdx.x * kOutRows, k = threadIdx.x;
+    pdl_wait();
     {
         const int r = k >> 3, c = k & 7;
         const uint4 *src = reinterpret_cast<const uint4 *>(a3 + (size_t)(r0 + r) * kHidden + c * 32);
@@ -542,6 +545,7 @@ __global__ void __launch_bounds__(256) finish_kernel(float *__restrict__ g, cons
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool adam = o.on;
     int blk = blockIdx.x;
+    pdl_wait();
     if (blk < kFinTiles) {
         const float *src = wg1;
         long long off = kOffW1;
@@ -717,6 +721,7 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float *__restr
     __shared__ unsigned int hist[256];
     __shared__ uint32_t s_prefix, s_need;
     __shared__ unsigned int s_out, s_eq;
+    pdl_wait();
     for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = float_key(y[i]);
     if (threadIdx.x == 0) { s_prefix = 0u; s_need = (uint32_t)k; s_out = s_eq = 0u; }
     for (int shift = 24; shift >= 0; shift -= 8) {
@@ -830,6 +835,7 @@ __global__ void neighbours_kernel(const int8_t *__restrict__ base, int beam, int
 {
     const int per = n * (n - 1) / 2 + n * (n - 1);
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (r >= beam * per) return;
     write_neighbour(base + r / per * kMaxK, n, r % per, out + (size_t)r * kMaxK);
 }
@@ -892,6 +898,7 @@ __global__ void __launch_bounds__(kDescendThreads) descend_kernel(KoDescent *s, 
 __global__ void gather_rows_kernel(const int8_t *src, int stride, const int *pick, int B, int8_t *dst)
 {
     const int b = blockIdx.x;
+    pdl_wait();
     if (b < B && threadIdx.x < stride) dst[(size_t)b * stride + threadIdx.x] = src[(size_t)pick[b] * stride + threadIdx.x];
 }
 
@@ -927,9 +934,8 @@ cudaError_t ko_mlp_encode(const int8_t *rows, int row_stride, const int *set_n, 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long blocks = ((long long)B + 32 * kEncWarps - 1) / (32 * kEncWarps);
     const int grid = (int)(blocks < (long long)sms * 8 ? blocks : (long long)sms * 8);
-    encode_kernel<<<grid, kEncWarps * 32, 0, st>>>(rows, row_stride, set_n, kfeat, gfeat, B, x);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(encode_kernel, dim3(grid), kEncWarps * 32, 0, st, rows, row_stride, set_n, kfeat, gfeat, B, x);
 }
 
 cudaError_t ko_mlp_batch(const int8_t *rows, int row_stride, const int *sid, const float *targets, long long pool,
@@ -937,10 +943,9 @@ cudaError_t ko_mlp_batch(const int8_t *rows, int row_stride, const int *sid, con
                          uint16_t *x, uint16_t *xt, float *t, cudaStream_t st)
 {
     if (B % kBatchRows) return cudaErrorInvalidValue;
-    batch_kernel<<<(unsigned)(B / kBatchRows), 256, 0, st>>>(rows, row_stride, sid, targets, pool, seed, set_n, kfeat,
-                                                            gfeat, B, x, xt, t);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(batch_kernel, dim3(B / kBatchRows), 256, 0, st, rows, row_stride, sid, targets, pool, seed,
+                        set_n, kfeat, gfeat, B, x, xt, t);
 }
 
 cudaError_t ko_mlp_features(const float *x, int B, uint16_t *xb, uint16_t *xt, cudaStream_t st)
@@ -962,9 +967,8 @@ cudaError_t ko_mlp_out_train(const uint16_t *a3, const uint16_t *w4, const float
                              uint16_t *dz, uint16_t *dzt, float *part, cudaStream_t st)
 {
     if (B % kOutRows) return cudaErrorInvalidValue;
-    out_train_kernel<<<(unsigned)(B / kOutRows), kHidden, 0, st>>>(a3, w4, b4, t, B, y, dz, dzt, part);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(out_train_kernel, dim3(B / kOutRows), kHidden, 0, st, a3, w4, b4, t, B, y, dz, dzt, part);
 }
 
 cudaError_t ko_mlp_relu_bwd(const float *da, const uint16_t *a, int B, uint16_t *dz, uint16_t *dzt, float *part,
@@ -980,10 +984,9 @@ cudaError_t ko_mlp_finish(float *g, const float *wg1, const float *wg2, const fl
                           const float *part_out, const float *part2, const float *part1, int B, float *loss_sum,
                           const KoMlpAdam &adam, cudaStream_t st)
 {
-    finish_kernel<<<kFinTiles + kFinSums, 256, 0, st>>>(g, wg1, wg2, wg3, slices, part_out, part2, part1,
-                                                       (int)ko_mlp_part_rows(B), loss_sum, adam);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(finish_kernel, dim3(kFinTiles + kFinSums), 256, 0, st, g, wg1, wg2, wg3, slices, part_out,
+                        part2, part1, (int)ko_mlp_part_rows(B), loss_sum, adam);
 }
 
 cudaError_t ko_mlp_weights_bf16(const float *w, int K, int N, uint16_t *wk, uint16_t *wt, cudaStream_t st)
@@ -997,9 +1000,8 @@ cudaError_t ko_mlp_topk(const float *y, long long n, int k, uint32_t *state, uns
                         unsigned int *counters, int *out, cudaStream_t st)
 {
     if (n <= kSmallTopk) {
-        select_small_kernel<<<1, 1024, 0, st>>>(y, (int)n, k, out);
         ko_count_launch();
-        return cudaGetLastError();
+        return launch_after(select_small_kernel, dim3(1), 1024, 0, st, y, (int)n, k, out);
     }
     select_init_kernel<<<1, 256, 0, st>>>(state, (uint32_t)k, hist, counters);
     ko_count_launch();
@@ -1041,9 +1043,8 @@ cudaError_t ko_mlp_neighbours(const int8_t *base, int beam, int n, int8_t *out, 
     const int per = n * (n - 1) / 2 + n * (n - 1);
     const int rows = beam * per;
     if (rows <= 0) return cudaSuccess;
-    neighbours_kernel<<<(rows + 127) / 128, 128, 0, st>>>(base, beam, n, out);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(neighbours_kernel, dim3((rows + 127) / 128), 128, 0, st, base, beam, n, out);
 }
 
 cudaError_t ko_mlp_descend(KoDescent *s, const int64_t *ms, int nq, int n, int8_t *rows, cudaStream_t st)
@@ -1056,7 +1057,6 @@ cudaError_t ko_mlp_descend(KoDescent *s, const int64_t *ms, int nq, int n, int8_
 cudaError_t ko_mlp_gather_rows(const int8_t *src, int stride, const int *pick, int B, int8_t *dst,
                                cudaStream_t st)
 {
-    gather_rows_kernel<<<B, 32, 0, st>>>(src, stride, pick, B, dst);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(gather_rows_kernel, dim3(B), 32, 0, st, src, stride, pick, B, dst);
 }

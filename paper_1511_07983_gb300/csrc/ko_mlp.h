@@ -6,6 +6,34 @@
 
 #include "ko_internal.h"
 
+// Launch that may begin while the kernel before it in the stream ends (programmatic
+// dependent launch): the network's kernels are 4 to 15 us each and follow each
+// other, so a launch's own start-up showed between them.  A kernel launched so
+// calls pdl_wait() before it touches memory that kernel wrote, or that it reads.
+template <typename... Par, typename... Arg>
+cudaError_t launch_after(void (*kernel)(Par...), dim3 grid, int threads, size_t smem, cudaStream_t st, Arg... arg)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait()
+{
+#ifdef __CUDA_ARCH__
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+#endif
+}
+#endif
+
 constexpr int kSlots = 24;        // position slots
 constexpr int kSlotFeat = 7;      // features per slot
 constexpr int kGlobals = 8;       // global features

@@ -216,6 +216,7 @@ tc_layer_kernel(const uint16_t *__restrict__ A, const uint16_t *__restrict__ Wt,
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(saddr(&mbar)));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
     }
+    pdl_wait();
     tc_fill(sb, Wt + (size_t)n0 * K, NT, NT, K, K);
     asm volatile("cp.async.commit_group;\n" ::);
     if (MODE != 3)
@@ -473,6 +474,7 @@ tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     const int ntiles = (int)blockIdx.x < tiles ? (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     // swizzled TMA destinations and the MMA atoms need 1024-byte aligned stages
     if (saddr(smem) & 1023u) {
+        pdl_wait();
         if (tid == 0) atomicExch(err, 1);
         return;
     }
@@ -495,6 +497,7 @@ tc_ws_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
     }
+    pdl_wait();
     for (int i = tid; i < kTileN; i += blockDim.x) sbias[i] = bias[i];
     float *sw4 = sbias + kTileN;    // OUT: w4 as floats, then 2 x 4 x 128 partial sums
     if (OUT)
@@ -706,6 +709,7 @@ tc_wgrad_kernel(const uint16_t *__restrict__ A, long long lda, const uint16_t *_
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(saddr(&mbar)));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::);
     }
+    pdl_wait();
     tc_fill(sa, A + (size_t)m0 * lda + k0, kTileM, M - m0, lda, kSliceK);
     tc_fill(sb, Bt + (size_t)n0 * ldb + k0, NT, NT, ldb, kSliceK);
     asm volatile("cp.async.commit_group;\n" ::);
@@ -761,9 +765,9 @@ cudaError_t launch_layer_nt(const uint16_t *A, const uint16_t *Wt, int M, int K,
     if (e != cudaSuccess) return e;
     const int tiles = M / kTileM, room = sm_count() / (kTileN / NT);
     const dim3 grid(tiles < room ? tiles : (room > 0 ? room : 1), kTileN / NT);
-    tc_layer_kernel<MODE, NT><<<grid, kThreadsTc, smem, st>>>(A, Wt, K, tiles, bias, act, out, out_t, ldt, part, err);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(tc_layer_kernel<MODE, NT>, grid, kThreadsTc, smem, st, A, Wt, K, tiles, bias, act, out, out_t,
+                        ldt, part, err);
 }
 
 // Columns per CTA: the fewest whose CTAs still run in one wave (see above).
@@ -810,9 +814,9 @@ cudaError_t launch_ws(const uint16_t *A, const uint16_t *Wt, int M, int K, const
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = M / kTileM;
     const int grid = tiles < sms ? tiles : sms;
-    tc_ws_kernel<OUT><<<grid, kWsThreads, smem, st>>>(tma, tmw, K, tiles, stages, bias, out, w4, b4, y, err);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(tc_ws_kernel<OUT>, dim3(grid), kWsThreads, smem, st, tma, tmw, K, tiles, stages, bias, out, w4,
+                        b4, y, err);
 }
 
 }  // namespace
@@ -869,10 +873,9 @@ cudaError_t launch_wgrad(const uint16_t *A, long long lda, const uint16_t *Bt, l
     if ((long long)smem > (long long)max_dyn_smem()) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(tc_wgrad_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    tc_wgrad_kernel<NT><<<dim3(mt, slices, kTileN / NT), kThreadsTc, smem, st>>>(A, lda, Bt, ldb, M, work,
-                                                                                2 * kTileM, err);
     ko_count_launch();
-    return cudaGetLastError();
+    return launch_after(tc_wgrad_kernel<NT>, dim3(mt, slices, kTileN / NT), kThreadsTc, smem, st, A, lda, Bt, ldb, M,
+                        work, 2 * kTileM, err);
 }
 
 }  // namespace

@@ -357,10 +357,12 @@ size_t slab_bytes(int levels)
     return sizeof(uint32_t) * (size_t)sms * lane_threads<SH>() * levels * SH::kSaveWords;
 }
 
-// Threads per block when a launch's work items cannot fill every SM with
-// full blocks: small blocks spread the items over all SMs, so each warp shares
-// its SM's issue slots with fewer warps (the simulation is latency-bound per
-// warp).
+// Threads per block when a launch's units cannot fill every SM with full blocks:
+// small blocks spread them over all SMs, so each warp shares its SM's issue slots
+// with fewer warps (the simulation is latency-bound per warp) -- as long as all
+// small blocks run at once.  A second wave of a few blocks costs a simulation's
+// time: 40,320 orders of an 8-kernel set are 630 blocks of the 14-run state where
+// 608 fit (four of 51 KB per SM): 342 us, and 253 in 140 full blocks.
 constexpr int kSmallT = 64;
 
 template <int T, class SH>
@@ -387,8 +389,12 @@ cudaError_t launch_lane(const KoWork &a, cudaStream_t st)
     if (a.space && a.item_list) work = (long long)sms * T;
     else if (a.space && work < (long long)sms * T) work *= kounits::parts(levels + 1, 2);
     const long long needed = (work + T - 1) / T;
-    if (needed < sms && work > 0) {
-        // fewer items than SMs x T: blocks of kSmallT threads, one item per thread at most
+    int smem_sm = 0;
+    cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    const long long small_at_once =
+        (long long)sms * (smem_sm / (SH::kWords * 4 * kSmallT + 1024)) * kSmallT;  // 1 KB a block is the system's
+    if (needed < sms && work > 0 && work <= small_at_once) {
+        // blocks of kSmallT threads, one unit per thread at most
         long long blocks = (work + kSmallT - 1) / kSmallT;
         const long long fit = a.gstack_words / ((long long)kSmallT * levels * SH::kSaveWords);
         if (blocks > fit) blocks = fit;  // the slab holds sms x T threads' node states, so fit >= needed

@@ -848,9 +848,12 @@ fast_kernel(KoWork a)
     if (sim.sg.lane == 0) st.flush(a.accs, st_set);
 }
 
-// Lists of abandoned units: one per pass that can abandon any (two one-thread
+// Lists of abandoned units: one per pass that can abandon any (three one-thread
 // passes, the 16-lane and the wide one).
-constexpr int kLists = 4;
+constexpr int kLists = 5;
+// Saved levels from which the items a one-thread pass abandons are tried once
+// more in parts: an item fails with the first of its nodes that is too large.
+constexpr int kFineLevels = 3;
 
 // Device buffer layout inside KoFastState::buf.
 struct FastBuf {
@@ -940,29 +943,24 @@ KoChoice ko_list_choice(const KoSet &h, long long count)
 }
 
 // Whole spaces: the work items of a space are its prefixes, each walked by one
-// simulation.  Up to 6! orders fill no chip however they are split, so a
-// warp takes one order (N=5, 148 SMs: 96 us; one 16-lane segment for the
-// whole space 3.9 ms).  Larger spaces go to one thread per item with the most
-// levels that still leave four items for every thread, and none where even
-// single orders do not (N=8, 13 SMs: 0.23 ms without levels, 0.31 with one, 6.4
-// with the state's default; N=9, 148 SMs: 2.1 ms with one level, 4.9 with three,
-// 22 with the default).  The 12-run state holds spaces on up to 16 SMs (N=9,
-// 13 SMs: 1.21 ms against 1.44 with 14 runs); on 148 SMs it hands on too many
-// items (N=10: 20.6 against 16.2 ms).  In a batch every set takes one thread per
-// item: its other sets fill the chip, and each choice is a launch of its own.
+// simulation.  Up to 7! orders fill no chip however they are split, so a warp
+// takes one order (N=5, 148 SMs: 96 us, one 16-lane segment for the whole space
+// 3.9 ms; N=7, 13 SMs: 92 us, one thread per order 183).  Larger spaces go to one
+// thread per item with two levels at eight kernels and three from nine on (a
+// pass cuts its last items, ko_units.cuh, so deep items do not idle the chip):
+// N=8, 148 SMs 0.38 ms with two, 0.42 with none, 13 with the state's default;
+// N=9, 148 SMs 2.10 ms with three, 2.33 with one, 22 with the default; N=10, 13
+// SMs 8.5 ms with three, 9.4 with two; N=11, 148 SMs 160 to 168 ms with three or
+// four, a set whose items are often too large 330 and 494).  The 12-run state holds spaces on up to 16 SMs
+// (N=9, 13 SMs: 1.30 ms against 1.41 with 14 runs); on 148 SMs it hands on too
+// many items (N=10: 17.6 against 15.0 ms).  In a batch every set takes one
+// thread per item: its other sets fill the chip, and each choice is a launch of
+// its own.
 KoChoice ko_space_choice(const KoSet &h, bool alone)
 {
     const int n = h.n;
-    if (n <= 6 && alone) return KoChoice{32, 0, 0};
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned long long want = 4ull * sms * 288;
-    const int deepest = h.S <= 16 ? 3 : 4;  // a deeper item that overflows hands on more orders
-    int levels = 0;
-    unsigned long long items = 1;
-    for (int i = 2; i <= n; i++) items *= (unsigned long long)i;
-    while (levels < deepest && levels + 1 < n && items / (levels + 2) >= want) items /= ++levels + 1;
+    if (n <= 7 && alone) return KoChoice{32, 0, 0};
+    const int levels = std::max(0, std::min(n - 6, 3));
     if (!packs(h)) return KoChoice{16, levels, 0};
     return KoChoice{1, levels, h.S <= 16 ? 1 : 0};
 }
@@ -1021,6 +1019,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     unsigned long long want = (unsigned long long)(w.n_items > w.reserve_items ? w.n_items : w.reserve_items);
     if (fs->lanes == 1 && w.space) {
         const unsigned long long threads = (unsigned long long)std::max(ko_lane_threads(fs->lane_shape), ko_lane_threads(0));
+        if (w.levels >= kFineLevels) want *= kounits::parts(w.levels + 1, 1);
         want += threads * kounits::parts(w.levels + 1, 1) + (threads + 1) * kounits::parts(w.levels + 1, 2);
     }
     want = ((want < 1024 ? 1024 : want) + 1023) & ~1023ull;
@@ -1103,31 +1102,23 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     if (lane) {
         // all items, one simulation per thread; what a smaller state cannot hold goes to the largest
         // one before any run-length pass (48 mixed sets in one graph: the 16-lane pass over what the
-        // 12-run state handed on took 51 of 180 ms)
+        // 12-run state handed on took 51 of 180 ms).  Long items are then tried once more in parts of
+        // six orders (an 11-kernel / 148-SM set of which half the 120-order items are too large:
+        // 857 -> 494 ms; with 24-order items 461 -> 330)
         KoWork w0 = w;
         w0.gstack = (int *)fs->lslab;
         w0.gstack_words = (long long)(fs->lslab_bytes / sizeof(int));
-        for (int shape = fs->lane_shape;; shape = 0) {
+        const int passes[3] = {fs->lane_shape, fs->lane_shape != 0 ? 0 : -1,
+                               w.space && w.levels >= kFineLevels ? 0 : -1};
+        for (int i = 0; i < 3; i++) {
+            if (passes[i] < 0) continue;
+            w0.fine = i == 2;
             next_pass(w0);
-            if ((e = ko_launch_lane(w0, shape, st)) != cudaSuccess) {
+            if ((e = ko_launch_lane(w0, passes[i], st)) != cudaSuccess) {
                 cudaGetLastError();
                 return KO_ERR_CUDA;
             }
-            if (shape == 0) break;
         }
-    }
-    if (warps) {
-        // its runs and groups are as many as the wide pass has
-        next_pass(w);
-        if ((e = ko_launch_warp(w, st)) == cudaSuccess) {
-            w.fb_counter = &fb->fb_counter;
-            e = ko_launch_fallback(w, fs->fb_scratch, fs->fb_bytes, max_slab_bytes, st);
-        }
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return KO_ERR_CUDA;
-        }
-        return KO_OK;
     }
     // all items, or those the one-thread passes abandoned: these first order by order, a warp each (a
     // few are done in one simulation's time: 100,003 orders of N=12, some 250 of them handed on, 2.2 ->

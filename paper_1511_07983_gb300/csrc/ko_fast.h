@@ -43,6 +43,7 @@ struct KoWork {
     const unsigned long long *item_count;
     int levels;                       // saved DFS levels per segment
     bool space;                       // the chunks are prefixes (mode 0): their items may be cut into parts
+    bool fine;                        // one-thread pass over a list: cut its items to walks of six orders
     bool singles_taken;               // list passes: the warp pass has taken a list it could cut to single orders
     int run_limit;                    // runs one simulation may hold
     int *gstack;                      // non-null: DFS node states in this global slab, not shared memory

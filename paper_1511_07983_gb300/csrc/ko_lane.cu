@@ -134,7 +134,8 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
     if (threadIdx.x == 0) {
         const int lv = a.space ? levels : 0;
         const unsigned long long threads = (unsigned long long)gridDim.x * T;
-        units = a.item_list ? kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, lv, threads)
+        units = a.item_list ? kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, lv, threads,
+                                                   a.fine ? a.ov_cap : 0ull)
                             : kounits::number_space((unsigned long long)a.n_items, lv, threads);
     }
     __syncthreads();

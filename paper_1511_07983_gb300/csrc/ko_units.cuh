@@ -71,8 +71,10 @@ __host__ __device__ inline Numbering number_space(unsigned long long items, int 
 }
 
 // A pass of `threads` simulations over `items` list entries, every one cut as
-// far as a thread is left for each part.
-__host__ __device__ inline Numbering number_list(unsigned long long items, int levels, unsigned long long threads)
+// far as a thread is left for each part; with `fine`, down to walks of at most
+// three kernels (six orders) where no more than `fine` parts come of it.
+__host__ __device__ inline Numbering number_list(unsigned long long items, int levels, unsigned long long threads,
+                                                 unsigned long long fine = 0)
 {
     Numbering u;
     const int m = levels + 1;
@@ -80,7 +82,7 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
     u.a = u.b = 0ull;
     u.x1 = u.x2 = 0;
     u.f1 = u.f2 = 1;
-    while (m - u.x2 > 1 && items * u.f2 * (unsigned)(m - u.x2) <= threads) {
+    while (m - u.x2 > 1 && items * u.f2 * (unsigned)(m - u.x2) <= (m - u.x2 > 3 && fine > threads ? fine : threads)) {
         u.f2 *= (unsigned)(m - u.x2);
         u.x2++;
     }
@@ -89,12 +91,14 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
 }
 
 // The numbering of a list as single orders, if there are few enough of them (and
-// no more than a list holds) that running each from the start, a warp per order,
-// beats walking the items: 65,536 orders take about 2 ms, as walking one item does.
+// no more than a list holds): run from the start, a warp per order, they take
+// 25 us a thousand, and none is too large for that pass, where walking them in
+// 16-lane segments abandons most of what one thread could not hold.
+constexpr unsigned long long kSinglesMax = 2ull << 20;
 __host__ __device__ inline bool number_singles(unsigned long long items, int levels, unsigned long long cap,
                                                Numbering &u)
 {
-    u = number_list(items, levels, cap < 65536ull ? cap : 65536ull);
+    u = number_list(items, levels, cap < kSinglesMax ? cap : kSinglesMax);
     return levels + 1 - u.x2 <= 1;
 }
 

@@ -199,7 +199,7 @@ def test_whole_space_items_beside_deeper_walks(ko, state):
 
 
 @pytest.mark.parametrize("workload,n,levels,state,run_limit", [
-    ("sets10", 8, 2, 0, 6), ("sets10", 8, 5, 1, 6), ("sets10", 7, 6, 2, 4),
+    ("sets10", 8, 2, 0, 6), ("sets10", 8, 5, 1, 6), ("sets10", 7, 6, 2, 4), ("sets10", 8, 4, 0, 5),
     ("single12", 9, 2, 0, 32), ("single12", 9, 3, 2, 32), ("single12", 9, 5, 1, 32), ("single12", 10, 2, 1, 32)])
 def test_cut_items_cover_the_space_once(ko, workload, n, levels, state, run_limit):
     """A pass cuts its last items (all of them below one item per thread) into

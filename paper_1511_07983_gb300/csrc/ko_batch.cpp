@@ -295,9 +295,9 @@ ko_status ko_batch_exec(ko_batch *b, ko_rank *out, uint64_t *hist, bool hist_dev
         cudaGetLastError();
         return KO_ERR_CUDA;
     }
-    // reset, the reference-order passes (two), each group's passes (three; with one-thread ones two or three more)
-    int launches = b->nsets * (b->nbins > 0 ? 1 : 0) + 3;
-    for (const ko_batch::Group &g : b->groups) launches += 3 + (g.lanes != 1 ? 0 : g.shape == 0 ? 2 : 3);
+    // reset, histograms, the reference-order passes, each group's passes
+    int launches = 1 + (b->nbins > 0 ? b->nsets : 0) + ko_fast_launches(32, 0, false, 1);
+    for (const ko_batch::Group &g : b->groups) launches += ko_fast_launches(g.lanes, g.shape, true, g.levels);
     ko_count_launch(launches);
     if (hist && b->nbins > 0) {
         const size_t bytes = sizeof(unsigned long long) * b->nbins * b->nsets;

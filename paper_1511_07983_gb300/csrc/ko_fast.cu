@@ -951,11 +951,11 @@ KoChoice ko_list_choice(const KoSet &h, long long count)
 // N=8, 148 SMs 0.38 ms with two, 0.42 with none, 13 with the state's default;
 // N=9, 148 SMs 2.10 ms with three, 2.33 with one, 22 with the default; N=10, 13
 // SMs 8.5 ms with three, 9.4 with two; N=11, 148 SMs 160 to 168 ms with three or
-// four, a set whose items are often too large 330 and 494).  The 12-run state holds spaces on up to 16 SMs
-// (N=9, 13 SMs: 1.30 ms against 1.41 with 14 runs); on 148 SMs it hands on too
-// many items (N=10: 17.6 against 15.0 ms).  In a batch every set takes one
-// thread per item: its other sets fill the chip, and each choice is a launch of
-// its own.
+// four, a set whose items are often too large 330 and 494).  The 12-run state
+// holds spaces on up to 16 SMs (N=9, 13 SMs: 1.30 ms against 1.41 with 14 runs);
+// on 148 SMs it hands on too many items (N=10: 17.6 against 15.0 ms).  In a batch
+// every set takes one thread per item: its other sets fill the chip, and each
+// choice is a launch of its own.
 KoChoice ko_space_choice(const KoSet &h, bool alone)
 {
     const int n = h.n;
@@ -1011,6 +1011,12 @@ KoRoute::~KoRoute()
     fs->levels = levels;
     fs->lane_shape = shape;
     fs->stack_global = stack;
+}
+
+int ko_fast_launches(int lanes, int shape, bool space, int levels)
+{
+    if (lanes == 32 && (!space || levels < 1)) return 2;
+    return 3 + (lanes != 1 ? 0 : 2 + (shape != 0 ? 1 : 0) + (space && levels >= kFineLevels ? 1 : 0));
 }
 
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st)
@@ -1119,6 +1125,19 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
                 return KO_ERR_CUDA;
             }
         }
+    }
+    if (warps) {
+        // its runs and groups are as many as the wide pass has
+        next_pass(w);
+        if ((e = ko_launch_warp(w, st)) == cudaSuccess) {
+            w.fb_counter = &fb->fb_counter;
+            e = ko_launch_fallback(w, fs->fb_scratch, fs->fb_bytes, max_slab_bytes, st);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return KO_ERR_CUDA;
+        }
+        return KO_OK;
     }
     // all items, or those the one-thread passes abandoned: these first order by order, a warp each (a
     // few are done in one simulation's time: 100,003 orders of N=12, some 250 of them handed on, 2.2 ->

@@ -116,6 +116,9 @@ struct KoRoute {
 // (a pass abandons a unit at most once).
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st);
 
+// Kernels ko_fast_launch enqueues for these options.
+int ko_fast_launches(int lanes, int shape, bool space, int levels);
+
 // One-thread-per-order pass (ko_lane.cu) over the items of `w` (counters and
 // the abandoned-item list already set; w.gstack = its node-state slab of
 // ko_lane_slab_bytes(w.levels, shape) bytes); shape as KoFastState::lane_shape.

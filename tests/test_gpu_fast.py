@@ -292,3 +292,20 @@ def test_captured_list_after_a_space_only(ko):
         got = out.cpu().numpy()
         want = g.eval_orders(orders=rows.cpu().numpy())
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("call,launches", [("list", 2), ("space7", 3), ("pinned16", 3), ("pinned1", 5)])
+def test_route_by_launches(ko, call, launches):
+    """The kernels a call enqueues tell its route: a warp per order is followed by
+    the simple simulator only; a space's accumulators are reset first."""
+    s = synth.gen_set("single8", 1, n=7)
+    rows = synth.random_orders(4, 7, 16).astype(np.int8)
+    with ko.Gpu.from_set(s) as g:
+        if call.startswith("pinned"):
+            g.configure(lanes=int(call[6:]))
+        before = ko.ko_kernel_launches()
+        if call == "space7":
+            _all(g, 7)
+        else:
+            g.eval_orders(orders=rows)
+        assert ko.ko_kernel_launches() - before == launches

@@ -711,19 +711,19 @@ __global__ void select_scan_kernel(uint32_t *state, int shift, unsigned int *his
     hist[threadIdx.x] = 0;
 }
 
-// Up to kSmallTopk keys: the four digits and the output in one block, the keys in
-// shared memory (the neighbourhoods of a search round; nine launches, two clears
-// and a copy before: 70 of a round's 340 us).
+// Up to kSmallTopk keys: the four digits in one block, the keys in shared memory
+// (the neighbourhoods of a search round; eight launches, two clears and a copy
+// before: 66 of a round's 340 us).
 constexpr int kSmallTopk = 8192;
-__global__ void __launch_bounds__(1024) select_small_kernel(const float *__restrict__ y, int n, int k, int *out)
+__global__ void __launch_bounds__(1024) select_small_kernel(const float *__restrict__ y, int n, int k, uint32_t *state,
+                                                            unsigned int *counters)
 {
     __shared__ uint32_t keys[kSmallTopk];
     __shared__ unsigned int hist[256];
     __shared__ uint32_t s_prefix, s_need;
-    __shared__ unsigned int s_out, s_eq;
     pdl_wait();
     for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = float_key(y[i]);
-    if (threadIdx.x == 0) { s_prefix = 0u; s_need = (uint32_t)k; s_out = s_eq = 0u; }
+    if (threadIdx.x == 0) { s_prefix = 0u; s_need = (uint32_t)k; }
     for (int shift = 24; shift >= 0; shift -= 8) {
         if (threadIdx.x < 256) hist[threadIdx.x] = 0u;
         __syncthreads();
@@ -743,14 +743,8 @@ __global__ void __launch_bounds__(1024) select_small_kernel(const float *__restr
         }
         __syncthreads();
     }
-    const uint32_t thr = s_prefix, quota = s_need;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const uint32_t key = keys[i];
-        if (key < thr || (key == thr && atomicAdd(&s_eq, 1u) < quota)) {
-            const unsigned int at = atomicAdd(&s_out, 1u);
-            if (at < (unsigned)k) out[at] = i;
-        }
-    }
+    if (threadIdx.x == 0) { state[0] = s_prefix; state[1] = s_need; }
+    if (threadIdx.x < 2) counters[threadIdx.x] = 0u;
 }
 
 // Write the indices of the k smallest keys: all keys below the threshold and
@@ -999,17 +993,19 @@ cudaError_t ko_mlp_weights_bf16(const float *w, int K, int N, uint16_t *wk, uint
 cudaError_t ko_mlp_topk(const float *y, long long n, int k, uint32_t *state, unsigned int *hist,
                         unsigned int *counters, int *out, cudaStream_t st)
 {
-    if (n <= kSmallTopk) {
-        ko_count_launch();
-        return launch_after(select_small_kernel, dim3(1), 1024, 0, st, y, (int)n, k, out);
-    }
-    select_init_kernel<<<1, 256, 0, st>>>(state, (uint32_t)k, hist, counters);
-    ko_count_launch();
     const int blocks = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        select_hist_kernel<<<blocks, 256, 0, st>>>(y, n, state, shift, hist);
-        select_scan_kernel<<<1, 256, 0, st>>>(state, shift, hist);
-        ko_count_launch(2);
+    if (n <= kSmallTopk) {
+        const cudaError_t e = launch_after(select_small_kernel, dim3(1), 1024, 0, st, y, (int)n, k, state, counters);
+        if (e != cudaSuccess) return e;
+        ko_count_launch();
+    } else {
+        select_init_kernel<<<1, 256, 0, st>>>(state, (uint32_t)k, hist, counters);
+        ko_count_launch();
+        for (int shift = 24; shift >= 0; shift -= 8) {
+            select_hist_kernel<<<blocks, 256, 0, st>>>(y, n, state, shift, hist);
+            select_scan_kernel<<<1, 256, 0, st>>>(state, shift, hist);
+            ko_count_launch(2);
+        }
     }
     select_emit_kernel<<<blocks, 256, 0, st>>>(y, n, state, counters, k, out);
     ko_count_launch();

@@ -186,17 +186,22 @@ ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t 
                         int32_t nbins, void *stream);
 
 /* Makespans of all N! orders in Lehmer-index order into makespans_out[N!]
- * (device memory), N <= 12.  Asynchronous on `stream`; the handle holds 16
- * bytes of device memory per work item (N! / (levels + 1)! items) for the
- * lists that carry abandoned items between passes. */
+ * (device memory), N <= 12.  Asynchronous on `stream`; the handle holds 40
+ * bytes of device memory per work item (N! / (levels + 1)! items; from three
+ * levels on, per item and kernel left in it) for the lists that carry
+ * abandoned items between passes, and about 20 MB of such lists at least. */
 ko_status ko_eval_all(ko_gpu *g, int64_t *makespans_out, void *stream);
 
 /* Tuning knobs of the device simulators (set by the tuner; per handle).
+ * While none of KO_OPT_LANES, KO_OPT_LEVELS, KO_OPT_STACK_GLOBAL and
+ * KO_OPT_LANE_STATE has been set or tuned, calls choose by their size instead:
+ * a warp or a thread per order for lists, and for spaces besides the levels.
  *   KO_OPT_LANES        threads per simulation: 1 = one thread per order,
- *                       its state in shared memory, followed by the
- *                       run-length passes for the work items it cannot hold;
- *                       16 or 32 = lanes sharing one run-length simulation,
- *                       its state packed in registers (default 16)
+ *                       its state in shared memory, followed by passes over
+ *                       the work items it cannot hold; 32 = a warp per order
+ *                       for lists and for spaces with no saved level; else 16
+ *                       or 32 = lanes sharing one run-length simulation, its
+ *                       state packed in registers (default 16)
  *   KO_OPT_LEVELS       prefix-sharing depth: exhaustive work items fix the
  *                       first N-1-levels kernels and walk the rest depth
  *                       first, saving `levels` states; 0..6 (default 4)
@@ -215,10 +220,11 @@ ko_status ko_eval_all(ko_gpu *g, int64_t *makespans_out, void *stream);
  *                       (288 simulations per SM, default), 1 = 12 runs and
  *                       40 slots (352), 2 = 10 runs and 32 slots (448).
  *                       Smaller states fit more simulations on an SM; work
- *                       items that need more move on to the run-length passes.
- *                       A launch with fewer work items than SMs x those
- *                       simulations runs in 64-thread blocks spread over
- *                       every SM instead (one item per thread)
+ *                       items that need more move on to the largest state and
+ *                       then to the passes above.  A launch with fewer work
+ *                       items than SMs x those simulations runs in 64-thread
+ *                       blocks spread over every SM instead (one item per
+ *                       thread) where all of them run at once
  * Results never depend on these knobs.  KO_ERR_ARG for an unknown key or
  * value. */
 #define KO_OPT_LANES 1
@@ -259,13 +265,12 @@ ko_status ko_autotune(ko_gpu *g, const char *cache_path, void *stream);
  * `stream`; results never depend on the choice. */
 ko_status ko_batch_autotune(ko_gpu *const *sets, int32_t nsets, const char *cache_path, void *stream);
 
-/* Work items the last exhaustive or index-list call moved from the
- * run-length simulator to its wider second pass (a simulation needed more runs
- * of distinct SM states than lanes, or more than 8 resident groups in a run;
- * what that pass cannot finish goes to the simple simulator); -1 for a NULL
- * handle.  Informational: results are exact either way, because the lists
- * that carry abandoned items between the passes hold every item of the call
- * (device memory: 16 bytes per work item, allocated by the call). */
+/* Work items the last exhaustive or list call could not finish in its first pass
+ * (a simulation needed more runs of distinct SM states or more groups of blocks
+ * than that pass's state holds) and moved on to the passes after it; -1 for a
+ * NULL handle.  Informational: results are exact either way, because the lists
+ * that carry abandoned items between the passes hold everything a pass may
+ * abandon. */
 int64_t ko_last_fallback_items(const ko_gpu *g);
 
 /* Number of CUDA kernels this library has launched in this process (all

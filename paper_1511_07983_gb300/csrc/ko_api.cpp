@@ -75,7 +75,7 @@ struct ko_gpu {
     unsigned long long *d_hist = nullptr;
     int hist_cap = 0;
     long long h2d = 0, d2h = 0;   // bytes copied by this handle
-    Meta *d_meta = nullptr;       // chunk lists, heuristic order, reference makespan (device)
+    Meta *d_meta = nullptr;       // the call's chunk (device)
     Meta h_meta{};
     KoFastState fast{};        // run-length simulator state (work list, overflow list)
     bool fast_pending = false; // an asynchronous run-length launch has not been inspected yet

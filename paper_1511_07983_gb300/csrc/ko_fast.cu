@@ -36,6 +36,9 @@
 //   kG groups in one run, abandons its work item and records it; a second
 //   pass with 32 lanes and 16 group slots re-runs the recorded items, and the
 //   simple simulator takes whatever that pass abandons, all on the stream.
+//
+// ko_fast_launch, below, also puts the other simulators' passes in order: one
+// thread per order (ko_lane.cu) or one warp per order (ko_warp.cu) first.
 #include <algorithm>
 
 #include "ko_fast.h"

@@ -33,7 +33,7 @@ struct KoWork {
     int perm_stride;                  // bytes between mode-2 rows (0: N of the row's set)
     int64_t *out;                     // makespans, or null
     unsigned long long *counter;      // next work item
-    unsigned long long *ov_count;     // items abandoned by the run-length simulator
+    unsigned long long *ov_count;     // units the pass abandoned
     unsigned long long *ov_list;      // their list entries (ko_units.cuh)
     unsigned long long *abandoned;    // work items the first pass abandoned (whole or in part)
     unsigned int *part_seen;          // first pass: items with an abandoned part, one bit each
@@ -51,7 +51,7 @@ struct KoWork {
     long long reserve_items;          // sizing only: abandoned-item lists for this many items
 };
 
-// Device-side state of the run-length simulator, owned by a handle or batch.
+// Device-side state of the simulators' passes, owned by a handle, batch or model.
 struct KoFastState {
     void *buf = nullptr;        // counters and the two passes' abandoned-item lists
     size_t cap = 0;

@@ -13,8 +13,9 @@
 //
 // Node states (the simulation after a DFS prefix, burst still open) are saved
 // to a per-thread slab in global memory (L2-resident), kSaveWords per level,
-// 16-byte stores.  A work item that needs more runs or group slots than one
-// simulation holds is recorded for the run-length simulator, which re-runs it.
+// 16-byte stores.  Work comes in units, whole items or parts of them
+// (ko_units.cuh); a unit that needs more runs or group slots than one simulation
+// holds is recorded for the passes that follow (ko_fast.cu).
 #include "ko_fast.h"
 #include "ko_lane_sim.cuh"
 #include "ko_units.cuh"

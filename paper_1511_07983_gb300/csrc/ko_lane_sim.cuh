@@ -28,13 +28,14 @@
 // warps per SM; it moves no data to speak of.  The loops over released runs
 // and their slots that an event step had before made a warp run as long as its
 // worst thread.  All 39.9M orders of an 11-kernel / 148-SM set: 470 ms with the
-// looping event step over ordered runs, 260 ms with this one; 3.6M orders of a
-// ten-kernel / 15-SM set 31.9 -> 22.6 ms.
+// looping event step over ordered runs, 260 ms with this one, 184 with a kernel's
+// first burst and the close of a burst as such steps too; 3.6M orders of a
+// ten-kernel / 15-SM set 31.9 -> 22.6 -> 15.3 ms.
 //
 // Measured on the N=12 / 148-SM set: about 11 runs and 34 groups live, 1.24
 // runs released per event, 34 events per order, a split every 15 events.  56
 // slots hold every group of about 99 % of the 120-order work items; the rest
-// move on to the run-length passes.
+// move on to other passes.
 //
 // Layout.  The state of one simulation is a column of kWords 32-bit words in
 // shared memory, word f of the thread's column at col[f * STRIDE]; with STRIDE

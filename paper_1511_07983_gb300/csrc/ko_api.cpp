@@ -199,12 +199,7 @@ ko_status fast_after_sync(ko_gpu *g)
     float ms = -1.0f;
     if (fs.ev0 && cudaEventElapsedTime(&ms, fs.ev0, fs.ev1) == cudaSuccess) fs.last_ms = ms;
     cudaGetLastError();
-    unsigned long long cnt = 0;
-    const unsigned long long *dc = ko_fast_overflow_counter(&fs);
-    if (dc && cudaMemcpy(&cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost) != cudaSuccess) return KO_ERR_CUDA;
-    fs.d2h += sizeof(cnt);
-    fs.last_overflow = cnt;
-    return cnt > fs.ov_cap ? KO_ERR_STATE : KO_OK;  // cannot happen: the lists hold every item
+    return ko_fast_check(&fs);
 }
 
 }  // namespace

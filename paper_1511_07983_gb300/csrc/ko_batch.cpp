@@ -306,11 +306,8 @@ ko_status ko_batch_exec(ko_batch *b, ko_rank *out, uint64_t *hist, bool hist_dev
             return KO_ERR_CUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return KO_ERR_CUDA;
-    unsigned long long cnt = 0;
-    const unsigned long long *dc = ko_fast_overflow_counter(&b->fast);
-    if (dc && cudaMemcpy(&cnt, dc, sizeof(cnt), cudaMemcpyDeviceToHost) == cudaSuccess)
-        b->fast.last_overflow = cnt;
-    if (cnt > b->fast.ov_cap) return KO_ERR_STATE;  // cannot happen
+    const ko_status s = ko_fast_check(&b->fast);
+    if (s) return s;
     for (int i = 0; i < b->nsets; i++) {
         const KoAccum &a = b->h_accs[i];
         const long long mh = b->h_refs[i];

@@ -658,7 +658,7 @@ fast_kernel(KoWork a)
             const unsigned long long have = *a.item_count < a.ov_cap ? *a.item_count : a.ov_cap;
             const int lv = a.space ? a.levels : 0;
             kounits::Numbering singles;
-            units = kounits::number_list(have, lv, (unsigned long long)gridDim.x * kSegs);
+            units = kounits::number_list(have, lv, (unsigned long long)gridDim.x * kSegs, a.ov_cap);
             if (a.singles_taken && kounits::number_singles(have, lv, a.ov_cap, singles)) units.units = 0;
         } else {
             units.units = (unsigned long long)a.n_items;
@@ -840,8 +840,7 @@ fast_kernel(KoWork a)
         }
         if (have && sim.sg.lane == 0) {
             if (sim.fail) {
-                const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                if (slot < a.ov_cap) a.ov_list[slot] = rec;
+                kounits::hand_on(a, rec);
                 if (!a.item_list) atomicAdd(a.abandoned, 1ull);
             } else {
                 st.add(is);
@@ -860,7 +859,8 @@ constexpr int kFineLevels = 3;
 
 // Device buffer layout inside KoFastState::buf.
 struct FastBuf {
-    unsigned long long counter[kLists + 1], ov_count[kLists], fb_counter, abandoned;
+    unsigned long long lost;         // units no list had room for (none); not cleared between launches
+    unsigned long long abandoned, counter[kLists + 1], ov_count[kLists], fb_counter;
     unsigned int part_seen[kPartSeen / 32];
     unsigned long long ov_list[1];   // KoFastState::ov_cap entries per list
 };
@@ -1047,6 +1047,7 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         }
         fs->cap = need;
         fs->ov_cap = want;
+        if (cudaMemsetAsync(fs->buf, 0, sizeof(FastBuf), st) != cudaSuccess) return KO_ERR_CUDA;
     }
     if (!fs->fb_scratch) {
         if (cudaMalloc(&fs->fb_scratch, kFallbackScratch) != cudaSuccess) {
@@ -1091,11 +1092,13 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
         }
     }
     FastBuf *fb = (FastBuf *)fs->buf;
-    if (cudaMemsetAsync(fb, 0, sizeof(FastBuf), st) != cudaSuccess) return KO_ERR_CUDA;
+    constexpr size_t kCleared = offsetof(FastBuf, abandoned);
+    if (cudaMemsetAsync((char *)fb + kCleared, 0, sizeof(FastBuf) - kCleared, st) != cudaSuccess) return KO_ERR_CUDA;
     w.run_limit = fs->run_limit;
     if (w.levels < 1) w.levels = 1;
     if (w.levels > kMaxLevels) w.levels = kMaxLevels;
     w.ov_cap = fs->ov_cap;
+    w.lost = &fb->lost;
     w.abandoned = &fb->abandoned;
     w.part_seen = fb->part_seen;
     int list = 0;  // list the next pass writes; it reads the one before
@@ -1188,9 +1191,17 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     return KO_OK;
 }
 
-const unsigned long long *ko_fast_overflow_counter(const KoFastState *fs)
+ko_status ko_fast_check(KoFastState *fs)
 {
-    return fs->buf ? &((const FastBuf *)fs->buf)->abandoned : nullptr;
+    static_assert(offsetof(FastBuf, lost) == 0 && offsetof(FastBuf, abandoned) == 8, "one copy brings both");
+    unsigned long long cnt[2] = {0, 0};
+    if (fs->buf && cudaMemcpy(cnt, fs->buf, sizeof(cnt), cudaMemcpyDeviceToHost) != cudaSuccess) {
+        cudaGetLastError();
+        return KO_ERR_CUDA;
+    }
+    fs->d2h += sizeof(cnt);
+    fs->last_overflow = cnt[1];
+    return cnt[0] ? KO_ERR_STATE : KO_OK;
 }
 
 void ko_fast_release(KoFastState *fs)

@@ -35,6 +35,7 @@ struct KoWork {
     unsigned long long *counter;      // next work item
     unsigned long long *ov_count;     // units the pass abandoned
     unsigned long long *ov_list;      // their list entries (ko_units.cuh)
+    unsigned long long *lost;         // units a full list dropped (none: a pass numbers no more than its list holds)
     unsigned long long *abandoned;    // work items the first pass abandoned (whole or in part)
     unsigned int *part_seen;          // first pass: items with an abandoned part, one bit each
     unsigned long long ov_cap;
@@ -131,8 +132,9 @@ long long ko_lane_threads(int shape);  // simulations a full launch runs at a ti
 // units, which it leaves alone where their single orders outnumber a list.
 cudaError_t ko_launch_warp(const KoWork &w, cudaStream_t st);
 
-// Device address of the count of items the first pass of the last launch abandoned.
-const unsigned long long *ko_fast_overflow_counter(const KoFastState *fs);
+// After the launches have ended: reads how many items the first pass of the last
+// one abandoned (last_overflow); KO_ERR_STATE if a list of any pass was too short.
+ko_status ko_fast_check(KoFastState *fs);
 
 void ko_fast_release(KoFastState *fs);
 

@@ -100,8 +100,7 @@ __device__ __forceinline__ void save_node(const SIM &sim, uint32_t *node)
 // abandoned: items from `cut_from` on may have several such parts.
 __device__ __forceinline__ void abandon(const KoWork &a, unsigned long long rec, unsigned long long cut_from)
 {
-    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-    if (slot < a.ov_cap) a.ov_list[slot] = rec;
+    kounits::hand_on(a, rec);
     if (a.item_list) return;
     const unsigned long long item = rec & kounits::kItemMask;
     bool seen = false;
@@ -136,7 +135,7 @@ __global__ void __launch_bounds__(T, 1) lane_kernel(KoWork a)
         const int lv = a.space ? levels : 0;
         const unsigned long long threads = (unsigned long long)gridDim.x * T;
         units = a.item_list ? kounits::number_list(*a.item_count < a.ov_cap ? *a.item_count : a.ov_cap, lv, threads,
-                                                   a.fine ? a.ov_cap : 0ull)
+                                                   a.ov_cap, a.fine)
                             : kounits::number_space((unsigned long long)a.n_items, lv, threads);
     }
     __syncthreads();

@@ -72,17 +72,21 @@ __host__ __device__ inline Numbering number_space(unsigned long long items, int 
 
 // A pass of `threads` simulations over `items` list entries, every one cut as
 // far as a thread is left for each part; with `fine`, down to walks of at most
-// three kernels (six orders) where no more than `fine` parts come of it.
+// three kernels (six orders) whatever the threads.  `room`, the entries of the
+// list the pass writes, bounds the units of either: a pass may abandon all it
+// numbers (840 two-level items in 2,520 parts against a list of 1,024 lost
+// 2,992 of 5,040 orders).
 __host__ __device__ inline Numbering number_list(unsigned long long items, int levels, unsigned long long threads,
-                                                 unsigned long long fine = 0)
+                                                 unsigned long long room, bool fine = false)
 {
     Numbering u;
     const int m = levels + 1;
+    if (threads > room) threads = room;
     u.items = items;
     u.a = u.b = 0ull;
     u.x1 = u.x2 = 0;
     u.f1 = u.f2 = 1;
-    while (m - u.x2 > 1 && items * u.f2 * (unsigned)(m - u.x2) <= (m - u.x2 > 3 && fine > threads ? fine : threads)) {
+    while (m - u.x2 > 1 && items * u.f2 * (unsigned)(m - u.x2) <= (m - u.x2 > 3 && fine ? room : threads)) {
         u.f2 *= (unsigned)(m - u.x2);
         u.x2++;
     }
@@ -95,10 +99,10 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
 // 25 us a thousand, and none is too large for that pass, where walking them in
 // 16-lane segments abandons most of what one thread could not hold.
 constexpr unsigned long long kSinglesMax = 2ull << 20;
-__host__ __device__ inline bool number_singles(unsigned long long items, int levels, unsigned long long cap,
+__host__ __device__ inline bool number_singles(unsigned long long items, int levels, unsigned long long room,
                                                Numbering &u)
 {
-    u = number_list(items, levels, cap < kSinglesMax ? cap : kSinglesMax);
+    u = number_list(items, levels, kSinglesMax, room);
     return levels + 1 - u.x2 <= 1;
 }
 
@@ -122,5 +126,17 @@ __host__ __device__ inline Unit cut_unit(unsigned long long item, unsigned part,
     const unsigned f = parts(left, cut);
     return Unit{item, part * f + s, x + cut, s < f};
 }
+
+#ifdef __CUDACC__
+// Record an abandoned unit for the next pass.  Every pass numbers at most as many
+// units as its list has entries; one that found its list full all the same is
+// counted, and the call's status tells.
+__device__ __forceinline__ void hand_on(const KoWork &a, unsigned long long entry)
+{
+    const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
+    if (slot < a.ov_cap) a.ov_list[slot] = entry;
+    else atomicAdd(a.lost, 1ull);
+}
+#endif
 
 }  // namespace kounits

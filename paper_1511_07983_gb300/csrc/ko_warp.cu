@@ -545,8 +545,7 @@ __global__ void __launch_bounds__(kWarps * 32) warp_kernel(KoWork a)
         for (int d = 0; ok && d < n; d++) ok = sim.place_kernel(__shfl_sync(kAll, mine, d), limit, run_limit);
         if (!ok) {
             if (lane == 0) {
-                const unsigned long long slot = atomicAdd(a.ov_count, 1ull);
-                if (slot < a.ov_cap) a.ov_list[slot] = kounits::entry_of(item, part, cut);
+                kounits::hand_on(a, kounits::entry_of(item, part, cut));
                 if (!a.item_list) atomicAdd(a.abandoned, 1ull);
             }
             continue;

@@ -182,3 +182,17 @@ def test_batch_autotune_per_class(ko, tmp_path):
         assert (ko.ko_get_option(g.h, ko.KO_OPT_LANES), ko.ko_get_option(g.h, ko.KO_OPT_LEVELS),
                 ko.ko_get_option(g.h, ko.KO_OPT_STACK_GLOBAL),
                 ko.ko_get_option(g.h, ko.KO_OPT_LANE_STATE)) == next(iter(by_class[_class_key(s)]))
+
+
+@pytest.mark.parametrize("lanes,n,levels", [(16, 7, 2), (32, 7, 2), (16, 8, 4)])
+def test_batch_with_pinned_lanes_forced_hand_over(ko, lanes, n, levels):
+    """One set whose every item is handed on and cut by the wide pass; the graph
+    counts every order once."""
+    s = synth.gen_set("sets10", 2, n=n)
+    g = ko.Gpu.from_set(s).configure(lanes=lanes, levels=levels, run_limit=1)
+    b = ko.Batch([g], nbins=0)
+    (r,), _ = b.run()
+    assert b.fallback_items() == math.factorial(n) // math.factorial(levels + 1)
+    st = _oracle_stats(s, 0)
+    assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
+        (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"])

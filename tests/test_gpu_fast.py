@@ -309,3 +309,32 @@ def test_route_by_launches(ko, call, launches):
         else:
             g.eval_orders(orders=rows)
         assert ko.ko_kernel_launches() - before == launches
+
+
+# --------------------------------------- hand-over of spaces with pinned 16 or 32 lanes
+
+@pytest.mark.parametrize("lanes", [16, 32])
+@pytest.mark.parametrize("run_limit", [1, 2])
+@pytest.mark.parametrize("n,levels", [(6, 1), (7, 1), (7, 2), (7, 3), (8, 2), (8, 4), (8, 6)])
+def test_cut_hand_over_loses_no_order(ko, n, levels, run_limit, lanes):
+    """(Nearly) every item fails the first pass and every part of it the wide one,
+    which cuts a list of 42 to 20,160 items as far as it has segments: no more
+    parts than the next list holds, so every order is written and counted."""
+    import torch
+    s = synth.gen_set("sets10", 2, n=n)
+    n_all = math.factorial(n)
+    want = oracle.makespans_idx(s.gpu, s.kernels, first=0, count=n_all)
+    h = oracle.heuristic(s.gpu, s.kernels)
+    st = oracle.exhaustive_stats(s.gpu, s.kernels, oracle.makespan(s.gpu, s.kernels, h), makespans=want)
+    with ko.Gpu.from_set(s) as g:
+        g.configure(lanes=lanes, levels=levels, run_limit=run_limit)
+        out = torch.full((n_all,), -7, dtype=torch.int64, device="cuda")
+        g.eval_all(out)
+        assert g.last_fallback_items() > 0
+        got = out.cpu().numpy()
+        assert (got == -7).sum() == 0
+        assert np.array_equal(got, want)
+        r, hist = g.rank_order(h, nbins=4096)
+    assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
+        (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"])
+    assert np.array_equal(hist, st["hist"])

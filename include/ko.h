@@ -180,16 +180,20 @@ ko_status ko_eval_orders_ps(ko_gpu *g, const int8_t *orders, int64_t n, double *
  * entries) it receives the histogram with
  *     bin = floor((M - min) * nbins / (max - min + 1)).
  * Synchronises `stream`; `out` is host memory.  The handle keeps the N!
- * makespans on the device (8 bytes per order) for the histogram, and 16 bytes
- * per work item for the lists that carry abandoned items between passes. */
+ * makespans on the device (8 bytes per order) for the histogram, besides what
+ * ko_eval_all holds. */
 ko_status ko_rank_order(ko_gpu *g, const int32_t *order, ko_rank *out, uint64_t *hist,
                         int32_t nbins, void *stream);
 
 /* Makespans of all N! orders in Lehmer-index order into makespans_out[N!]
- * (device memory), N <= 12.  Asynchronous on `stream`; the handle holds 40
- * bytes of device memory per work item (N! / (levels + 1)! items; from three
- * levels on, per item and kernel left in it) for the lists that carry
- * abandoned items between passes, and about 20 MB of such lists at least. */
+ * (device memory), N <= 12.  Asynchronous on `stream`; the handle holds 16
+ * bytes of device memory per work item (N! / (levels + 1)! items) for the two
+ * lists that carry abandoned items between passes.  With one thread per item
+ * and m = levels + 1, the lists have 16 bytes more for m + m (m - 1) parts per
+ * thread of a full launch (288 to 448 per SM: 3 MB at one level, 11 at three, 34
+ * at six on 152 SMs) and, from three levels on, for m - 1 parts per item, 2^21
+ * of them at most.  The simple simulator's scratch is 256 MB, the saved node
+ * states of the one-thread pass 36 MB per level. */
 ko_status ko_eval_all(ko_gpu *g, int64_t *makespans_out, void *stream);
 
 /* Tuning knobs of the device simulators (set by the tuner; per handle).

@@ -192,6 +192,22 @@ ko_status fast_launch_timed(ko_gpu *g, const KoWork &w, cudaStream_t st)
     return s;
 }
 
+// Runs `launch` with the choice for the call's size, where the handle's options
+// were left alone, and with those options where the device has no memory for the
+// choice (a 12-kernel space: 0.76 GB, with the options 0.37).
+template <class F>
+ko_status by_size(ko_gpu *g, KoChoice c, cudaStream_t st, F launch)
+{
+    ko_status s;
+    {
+        KoRoute route(&g->fast, c, st);
+        s = launch();
+    }
+    if (s != KO_ERR_NOMEM || g->fast.chosen) return s;
+    ko_fast_release(&g->fast);
+    return launch();
+}
+
 // After a synchronise: read the event time and the abandoned-item count.
 ko_status fast_after_sync(ko_gpu *g)
 {
@@ -388,13 +404,16 @@ ko_status ko_eval_orders(ko_gpu *g, const uint64_t *idx, const int8_t *orders, i
         c.count = n;
         c.d0 = N;
         c.mode = idx ? 1 : 2;
-        KoRoute route(&g->fast, ko_list_choice(g->h, n), st);
-        if ((s = upload_meta(g, st))) return fail(s);
-        KoWork w = work_for(g);
-        w.idx = idx ? (const uint64_t *)d_in : nullptr;
-        w.perms = idx ? nullptr : (const int8_t *)d_in;
-        w.out = d_out;
-        if ((s = fast_launch_timed(g, w, st))) return fail(s);
+        s = by_size(g, ko_list_choice(g->h, n), st, [&]() -> ko_status {
+            ko_status e = upload_meta(g, st);
+            if (e) return e;
+            KoWork w = work_for(g);
+            w.idx = idx ? (const uint64_t *)d_in : nullptr;
+            w.perms = idx ? nullptr : (const int8_t *)d_in;
+            w.out = d_out;
+            return fast_launch_timed(g, w, st);
+        });
+        if (s) return fail(s);
         used_fast = true;
         g->fast_pending = true;
     } else {
@@ -431,16 +450,18 @@ ko_status exhaustive(ko_gpu *g, int64_t *d_out, KoAccum *d_acc, cudaStream_t st)
     ko_status s = check_cuda(ko_launch_accum_reset(d_acc, 1, st));
     if (s) return s;
     if (fast_ok(g)) {
-        KoRoute route(&g->fast, ko_space_choice(g->h), st);
-        KoWork lv;
-        exhaustive_chunk(g, &lv);
-        if ((s = upload_meta(g, st))) return s;
-        KoWork w = work_for(g);
-        w.levels = lv.levels;
-        w.space = true;
-        w.accs = d_acc;
-        w.out = d_out;
-        return fast_launch_timed(g, w, st);
+        return by_size(g, ko_space_choice(g->h), st, [&]() -> ko_status {
+            KoWork lv;
+            exhaustive_chunk(g, &lv);
+            ko_status e = upload_meta(g, st);
+            if (e) return e;
+            KoWork w = work_for(g);
+            w.levels = lv.levels;
+            w.space = true;
+            w.accs = d_acc;
+            w.out = d_out;
+            return fast_launch_timed(g, w, st);
+        });
     }
     if ((s = simple_scratch(g, total))) return s;
     return check_cuda(ko_launch_simple(g->d_set, g->h, nullptr, nullptr, 0, total, d_out, d_acc,
@@ -685,6 +706,16 @@ ko_batch *ko_batch_create(ko_gpu *const *sets, int32_t nsets, int32_t nbins)
     ko_status err = KO_OK;
     ko_batch *b = ko_batch_build(hs.data(), levels.data(), lanes.data(), stack.data(), shape.data(), nsets, nbins,
                                  sets[0]->fast.run_limit, &err);
+    if (!b && err == KO_ERR_NOMEM) {  // the handles' own options need less
+        for (int i = 0; i < nsets; i++) {
+            levels[i] = sets[i]->fast.levels;
+            lanes[i] = sets[i]->fast.lanes;
+            stack[i] = sets[i]->fast.stack_global;
+            shape[i] = sets[i]->fast.lane_shape;
+        }
+        b = ko_batch_build(hs.data(), levels.data(), lanes.data(), stack.data(), shape.data(), nsets, nbins,
+                           sets[0]->fast.run_limit, &err);
+    }
     if (!b) fail(err);
     else ok();
     return b;

@@ -254,11 +254,12 @@ ko_batch *ko_batch_build(const KoSet *const *sets, const int *levels, const int 
         b->fast.lanes = gr.lanes;
         b->fast.stack_global = gr.stack;
         b->fast.lane_shape = gr.shape;
-        if (ko_fast_launch(&b->fast, none, b->slab, b->cap_stream) != KO_OK ||
-            cudaStreamSynchronize(b->cap_stream) != cudaSuccess) {
+        ko_status s = ko_fast_launch(&b->fast, none, b->slab, b->cap_stream);
+        if (!s && cudaStreamSynchronize(b->cap_stream) != cudaSuccess) s = KO_ERR_CUDA;
+        if (s) {
             cudaGetLastError();
             delete b;
-            *err = KO_ERR_CUDA;
+            *err = s == KO_ERR_NOMEM ? s : KO_ERR_CUDA;
             return nullptr;
         }
     }

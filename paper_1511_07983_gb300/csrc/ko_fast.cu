@@ -850,19 +850,27 @@ fast_kernel(KoWork a)
     if (sim.sg.lane == 0) st.flush(a.accs, st_set);
 }
 
-// Lists of abandoned units: one per pass that can abandon any (three one-thread
-// passes, the 16-lane and the wide one).
+// Passes that can abandon units (three one-thread passes, the 16-lane and the wide
+// one).  Each reads the list of the one before it and writes its own, so two lists
+// are enough, taken in turn.
 constexpr int kLists = 5;
 // Saved levels from which the items a one-thread pass abandons are tried once
 // more in parts: an item fails with the first of its nodes that is too large.
 constexpr int kFineLevels = 3;
+
+// Entries of a list beyond the units a first pass numbers: room for the parts of
+// that pass over abandoned items (as many as they can come to, up to these), which
+// cuts as many of them as fit.  11-kernel spaces of which 40 % of the 24-order
+// items are abandoned still cut every one (330 ms as with room for all parts of all
+// items); a 12-kernel space holds 0.36 GB of lists instead of 3.2.
+constexpr unsigned long long kFineRoom = 2ull << 20;
 
 // Device buffer layout inside KoFastState::buf.
 struct FastBuf {
     unsigned long long lost;         // units no list had room for (none); not cleared between launches
     unsigned long long abandoned, counter[kLists + 1], ov_count[kLists], fb_counter;
     unsigned int part_seen[kPartSeen / 32];
-    unsigned long long ov_list[1];   // KoFastState::ov_cap entries per list
+    unsigned long long ov_list[1];   // two lists of KoFastState::ov_cap entries
 };
 
 constexpr size_t kFallbackScratch = size_t(256) << 20;
@@ -1024,19 +1032,21 @@ int ko_fast_launches(int lanes, int shape, bool space, int levels)
 
 ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaStream_t st)
 {
-    // a pass abandons a unit at most once, so lists as long as the units a pass may number lose none
+    // a pass abandons a unit at most once, so lists as long as the units the first pass may number lose
+    // none; the passes over abandoned units number no more than that either
     unsigned long long want = (unsigned long long)(w.n_items > w.reserve_items ? w.n_items : w.reserve_items);
     if (fs->lanes == 1 && w.space) {
         const unsigned long long threads = (unsigned long long)std::max(ko_lane_threads(fs->lane_shape), ko_lane_threads(0));
-        if (w.levels >= kFineLevels) want *= kounits::parts(w.levels + 1, 1);
-        want += threads * kounits::parts(w.levels + 1, 1) + (threads + 1) * kounits::parts(w.levels + 1, 2);
+        const unsigned long long f1 = kounits::parts(w.levels + 1, 1);
+        if (w.levels >= kFineLevels) want += std::min(want * (f1 - 1), kFineRoom);
+        want += threads * f1 + (threads + 1) * kounits::parts(w.levels + 1, 2);
     }
     want = ((want < 1024 ? 1024 : want) + 1023) & ~1023ull;
     if (fs->ov_cap < want) {
         // a stream being captured cannot take a free or a malloc: the caller
         // must size the lists with an uncaptured launch first
         if (capturing(st)) return KO_ERR_STATE;
-        const size_t need = sizeof(FastBuf) + sizeof(unsigned long long) * kLists * (size_t)want;
+        const size_t need = sizeof(FastBuf) + sizeof(unsigned long long) * 2 * (size_t)want;
         cudaFree(fs->buf);
         fs->buf = nullptr;
         fs->cap = 0;
@@ -1104,10 +1114,10 @@ ko_status ko_fast_launch(KoFastState *fs, KoWork w, size_t max_slab_bytes, cudaS
     int list = 0;  // list the next pass writes; it reads the one before
     auto next_pass = [&](KoWork &x) {
         x.counter = &fb->counter[list];
-        x.item_list = list ? fb->ov_list + (list - 1) * fs->ov_cap : nullptr;
+        x.item_list = list ? fb->ov_list + (list - 1) % 2 * fs->ov_cap : nullptr;
         x.item_count = list ? &fb->ov_count[list - 1] : nullptr;
         x.ov_count = &fb->ov_count[list];
-        x.ov_list = fb->ov_list + list * fs->ov_cap;
+        x.ov_list = fb->ov_list + list % 2 * fs->ov_cap;
         list++;
     };
     cudaError_t e = cudaSuccess;
@@ -1223,5 +1233,6 @@ void ko_fast_release(KoFastState *fs)
     fs->buf = nullptr;
     fs->fb_scratch = nullptr;
     fs->cap = 0;
+    fs->ov_cap = 0;
     fs->fb_bytes = 0;
 }

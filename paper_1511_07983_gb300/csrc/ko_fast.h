@@ -54,9 +54,9 @@ struct KoWork {
 
 // Device-side state of the simulators' passes, owned by a handle, batch or model.
 struct KoFastState {
-    void *buf = nullptr;        // counters and the two passes' abandoned-item lists
+    void *buf = nullptr;        // counters and the two lists of abandoned units
     size_t cap = 0;
-    unsigned long long ov_cap = 0;  // entries of each abandoned-item list
+    unsigned long long ov_cap = 0;  // entries of each list
     void *fb_scratch = nullptr; // fallback slabs
     size_t fb_bytes = 0;
     unsigned long long last_overflow = 0;

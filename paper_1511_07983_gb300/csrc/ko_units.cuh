@@ -72,8 +72,9 @@ __host__ __device__ inline Numbering number_space(unsigned long long items, int 
 
 // A pass of `threads` simulations over `items` list entries, every one cut as
 // far as a thread is left for each part; with `fine`, down to walks of at most
-// three kernels (six orders) whatever the threads.  `room`, the entries of the
-// list the pass writes, bounds the units of either: a pass may abandon all it
+// three kernels (six orders) whatever the threads, or as many of them as there
+// is room for by one kernel more than the rest.  `room`, the entries of the
+// list the pass writes, bounds the units of any: a pass may abandon all it
 // numbers (840 two-level items in 2,520 parts against a list of 1,024 lost
 // 2,992 of 5,040 orders).
 __host__ __device__ inline Numbering number_list(unsigned long long items, int levels, unsigned long long threads,
@@ -90,7 +91,13 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
         u.f2 *= (unsigned)(m - u.x2);
         u.x2++;
     }
-    u.units = items * u.f2;
+    if (fine && m - u.x2 > 3 && items) {  // the last items one kernel further
+        u.x1 = u.x2++;
+        u.f1 = u.f2;
+        u.f2 *= (unsigned)(m - u.x1);
+        u.b = items - (room - items * u.f1) / (u.f2 - u.f1);
+    }
+    u.units = u.b * u.f1 + (items - u.b) * u.f2;
     return u;
 }
 

@@ -338,3 +338,45 @@ def test_cut_hand_over_loses_no_order(ko, n, levels, run_limit, lanes):
     assert (r["min"], r["max"], r["n_better"], r["n_equal"], r["n_worse"]) == \
         (st["min"], st["max"], st["n_better"], st["n_equal"], st["n_worse"])
     assert np.array_equal(hist, st["hist"])
+
+
+# ------------------------------------------------------- device memory of a space
+
+def test_lists_of_a_large_space_stay_small(ko):
+    """12 kernels, options left alone (20M items): the lists between the passes,
+    node states and the simple simulator's scratch hold less than 1 GB."""
+    import torch
+    s = synth.gen_set("single12")
+    out = torch.empty(math.factorial(12), dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    with ko.Gpu.from_set(s) as g:
+        g.eval_all(out)
+        torch.cuda.synchronize()
+        held = free - torch.cuda.mem_get_info()[0]
+    assert held < 1 << 30, held
+
+
+def test_space_takes_the_handles_options_where_memory_is_short(ko):
+    """400 MB left on the device: the choice by size (0.45 GB for this space) does
+    not fit, the handle's own options (0.31 GB) do."""
+    import torch
+    s = synth.gen_set("sets10", 4, n=11)
+    n_all = math.factorial(11)
+    want = torch.empty(n_all, dtype=torch.int64, device="cuda")
+    out = torch.full((n_all,), -7, dtype=torch.int64, device="cuda")
+    for cfg in ({}, dict(lanes=16, levels=4)):      # both routes' kernels are loaded now
+        with ko.Gpu.from_set(s) as g:
+            g.configure(**cfg)
+            g.eval_all(want)
+            torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (400 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with ko.Gpu.from_set(s) as g:
+            g.eval_all(out)
+            torch.cuda.synchronize()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert torch.equal(out, want)

@@ -103,7 +103,7 @@ __host__ __device__ inline Numbering number_list(unsigned long long items, int l
 
 // The numbering of a list as single orders, if there are few enough of them (and
 // no more than a list holds): run from the start, a warp per order, they take
-// 25 us a thousand, and none is too large for that pass, where walking them in
+// 10 to 50 us a thousand, and none is too large for that pass, where walking them in
 // 16-lane segments abandons most of what one thread could not hold.
 constexpr unsigned long long kSinglesMax = 2ull << 20;
 __host__ __device__ inline bool number_singles(unsigned long long items, int levels, unsigned long long room,

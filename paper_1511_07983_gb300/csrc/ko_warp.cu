@@ -571,8 +571,12 @@ cudaError_t ko_launch_warp(const KoWork &a, cudaStream_t st)
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // as few warps per block as give every warp one order, up to one per sub-partition
-    const long long work = a.item_list ? (long long)sms * kWarps : a.n_items;
+    // as few warps per block as give every warp one order, up to one per sub-partition.  A list's
+    // length is not known here: its pass gets the warps that are resident at once (96 registers a
+    // thread: 5 blocks per SM; an empty list costs no more than with one).  100,003 orders that the
+    // one-thread pass hands on for their set's limits, us with one block per SM / with five: N=8 on
+    // 13 SMs 3520 / 1048, N=12 on 148 SMs 7280 / 2267; in 16 lanes 2081 and 5889
+    const long long work = a.item_list ? (long long)sms * 5 * kWarps : a.n_items;
     const long long per_sm = (work + sms - 1) / sms;
     const int warps = per_sm < 1 ? 1 : per_sm < kWarps ? (int)per_sm : kWarps;
     long long blocks = (work + warps - 1) / warps;

@@ -223,3 +223,33 @@ def test_cut_items_cover_the_space_once(ko, workload, n, levels, state, run_limi
     assert torch.equal(got, want)
     assert rg == rw and np.array_equal(hg, hw)
     assert moved <= n_all // math.factorial(min(levels, n - 1) + 1) and (run_limit == 32 or moved > 0)
+
+
+def test_orders_handed_on_run_as_wide_as_a_list(ko):
+    """A set outside the packed usage word, one thread per order pinned: every
+    order of a long list is handed on, and the pass that takes them fills the
+    chip (no slower than the same list in 16 lanes)."""
+    import time
+
+    import torch
+    s = synth.gen_set("single8", 7)
+    k = s.kernels.copy()
+    k[:, 0] *= 16
+    s = synth.KernelSet(gpu=(s.gpu[0], 1 << 20) + tuple(s.gpu[2:]), kernels=k)
+    rows = torch.from_numpy(synth.random_orders(3, 8, 100003).astype(np.int8)).cuda()
+    out = {}
+    best = {}
+    for lanes in (1, 16):
+        out[lanes] = torch.full((100003,), -7, dtype=torch.int64, device="cuda")
+        with ko.Gpu.from_set(s) as g:
+            g.configure(lanes=lanes)
+            best[lanes] = 1e9
+            for _ in range(5):
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                g.eval_orders(orders=rows, out=out[lanes])
+                torch.cuda.synchronize()
+                best[lanes] = min(best[lanes], time.perf_counter() - t0)
+            assert g.last_fallback_items() == (100003 if lanes == 1 else 0)
+    assert torch.equal(out[1], out[16])
+    assert best[1] < 1.25 * best[16], best

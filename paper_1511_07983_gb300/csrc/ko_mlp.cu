@@ -298,7 +298,8 @@ __global__ void __launch_bounds__(256) batch_kernel(const int8_t *__restrict__ r
 {
     __shared__ int s_src[kBatchRows], s_set[kBatchRows], s_n[kBatchRows];
     __shared__ int8_t s_kern[kBatchRows][kSlots];
-    __shared__ uint16_t tile[kBatchRows * kBatchPitch];
+    __shared__ __align__(16) uint16_t tile[kBatchRows * kBatchPitch];
+    static_assert(__alignof__(tile) >= sizeof(uint32_t), "read as words below");
     const int r0 = blockIdx.x * kBatchRows;
     pdl_wait();
     if (threadIdx.x < kBatchRows) {
@@ -355,7 +356,8 @@ constexpr int kFeatRows = 64, kFeatPitch = kFeatRows + 2;
 __global__ void __launch_bounds__(256) features_bf16_kernel(const float *__restrict__ x, int B, uint16_t *xb,
                                                             uint16_t *xt)
 {
-    __shared__ uint16_t tile[kMlpIn * kFeatPitch];
+    __shared__ __align__(16) uint16_t tile[kMlpIn * kFeatPitch];
+    static_assert(__alignof__(tile) >= sizeof(uint32_t), "read as words below");
     const long long row0 = (long long)blockIdx.x * kFeatRows;
     constexpr int kQuads = kMlpIn / 4;
     for (int i = threadIdx.x; i < kFeatRows * kQuads; i += blockDim.x) {

@@ -390,17 +390,18 @@ ko_status ko_surrogate_propose(ko_model *m, ko_gpu *g, int64_t n_cand, int32_t t
  * steepest descent from the best order found (KO_MODEL_OPT_POLISH steps at
  * most).  Returns the best exact order found (host, N ids); gpu_ms =
  * device-timeline duration of the whole search including the host's
- * per-round and per-step bookkeeping. */
+ * per-round and per-step bookkeeping.  The model keeps the workspace of its
+ * proposals and searches (about 30 bytes per candidate) for the next one, up
+ * to 256 MB; ko_model_destroy frees it. */
 ko_status ko_surrogate_search(ko_model *m, ko_gpu *g, int64_t n_cand, int32_t top_k, int32_t rounds,
                               int32_t beam, uint64_t seed, int32_t *best_order, int64_t *best_makespan,
                               double *gpu_ms, void *stream);
 
 /* Plain random search, the baseline of the surrogate: n_orders uniform random
  * orders simulated exactly; the best one is returned.  Like the exact
- * rescoring of the surrogate calls and ko_local_search, it picks the threads
- * per simulation by list length and N_SM (32 for more than 32 SMs or up to
- * 4096 orders, 16 up to 32768, one thread per order beyond) instead of the
- * handle's KO_OPT_LANES, which ko_eval_orders and the exhaustive calls use. */
+ * rescoring of the surrogate calls and ko_local_search, it picks a warp or a
+ * thread per order by list length, N and N_SM as ko_eval_orders does where
+ * options were left alone, whatever options the handle has. */
 ko_status ko_random_search(ko_gpu *g, int64_t n_orders, uint64_t seed, int32_t *best_order,
                            int64_t *best_makespan, double *gpu_ms, void *stream);
 

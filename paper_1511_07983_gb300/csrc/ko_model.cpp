@@ -473,6 +473,25 @@ struct ArenaUse {
     }
 };
 
+// Device workspace of a descent over the neighbours of one order.
+struct DescentWork {
+    KoDescent *state = nullptr;
+    int8_t *rows = nullptr;
+    int64_t *ms = nullptr;
+    KoChunk *chunk = nullptr;
+    void carve(Carve &c, int n)
+    {
+        const size_t per = (size_t)(n * (n - 1) / 2 + n * (n - 1));
+        state = c.take<KoDescent>(1);
+        rows = c.take<int8_t>((per + 1) * kMaxK);
+        ms = c.take<int64_t>(per + 1);
+        chunk = c.take<KoChunk>(1);
+    }
+};
+static ko_status descend(KoFastState *fs, const KoSet &h, const int32_t *start, bool moves, int max_iters,
+                         int32_t *order_out, int64_t *makespan_out, int32_t *steps_out, int64_t *evals_out,
+                         double *gpu_ms, cudaStream_t st, const DescentWork &work);
+
 // Device copies of the sets and what the encoder reads of them, in one block.
 struct SetTables {
     void *mem = nullptr;
@@ -785,6 +804,7 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
     uint32_t *sel_state;
     unsigned int *sel_hist, *sel_cnt;
     KoChunk *d_chunk;
+    DescentWork polish;  // its own: the descent leaves the search's buffers alone
     auto carve = [&](Carve &c) {
         rows = c.take<int8_t>((size_t)padded * kMaxK);
         y_all = c.take<float>((size_t)std::max<long long>(n_cand, nb_pad));
@@ -797,6 +817,7 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
         sel_hist = c.take<unsigned int>(256);
         sel_cnt = c.take<unsigned int>(2);
         d_chunk = c.take<KoChunk>(1);
+        polish.carve(c, n);
     };
     Carve need(nullptr);
     carve(need);
@@ -884,8 +905,8 @@ ko_status ko_model_search_set(ko_model *md, const KoSet &h, long long n_cand, in
             int64_t pms = -1, evals = 0;
             int32_t steps = 0;
             double lms = 0.0;
-            if (!s) s = ko_local_search_set(&md->fast, h, start.data(), true, md->polish, out.data(), &pms, &steps,
-                                            &evals, &lms, st);
+            if (!s) s = descend(&md->fast, h, start.data(), true, md->polish, out.data(), &pms, &steps, &evals, &lms,
+                                st, polish);
             if (!s && pms >= 0 && pms < pool[0].ms) {
                 pool[0].ms = pms;
                 for (int i = 0; i < n; i++) pool[0].row[i] = (int8_t)out[i];
@@ -961,6 +982,22 @@ ko_status ko_local_search_set(KoFastState *fs, const KoSet &h, const int32_t *st
                               int32_t *order_out, int64_t *makespan_out, int32_t *steps_out, int64_t *evals_out,
                               double *gpu_ms, cudaStream_t st)
 {
+    if (h.n < 1) return KO_ERR_ARG;
+    DescentWork work;
+    Carve need(nullptr);
+    work.carve(need, h.n);
+    ArenaUse use{fs, st};
+    const ko_status s = ensure_arena(fs, need.size);
+    if (s) return s;
+    Carve mem(fs->arena);
+    work.carve(mem, h.n);
+    return descend(fs, h, start, moves, max_iters, order_out, makespan_out, steps_out, evals_out, gpu_ms, st, work);
+}
+
+static ko_status descend(KoFastState *fs, const KoSet &h, const int32_t *start, bool moves, int max_iters,
+                         int32_t *order_out, int64_t *makespan_out, int32_t *steps_out, int64_t *evals_out,
+                         double *gpu_ms, cudaStream_t st, const DescentWork &work)
+{
     constexpr int kAhead = 3;
     const int n = h.n;
     if (n < 1 || max_iters < 0 || max_iters > (1 << 20)) return KO_ERR_ARG;
@@ -982,22 +1019,10 @@ ko_status ko_local_search_set(KoFastState *fs, const KoSet &h, const int32_t *st
     if (s) return s;
     const int swaps = n * (n - 1) / 2, per = swaps + n * (n - 1);
     const int nq = max_iters > 0 ? (moves ? per : swaps) : 0;
-    Carve need(nullptr);
-    auto carve = [&](Carve &c, KoDescent **state, int8_t **rows, int64_t **ms, KoChunk **chunk) {
-        *state = c.take<KoDescent>(1);
-        *rows = c.take<int8_t>((size_t)(per + 1) * kMaxK);  // the neighbours kernel writes all of them
-        *ms = c.take<int64_t>((size_t)nq + 1);
-        *chunk = c.take<KoChunk>(1);
-    };
-    KoDescent *state;
-    int8_t *rows;
-    int64_t *ms;
-    KoChunk *d_chunk;
-    carve(need, &state, &rows, &ms, &d_chunk);
-    ArenaUse use{fs, st};
-    if ((s = ensure_arena(fs, need.size))) return s;
-    Carve mem(fs->arena);
-    carve(mem, &state, &rows, &ms, &d_chunk);
+    KoDescent *const state = work.state;
+    int8_t *const rows = work.rows;
+    int64_t *const ms = work.ms;
+    KoChunk *const d_chunk = work.chunk;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if ((s = make_events(&e0, &e1))) return s;
     cudaEventRecord(e0, st);

@@ -380,3 +380,22 @@ def test_space_takes_the_handles_options_where_memory_is_short(ko):
         del hold
         torch.cuda.empty_cache()
     assert torch.equal(out, want)
+
+
+# ----------------------------------- a warp per order: run pointers, capacities, limits
+
+@pytest.mark.parametrize("n_sm", [1, 2, 31, 148, 1023, 1024])
+@pytest.mark.parametrize("caps", [(32768, 32768), (3000, 7001), (32768, 5000)])
+@pytest.mark.parametrize("n", [2, 11, 24])
+def test_warp_per_order_edges(ko, n_sm, caps, n):
+    """Up to 1,024 SMs (the pointer's field in a warp's keys), capacities that are
+    no power of two, kernels alike enough that several runs end together."""
+    s = synth.random_set(900 + n, n, gpu=(n_sm, 65536, 98304, 64, 16), blk=(1, 3 * n_sm + 5), c=(500, 520),
+                         c_cap=caps[0], m_cap=caps[1])
+    k = s.kernels.copy()
+    k[::2, 4:6] = k[0, 4:6]
+    s = synth.KernelSet(gpu=s.gpu, kernels=k)
+    rows = synth.random_orders(n, n, 40)
+    with ko.Gpu.from_set(s) as g:
+        got = g.eval_orders(orders=rows.astype(np.int8))
+    assert np.array_equal(got, oracle.makespans_orders(s.gpu, s.kernels, rows.astype(np.int32)))

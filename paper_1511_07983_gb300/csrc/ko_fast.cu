@@ -860,8 +860,8 @@ constexpr int kFineLevels = 3;
 
 // Entries of a list beyond the units a first pass numbers: room for the parts of
 // that pass over abandoned items (as many as they can come to, up to these), which
-// cuts as many of them as fit.  11-kernel spaces of which 40 % of the 24-order
-// items are abandoned still cut every one (330 ms as with room for all parts of all
+// cuts as many of them as fit.  An 11-kernel space of which 30 % of the 24-order
+// items are abandoned still cuts every one (330 ms as with room for all parts of all
 // items); a 12-kernel space holds 0.36 GB of lists instead of 3.2.
 constexpr unsigned long long kFineRoom = 2ull << 20;
 

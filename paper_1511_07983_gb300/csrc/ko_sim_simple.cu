@@ -406,9 +406,9 @@ constexpr int kHistPerThread = 4;   // makespans per thread of a full grid's fir
 
 // Histogram of stored makespans and, with `counts`, how many are below, equal to
 // and above the one at `ref_at` (also written to counts->min).  One read of the
-// makespans, so the ranked order needs no simulation of its own: that pass cost a
-// single simulation's latency and three empty hand-over passes (a 40,320-order ranking
-// 505 -> 430 us at the same set).
+// makespans, so the ranked order needs no simulation of its own: a pass for it, as
+// there was, cost a single simulation's latency and the empty passes behind it (a
+// 40,320-order ranking 505 -> 430 us at the same set).
 __global__ void __launch_bounds__(kHistThreads)
 hist_kernel(const int64_t *__restrict__ ms, long long count, const KoAccum *acc,
             unsigned long long *hist, int nbins, long long ref_at, KoAccum *counts)

@@ -9,22 +9,23 @@
 //     registers and its groups (end, descriptor) in its own column of shared
 //     memory, free of bank conflicts; an event reads the column once, in one
 //     burst of independent loads, for what ends and for the next end;
-//   * between a kernel's first and last burst an event changes only the lanes
-//     whose groups end, and those take their full capacity, so the event is
-//     three warp reductions (next end, blocks taken, pointer) and one lane's
-//     work; the joint water-fill runs once per kernel, for the burst that
-//     empties the queue.
+//   * between a kernel's first and last burst an event changes only the run
+//     whose groups end, and that one takes its full capacity, so every lane has
+//     its next event worked out ahead (release, room, the new group's duration)
+//     and a turn takes the events of all lanes that come before the earliest
+//     one not worked out yet: four warp reductions, three more where several
+//     runs end together and decide the pointer.  The joint water-fill runs once
+//     per kernel, for the burst that empties the queue.
 //   * the slot and descriptor of a lane's next group to end are at hand, so its
-//     release does not wait for a look through the column; its room and the
-//     duration of what it takes come before the reductions that decide whether
-//     the queue runs empty.
+//     release does not wait for a look through the column.
 // It is bound by instruction latency (570 orders of N=20 on 13 SMs, one warp per
-// SM sub-partition: 229 warp instructions per event at 4.2 cycles each, half of
-// that waits for the previous instruction).  The run-length kernel took 3,200
-// cycles per event here (its groups in registers behind select chains, two
-// reductions more per event, lanes shifted by every split).  570 orders, us
-// before -> after: N=8 on 13 SMs 124 -> 60, N=20 on 13 SMs 608 -> 268, N=20 on
-// 148 SMs 573 -> 283.
+// SM sub-partition: 145 warp instructions per event at 4.2 cycles each, half of
+// that waits for the previous instruction; 229 while a turn took one event
+// time).  The run-length kernel took 3,200 cycles per event here (its groups in
+// registers behind select chains, more reductions per event, lanes shifted by
+// every split).  570 orders, us before -> with one event time a turn -> now:
+// N=8 on 13 SMs 124 -> 60 -> 55, N=20 on 13 SMs 608 -> 268 -> 185, N=20 on 148
+// SMs 573 -> 283 -> 146.
 #include "ko_fast.h"
 #include "ko_units.cuh"
 
